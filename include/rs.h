@@ -77,9 +77,9 @@ RS_API rs_status rs_async_status(rs_ctx* ctx, void* stream);
  * Whether a given shape runs on them is answered by the two queries below. */
 RS_API int rs_uses_tensor_cores(const rs_ctx* ctx, rs_dtype dtype);
 /* Which kernels a call would run, by shape (Eq. att / Eq. MLP contractions and Eq. sa): 1 = the
- * tcgen05 kernels, 0 = the fp32-FMA kernels.  The tensor-core GEMM needs RS_BF16, N % 128 == 0 and
+ * tcgen05 kernels, 0 = the fp32-FMA kernels.  The tensor-core GEMM needs RS_BF16, N a multiple of 128 or 192 and
  * K % 64 == 0; a block runs on the tensor cores only if all four of its projections qualify
- * (D % 128 == 0, D_mlp % 128 == 0).  Every other valid shape still computes the same result on
+ * (D and D_mlp multiples of 128 or of 192).  Every other valid shape still computes the same result on
  * the fp32-FMA kernels, far slower.  With RS_REQUIRE_TC=1 in the environment at rs_create such a
  * call returns RS_ERR_UNSUPPORTED instead of taking the slow kernels. */
 RS_API int rs_linear_uses_tensor_cores(const rs_ctx* ctx, rs_dtype dtype, long long M, int N, int K);
@@ -111,8 +111,8 @@ RS_API rs_status rs_attn_fwd(rs_ctx* ctx, const rs_attn_desc* desc /*host*/, con
  *   RS_LIN_BIAS           out in `dtype`
  *   RS_LIN_BIAS_GELU      exact-erf GELU, out in `dtype`
  *   RS_LIN_BIAS_RESIDUAL  + residual[M, N] (of `dtype`), out in fp32 (the residual stream x')
- * A, W, residual, out (dev); bias (dev, fp32, may be NULL).  With RS_BF16 and N % 128 == 0,
- * K % 64 == 0 the tensor-core kernel runs, otherwise the fp32-FMA kernel. */
+ * A, W, residual, out (dev); bias (dev, fp32, may be NULL).  With RS_BF16, N a multiple of 128 or 192
+ * and K of 64 the tensor-core kernel runs, otherwise the fp32-FMA kernel. */
 typedef enum { RS_LIN_BIAS = 0, RS_LIN_BIAS_GELU = 1, RS_LIN_BIAS_RESIDUAL = 2 } rs_linear_epilogue;
 RS_API rs_status rs_linear_fwd(rs_ctx* ctx, rs_dtype dtype, rs_linear_epilogue epilogue, long long M, int N,
                                int K, const void* A, const void* W, const float* bias, const void* residual,
@@ -190,7 +190,7 @@ typedef struct {           /* all dev pointers */
  * into caller buffers; put them in rs_block_weights and the layer loop uses the folded form for every
  * block but the first: the sums come from the previous block's FC2 epilogue when that block drops no
  * token, else from the kernel that moves the kept rows (which then copies them instead of normalising
- * them, into a dense buffer).  RS_BF16 only; D a multiple of 128.  Results differ from
+ * them, into a dense buffer).  RS_BF16 only; D a multiple of 128 or 192.  Results differ from
  * the unfolded loop by rounding (W g is rounded once more, LN(x) is not rounded to bf16). */
 RS_API rs_status rs_prepare_ln1_fold(rs_ctx* ctx, rs_dtype dtype, int D, const void* w_qkv, const float* b_qkv,
                                      const float* ln1_g, const float* ln1_b, void* w_out, float* c_out,
@@ -270,7 +270,7 @@ RS_API rs_status rs_vit_fwd(rs_ctx* ctx, const rs_vit_desc* desc /*host*/,
  * x_full) are unspecified but finite there.  seq_lens, drops, lens_out (dev): [B] int32.  Values are
  * read on the device and clamped there: seq_lens to [1, N], drops to [0, seq_lens[b] - 1], and the
  * kept count seq_lens[b] - drops[b] to at most the row stride of the outputs.  Tensor-core path only
- * (RS_BF16, head_dim 64; for the block D and D_mlp multiples of 128) and N <= 4608:
+ * (RS_BF16, head_dim 64; for the block D and D_mlp multiples of 128 or 192) and N <= 4608:
  * RS_ERR_UNSUPPORTED otherwise, before any launch.
  *
  * rs_attn_fwd_ragged: rs_attn_fwd where sample b attends over its first seq_lens[b] tokens (Eq. sa

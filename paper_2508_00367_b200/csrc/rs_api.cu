@@ -255,7 +255,7 @@ rs_status rs_linear_fwd(rs_ctx* ctx, rs_dtype dtype, rs_linear_epilogue epi, lon
     cudaStream_t st = (cudaStream_t)stream;
     const rs_dtype out_dtype = epi == RS_LIN_BIAS_RESIDUAL ? RS_F32 : dtype;
     if (ctx->require_tc && dtype == RS_BF16 && !rs_linear_uses_tensor_cores(ctx, dtype, M, N, K))
-        return fail(ctx, RS_ERR_UNSUPPORTED, "rs_linear_fwd: shape outside the tensor-core kernel (N %% 128, K %% 64) and RS_REQUIRE_TC is set");
+        return fail(ctx, RS_ERR_UNSUPPORTED, "rs_linear_fwd: shape outside the tensor-core kernel (N a multiple of 128 or 192, K of 64) and RS_REQUIRE_TC is set");
     if (ctx->use_tc && dtype == RS_BF16 && rs::gemm_tc_supported(M, N, K)) {
         const int e = epi == RS_LIN_BIAS ? rs::RS_EPI_BIAS : epi == RS_LIN_BIAS_GELU ? rs::RS_EPI_BIAS_GELU : rs::RS_EPI_RESID;
         RS_CHECK_LAUNCH(ctx, RS_K_GEMM, st, rs::launch_gemm_tc(ctx, e, A, W, bias, residual, nullptr, nullptr, out, out_dtype, nullptr, 0, 0, M, N, K, st), "tensor-core GEMM");
@@ -430,10 +430,10 @@ static rs_status block_fwd_impl(rs_ctx* ctx, const rs_block_desc* d, const rs_bl
 
     const bool tc = rs_block_uses_tensor_cores(ctx, d) != 0;
     if (ctx->require_tc && d->dtype == RS_BF16 && !tc)
-        return fail(ctx, RS_ERR_UNSUPPORTED, "rs_block_fwd: shape outside the tensor-core kernels (D, D_mlp multiples of 128) and RS_REQUIRE_TC is set");
+        return fail(ctx, RS_ERR_UNSUPPORTED, "rs_block_fwd: shape outside the tensor-core kernels (D, D_mlp multiples of 128 or 192) and RS_REQUIRE_TC is set");
     const int32_t* in_map = hk ? hk->in_map : nullptr;
     if (in_map && !tc) return fail(ctx, RS_ERR_UNSUPPORTED, "rs_block_fwd: a row-mapped input needs the tensor-core kernels");
-    if (ragged && (!tc || d->N > 4608)) return fail(ctx, RS_ERR_UNSUPPORTED, "rs_block_fwd_ragged: needs the tensor-core kernels (bf16, D and D_mlp multiples of 128) and N <= 4608");
+    if (ragged && (!tc || d->N > 4608)) return fail(ctx, RS_ERR_UNSUPPORTED, "rs_block_fwd_ragged: needs the tensor-core kernels (bf16, D and D_mlp multiples of 128 or 192) and N <= 4608");
     const size_t sz = rs::dtype_size(d->dtype);
     rs_attn_desc ad;
     ad.dtype = d->dtype; ad.B = d->B; ad.N = d->N; ad.H = d->H; ad.head_dim = 64; ad.scale = d->scale;
@@ -695,7 +695,7 @@ rs_status rs_prepare_ln1_fold(rs_ctx* ctx, rs_dtype dtype, int D, const void* w_
                               void* stream) {
     if (!ctx) return RS_ERR_INVALID_ARG;
     if (!w_qkv || !ln1_g || !ln1_b || !w_out || !c_out || !b_out) return fail(ctx, RS_ERR_INVALID_ARG, "rs_prepare_ln1_fold: null argument");
-    if (dtype != RS_BF16 || D < 128 || (D % 128)) return fail(ctx, RS_ERR_UNSUPPORTED, "rs_prepare_ln1_fold: bf16 and D a multiple of 128 only");
+    if (dtype != RS_BF16 || D < 128 || ((D % 128) && (D % 192))) return fail(ctx, RS_ERR_UNSUPPORTED, "rs_prepare_ln1_fold: bf16 and D a multiple of 128 or 192 only");
     if (!aligned16(w_qkv) || !aligned16(w_out)) return fail(ctx, RS_ERR_INVALID_ARG, "rs_prepare_ln1_fold: misaligned pointer");
     cudaError_t e = rs::launch_ln_fold_prep(w_qkv, b_qkv, ln1_g, ln1_b, 3 * D, D, w_out, c_out, b_out, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "rs_prepare_ln1_fold");
