@@ -53,7 +53,7 @@ bool valid_dtype(int t) { return t == RS_F32 || t == RS_BF16; }
 
 // Scratch layout of one block.  Every buffer starts on a 256-byte boundary.
 struct BlockWs {
-    size_t u, qkv, o, x_prime, h, m, x_hat, scores, keep, flags, total;
+    size_t u, qkv, o, x_prime, h, m, x_hat, scores, keep, total;
 };
 
 bool block_layout(const rs_block_desc& d, BlockWs* ws) {
@@ -72,7 +72,6 @@ bool block_layout(const rs_block_desc& d, BlockWs* ws) {
     ws->x_hat = take(T * D * osz);       // un-pruned block output when the caller gives no x_full
     ws->scores = take(T * 4);            // when the caller gives no scores buffer
     ws->keep = take((size_t)d.B * (size_t)(d.N) * 4);
-    ws->flags = take(T + 4 * (T / 64 + 2 * (size_t)d.B) + 16);   // slice counts and keep flags between the ranking kernel and the mover
     ws->total = off;
     return true;
 }
@@ -101,13 +100,11 @@ rs_status rs_create(rs_ctx** out, int device) {
         return RS_ERR_UNSUPPORTED;
     }
     ctx->sm_count = prop.multiProcessorCount;
-    if (cudaMalloc(&ctx->d_status, 256 + kFlagScratch) != cudaSuccess || cudaMemset(ctx->d_status, 0, 256) != cudaSuccess ||
-        rs::select_init() != cudaSuccess) {
+    if (cudaMalloc(&ctx->d_status, 256) != cudaSuccess || cudaMemset(ctx->d_status, 0, 256) != cudaSuccess) {
         if (ctx->d_status) cudaFree(ctx->d_status);
         free(ctx);
         return RS_ERR_CUDA;
     }
-    ctx->d_flags = (unsigned char*)ctx->d_status + 256;
     // RS_DISABLE_TC=1 routes bf16 through the fp32-FMA kernels (cross-check of the tcgen05 path).
     const char* no_tc = getenv("RS_DISABLE_TC");
     ctx->encode_tiled = rs::tc_get_encode_fn();
@@ -301,14 +298,7 @@ rs_status rs_topk_compact(rs_ctx* ctx, rs_dtype dtype, int B, int N, int D, int 
         const size_t xbytes = (size_t)B * N * D * sz, obytes = (size_t)B * K * D * sz;
         if (xa < xo + obytes && xo < xa + xbytes) return fail(ctx, RS_ERR_INVALID_ARG, "rs_topk_compact: x_out overlaps x");
     }
-    int nl = 1;
-    if (x && rs::prune_fusable(N, K, kFlagScratch)) {
-        RS_CHECK_LAUNCH(ctx, RS_K_GATHER, st, rs::launch_prune(scores, 0, nullptr, B, N, K, has_cls ? 1 : 0, keep_idx, nullptr, dtype, x, D, x_out, nullptr, ctx->d_flags, kFlagScratch, ctx->sm_count, st, &nl, nullptr, nullptr, nullptr), "select+gather launch");
-        ctx->launches += nl - 1;
-        return RS_OK;
-    }
-    RS_CHECK_LAUNCH(ctx, RS_K_SELECT, st, rs::launch_select(scores, 0, nullptr, B, N, K, has_cls ? 1 : 0, keep_idx, nullptr, ctx->d_flags, kFlagScratch, ctx->sm_count, st, &nl), "select launch");
-    ctx->launches += nl - 1;
+    RS_CHECK_LAUNCH(ctx, RS_K_SELECT, st, rs::launch_select(scores, 0, nullptr, B, N, K, has_cls ? 1 : 0, keep_idx, nullptr, st), "select launch");
     if (x) RS_CHECK_LAUNCH(ctx, RS_K_GATHER, st, rs::launch_gather(dtype, x, keep_idx, B, N, K, D, x_out, nullptr, st), "gather launch");
     return RS_OK;
 }
@@ -505,26 +495,15 @@ static rs_status block_fwd_impl(rs_ctx* ctx, const rs_block_desc* d, const rs_bl
     int32_t* out_map = (hk && moves) ? hk->out_map : nullptr;
     void* dense = dense_out ? x_out : nullptr;
     const int cls = d->has_cls ? 1 : 0;
-    uint8_t* flags = (uint8_t*)(base + ws.flags);
     if (ragged) {
         // per-sample counts: sample b keeps lens[b] - drops[b] of its first lens[b] tokens; K is the row stride
-        int nlr = 0;
-        const size_t fb = (size_t)T + 4 * ((size_t)T / 64 + 2 * (size_t)d->B) + 16;
-        RS_CHECK_LAUNCH(ctx, RS_K_GATHER, st, rs::launch_prune(sel_in, sel_enc, sel_out, d->B, d->N, K, cls, keep, nullptr, d->out_dtype, x_hat, D, x_out, nullptr, flags, fb, ctx->sm_count, st, &nlr, hk->seq_lens, hk->drops, hk->lens_out), "select+gather (per-sample counts)");
-        ctx->launches += nlr - 1;
-        return RS_OK;
-    }
-    const size_t flags_bytes = (size_t)T + 4 * ((size_t)T / 64 + 2 * (size_t)d->B) + 16;
-    int nl = 1;
-    if (moves && rs::prune_fusable(d->N, K, flags_bytes) && (dense || ln)) {
-        RS_CHECK_LAUNCH(ctx, RS_K_GATHER, st, rs::launch_prune(sel_in, sel_enc, sel_out, d->B, d->N, K, cls, keep, out_map, d->out_dtype, x_hat, D, dense, ln, flags, flags_bytes, ctx->sm_count, st, &nl, nullptr, nullptr, nullptr), "select+gather");
-        ctx->launches += nl - 1;
+        RS_CHECK_LAUNCH(ctx, RS_K_SELECT, st, rs::launch_select(sel_in, sel_enc, sel_out, d->B, d->N, K, cls, keep, nullptr, st, hk->seq_lens, hk->drops, hk->lens_out), "select (per-sample counts)");
+        RS_CHECK_LAUNCH(ctx, RS_K_GATHER, st, rs::launch_gather(d->out_dtype, x_hat, keep, d->B, d->N, K, D, x_out, nullptr, st), "gather (per-sample counts)");
         return RS_OK;
     }
     // nothing dropped and neither the scores nor the (identity) index list asked for: nothing left to do
     if (!moves && hk && !scores && !keep_idx) return RS_OK;
-    RS_CHECK_LAUNCH(ctx, RS_K_SELECT, st, rs::launch_select(sel_in, sel_enc, sel_out, d->B, d->N, K, cls, keep, out_map, flags, flags_bytes, ctx->sm_count, st, &nl), "select");
-    ctx->launches += nl - 1;
+    RS_CHECK_LAUNCH(ctx, RS_K_SELECT, st, rs::launch_select(sel_in, sel_enc, sel_out, d->B, d->N, K, cls, keep, out_map, st), "select");
     if (moves && (dense || ln))
         RS_CHECK_LAUNCH(ctx, RS_K_GATHER, st, rs::launch_gather(d->out_dtype, x_hat, keep, d->B, d->N, K, D, dense, ln, st), "gather");
     return RS_OK;
@@ -580,10 +559,9 @@ rs_status rs_topk_compact_ragged(rs_ctx* ctx, rs_dtype dtype, int B, int N, int 
         const size_t xbytes = (size_t)B * N * D * sz, obytes = (size_t)B * K_pad * D * sz;
         if (xa < xo + obytes && xo < xa + xbytes) return fail(ctx, RS_ERR_INVALID_ARG, "rs_topk_compact_ragged: x_out overlaps x");
     }
-    int nl = 1;
     cudaStream_t st = (cudaStream_t)stream;
-    RS_CHECK_LAUNCH(ctx, RS_K_GATHER, st, rs::launch_prune(scores, 0, nullptr, B, N, K_pad, has_cls ? 1 : 0, keep_idx, nullptr, dtype, x, D, x_out, nullptr, ctx->d_flags, kFlagScratch, ctx->sm_count, st, &nl, seq_lens, drops, lens_out), "select+gather launch (per-sample counts)");
-    ctx->launches += nl - 1;
+    RS_CHECK_LAUNCH(ctx, RS_K_SELECT, st, rs::launch_select(scores, 0, nullptr, B, N, K_pad, has_cls ? 1 : 0, keep_idx, nullptr, st, seq_lens, drops, lens_out), "select launch (per-sample counts)");
+    if (x) RS_CHECK_LAUNCH(ctx, RS_K_GATHER, st, rs::launch_gather(dtype, x, keep_idx, B, N, K_pad, D, x_out, nullptr, st), "gather launch (per-sample counts)");
     return RS_OK;
 }
 

@@ -32,7 +32,6 @@ struct rs_ctx {
     int use_tc;            // tcgen05 kernels enabled for bf16
     int require_tc;        // RS_REQUIRE_TC=1: a bf16 shape the tensor-core kernels cannot take is an error
     int* d_status;         // device status word (0 = ok), first bytes of a small allocation made by rs_create
-    unsigned char* d_flags; // keep-flag scratch of rs_topk_compact (kFlagScratch bytes, same allocation)
     int log, nvtx;          // RS_LOG=1: a line per launch on stderr; RS_NVTX=1: an NVTX range around each launch call
     int attn_kernel;        // RS_ATTN_KERNEL: 0 the faster attention kernel per shape (cost model), 2 / 3 always that one
     long long launches;    // kernels launched through this context
@@ -47,7 +46,6 @@ struct rs_ctx {
 };
 
 enum { kMaxTimed = 8192 };
-enum { kFlagScratch = 1 << 20 };
 
 // Device status word values.
 enum { RS_DEV_OK = 0, RS_DEV_TIMEOUT = 1, RS_DEV_SMEM_ALIGN = 2 };
@@ -98,39 +96,27 @@ cudaError_t launch_residual_score(const float* m, const float* x_prime, const vo
 // from which the score is finished here (and written to scores_out when non-null).
 // row_map (optional, [B, K] int32): flat source row b * N + keep_idx[b, j] of every kept token, with
 // which the next block reads the un-pruned rows in place.
-// flags / flags_bytes: 4-byte aligned scratch between the flag kernel and the row kernel (a byte
-// per token and a count per 64 or 128 tokens; with less than the whole batch needs, the batch is
-// processed in several passes, with less than one sample needs the radix kernel runs instead).
-// *launches (optional) receives the number of kernels launched.
-cudaError_t launch_select(const float* scores, int nparts, float* scores_out, int B, int N, int K,
-                          int has_cls, int32_t* keep_idx, int32_t* row_map, uint8_t* flags, size_t flags_bytes,
-                          int sm_count, cudaStream_t st, int* launches);
+// seq_lens, drops (optional, dev [B]): per-sample token counts (rs_topk_compact_ragged); index -1 past a sample's
+// count; lens_out (optional, dev [B]) receives the kept counts.
+cudaError_t launch_select(const float* scores, int nparts, float* scores_out, int B, int N, int K, int has_cls,
+                          int32_t* keep_idx, int32_t* row_map, cudaStream_t st, const int32_t* seq_lens = nullptr,
+                          const int32_t* drops = nullptr, int32_t* lens_out = nullptr);
 // The compaction kernels can also write LN(x_out) for the block that follows (its LN1 of Eq. att):
 // the warp that copies a kept row has it in registers.  out: [B, K, D] of the rows' dtype.
 // gamma == null with stats set: no LayerNorm; the kept rows are copied and the sum and sum of squares of each
 // copied row's bf16 values go to stats[2 * row], stats[2 * row + 1] (for a LayerNorm folded into the next product).
 struct LnFuse { const float* gamma; const float* beta; float eps; void* out; float* stats; };
 bool ln_fusable(rs_dtype dtype, int D);   // the row fits the registers of one warp
-// x_out may be null when ln is given: only the normalised rows are written (no dense copy).
+// x_out may be null when ln is given: only the normalised rows are written (no dense copy).  Rows with index -1
+// become zeros.
 cudaError_t launch_gather(rs_dtype dtype, const void* x, const int32_t* keep_idx, int B, int N, int K,
                           int D, void* x_out, const LnFuse* ln /*null: none*/, cudaStream_t st);
-// Selection, index lists and the rows' move (N <= 4608 and something is dropped): a kernel that finds
-// the cut of every sample and flags its kept tokens (a CTA per sample), then a warp per kept row.
-// x null: indices only.  x given: x_out (dense copy) and / or ln (normalised rows) must be given.
-bool prune_fusable(int N, int K, size_t flags_bytes);
-cudaError_t launch_prune(const float* scores, int nparts, float* scores_out, int B, int N, int K, int has_cls,
-                         int32_t* keep_idx, int32_t* row_map, rs_dtype dtype, const void* x, int D, void* x_out,
-                         const LnFuse* ln /*null: none*/, uint8_t* flags, size_t flags_bytes, int sm_count,
-                         cudaStream_t st, int* launches, const int32_t* seq_lens /*dev [B] or null*/,
-                         const int32_t* drops /*dev [B], with seq_lens*/, int32_t* lens_out /*dev [B] or null*/);
 // Line-wise pruning of a 2-D token grid: keep_rows [B, Hk], keep_cols [B, Wk] and, when x is given,
 // x_out[b, i, j, :] = x[b, keep_rows[b, i], keep_cols[b, j], :].  H, W <= linewise_max_lines().
 int linewise_max_lines();
 cudaError_t launch_linewise(const float* scores, int B, int H, int W, int Hk, int Wk, int32_t* keep_rows,
                             int32_t* keep_cols, rs_dtype dtype, const void* x, int D, void* x_out, int sm_count,
                             cudaStream_t st);
-size_t select_smem_bytes(int N);
-cudaError_t select_init();   // opt in to large dynamic shared memory, once per device (the current one)
 
 // ---- SIMT contraction path (rs_simt.cu): fp32 FMA, used for RS_F32 and as a cross-check ----
 // out[M, N] = act(A[M, K] * W[N, K]^T + bias) + residual.

@@ -31,8 +31,7 @@ void say(char* err, size_t err_len, const char* msg) {
     if (err && err_len) snprintf(err, err_len, "%s", msg);
 }
 
-// First call on a device: resolve the array's device address and opt the selection
-// kernel in to its shared-memory size.  Neither call allocates.
+// First call on a device: resolve the array's device address (which allocates nothing).
 rs_status setup_device(int dev, void** scratch, int** status, void** encode, char* err, size_t err_len) {
     std::lock_guard<std::mutex> lock(g_mu);
     if (!g_encode_done) {
@@ -49,11 +48,6 @@ rs_status setup_device(int dev, void** scratch, int** status, void** encode, cha
             return RS_ERR_CUDA;
         }
         g_status[dev] = (int*)ps;
-        e = rs::select_init();
-        if (e != cudaSuccess) {
-            say(err, err_len, cudaGetErrorString(e));
-            return RS_ERR_CUDA;
-        }
         g_scratch[dev] = p;
         g_ready[dev] = true;
     }
