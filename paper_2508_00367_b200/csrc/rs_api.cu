@@ -334,8 +334,8 @@ rs_status rs_linewise_compact(rs_ctx* ctx, rs_dtype dtype, int B, int H, int W, 
         if (xa < xo + obytes && xo < xa + xbytes) return fail(ctx, RS_ERR_INVALID_ARG, "rs_linewise_compact: x_out overlaps x");
     }
     cudaStream_t st = (cudaStream_t)stream;
-    RS_CHECK_LAUNCH(ctx, RS_K_GATHER, st, rs::launch_linewise(scores, B, H, W, Hk, Wk, keep_rows, keep_cols, dtype, x, D, x_out, ctx->sm_count, st),
-                    "line-wise select+gather launch");
+    RS_CHECK_LAUNCH(ctx, RS_K_SELECT, st, rs::launch_line_select(scores, B, H, W, Hk, Wk, keep_rows, keep_cols, st), "line selection launch");
+    if (x) RS_CHECK_LAUNCH(ctx, RS_K_GATHER, st, rs::launch_line_gather(dtype, x, keep_rows, keep_cols, B, H, W, Hk, Wk, D, x_out, st), "line gather launch");
     return RS_OK;
 }
 

@@ -39,60 +39,110 @@ layernorm_kernel(const TI* __restrict__ x, const float* __restrict__ gamma,
 
 // ---------------------------------------------------------------- shift score
 // s = D(F(x), x) per token (Sec. 3.2); DIST 0: L2, 1: L1, 2: cosine distance.
-// One warp per token.  The 16-byte pieces stay packed in registers until they are reduced, so
-// that eight loads per lane are in flight at about 48 registers per thread and enough warps
-// fit an SM to cover the HBM latency.
+// Bound by HBM.  The 16-byte pieces stay packed in registers until they are reduced, so that eight loads per
+// lane are in flight at about 48 registers per thread and enough warps fit an SM to cover the HBM latency.
+// `before` is read with an evict-first hint: what the L2 can keep of the two is then `after`, whose kept rows
+// the compaction reads next.
+template <typename T, int DIST> struct ShiftSums {
+    float acc = 0.f, aa = 0.f, bb = 0.f;
+    __device__ __forceinline__ void add(const uint4& ra, const uint4& rb) {
+        constexpr int VN = Vec16<T>::N;
+        float va[VN], vb[VN];
+        unpack16<T>(ra, va);
+        unpack16<T>(rb, vb);
+#pragma unroll
+        for (int e = 0; e < VN; ++e) {
+            if (DIST == 0) { const float d = va[e] - vb[e]; acc = fmaf(d, d, acc); }
+            else if (DIST == 1) { acc += fabsf(va[e] - vb[e]); }
+            else {
+                acc = fmaf(va[e], vb[e], acc);
+                aa = fmaf(va[e], va[e], aa);
+                bb = fmaf(vb[e], vb[e], bb);
+            }
+        }
+    }
+    // over the lanes whose numbers differ below `width` (a power of two)
+    __device__ __forceinline__ float finish(int width) {
+        for (int o = width >> 1; o > 0; o >>= 1) {
+            acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (DIST == 2) {
+                aa += __shfl_xor_sync(0xffffffffu, aa, o);
+                bb += __shfl_xor_sync(0xffffffffu, bb, o);
+            }
+        }
+        return DIST == 0 ? sqrtf(acc) : DIST == 1 ? acc : 1.f - acc / fmaxf(sqrtf(aa) * sqrtf(bb), 1e-12f);
+    }
+};
+
+// One warp per token.
 template <typename T, int DIST>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, 5)
 shift_score_kernel(const T* __restrict__ after, const T* __restrict__ before, long long rows, int D,
                    float* __restrict__ scores) {
-    constexpr int VN = Vec16<T>::N;
     constexpr int UNROLL = 4;
     grid_dep_launch();
     grid_dep_wait();
+    const uint64_t once = evict_first_policy();
     const int lane = threadIdx.x & 31;
     const long long row = (long long)blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
     if (row >= rows) return;
-    const int nvec = D / VN;
+    const int nvec = D / Vec16<T>::N;
     const uint4* a = reinterpret_cast<const uint4*>(after + row * D);
     const uint4* b = reinterpret_cast<const uint4*>(before + row * D);
-    float acc = 0.f, aa = 0.f, bb = 0.f;
+    ShiftSums<T, DIST> s;
     for (int base = 0; base < nvec; base += 32 * UNROLL) {
         uint4 ra[UNROLL], rb[UNROLL];
 #pragma unroll
         for (int u = 0; u < UNROLL; ++u) {
             const int iv = base + u * 32 + lane;
-            if (iv < nvec) { ra[u] = ld_stream(a + iv); rb[u] = ld_stream(b + iv); }
+            if (iv < nvec) { ra[u] = ld_stream(a + iv); rb[u] = ld_stream(b + iv, once); }
         }
 #pragma unroll
-        for (int u = 0; u < UNROLL; ++u) {
-            const int iv = base + u * 32 + lane;
-            if (iv < nvec) {
-                float va[VN], vb[VN];
-                unpack16<T>(ra[u], va);
-                unpack16<T>(rb[u], vb);
+        for (int u = 0; u < UNROLL; ++u)
+            if (base + u * 32 + lane < nvec) s.add(ra[u], rb[u]);
+    }
+    const float d = s.finish(32);
+    if (lane == 0) scores[row] = d;
+}
+
+// Tokens of at most 32 * VPR pieces (VPR 1 or 2): 4 / VPR groups of 32 >> lsh tokens side by side per warp, 1 << lsh
+// lanes per token, so that a lane has eight loads in flight here too (a warp per token of 256 bf16 had two:
+// 64 x 56 x 56 positions took 56 us = 3.7 TB/s; this takes 36 = 5.7 TB/s).
+template <typename T, int DIST, int VPR>
+__global__ void __launch_bounds__(kWarpsPerCta * 32, 5)
+shift_score_short_kernel(const T* __restrict__ after, const T* __restrict__ before, long long rows, int D, int lsh,
+                         float* __restrict__ scores) {
+    constexpr int U = 4 / VPR;
+    grid_dep_launch();
+    grid_dep_wait();
+    const uint64_t once = evict_first_policy();
+    const int lane = threadIdx.x & 31;
+    if (VPR > 1) lsh = 5;
+    const int nvec = D / Vec16<T>::N, side = 32 >> lsh, v0 = lane & ((1 << lsh) - 1);
+    const long long row0 = ((long long)blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5)) * (U * side) + (lane >> lsh);
+    uint4 ra[U][VPR], rb[U][VPR];
 #pragma unroll
-                for (int e = 0; e < VN; ++e) {
-                    if (DIST == 0) { const float d = va[e] - vb[e]; acc = fmaf(d, d, acc); }
-                    else if (DIST == 1) { acc += fabsf(va[e] - vb[e]); }
-                    else {
-                        acc = fmaf(va[e], vb[e], acc);
-                        aa = fmaf(va[e], va[e], aa);
-                        bb = fmaf(vb[e], vb[e], bb);
-                    }
-                }
+    for (int u = 0; u < U; ++u) {
+        const long long row = row0 + u * side;
+#pragma unroll
+        for (int j = 0; j < VPR; ++j) {
+            const int iv = j * 32 + v0;
+            ra[u][j] = rb[u][j] = make_uint4(0u, 0u, 0u, 0u);
+            if (row < rows && iv < nvec) {
+                ra[u][j] = ld_stream(reinterpret_cast<const uint4*>(after + row * D) + iv);
+                rb[u][j] = ld_stream(reinterpret_cast<const uint4*>(before + row * D) + iv, once);
             }
         }
     }
-    acc = warp_sum(acc);
-    float s;
-    if (DIST == 0) s = sqrtf(acc);
-    else if (DIST == 1) s = acc;
-    else {
-        aa = warp_sum(aa); bb = warp_sum(bb);
-        s = 1.f - acc / fmaxf(sqrtf(aa) * sqrtf(bb), 1e-12f);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const long long row = row0 + u * side;
+        ShiftSums<T, DIST> s;
+#pragma unroll
+        for (int j = 0; j < VPR; ++j) s.add(ra[u][j], rb[u][j]);
+        const float d = s.finish(1 << lsh);
+        if (v0 == 0 && row < rows) scores[row] = d;
     }
-    if (lane == 0) scores[row] = s;
 }
 
 // ---------------------------------------------------------------- residual add + score
@@ -168,9 +218,15 @@ cudaError_t launch_layernorm(rs_dtype in_dtype, rs_dtype out_dtype, const void* 
 cudaError_t launch_shift_score(rs_dtype dtype, rs_dist dist, long long T, int D, const void* after,
                                const void* before, float* scores, cudaStream_t st) {
     if (T == 0) return cudaSuccess;
-    const dim3 grid(row_grid(T)), block(kWarpsPerCta * 32);
-#define RS_SCORE_CASE(TT, DD)                                                                   \
-    return launch_pdl(shift_score_kernel<TT, DD>, grid, block, 0, st, (const TT*)after, (const TT*)before, T, D, scores)
+    const int nvec = (int)((size_t)D * dtype_size(dtype) / 16);
+    int lsh = 0;
+    while (lsh < 5 && (1 << lsh) < nvec) ++lsh;
+    const long long per_cta = kWarpsPerCta * (nvec <= 32 ? 4 * (32 >> lsh) : nvec <= 64 ? 2 : 1);
+    const dim3 grid((unsigned)((T + per_cta - 1) / per_cta)), block(kWarpsPerCta * 32);
+#define RS_SCORE_CASE(TT, DD)                                                                                                        \
+    return nvec <= 32   ? launch_pdl(shift_score_short_kernel<TT, DD, 1>, grid, block, 0, st, (const TT*)after, (const TT*)before, T, D, lsh, scores) \
+           : nvec <= 64 ? launch_pdl(shift_score_short_kernel<TT, DD, 2>, grid, block, 0, st, (const TT*)after, (const TT*)before, T, D, lsh, scores) \
+                        : launch_pdl(shift_score_kernel<TT, DD>, grid, block, 0, st, (const TT*)after, (const TT*)before, T, D, scores)
     if (dtype == RS_BF16) {
         if (dist == RS_DIST_L2) RS_SCORE_CASE(__nv_bfloat16, 0);
         else if (dist == RS_DIST_L1) RS_SCORE_CASE(__nv_bfloat16, 1);

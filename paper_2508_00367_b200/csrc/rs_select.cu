@@ -247,6 +247,18 @@ select_kernel(const float* __restrict__ scores, int nparts, float* __restrict__ 
         for (int j = k_b + tid; j < K; j += nt) out[j] = -1;
 }
 
+// Adds the eight bf16 values of a 16-byte piece and their squares: the statistics of a LayerNorm folded into the
+// next product.
+__device__ __forceinline__ void add_row_sums(const uint4& v, float& s1, float& s2) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float y0 = __uint_as_float(w[e] << 16), y1 = __uint_as_float(w[e] & 0xffff0000u);
+        s1 += y0 + y1;
+        s2 = fmaf(y0, y0, fmaf(y1, y1, s2));
+    }
+}
+
 // One warp moves one kept row (16-byte pieces, all loads of a pass issued before its first store):
 // to row `orow` of x_out when x_out is given, and, with LT given, LN of the row to the same row of
 // ln.out.
@@ -268,15 +280,7 @@ __device__ __forceinline__ void copy_row(const uint4* __restrict__ src, long lon
                 const int iv = base + j * 32 + lane;
                 if (iv < row_vecs) {
                     dst[iv] = v[j];
-                    if (ln.stats) {                  // bf16 rows only (the caller's business)
-                        const uint32_t w[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float y0 = __uint_as_float(w[e] << 16), y1 = __uint_as_float(w[e] & 0xffff0000u);
-                            s1 += y0 + y1;
-                            s2 = fmaf(y0, y0, fmaf(y1, y1, s2));
-                        }
-                    }
+                    if (ln.stats) add_row_sums(v[j], s1, s2);    // bf16 rows only (the caller's business)
                 }
             }
         }
@@ -308,26 +312,6 @@ __device__ __forceinline__ void copy_row(const uint4* __restrict__ src, long lon
     }
 }
 
-// Sum and sum of squares of a row of bf16 values held by a warp as 16-byte pieces (zeros where a lane has none),
-// to out[0], out[1]: the statistics of a LayerNorm folded into the next product.
-template <int NV>
-__device__ __forceinline__ void row_sums(const uint4 (&v)[NV], int lane, float* __restrict__ out) {
-    float s1 = 0.f, s2 = 0.f;
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-        const uint32_t w[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float y0 = __uint_as_float(w[e] << 16), y1 = __uint_as_float(w[e] & 0xffff0000u);
-            s1 += y0 + y1;
-            s2 = fmaf(y0, y0, fmaf(y1, y1, s2));
-        }
-    }
-    s1 = warp_sum(s1);
-    s2 = warp_sum(s2);
-    if (lane == 0) { out[0] = s1; out[1] = s2; }
-}
-
 // Nothing dropped (K == N): every token is kept, in order; only the scores remain to be
 // finished when they arrive as per-tile partial sums of squares.
 __global__ void __launch_bounds__(256)
@@ -341,163 +325,177 @@ keep_all_kernel(const float* __restrict__ scores, int nparts, float* __restrict_
     keep_idx[t] = (int32_t)(t % N);
 }
 
-// x_out[b, j, :] = x[b, keep_idx[b, j], :] (zeros where the index is -1); with LT given, LN of the row to ln.out.
-// One warp per row, 16-byte pieces, all loads of a row issued before the first store.
-template <int MAXV, typename LT>
+// Source row of output row `row` (-1: the output row is zeros).  TokenRows: row j of sample b is token
+// keep_idx[b, j].  GridRows: position (i, j) of the kept grid is position (keep_rows[i], keep_cols[j]).
+struct TokenRows {
+    const int32_t* keep_idx;
+    unsigned K;
+    int N;
+    __device__ __forceinline__ long long operator()(unsigned row) const {
+        const int t = __ldg(keep_idx + row);
+        return t < 0 ? -1 : (long long)(row / K) * N + t;
+    }
+};
+struct GridRows {
+    const int32_t *keep_rows, *keep_cols;
+    unsigned Hk, Wk;
+    int H, W;
+    __device__ __forceinline__ long long operator()(unsigned row) const {
+        const unsigned line = row / Wk, j = row - line * Wk, b = line / Hk;        // line = b * Hk + i
+        return ((long long)b * H + __ldg(keep_rows + line)) * W + __ldg(keep_cols + b * Wk + j);
+    }
+};
+
+// x_out[row, :] = x[src(row), :]; with LT given, LN of the row to ln.out.
+// One warp per row, 16-byte pieces, all loads of a row issued before the first store.  CTAs take the rows from
+// the last to the first: what the kernel before this one touched last is what the L2 still holds of an input
+// larger than it (512 x 197 tokens of 768 bf16 after their scores: 43 -> 41 us, 6.9 TB/s read and written; an
+// evict-first hint on the writes as well cost 2 us).
+template <int MAXV, typename LT, typename Src>
 __global__ void __launch_bounds__(256)
-gather_kernel(const uint4* __restrict__ x, const int32_t* __restrict__ keep_idx, unsigned rows, int N,
-              unsigned K, int row_vecs, uint4* __restrict__ x_out, const LnFuse ln) {
+gather_kernel(const uint4* __restrict__ x, const Src src_of, unsigned rows, int row_vecs, uint4* __restrict__ x_out, const LnFuse ln) {
     grid_dep_launch();
     grid_dep_wait();
     const int lane = threadIdx.x & 31;
-    const unsigned row = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const unsigned row = (gridDim.x - 1 - blockIdx.x) * 8 + (threadIdx.x >> 5);
     if (row >= rows) return;
-    const int src = __ldg(keep_idx + row);
+    const long long src = src_of(row);
     if (src < 0) {
         if (x_out)
             for (int iv = lane; iv < row_vecs; iv += 32) x_out[(long long)row * row_vecs + iv] = make_uint4(0u, 0u, 0u, 0u);
         return;
     }
-    copy_row<MAXV, LT>(x + ((long long)(row / K) * N + src) * row_vecs, row, row_vecs, lane, x_out, ln);
+    copy_row<MAXV, LT>(x + src * row_vecs, row, row_vecs, lane, x_out, ln);
 }
 
-// The same for rows of at most 32 * VPR pieces, RPW = 4 / VPR rows per warp, so that a lane has four loads in
-// flight whatever the width (a row of 192 bf16 is 24 pieces: one load per lane).  Bound by HBM / L2: 256 x 181 rows
-// of 192 bf16 3.8 us after the selection = 9.3 TB/s out of L2.
-template <int VPR>
+// The same copy for rows of at most 32 * VPR pieces: a lane keeps four loads in flight whatever the width.
+// VPR 2: two rows per warp.  VPR 1: four groups of 32 >> lsh rows side by side, 1 << lsh lanes (the pieces of a
+// row rounded up to a power of two) per row.  Bound by HBM / L2: 256 x 181 rows of 192 bf16 take 3.8 us after the
+// selection = 9.3 TB/s out of L2.
+template <int VPR, typename Src>
 __global__ void __launch_bounds__(256)
-gather_short_kernel(const uint4* __restrict__ x, const int32_t* __restrict__ keep_idx, unsigned rows, int N,
-                    unsigned K, int row_vecs, uint4* __restrict__ x_out, float* __restrict__ stats) {
-    constexpr int RPW = 4 / VPR;
+gather_short_kernel(const uint4* __restrict__ x, const Src src_of, unsigned rows, int row_vecs, int lsh,
+                    uint4* __restrict__ x_out, float* __restrict__ stats) {
+    constexpr int U = 4 / VPR;
     grid_dep_launch();
     grid_dep_wait();
     const int lane = threadIdx.x & 31;
-    const unsigned row0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * RPW;
-    if (row0 >= rows) return;
-    const int mine = lane < RPW && row0 + lane < rows ? __ldg(keep_idx + row0 + lane) : -1;
-    uint4 v[RPW][VPR];
+    if (VPR > 1) lsh = 5;
+    const unsigned side = 32u >> lsh, sub = (unsigned)lane >> lsh;
+    const int v0 = lane & ((1 << lsh) - 1);
+    const unsigned row0 = ((gridDim.x - 1 - blockIdx.x) * 8 + (threadIdx.x >> 5)) * U * side + sub;
+    uint4 v[U][VPR];
 #pragma unroll
-    for (int r = 0; r < RPW; ++r) {
-        const int src = __shfl_sync(0xffffffffu, mine, r);
-        const uint4* s = x + ((long long)((row0 + r) / K) * N + (src < 0 ? 0 : src)) * row_vecs;
+    for (int u = 0; u < U; ++u) {
+        const unsigned row = row0 + u * side;
+        const long long src = row < rows ? src_of(row) : -1;
 #pragma unroll
         for (int j = 0; j < VPR; ++j) {
-            v[r][j] = make_uint4(0u, 0u, 0u, 0u);
-            if (src >= 0 && j * 32 + lane < row_vecs) v[r][j] = __ldg(s + j * 32 + lane);
+            v[u][j] = make_uint4(0u, 0u, 0u, 0u);
+            if (src >= 0 && j * 32 + v0 < row_vecs) v[u][j] = __ldg(x + src * row_vecs + j * 32 + v0);
         }
     }
 #pragma unroll
-    for (int r = 0; r < RPW; ++r) {
-        if (row0 + r >= rows) break;
-        uint4* dst = x_out + (long long)(row0 + r) * row_vecs;
+    for (int u = 0; u < U; ++u) {
+        const unsigned row = row0 + u * side;
 #pragma unroll
         for (int j = 0; j < VPR; ++j)
-            if (j * 32 + lane < row_vecs) dst[j * 32 + lane] = v[r][j];
-        if (stats) row_sums<VPR>(v[r], lane, stats + 2 * (long long)(row0 + r));
+            if (row < rows && j * 32 + v0 < row_vecs) x_out[(long long)row * row_vecs + j * 32 + v0] = v[u][j];
+        if (stats) {
+            float s1 = 0.f, s2 = 0.f;
+#pragma unroll
+            for (int j = 0; j < VPR; ++j) add_row_sums(v[u][j], s1, s2);
+            for (int o = 1 << lsh >> 1; o > 0; o >>= 1) {
+                s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+                s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+            }
+            if (v0 == 0 && row < rows) reinterpret_cast<float2*>(stats)[row] = make_float2(s1, s2);
+        }
     }
 }
 
 // Line-wise pruning of an H x W token grid (Sec. 4, CNN variant L-W): the shift is averaged over
-// every row and every column of the full grid, and the lines with the lowest averages go.  Grid
-// (G, B): every CTA of sample b repeats the cheap part — one thread per line sums its line in
-// fp64 in index order (the order a plain loop takes, so the averages are the same doubles on any
-// machine), ranks it among its peers by counting (larger average first, lower index on a tie, NaN
-// last) and the kept lines are numbered by a count over the flags — and then copies its share of
-// the Hk x Wk kept positions, a warp per position.  CTA 0 of the sample writes the two index lists.
+// every row and every column of the full grid, and the lines with the lowest averages go.  One CTA per
+// sample finds the kept lines -- one thread per line sums it in fp64 in index order (the order a plain loop
+// takes, so the averages are the same doubles on any machine), ranks it among its peers by counting (larger
+// average first, lower index on a tie, NaN last) and takes its position from the flags' ballots -- and the
+// gather kernels above move the kept positions.  (Repeating the selection in every CTA that copied positions
+// left room for five CTAs of 256 threads per SM and made all of them start with it: 64 maps of 56 x 56 x 256
+// took 52 us that way, 150 MB at 2.9 TB/s; the two kernels take 30.)
 constexpr int kLineMax = 256;
-constexpr int kMapMax = 8192;               // scores of one sample staged in shared memory (32 KB)
+constexpr int kMapMax = 8192;               // scores of one sample staged in shared memory (33 KB)
 
-__device__ __forceinline__ bool line_outranks(double a, int ia, double b, int ib) {
-    if (a != a) return (b != b) && ia < ib;
-    if (b != b) return true;
-    return a > b || (a == b && ia < ib);
+// A double as a key that sorts like it: NaN below every number, -0 = +0.
+__device__ __forceinline__ unsigned long long line_key(double a) {
+    if (a != a) return 0ull;
+    if (a == 0.0) a = 0.0;
+    const unsigned long long b = (unsigned long long)__double_as_longlong(a);
+    return b >> 63 ? ~b : b | (1ull << 63);
 }
 
-template <int MAXV>
-__global__ void __launch_bounds__(256)
-linewise_kernel(const float* __restrict__ scores, int H, int W, int Hk, int Wk, int32_t* __restrict__ keep_rows,
-                int32_t* __restrict__ keep_cols, const uint4* __restrict__ x, int row_vecs, uint4* __restrict__ x_out) {
-    __shared__ double mean[2 * kLineMax];      // rows, then columns
-    __shared__ int32_t kept[2 * kLineMax];
-    __shared__ unsigned char flag[2 * kLineMax];
-    __shared__ float smap[kMapMax];
+__global__ void __launch_bounds__(2 * kLineMax)
+line_select_kernel(const float* __restrict__ scores, int H, int W, int Hk, int Wk, int32_t* __restrict__ keep_rows,
+                   int32_t* __restrict__ keep_cols) {
+    __shared__ unsigned long long key[2][kLineMax];    // rows, then columns
+    __shared__ unsigned mask[2][kLineMax / 32];
+    __shared__ float smap[kMapMax + kLineMax];
     grid_dep_launch();
     grid_dep_wait();
-    const int b = blockIdx.y;
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     const float* s = scores + (long long)b * H * W;
-    // a map of up to kMapMax scores is staged in shared memory first (coalesced, all threads), so
-    // that the per-line loops below do not wait on global memory one element at a time
+    // a map of up to kMapMax scores is staged in shared memory first (coalesced, all threads; an odd row
+    // stride keeps the row sums free of bank conflicts), so that the sums do not wait on global memory
     const bool staged = H * W <= kMapMax;
+    const int ld = staged ? W | 1 : W;
     if (staged) {
-        for (int i = threadIdx.x; i < H * W; i += blockDim.x) smap[i] = s[i];
+        for (int i = tid; i < H * W; i += 2 * kLineMax) {
+            const int r = i / W;
+            smap[r * ld + (i - r * W)] = s[i];
+        }
         __syncthreads();
     }
     const float* sv = staged ? smap : s;
-    for (int l = threadIdx.x; l < H + W; l += blockDim.x) {
+    const int kind = tid / kLineMax, l = tid - kind * kLineMax;        // threads 0 .. 255: rows, the rest: columns
+    const int n = kind ? W : H, len = kind ? H : W, want = kind ? Wk : Hk;
+    if (l < n) {
+        const float* p = sv + (kind ? l : l * ld);
+        const int step = kind ? ld : 1;
         double acc = 0.0;
-        if (l < H) {
-            for (int w = 0; w < W; ++w) acc += (double)sv[l * W + w];
-            mean[l] = acc / (double)W;
-        } else {
-            const int c = l - H;
-            for (int h = 0; h < H; ++h) acc += (double)sv[h * W + c];
-            mean[kLineMax + c] = acc / (double)H;
-        }
+#pragma unroll 8
+        for (int e = 0; e < len; ++e) acc += (double)p[e * step];
+        key[kind][l] = line_key(acc / (double)len);
     }
     __syncthreads();
-    for (int l = threadIdx.x; l < H + W; l += blockDim.x) {
-        const bool row = l < H;
-        const int i = row ? l : l - H, n = row ? H : W, want = row ? Hk : Wk;
-        const double* m = mean + (row ? 0 : kLineMax);
-        const double mine = m[i];
+    bool keep = false;
+    if (l < n) {
+        const unsigned long long mine = key[kind][l];
         int rank = 0;
-        for (int j = 0; j < n; ++j) rank += (j != i) && line_outranks(m[j], j, mine, i);
-        flag[(row ? 0 : kLineMax) + i] = rank < want;
+#pragma unroll 4
+        for (int j = 0; j < n; ++j) rank += key[kind][j] > mine || (key[kind][j] == mine && j < l);
+        keep = rank < want;
     }
+    const unsigned m = __ballot_sync(0xffffffffu, keep);
+    if (lane == 0) mask[kind][l >> 5] = m;
     __syncthreads();
-    for (int l = threadIdx.x; l < H + W; l += blockDim.x) {
-        const bool row = l < H;
-        const int i = row ? l : l - H, off = row ? 0 : kLineMax;
-        if (!flag[off + i]) continue;
-        int pos = 0;
-        for (int j = 0; j < i; ++j) pos += flag[off + j];
-        kept[off + pos] = i;
-        if (blockIdx.x == 0) (row ? keep_rows + (long long)b * Hk : keep_cols + (long long)b * Wk)[pos] = i;
+    if (!keep) return;
+    int pos = __popc(m & ((1u << lane) - 1u));
+    for (int w = 0; w < l >> 5; ++w) pos += __popc(mask[kind][w]);
+    (kind ? keep_cols + (long long)b * Wk : keep_rows + (long long)b * Hk)[pos] = l;
+}
+
+// Launch of the copy: several narrow rows per warp, else a warp per row.
+template <typename Src>
+cudaError_t launch_copy(const void* x, const Src& src, long long rows, int row_vecs, void* x_out, const LnFuse& ln, cudaStream_t st) {
+    if (row_vecs <= 64) {
+        const int vpr = row_vecs <= 32 ? 1 : 2;
+        int lsh = 0;
+        while (lsh < 5 && (1 << lsh) < row_vecs) ++lsh;
+        const unsigned per_cta = vpr == 1 ? 8 * 4 * (32u >> lsh) : 16;
+        const dim3 grid((unsigned)((rows + per_cta - 1) / per_cta));
+        return vpr == 1 ? launch_pdl(gather_short_kernel<1, Src>, grid, dim3(256), 0, st, (const uint4*)x, src, (unsigned)rows, row_vecs, lsh, (uint4*)x_out, ln.stats)
+                        : launch_pdl(gather_short_kernel<2, Src>, grid, dim3(256), 0, st, (const uint4*)x, src, (unsigned)rows, row_vecs, lsh, (uint4*)x_out, ln.stats);
     }
-    __syncthreads();
-    if (!x) return;
-    const int P = Hk * Wk, G = gridDim.x, per = (P + G - 1) / G;
-    const int lo = blockIdx.x * per, hi = min(lo + per, P);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const LnFuse none = {nullptr, nullptr, 0.f, nullptr, nullptr};
-    auto src_of = [&](int p) {
-        const int i = p / Wk, j = p - i * Wk;
-        return x + (((long long)b * H + kept[i]) * W + kept[kLineMax + j]) * row_vecs;
-    };
-    if (row_vecs <= 32) {
-        // short rows (up to 512 bytes): a warp takes 32 / rv positions side by side (rv = the row's
-        // 16-byte pieces rounded up to a power of two) and four such groups per step, so that every
-        // lane has four loads in flight
-        int rv = 1;
-        while (rv < row_vecs) rv <<= 1;
-        const int side = 32 / rv, sub = lane / rv, v = lane - sub * rv, step = side * 4;
-        for (int p0 = lo + warp * step; p0 < hi; p0 += nwarps * step) {
-            uint4 val[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int p = p0 + u * side + sub;
-                if (p < hi && v < row_vecs) val[u] = __ldg(src_of(p) + v);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int p = p0 + u * side + sub;
-                if (p < hi && v < row_vecs) x_out[((long long)b * P + p) * row_vecs + v] = val[u];
-            }
-        }
-        return;
-    }
-    for (int p = lo + warp; p < hi; p += nwarps)
-        copy_row<MAXV, void>(src_of(p), (long long)b * P + p, row_vecs, lane, x_out, none);
+    return launch_pdl(gather_kernel<4, void, Src>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, (const uint4*)x, src, (unsigned)rows, row_vecs, (uint4*)x_out, ln);
 }
 
 }  // namespace
@@ -537,36 +535,30 @@ cudaError_t launch_gather(rs_dtype dtype, const void* x, const int32_t* keep_idx
     const bool norm = ln && ln->gamma;               // else ln, if given, only asks for the row sums of the copy
     if ((norm && !ln_fusable(dtype, D)) || (!x_out && !norm)) return cudaErrorInvalidValue;
     const LnFuse none = {nullptr, nullptr, 0.f, nullptr, nullptr};
-#define RS_G_CASE(LT)                                                                                                 \
-    launch_pdl(gather_kernel<4, LT>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, (const uint4*)x, keep_idx,   \
-               (unsigned)rows, N, (unsigned)K, row_vecs, (uint4*)x_out, ln ? *ln : none)
-#define RS_GS_CASE(VPR)                                                                                               \
-    launch_pdl(gather_short_kernel<VPR>, dim3((unsigned)((rows + 32 / VPR - 1) / (32 / VPR))), dim3(256), 0, st,      \
-               (const uint4*)x, keep_idx, (unsigned)rows, N, (unsigned)K, row_vecs, (uint4*)x_out, ln ? ln->stats : nullptr)
-    if (!norm) return row_vecs <= 32 ? RS_GS_CASE(1) : row_vecs <= 64 ? RS_GS_CASE(2) : RS_G_CASE(void);
-    return dtype == RS_BF16 ? RS_G_CASE(__nv_bfloat16) : RS_G_CASE(float);
-#undef RS_GS_CASE
-#undef RS_G_CASE
+    const TokenRows src = {keep_idx, (unsigned)K, N};
+    if (!norm) return launch_copy(x, src, rows, row_vecs, x_out, ln ? *ln : none, st);
+    const dim3 grid((unsigned)((rows + 7) / 8));
+    if (dtype == RS_BF16)
+        return launch_pdl(gather_kernel<4, __nv_bfloat16, TokenRows>, grid, dim3(256), 0, st, (const uint4*)x, src, (unsigned)rows, row_vecs, (uint4*)x_out, *ln);
+    return launch_pdl(gather_kernel<4, float, TokenRows>, grid, dim3(256), 0, st, (const uint4*)x, src, (unsigned)rows, row_vecs, (uint4*)x_out, *ln);
 }
 
 int linewise_max_lines() { return kLineMax; }
 
-cudaError_t launch_linewise(const float* scores, int B, int H, int W, int Hk, int Wk, int32_t* keep_rows,
-                            int32_t* keep_cols, rs_dtype dtype, const void* x, int D, void* x_out, int sm_count,
-                            cudaStream_t st) {
+cudaError_t launch_line_select(const float* scores, int B, int H, int W, int Hk, int Wk, int32_t* keep_rows,
+                               int32_t* keep_cols, cudaStream_t st) {
     if (B == 0) return cudaSuccess;
-    const int row_vecs = x ? (int)((size_t)D * dtype_size(dtype) / 16) : 0;
-    // about eight CTAs per SM in all (measured best between six and twelve), at least 16 positions
-    // each; one CTA per sample for the indices alone
-    int G = 1;
-    if (x) {
-        G = (8 * sm_count + B - 1) / B;
-        const int cap = (Hk * Wk + 15) / 16;
-        if (G > cap) G = cap;
-        if (G < 1) G = 1;
-    }
-    return launch_pdl(linewise_kernel<4>, dim3(G, B), dim3(256), 0, st, scores, H, W, Hk, Wk, keep_rows, keep_cols,
-                      (const uint4*)x, row_vecs, (uint4*)x_out);
+    return launch_pdl(line_select_kernel, dim3(B), dim3(2 * kLineMax), 0, st, scores, H, W, Hk, Wk, keep_rows, keep_cols);
+}
+
+cudaError_t launch_line_gather(rs_dtype dtype, const void* x, const int32_t* keep_rows, const int32_t* keep_cols, int B, int H,
+                               int W, int Hk, int Wk, int D, void* x_out, cudaStream_t st) {
+    const long long rows = (long long)B * Hk * Wk;
+    if (rows == 0) return cudaSuccess;
+    if (rows >= (1ll << 31)) return cudaErrorInvalidValue;
+    const GridRows src = {keep_rows, keep_cols, (unsigned)Hk, (unsigned)Wk, H, W};
+    const LnFuse none = {nullptr, nullptr, 0.f, nullptr, nullptr};
+    return launch_copy(x, src, rows, (int)((size_t)D * dtype_size(dtype) / 16), x_out, none, st);
 }
 
 }  // namespace rs

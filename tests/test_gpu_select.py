@@ -33,3 +33,33 @@ def test_rows_of_every_width_class(ctx, pieces, B, N, r):   # noqa: F811
     np.testing.assert_array_equal(keep.cpu().numpy(), want)
     assert torch.equal(xo.cpu(), torch.stack([x[b][torch.from_numpy(want[b]).long()] for b in range(B)]))
     assert (buf[:64] == -7).all() and (buf[-64:] == -7).all()
+
+
+@pytest.mark.parametrize("dist", ["l2", "l1", "cos"])
+@pytest.mark.parametrize("pieces", [1, 2, 3, 16, 17, 32, 33, 64, 65])
+def test_score_of_every_width_class(ctx, pieces, dist):   # noqa: F811
+    D, rows = 8 * pieces, 131                                   # a row count that leaves a warp partly filled
+    g = torch.Generator().manual_seed(pieces)
+    a, b = torch.randn(1, rows, D, generator=g).bfloat16(), torch.randn(1, rows, D, generator=g).bfloat16()
+    buf = torch.full((rows + 2,), -7.0, device="cuda")
+    got = ctx.shift_score(a.cuda(), b.cuda(), dist, out=buf[1:-1].view(1, rows))
+    want = orc.shift_score(a.double().numpy(), b.double().numpy(), dist)
+    if dist == "cos":
+        np.testing.assert_allclose(got.cpu().double().numpy(), want, rtol=0, atol=2e-6)    # 1 - cos cancels: an absolute bound
+    else:
+        np.testing.assert_allclose(got.cpu().double().numpy(), want, rtol=2e-6, atol=0)    # fp32 sum of D <= 520 terms
+    assert buf[0] == -7 and buf[-1] == -7
+
+
+@pytest.mark.parametrize("pieces", [2, 3, 32, 33, 64, 65])
+@pytest.mark.parametrize("H,W,dr,dc", [(7, 5, 2, 1), (90, 91, 30, 40), (91, 91, 1, 90)])   # staged scores up to 8192
+def test_grid_rows_of_every_width_class(ctx, pieces, H, W, dr, dc):   # noqa: F811
+    D = 8 * pieces
+    s = _scores(2, H * W, "normal", pieces).reshape(2, H, W)
+    x = torch.randn(2, H, W, D, generator=torch.Generator().manual_seed(pieces)).bfloat16()
+    xo, kr, kc = ctx.linewise_compact(torch.from_numpy(s).cuda(), x.cuda(), dr, dc)
+    want_r, want_c = orc.linewise(s.astype(np.float64), dr, dc)
+    np.testing.assert_array_equal(kr.cpu().numpy(), want_r)
+    np.testing.assert_array_equal(kc.cpu().numpy(), want_c)
+    for b in range(2):
+        assert torch.equal(xo[b].cpu(), x[b][torch.from_numpy(want_r[b]).long()][:, torch.from_numpy(want_c[b]).long()])
