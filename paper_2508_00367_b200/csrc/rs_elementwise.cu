@@ -153,6 +153,8 @@ template <typename TO, typename TX, int MODE>
 __global__ void __launch_bounds__(kWarpsPerCta * 32)
 residual_score_kernel(const float* __restrict__ m, const float* __restrict__ xp, const TX* __restrict__ x0,
                       long long rows, int D, int dist, TO* __restrict__ x_hat, float* __restrict__ scores) {
+    grid_dep_launch();
+    grid_dep_wait();
     const int lane = threadIdx.x & 31;
     const long long row = (long long)blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
     if (row >= rows) return;
@@ -246,7 +248,7 @@ cudaError_t launch_residual_score(const float* m, const float* x_prime, const vo
     if (T == 0) return cudaSuccess;
     const dim3 grid(row_grid(T)), block(kWarpsPerCta * 32);
 #define RS_RES_CASE(TO, TX, MD)                                                                                  \
-    residual_score_kernel<TO, TX, MD><<<grid, block, 0, st>>>(m, x_prime, (const TX*)x, T, D, (int)dist, (TO*)x_hat, scores)
+    return launch_pdl(residual_score_kernel<TO, TX, MD>, grid, block, 0, st, m, x_prime, (const TX*)x, T, D, (int)dist, (TO*)x_hat, scores)
 #define RS_RES_MODE(TO, TX)                                     \
     do {                                                        \
         if (mode == RS_SCORE_MLP) RS_RES_CASE(TO, TX, 0);       \
