@@ -1,0 +1,77 @@
+// What the two tensor-core GEMM kernels share: the epilogues' names, arguments and arithmetic (Eq. att, Eq. MLP, Sec. 3.2).
+#pragma once
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "rs.h"
+
+namespace rs {
+namespace gemm {
+
+// EPI_SCORE_STATS: EPI_SCORE that also leaves, per row and column half of a tile, the sum and the sum of
+// squares of the (rounded) output values -- the row statistics of the next block's LayerNorm.
+// EPI_BIAS_LN: the LayerNorm of the A operand folded into the product: with W' = W * gamma (column-wise),
+// c_n = sum_k W'_nk and b'_n = b_n + sum_k W_nk beta_k,  LN(x) W^T + b = rstd (x W'^T - mu c) + b';  mu and
+// rstd of a row come from the statistics above, acc = x W'^T from the tensor cores.
+enum { EPI_BIAS = 0, EPI_BIAS_GELU = 1, EPI_RESID = 2, EPI_SCORE = 3, EPI_SCORE_STATS = 4, EPI_BIAS_LN = 5 };
+
+struct GemmArgs {
+    int M, N, K;
+    const float* bias;        // [N] or null
+    const void* residual;     // EPI_RESID: bf16 [M, N];  EPI_SCORE: fp32 [M, N]
+    const void* residual2;    // EPI_SCORE, score_kind 2: bf16 [M, N] block input x
+    const int* row_map;       // optional [M]: row t of the block input (EPI_RESID's residual, EPI_SCORE's residual2)
+                              // is row row_map[t] of that matrix (the previous block's un-pruned output, read in place)
+    float* partials;          // EPI_SCORE (and EPI_RESID when non-null): [M, 2 * N / BN] sums of squares
+    int score_kind;           // EPI_SCORE: scored pair (u, v) = 0: (m, x'), 1: (x^, x'), 2: (x^, x)
+    int dist;                 // rs_dist of the score: L2 / L1 sums of (u - v)^2 / |u - v|, cosine sums of u.v, u.u, v.v
+    float* stats_out;         // EPI_SCORE_STATS: [M, 2 * N / BN][2] = (sum, sum of squares) of the row's outputs in that half tile
+    const float* stats_in;    // EPI_BIAS_LN: such statistics of the A operand's rows, stats_parts pairs per row over ln_dim = K values
+    const float* colsum;      // EPI_BIAS_LN: c [N]
+    int stats_parts;
+    float ln_eps;
+    int* status;
+};
+
+// Exact-erf GELU, v * Phi(v), to fp32 accuracy (max abs error 8e-7 over all v) without erff:
+// with q(t) = -log2(Phi(-t)) for t >= 0,  Phi(v) = 2^-q(|v|) for v < 0 and 1 - 2^-q(|v|) for
+// v >= 0.  q is smooth (about t^2/2 * log2(e) plus slow terms) and a degree-5 polynomial fitted
+// on [0, 7] with weight t * Phi(-t) reproduces GELU to that accuracy; its positive leading
+// coefficient keeps 2^-q -> 0 for large |v|.  Coefficients from csrc/fit_gelu.py.
+__device__ __forceinline__ float gelu_erf(float v) {
+    const float a = fabsf(v);
+    float q = 0.00047694556997157633f;
+    q = fmaf(q, a, -0.00711308466270566f);
+    q = fmaf(q, a, 0.05190887302160263f);
+    q = fmaf(q, a, 0.4598882496356964f);
+    q = fmaf(q, a, 1.1508461236953735f);
+    q = fmaf(q, a, 1.0000265836715698f);
+    float e;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(-q));
+    return v * (v >= 0.f ? 1.f - e : e);
+}
+
+// Adds one element of the scored pair (u, v) to the running sums of the chosen distance (Sec. 3.3).
+__device__ __forceinline__ void score_acc(int dist, float u, float v, float& s0, float& s1, float& s2) {
+    if (dist == RS_DIST_L2) { const float d = u - v; s0 = fmaf(d, d, s0); }
+    else if (dist == RS_DIST_L1) { s0 += fabsf(u - v); }
+    else { s0 = fmaf(u, v, s0); s1 = fmaf(u, u, s1); s2 = fmaf(v, v, s2); }
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+    __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<uint32_t*>(&h);
+}
+
+}  // namespace gemm
+
+// The kernel for few rows (rs_gemm_small.cu): whether a shape goes there, and the CTAs that share the K of a tile.
+// tmA: boxes of 128 rows; tmB: boxes of kSmallBN rows; both 64 columns, 128-byte swizzle.
+constexpr int kSmallBN = 64;
+struct SmallPlan { bool use; int splits; };
+SmallPlan gemm_small_plan(long long M, int N, int K, int sm_count);
+cudaError_t launch_gemm_small(int epi, const CUtensorMap& tmA, const CUtensorMap& tmB, const gemm::GemmArgs& args, int splits, void* out,
+                              rs_dtype out_dtype, bool weights_ready, cudaStream_t st);
+}  // namespace rs

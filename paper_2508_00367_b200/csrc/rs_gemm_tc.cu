@@ -21,6 +21,7 @@
 #include <string.h>
 
 #include "rs_internal.h"
+#include "rs_gemm.cuh"
 #include "rs_device.cuh"
 #include "rs_once.h"
 #include "rs_tc.cuh"
@@ -30,13 +31,7 @@ namespace rs {
 namespace {
 
 using namespace tc;
-
-// EPI_SCORE_STATS: EPI_SCORE that also leaves, per row and column half of a tile, the sum and the sum of
-// squares of the (rounded) output values -- the row statistics of the next block's LayerNorm.
-// EPI_BIAS_LN: the LayerNorm of the A operand folded into the product: with W' = W * gamma (column-wise),
-// c_n = sum_k W'_nk and b'_n = b_n + sum_k W_nk beta_k,  LN(x) W^T + b = rstd (x W'^T - mu c) + b';  mu and
-// rstd of a row come from the statistics above, acc = x W'^T from the tensor cores.
-enum { EPI_BIAS = 0, EPI_BIAS_GELU = 1, EPI_RESID = 2, EPI_SCORE = 3, EPI_SCORE_STATS = 4, EPI_BIAS_LN = 5 };
+using namespace gemm;
 
 constexpr int BM = 128;                       // rows per CTA; the pair's tile has 2 * BM rows
 constexpr int BK = 64;
@@ -68,54 +63,6 @@ template <int BN, int EPI> struct Cfg {
     static constexpr size_t SMEM = (size_t)OFF_BIAS + (LN ? 4096 : 2048);   // the window itself must be 1024-byte aligned
     static_assert(SMEM <= 227 * 1024, "shared memory of one CTA");
 };
-
-struct GemmArgs {
-    int M, N, K;
-    const float* bias;        // [N] or null
-    const void* residual;     // EPI_RESID: bf16 [M, N];  EPI_SCORE: fp32 [M, N]
-    const void* residual2;    // EPI_SCORE, score_kind 2: bf16 [M, N] block input x
-    const int* row_map;       // optional [M]: row t of the block input (EPI_RESID's residual, EPI_SCORE's residual2)
-                              // is row row_map[t] of that matrix (the previous block's un-pruned output, read in place)
-    float* partials;          // EPI_SCORE (and EPI_RESID when non-null): [M, 2 * N / BN] sums of squares
-    int score_kind;           // EPI_SCORE: scored pair (u, v) = 0: (m, x'), 1: (x^, x'), 2: (x^, x)
-    int dist;                 // rs_dist of the score: L2 / L1 sums of (u - v)^2 / |u - v|, cosine sums of u.v, u.u, v.v
-    float* stats_out;         // EPI_SCORE_STATS: [M, 2 * N / BN][2] = (sum, sum of squares) of the row's outputs in that half tile
-    const float* stats_in;    // EPI_BIAS_LN: such statistics of the A operand's rows, stats_parts pairs per row over ln_dim = K values
-    const float* colsum;      // EPI_BIAS_LN: c [N]
-    int stats_parts;
-    float ln_eps;
-    int* status;
-};
-
-// Exact-erf GELU, v * Phi(v), to fp32 accuracy (max abs error 8e-7 over all v) without erff:
-// with q(t) = -log2(Phi(-t)) for t >= 0,  Phi(v) = 2^-q(|v|) for v < 0 and 1 - 2^-q(|v|) for
-// v >= 0.  q is smooth (about t^2/2 * log2(e) plus slow terms) and a degree-5 polynomial fitted
-// on [0, 7] with weight t * Phi(-t) reproduces GELU to that accuracy; its positive leading
-// coefficient keeps 2^-q -> 0 for large |v|.  Coefficients from csrc/fit_gelu.py.
-__device__ __forceinline__ float gelu_erf(float v) {
-    const float a = fabsf(v);
-    float q = 0.00047694556997157633f;
-    q = fmaf(q, a, -0.00711308466270566f);
-    q = fmaf(q, a, 0.05190887302160263f);
-    q = fmaf(q, a, 0.4598882496356964f);
-    q = fmaf(q, a, 1.1508461236953735f);
-    q = fmaf(q, a, 1.0000265836715698f);
-    float e;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(-q));
-    return v * (v >= 0.f ? 1.f - e : e);
-}
-
-// Adds one element of the scored pair (u, v) to the running sums of the chosen distance (Sec. 3.3).
-__device__ __forceinline__ void score_acc(int dist, float u, float v, float& s0, float& s1, float& s2) {
-    if (dist == RS_DIST_L2) { const float d = u - v; s0 = fmaf(d, d, s0); }
-    else if (dist == RS_DIST_L1) { s0 += fabsf(u - v); }
-    else { s0 = fmaf(u, v, s0); s1 = fmaf(u, u, s1); s2 = fmaf(v, v, s2); }
-}
-
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-    __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<uint32_t*>(&h);
-}
 
 template <int BN, int EPI, typename OutT>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -648,25 +595,26 @@ bool gemm_tc_supported(long long M, int N, int K) {
     return M >= 1 && M < (1ll << 31) && N >= 128 && ((N % 128) == 0 || (N % 192) == 0) && K >= 64 && (K % 64) == 0;
 }
 
-int gemm_tc_score_parts(const rs_ctx* ctx, long long M, int N) {
-    return 2 * (N / pick_bn(M, N, ctx->sm_count));
+int gemm_tc_score_parts(const rs_ctx* ctx, long long M, int N, int K) {
+    return 2 * (N / (gemm_small_plan(M, N, K, ctx->sm_count).use ? kSmallBN : pick_bn(M, N, ctx->sm_count)));
 }
 
 cudaError_t launch_gemm_tc(rs_ctx* ctx, int epi, const void* A, const void* W, const float* bias,
                            const void* residual, const void* residual2, const int32_t* row_map, void* out, rs_dtype out_dtype,
                            float* partials, int score_kind, int dist, long long M, int N, int K, cudaStream_t st,
-                           const GemmLn* ln) {
+                           const GemmLn* ln, bool weights_ready) {
     if (!ctx->encode_tiled) return cudaErrorNotSupported;
     if (ln && epi == EPI_SCORE && ln->stats_out && out_dtype == RS_BF16) epi = EPI_SCORE_STATS;
     if (ln && epi == EPI_BIAS && ln->stats_in) epi = EPI_BIAS_LN;
-    const int bn = pick_bn(M, N, ctx->sm_count);
+    const SmallPlan small = gemm_small_plan(M, N, K, ctx->sm_count);
+    const int bn = small.use ? kSmallBN : pick_bn(M, N, ctx->sm_count);
     const int out_bytes = (epi == EPI_RESID || (epi == EPI_SCORE && out_dtype == RS_F32)) ? 4 : 2;
     if (epi == EPI_SCORE_STATS && ln->stats_parts_out) *ln->stats_parts_out = 2 * (N / bn);
     CUtensorMap tmA, tmB, tmOut, tmRes;
-    if (epi == EPI_RESID && !row_map && !make_tmap_res(ctx, &tmRes, residual, (uint64_t)M, (uint64_t)N)) return cudaErrorInvalidValue;
+    if (epi == EPI_RESID && !row_map && !small.use && !make_tmap_res(ctx, &tmRes, residual, (uint64_t)M, (uint64_t)N)) return cudaErrorInvalidValue;
     if (!make_tmap_2d(ctx, &tmA, A, 2, (uint64_t)M, (uint64_t)K, BM) ||
-        !make_tmap_2d(ctx, &tmB, W, 2, (uint64_t)N, (uint64_t)K, (uint32_t)(bn / 2)) ||
-        !make_tmap_2d(ctx, &tmOut, out, out_bytes, (uint64_t)M, (uint64_t)N, 32))
+        !make_tmap_2d(ctx, &tmB, W, 2, (uint64_t)N, (uint64_t)K, (uint32_t)(small.use ? bn : bn / 2)) ||
+        (!small.use && !make_tmap_2d(ctx, &tmOut, out, out_bytes, (uint64_t)M, (uint64_t)N, 32)))
         return cudaErrorInvalidValue;
     if (epi != EPI_RESID || row_map) tmRes = tmOut;  // unused by the other epilogues and by the mapped residual
     GemmArgs args;
@@ -677,6 +625,7 @@ cudaError_t launch_gemm_tc(rs_ctx* ctx, int epi, const void* A, const void* W, c
     args.colsum = ln ? ln->colsum : nullptr;
     args.stats_parts = ln ? ln->stats_parts : 0;
     args.ln_eps = ln ? ln->eps : 0.f;
+    if (small.use) return launch_gemm_small(epi, tmA, tmB, args, small.splits, out, out_dtype, weights_ready, st);
     const int sms = ctx->sm_count;
 #define RS_GEMM_CASE(E, T)                                                                       \
     return bn == 256   ? launch_one<256, E, T>(tmA, tmB, tmOut, tmRes, args, sms, st)           \

@@ -77,9 +77,11 @@ inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // ---- memory-bound kernels (rs_elementwise.cu) ----
 // LayerNorm over the last dimension: x [T, D] (in_dtype) -> out [T, D] (out_dtype); fp32 math.
 // row_map (optional, [T] int32): output row t normalises input row row_map[t] instead of row t.
+// first: the first kernel of a call.  It lets its successor start only once its own predecessor has completed, so
+// that every later kernel of the call knows that what ran before the call (and may have written the weights) is done.
 cudaError_t launch_layernorm(rs_dtype in_dtype, rs_dtype out_dtype, const void* x, const float* gamma,
                              const float* beta, float eps, long long T, int D, void* out,
-                             const int32_t* row_map, cudaStream_t st);
+                             const int32_t* row_map, bool first, cudaStream_t st);
 // s[t] = D(after[t,:], before[t,:]).
 cudaError_t launch_shift_score(rs_dtype dtype, rs_dist dist, long long T, int D, const void* after,
                                const void* before, float* scores, cudaStream_t st);
@@ -135,7 +137,7 @@ void* tc_get_encode_fn();                       // cuTensorMapEncodeTiled via th
 bool tc_encode_cached(rs_ctx* ctx, CUtensorMap* out, const void* base, int rank, int dtype, const unsigned long long* dims,
                       const unsigned long long* strides, const unsigned int* box, int swizzle_bytes);
 bool gemm_tc_supported(long long M, int N, int K);
-int gemm_tc_score_parts(const rs_ctx* ctx, long long M, int N);   // partial sums per row written by RS_EPI_SCORE
+int gemm_tc_score_parts(const rs_ctx* ctx, long long M, int N, int K);   // partial sums per row written by RS_EPI_SCORE / RS_EPI_RESID
 // out[M, N] = epilogue(A[M, K] . W[N, K]^T); see rs_gemm_tc.cu for the epilogues.
 // row_map (optional, [M] int32): row t of the block input (the bf16 residual of RS_EPI_RESID, residual2
 // of RS_EPI_SCORE) is row row_map[t] of the given matrix -- the un-pruned output of the previous block.
@@ -153,10 +155,12 @@ struct GemmLn {
     const float* colsum;
     float eps;
 };
+// weights_ready: nothing that may still be running when this kernel starts writes W (every earlier kernel that
+// could has completed), so W may be read before the kernel waits for its predecessor.
 cudaError_t launch_gemm_tc(rs_ctx* ctx, int epi, const void* A, const void* W, const float* bias,
                            const void* residual, const void* residual2, const int32_t* row_map, void* out,
                            rs_dtype out_dtype, float* partials, int score_kind, int dist, long long M, int N, int K,
-                           cudaStream_t st, const GemmLn* ln = nullptr);
+                           cudaStream_t st, const GemmLn* ln = nullptr, bool weights_ready = false);
 
 // ---- tcgen05 attention (rs_attn_tc.cu): bf16, head dimension 64 ----
 bool attn_tc_supported(const rs_attn_desc& d);
