@@ -113,6 +113,11 @@ __device__ __forceinline__ float row_max64(const uint32_t (&r)[BKV], int valid) 
 
 // p_i = exp2(s_i * sl + mneg) for the first `valid` of the 64 keys (0 for the rest), packed to bf16
 // pairs in place (r[0 .. 32) on return); returns the sum of the unrounded p_i.
+// Six pairs of the 32 go through the FMA pipes: the special-function unit (8 cycles per warp and exponential) is the
+// busiest pipe of this kernel, and its idle time does not line up between the three warps of a scheduler.  4 x 16 x
+// 4097: 380 us with none, 379 / 371 / 368 / 371 / 382 with 2 / 5 / 6 / 8 / 11 pairs, 435 with all second pairs of four
+// elements; 16 x 12 x 1569 195 -> 190, 32 x 16 x 577 94.3 -> 91.4.  (In the two-tile kernel any share is slower: its two
+// warps per scheduler have no issue slots to spare for it.)
 template <bool MASKED>
 __device__ __forceinline__ float exp_pass64(uint32_t (&r)[BKV], float sl, float mneg, int valid) {
     const uint64_t sl2 = pack2(sl, sl), mneg2 = pack2(mneg, mneg);
@@ -128,7 +133,11 @@ __device__ __forceinline__ float exp_pass64(uint32_t (&r)[BKV], float sl, float 
             if (i + 2 >= valid) x2 = -INFINITY;
             if (i + 3 >= valid) x3 = -INFINITY;
         }
-        const float p0 = ex2(x0), p1 = ex2(x1), p2 = ex2(x2), p3 = ex2(x3);   // ex2(-inf) = 0
+        const float p0 = ex2(x0), p1 = ex2(x1);   // ex2(-inf) = 0
+        float p2, p3;
+        constexpr int kByFma = 0x52;                     // which of eight consecutive groups of four send their second pair there
+        if (!MASKED && ((kByFma >> ((i / 4) % 8)) & 1)) ex2_pair_fma(pack2(x2, x3), p2, p3);
+        else { p2 = ex2(x2); p3 = ex2(x3); }
         l01 = fadd2(l01, pack2(p0, p1));
         l23 = fadd2(l23, pack2(p2, p3));
         r[i >> 1] = pack_bf16(p0, p1);

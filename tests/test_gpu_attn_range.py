@@ -1,0 +1,28 @@
+"""Attention weights over the whole range of the exponential: rows whose scores lie up to hundreds of octaves below
+their maximum, maxima that rise from key tile to key tile, and sums of very many small weights."""
+import numpy as np
+import pytest
+import torch
+
+import parity
+from oracle import rs_oracle as orc
+from test_gpu_parts import ctx, pinned   # noqa: F401  (the module's context fixtures)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("kernel", [2, 3])
+@pytest.mark.parametrize("gain", [0.02, 1.0, 8.0, 30.0])
+def test_weights_over_the_range_of_exp2(pinned, kernel, gain):   # noqa: F811
+    B, N, H = 1, 450, 2
+    g = torch.Generator().manual_seed(int(gain * 100))
+    qkv = torch.randn(B, N, 3, H, 64, generator=g)
+    qkv[:, :, 0] *= gain                                         # scores with a standard deviation of `gain` nats
+    qkv[:, :, 1] *= torch.linspace(0.3, 1.7, N)[None, :, None, None]     # later keys reach higher
+    qkv = qkv.to(torch.bfloat16)
+    dq = qkv.cuda()
+    got = pinned[kernel].attn_fwd(dq[:, :, 0], dq[:, :, 1], dq[:, :, 2]).cpu().double().numpy()
+    f = qkv.double().numpy()
+    want = orc.attn(f[:, :, 0], f[:, :, 1], f[:, :, 2]).reshape(B, N, H * 64)
+    # weights rounded to bf16 (2^-9 each, they sum to one), values up to |v|max; one rounding of the output
+    assert np.abs(got - want).max() < (2.0 ** -8) * np.abs(f[:, :, 2]).max()
