@@ -3,6 +3,7 @@
 // token row; rows move as 16-byte vectors, several in flight per lane.
 #include "rs_internal.h"
 #include "rs_device.cuh"
+#include "rs_gemm.cuh"
 
 namespace rs {
 
@@ -18,7 +19,7 @@ template <typename TI, typename TO, int MAXV>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, MAXV <= 4 ? 5 : 4)
 layernorm_kernel(const TI* __restrict__ x, const float* __restrict__ gamma,
                  const float* __restrict__ beta, float eps, long long T, int D, TO* __restrict__ out,
-                 const int32_t* __restrict__ row_map, const int first) {
+                 const int32_t* __restrict__ row_map, const int first, const int32_t* __restrict__ lens, unsigned seq_n) {
     constexpr int VN = Vec16<TI>::N;
     if (!first) grid_dep_launch();
     grid_dep_wait();
@@ -26,6 +27,10 @@ layernorm_kernel(const TI* __restrict__ x, const float* __restrict__ gamma,
     const int lane = threadIdx.x & 31;
     const long long row = (long long)blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
     if (row >= T) return;
+    if (lens) {                                  // padding that neither the products nor attention read
+        const unsigned b = (unsigned)row / seq_n, i = (unsigned)row - b * seq_n;
+        if ((int)i >= max(__ldg(lens + b), 1) + gemm::kPadRows) return;
+    }
     const int nvec = D / VN;
     const long long src = row_map ? (long long)row_map[row] : row;
     const uint4* xr = reinterpret_cast<const uint4*>(x + src * D);
@@ -196,13 +201,13 @@ inline unsigned row_grid(long long rows) { return (unsigned)((rows + kWarpsPerCt
 
 template <typename TI, typename TO>
 cudaError_t ln_dispatch(const void* x, const float* g, const float* b, float eps, long long T, int D,
-                        void* out, const int32_t* row_map, bool first, cudaStream_t st) {
+                        void* out, const int32_t* row_map, bool first, cudaStream_t st, const int32_t* lens, int seq_n) {
     const int nvec = D / Vec16<TI>::N;
     const dim3 grid(row_grid(T)), block(kWarpsPerCta * 32);
     if (nvec <= 32 * 4)
-        return launch_pdl(layernorm_kernel<TI, TO, 4>, grid, block, 0, st, (const TI*)x, g, b, eps, T, D, (TO*)out, row_map, (int)first);
+        return launch_pdl(layernorm_kernel<TI, TO, 4>, grid, block, 0, st, (const TI*)x, g, b, eps, T, D, (TO*)out, row_map, (int)first, lens, (unsigned)seq_n);
     else if (nvec <= 32 * 8)
-        return launch_pdl(layernorm_kernel<TI, TO, 8>, grid, block, 0, st, (const TI*)x, g, b, eps, T, D, (TO*)out, row_map, (int)first);
+        return launch_pdl(layernorm_kernel<TI, TO, 8>, grid, block, 0, st, (const TI*)x, g, b, eps, T, D, (TO*)out, row_map, (int)first, lens, (unsigned)seq_n);
     return cudaErrorInvalidValue;
 }
 
@@ -210,12 +215,12 @@ cudaError_t ln_dispatch(const void* x, const float* g, const float* b, float eps
 
 cudaError_t launch_layernorm(rs_dtype in_dtype, rs_dtype out_dtype, const void* x, const float* gamma,
                              const float* beta, float eps, long long T, int D, void* out,
-                             const int32_t* row_map, bool first, cudaStream_t st) {
+                             const int32_t* row_map, bool first, cudaStream_t st, const int32_t* lens, int seq_n) {
     if (T == 0) return cudaSuccess;
-    if (in_dtype == RS_F32 && out_dtype == RS_F32) return ln_dispatch<float, float>(x, gamma, beta, eps, T, D, out, row_map, first, st);
-    if (in_dtype == RS_F32 && out_dtype == RS_BF16) return ln_dispatch<float, __nv_bfloat16>(x, gamma, beta, eps, T, D, out, row_map, first, st);
-    if (in_dtype == RS_BF16 && out_dtype == RS_BF16) return ln_dispatch<__nv_bfloat16, __nv_bfloat16>(x, gamma, beta, eps, T, D, out, row_map, first, st);
-    return ln_dispatch<__nv_bfloat16, float>(x, gamma, beta, eps, T, D, out, row_map, first, st);
+    if (in_dtype == RS_F32 && out_dtype == RS_F32) return ln_dispatch<float, float>(x, gamma, beta, eps, T, D, out, row_map, first, st, lens, seq_n);
+    if (in_dtype == RS_F32 && out_dtype == RS_BF16) return ln_dispatch<float, __nv_bfloat16>(x, gamma, beta, eps, T, D, out, row_map, first, st, lens, seq_n);
+    if (in_dtype == RS_BF16 && out_dtype == RS_BF16) return ln_dispatch<__nv_bfloat16, __nv_bfloat16>(x, gamma, beta, eps, T, D, out, row_map, first, st, lens, seq_n);
+    return ln_dispatch<__nv_bfloat16, float>(x, gamma, beta, eps, T, D, out, row_map, first, st, lens, seq_n);
 }
 
 cudaError_t launch_shift_score(rs_dtype dtype, rs_dist dist, long long T, int D, const void* after,

@@ -32,8 +32,13 @@ struct GemmArgs {
     const float* colsum;      // EPI_BIAS_LN: c [N]
     int stats_parts;
     float ln_eps;
+    const int* lens;          // optional [M / seq_n]: rows come as samples of seq_n, sample b's first lens[b] are in use;
+    int seq_n;                // rows past them (and past kPadRows more) need not be computed
     int* status;
 };
+// Rows behind a sample's own that are computed all the same: attention multiplies values of up to 15 of them by zero
+// weights, so they have to be finite.
+constexpr int kPadRows = 16;
 
 // Exact-erf GELU, v * Phi(v), to fp32 accuracy (max abs error 8e-7 over all v) without erff:
 // with q(t) = -log2(Phi(-t)) for t >= 0,  Phi(v) = 2^-q(|v|) for v < 0 and 1 - 2^-q(|v|) for

@@ -41,6 +41,21 @@ constexpr int A_BYTES = BM * BK * 2;          // 16 KB
 constexpr int STG_BYTES = 32 * 128;           // one staged output block of a warp: its 32 rows of 128 bytes
 constexpr int RES_BOX_BYTES = 32 * 64;         // residual of one 32-column chunk of a warp: 32 rows of 32 bf16
 
+// Batches with a count per sample: row tiles that hold padding alone are left out.  Up to this many row tiles of 256.
+constexpr int kMaskWords = 32, kMaskTiles = 32 * kMaskWords;
+// The k-th row tile in use, for a caller whose k never decreases.
+struct RowTiles {
+    const uint32_t* mask;    // null: all
+    int word = 0, before = 0;
+    __device__ __forceinline__ int at(int k) {
+        if (!mask) return k;
+        while (word < kMaskWords - 1 && before + __popc(mask[word]) <= k) before += __popc(mask[word++]);
+        uint32_t m = mask[word];
+        for (int i = before; i < k; ++i) m &= m - 1;
+        return word * 32 + __ffs(m) - 1;
+    }
+};
+
 // EPI_RESID brings the bf16 residual of a warp's rows in by TMA (a row per lane read straight from
 // global memory touches 32 lines per load instruction and cost a fifth of the projection's time):
 // one buffer per warp for a whole tile, loaded while the previous tile's main loop runs.  It pays
@@ -60,7 +75,8 @@ template <int BN, int EPI> struct Cfg {
     static constexpr int OFF_BAR = OFF_RES + kEpiWarps * RES_WARP_BYTES;
     static constexpr int OFF_BIAS = OFF_BAR + 256;                 // float [2 tile parities][2 halves][128]: bias slices
     static constexpr int OFF_COLSUM = OFF_BIAS + 2048;             // EPI_BIAS_LN: float [2][2][128] like the bias slices
-    static constexpr size_t SMEM = (size_t)OFF_BIAS + (LN ? 4096 : 2048);   // the window itself must be 1024-byte aligned
+    static constexpr int OFF_MASK = OFF_BIAS + (LN ? 4096 : 2048);  // one bit per row tile (batches with a count per sample)
+    static constexpr size_t SMEM = (size_t)OFF_MASK + kMaskWords * 4;   // the window itself must be 1024-byte aligned
     static_assert(SMEM <= 227 * 1024, "shared memory of one CTA");
 };
 
@@ -91,7 +107,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();     // 0 = leader of the pair
     const int num_m = (args.M + 2 * BM - 1) / (2 * BM), num_n = args.N / BN;
-    const int tiles = num_m * num_n, kblocks = args.K / BK;
+    const int kblocks = args.K / BK;
     const int pair = (int)cluster_id_x(), npairs = (int)cluster_count_x();
 
     if (threadIdx.x == 0) {
@@ -123,13 +139,31 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     grid_dep_launch();
     grid_dep_wait();
 
+    int tiles = num_m * num_n;
+    uint32_t* mask = args.lens ? reinterpret_cast<uint32_t*>(smem + C::OFF_MASK) : nullptr;
+    if (mask) {                                  // which row tiles hold rows in use (num_m <= kMaskTiles)
+        for (int t0 = warp * 32; t0 < kMaskTiles; t0 += kThreads) {
+            const int r0 = (t0 + lane) * 2 * BM, r1 = min(r0 + 2 * BM, args.M);
+            bool used = false;
+            for (int b = r0 / args.seq_n; r0 < args.M && b * args.seq_n < r1 && !used; ++b)
+                used = b * args.seq_n + min(min(max(__ldg(args.lens + b), 1), args.seq_n) + kPadRows, args.seq_n) > r0;
+            const uint32_t w = __ballot_sync(0xffffffffu, used);
+            if (lane == 0) mask[t0 / 32] = w;
+        }
+        __syncthreads();
+        tiles = 0;
+        for (int w = 0; w < kMaskWords; ++w) tiles += __popc(mask[w]);
+        tiles *= num_n;
+    }
+    RowTiles row_tiles = {mask};                 // (each role walks its own copy)
+
     if (warp == 0) {
         // ---------------- TMA producer (both CTAs; each loads its own halves) ----------------
         if (elect_one()) {
             uint32_t it = 0;
             bool ok = true;
             for (int tile = pair; tile < tiles && ok; tile += npairs) {
-                const int m0 = (tile / num_n) * (2 * BM) + (int)rank * BM;
+                const int m0 = row_tiles.at(tile / num_n) * (2 * BM) + (int)rank * BM;
                 const int n0 = (tile % num_n) * BN + (int)rank * (BN / 2);
                 for (int kb = 0; kb < kblocks; ++kb, ++it) {
                     const int s = it % C::STAGES;
@@ -194,8 +228,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // EPI_RESID: the residual of this warp's 32 rows x its half's columns of a tile, one 64-byte-
         // swizzled box per 32-column chunk (rows past M arrive as zeros)
         uint8_t* res_buf = smem + C::OFF_RES + (warp - 2) * C::RES_WARP_BYTES;
+        RowTiles ahead_tiles = row_tiles;                // the walk of what is fetched a tile ahead
         auto issue_res = [&](int tile) {
-            const int rm0 = (tile / num_n) * (2 * BM) + (int)rank * BM + q * 32, rn0 = (tile % num_n) * BN;
+            const int rm0 = ahead_tiles.at(tile / num_n) * (2 * BM) + (int)rank * BM + q * 32, rn0 = (tile % num_n) * BN;
             mbar_expect_tx(&res_full[warp - 2], (uint32_t)((c_end - c_begin) / 32) * RES_BOX_BYTES);
             for (int c = c_begin; c < c_end; c += 32)
                 tma_load_2d(res_buf + ((c - c_begin) / 32) * RES_BOX_BYTES, &tmRes, &res_full[warp - 2], rn0 + c, rm0);
@@ -204,7 +239,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // warp's row l; 16-byte asynchronous copies, a row's pieces by neighbouring lanes, land in the
         // layout the tensor map's 64-byte swizzle would give; rows past M are zero-filled.
         auto issue_res_mapped = [&](int tile) {      // whole warp
-            const int rm0 = (tile / num_n) * (2 * BM) + (int)rank * BM + q * 32, rn0 = (tile % num_n) * BN;
+            const int rm0 = ahead_tiles.at(tile / num_n) * (2 * BM) + (int)rank * BM + q * 32, rn0 = (tile % num_n) * BN;
             const int src_row = rm0 + lane < args.M ? __ldg(args.row_map + rm0 + lane) : -1;
             const int ppr = (c_end - c_begin) / 8, total = 32 * ppr;          // 16-byte pieces per row
             const __nv_bfloat16* base = reinterpret_cast<const __nv_bfloat16*>(args.residual) + rn0 + c_begin;
@@ -228,7 +263,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         constexpr int kLnPre = EPI == EPI_BIAS_LN ? 16 : 1;
         float2 ln_pre[kLnPre];
         auto ln_fetch = [&](int tile) {
-            const int frow = (tile / num_n) * (2 * BM) + (int)rank * BM + trow;
+            const int frow = (tile < tiles ? ahead_tiles.at(tile / num_n) : 0) * (2 * BM) + (int)rank * BM + trow;
             const bool ok = tile < tiles && frow < args.M && args.stats_parts <= kLnPre;
             const float2* sp = reinterpret_cast<const float2*>(args.stats_in) + (size_t)(ok ? frow : 0) * args.stats_parts;
 #pragma unroll
@@ -236,7 +271,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         };
         if (EPI == EPI_BIAS_LN) ln_fetch(pair);
         for (int tile = pair; tile < tiles; tile += npairs, ++tl) {
-            const int m0 = (tile / num_n) * (2 * BM) + (int)rank * BM, nt = tile % num_n, n0 = nt * BN;
+            const int m0 = row_tiles.at(tile / num_n) * (2 * BM) + (int)rank * BM, nt = tile % num_n, n0 = nt * BN;
             const uint32_t a = tl & 1u, aph = (tl >> 1) & 1u;
             const int row = m0 + trow;
             const bool valid = row < args.M;
@@ -602,7 +637,7 @@ int gemm_tc_score_parts(const rs_ctx* ctx, long long M, int N, int K) {
 cudaError_t launch_gemm_tc(rs_ctx* ctx, int epi, const void* A, const void* W, const float* bias,
                            const void* residual, const void* residual2, const int32_t* row_map, void* out, rs_dtype out_dtype,
                            float* partials, int score_kind, int dist, long long M, int N, int K, cudaStream_t st,
-                           const GemmLn* ln, bool weights_ready) {
+                           const GemmLn* ln, bool weights_ready, const GemmRows* rows) {
     if (!ctx->encode_tiled) return cudaErrorNotSupported;
     if (ln && epi == EPI_SCORE && ln->stats_out && out_dtype == RS_BF16) epi = EPI_SCORE_STATS;
     if (ln && epi == EPI_BIAS && ln->stats_in) epi = EPI_BIAS_LN;
@@ -625,6 +660,9 @@ cudaError_t launch_gemm_tc(rs_ctx* ctx, int epi, const void* A, const void* W, c
     args.colsum = ln ? ln->colsum : nullptr;
     args.stats_parts = ln ? ln->stats_parts : 0;
     args.ln_eps = ln ? ln->eps : 0.f;
+    const bool skips = rows && rows->lens && (M + 2 * BM - 1) / (2 * BM) <= kMaskTiles;
+    args.lens = skips ? rows->lens : nullptr;
+    args.seq_n = skips ? rows->seq_n : 0;
     if (small.use) return launch_gemm_small(epi, tmA, tmB, args, small.splits, out, out_dtype, weights_ready, st);
     const int sms = ctx->sm_count;
 #define RS_GEMM_CASE(E, T)                                                                       \

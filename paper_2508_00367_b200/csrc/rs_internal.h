@@ -77,11 +77,12 @@ inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // ---- memory-bound kernels (rs_elementwise.cu) ----
 // LayerNorm over the last dimension: x [T, D] (in_dtype) -> out [T, D] (out_dtype); fp32 math.
 // row_map (optional, [T] int32): output row t normalises input row row_map[t] instead of row t.
+// lens, seq_n (optional): as for the products below; rows that no kernel needs are left out.
 // first: the first kernel of a call.  It lets its successor start only once its own predecessor has completed, so
 // that every later kernel of the call knows that what ran before the call (and may have written the weights) is done.
 cudaError_t launch_layernorm(rs_dtype in_dtype, rs_dtype out_dtype, const void* x, const float* gamma,
                              const float* beta, float eps, long long T, int D, void* out,
-                             const int32_t* row_map, bool first, cudaStream_t st);
+                             const int32_t* row_map, bool first, cudaStream_t st, const int32_t* lens = nullptr, int seq_n = 0);
 // s[t] = D(after[t,:], before[t,:]).
 cudaError_t launch_shift_score(rs_dtype dtype, rs_dist dist, long long T, int D, const void* after,
                                const void* before, float* scores, cudaStream_t st);
@@ -155,12 +156,15 @@ struct GemmLn {
     const float* colsum;
     float eps;
 };
+// rows (optional): the rows are samples of seq_n of which the first lens[b] (dev) are in use; output rows past them
+// are unspecified, and whole tiles of them are not computed.
+struct GemmRows { const int32_t* lens; int seq_n; };
 // weights_ready: nothing that may still be running when this kernel starts writes W (every earlier kernel that
 // could has completed), so W may be read before the kernel waits for its predecessor.
 cudaError_t launch_gemm_tc(rs_ctx* ctx, int epi, const void* A, const void* W, const float* bias,
                            const void* residual, const void* residual2, const int32_t* row_map, void* out,
                            rs_dtype out_dtype, float* partials, int score_kind, int dist, long long M, int N, int K,
-                           cudaStream_t st, const GemmLn* ln = nullptr, bool weights_ready = false);
+                           cudaStream_t st, const GemmLn* ln = nullptr, bool weights_ready = false, const GemmRows* rows = nullptr);
 
 // ---- tcgen05 attention (rs_attn_tc.cu): bf16, head dimension 64 ----
 bool attn_tc_supported(const rs_attn_desc& d);

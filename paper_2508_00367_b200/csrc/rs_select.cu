@@ -149,7 +149,10 @@ select_kernel(const float* __restrict__ scores, int nparts, float* __restrict__ 
         key[e] = 0u;
         if (i < N) {
             float s;
-            if (nparts > 0) {              // partial sums from the GEMM epilogue
+            if (i >= n_b) {                // padding of a batch with a count per sample: its rows may not even have been computed
+                s = 0.f;
+                if (nparts > 0 && scores_out) scores_out[(long long)b * N + i] = s;
+            } else if (nparts > 0) {       // partial sums from the GEMM epilogue
                 s = finish_score(scores + ((long long)b * N + i) * partial_stride(nparts), nparts);
                 if (scores_out) scores_out[(long long)b * N + i] = s;
             } else {
