@@ -456,7 +456,7 @@ static rs_status block_fwd_impl(rs_ctx* ctx, const rs_block_desc* d, const rs_bl
         RS_CHECK_LAUNCH(ctx, RS_K_ATTN, st, rs::launch_attn_tc(ctx, ad, qkv, kp, vp, o, hk ? hk->seq_lens : nullptr, st), "attention");
         // shift through attention (operation choice (i)): partial sums of (SA(LN(x)) - x)^2 from this epilogue
         const bool attn_score = d->score_mode == RS_SCORE_ATTN;
-        nparts = rs::gemm_tc_score_parts(ctx, T, D, attn_score ? D : Dm);
+        nparts = rs::gemm_tc_score_parts(D);
         float* attn_parts = attn_score ? m : nullptr;
         RS_CHECK_LAUNCH(ctx, RS_K_GEMM, st, rs::launch_gemm_tc(ctx, rs::RS_EPI_RESID, o, w->w_o, w->b_o, x, nullptr, in_map, x_prime, RS_F32, attn_parts, 0, (int)d->dist, T, D, D, st, nullptr, true, &in_use), "proj");
     } else {
@@ -593,8 +593,8 @@ bool vit_plan(const rs_vit_desc& d, const int* drops, VitPlan* p) {
     p->block_ws = rs::align_up(block_ws, 256);
     p->act_bytes = rs::align_up((size_t)d.B * d.N * d.D * rs::dtype_size(d.dtype), 256);
     p->map_bytes = rs::align_up((size_t)d.B * d.N * sizeof(int32_t), 256);
-    // row sums for a LayerNorm folded into the next block's QKV: up to 2 * D / 64 pairs of floats per row
-    p->stats_bytes = rs::align_up((size_t)d.B * d.N * (2 * (size_t)d.D / 64 + 2) * 8, 256);
+    // row sums for a LayerNorm folded into the next block's QKV: up to D / 64 pairs of floats per row
+    p->stats_bytes = rs::align_up((size_t)d.B * d.N * ((size_t)d.D / 64 + 1) * 8, 256);
     // block scratch, two token buffers, one LN buffer, two row maps, two row-sum buffers
     p->total = p->block_ws + 3 * p->act_bytes + 2 * p->map_bytes + 2 * p->stats_bytes;
     p->n_final = n;

@@ -10,7 +10,7 @@
 namespace rs {
 namespace gemm {
 
-// EPI_SCORE_STATS: EPI_SCORE that also leaves, per row and column half of a tile, the sum and the sum of
+// EPI_SCORE_STATS: EPI_SCORE that also leaves, per row and 64 columns, the sum and the sum of
 // squares of the (rounded) output values -- the row statistics of the next block's LayerNorm.
 // EPI_BIAS_LN: the LayerNorm of the A operand folded into the product: with W' = W * gamma (column-wise),
 // c_n = sum_k W'_nk and b'_n = b_n + sum_k W_nk beta_k,  LN(x) W^T + b = rstd (x W'^T - mu c) + b';  mu and
@@ -24,10 +24,10 @@ struct GemmArgs {
     const void* residual2;    // EPI_SCORE, score_kind 2: bf16 [M, N] block input x
     const int* row_map;       // optional [M]: row t of the block input (EPI_RESID's residual, EPI_SCORE's residual2)
                               // is row row_map[t] of that matrix (the previous block's un-pruned output, read in place)
-    float* partials;          // EPI_SCORE (and EPI_RESID when non-null): [M, 2 * N / BN] sums of squares
+    float* partials;          // EPI_SCORE (and EPI_RESID when non-null): [M, N / 64] sums, one per 64 columns
     int score_kind;           // EPI_SCORE: scored pair (u, v) = 0: (m, x'), 1: (x^, x'), 2: (x^, x)
     int dist;                 // rs_dist of the score: L2 / L1 sums of (u - v)^2 / |u - v|, cosine sums of u.v, u.u, v.v
-    float* stats_out;         // EPI_SCORE_STATS: [M, 2 * N / BN][2] = (sum, sum of squares) of the row's outputs in that half tile
+    float* stats_out;         // EPI_SCORE_STATS: [M, N / 64][2] = (sum, sum of squares) of the row's outputs in those 64 columns
     const float* stats_in;    // EPI_BIAS_LN: such statistics of the A operand's rows, stats_parts pairs per row over ln_dim = K values
     const float* colsum;      // EPI_BIAS_LN: c [N]
     int stats_parts;

@@ -243,10 +243,10 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                 st2 = fmaf(y, y, st2);
             }
         }
-        // one set of sums per row and column half of the tile (eight lanes)
+        // one set of sums per row of the tile (sixteen lanes)
         if (SCORE || (EPI == EPI_RESID && args.partials)) {
 #pragma unroll
-            for (int o = 4; o > 0; o >>= 1) {
+            for (int o = 8; o > 0; o >>= 1) {
                 sq += __shfl_xor_sync(0xffffffffu, sq, o);
                 if (args.dist == RS_DIST_COS) {
                     sq1 += __shfl_xor_sync(0xffffffffu, sq1, o);
@@ -257,8 +257,8 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                     st2 += __shfl_xor_sync(0xffffffffu, st2, o);
                 }
             }
-            if (valid && (tid & 7) == 0) {
-                const size_t pi = (size_t)row * (2 * num_n) + 2 * blockIdx.y + ((tid >> 3) & 1);
+            if (valid && (tid & 15) == 0) {
+                const size_t pi = (size_t)row * num_n + blockIdx.y;
                 if (args.dist == RS_DIST_COS) {
                     args.partials[3 * pi] = sq; args.partials[3 * pi + 1] = sq1; args.partials[3 * pi + 2] = sq2;
                 } else {

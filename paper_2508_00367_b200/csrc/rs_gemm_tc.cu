@@ -56,6 +56,32 @@ struct RowTiles {
     }
 };
 
+// The list of work of a launch.  Whole tiles go to the pairs round robin; 256-wide tiles left for a last round that
+// half of the pairs or fewer would work on are cut in two, so that the round takes a part of a tile's time.  A
+// 128-column piece costs about 0.65 of a whole tile: it moves more operand bytes per FLOP and the ring's five stages hold
+// less of it in flight, which is why tiles are not narrow to begin with; quarters (0.75 to 0.9) gain nothing more.
+// 25104 x 768 x 3072 110 -> 98 us (one tile more than four rounds), 12608 x 768 x 768 24.1 -> 21.5.
+template <int BN> struct WorkList {
+    int full, rest, pieces, num_n;     // tiles of the full rounds, tiles of the last, the pieces of each of those, tiles per row tile
+    __device__ __forceinline__ WorkList(int tiles, int num_n_, int npairs) : num_n(num_n_) {
+        full = tiles / npairs * npairs;
+        rest = tiles - full;
+        pieces = BN == 256 && rest * 2 <= npairs ? 2 : 1;
+    }
+    __device__ __forceinline__ int count() const { return full + rest * pieces; }
+    struct Piece { int row_tile, n0, width; };
+    __device__ __forceinline__ Piece at(int i) const {
+        int tile = i, part = 0, width = BN;
+        if (i >= full && pieces > 1) {
+            tile = full + ((i - full) >> 1);
+            part = (i - full) & 1;
+            width = BN / 2;
+        }
+        const int mt = tile / num_n;
+        return {mt, (tile - mt * num_n) * BN + part * width, width};
+    }
+};
+
 // EPI_RESID brings the bf16 residual of a warp's rows in by TMA (a row per lane read straight from
 // global memory touches 32 lines per load instruction and cost a fifth of the projection's time):
 // one buffer per warp for a whole tile, loaded while the previous tile's main loop runs.  It pays
@@ -67,7 +93,7 @@ template <int BN, int EPI> struct Cfg {
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
     static constexpr int STAGES = (BN == 128) ? 6 : RES_TMA ? 4 : 5;
     static constexpr int TMEM_COLS = (BN == 128) ? 256 : 512;      // two accumulators, a power of two
-    static constexpr int SPLIT = (BN == 128) ? 64 : 128;           // epilogue warps 2-5 take columns [0, SPLIT)
+    static constexpr int SPLIT = (BN == 128) ? 64 : 128;           // epilogue warps 2-5 take columns [0, SPLIT) of a whole tile
     static constexpr int STG_PER_WARP = (RES_TMA || LN) ? 1 : 2;
     static constexpr int RES_WARP_BYTES = RES_TMA ? (SPLIT / 32) * RES_BOX_BYTES : 0;   // the wider half's chunks
     static constexpr int OFF_STG = STAGES * STAGE_BYTES;
@@ -83,8 +109,8 @@ template <int BN, int EPI> struct Cfg {
 template <int BN, int EPI, typename OutT>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-               const __grid_constant__ CUtensorMap tmOut, const __grid_constant__ CUtensorMap tmRes,
-               const GemmArgs args) {
+               const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ CUtensorMap tmOut,
+               const __grid_constant__ CUtensorMap tmRes, const GemmArgs args) {
     using C = Cfg<BN, EPI>;
     // The 128-byte swizzle wants 1024-byte aligned stage and staging buffers, and the layout leaves no
     // room to round the base up: a window that is not aligned is reported, and nothing else is done.
@@ -156,24 +182,27 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         tiles *= num_n;
     }
     RowTiles row_tiles = {mask};                 // (each role walks its own copy)
+    const WorkList<BN> list(tiles, num_n, npairs);
+    const int works = list.count();
 
     if (warp == 0) {
         // ---------------- TMA producer (both CTAs; each loads its own halves) ----------------
         if (elect_one()) {
             uint32_t it = 0;
             bool ok = true;
-            for (int tile = pair; tile < tiles && ok; tile += npairs) {
-                const int m0 = row_tiles.at(tile / num_n) * (2 * BM) + (int)rank * BM;
-                const int n0 = (tile % num_n) * BN + (int)rank * (BN / 2);
+            for (int i = pair; i < works && ok; i += npairs) {
+                const auto wk = list.at(i);
+                const int m0 = row_tiles.at(wk.row_tile) * (2 * BM) + (int)rank * BM;
+                const int n0 = wk.n0 + (int)rank * (wk.width / 2);
                 for (int kb = 0; kb < kblocks; ++kb, ++it) {
                     const int s = it % C::STAGES;
                     const uint32_t ph = (it / C::STAGES) & 1u;
                     if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag)) { ok = false; break; }
                     uint8_t* sa = smem + (size_t)s * C::STAGE_BYTES;
                     const uint32_t lead_full = map_to_cta(smem_u32(&full[s]), 0);
-                    if (rank == 0) mbar_expect_tx(&full[s], 2 * C::STAGE_BYTES);
+                    if (rank == 0) mbar_expect_tx(&full[s], 2 * A_BYTES + wk.width * BK * 2);
                     tma_load_2d_pair(sa, &tmA, lead_full, kb * BK, m0);
-                    tma_load_2d_pair(sa + A_BYTES, &tmB, lead_full, kb * BK, n0);
+                    tma_load_2d_pair(sa + A_BYTES, wk.width == BN ? &tmB : &tmBh, lead_full, kb * BK, n0);
                 }
             }
             // Every stage this thread filled must have been consumed (which implies its copies
@@ -188,10 +217,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     } else if (warp == 1) {
         // ---------------- MMA issuer (leader CTA only) ----------------
         if (rank == 0 && elect_one()) {
-            constexpr uint32_t idesc = idesc_bf16(2 * BM, BN, 0, 0);
             uint32_t it = 0, tl = 0;
             bool ok = true;
-            for (int tile = pair; tile < tiles && ok; tile += npairs, ++tl) {
+            for (int i = pair; i < works && ok; i += npairs, ++tl) {
+                const uint32_t idesc = idesc_bf16(2 * BM, list.at(i).width, 0, 0);
                 const uint32_t a = tl & 1u, aph = (tl >> 1) & 1u;
                 if (!mbar_wait(&tempty[a], aph ^ 1u, abort_flag)) { ok = false; break; }
                 tc_fence_after();
@@ -216,7 +245,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // ---------------- epilogue (both CTAs; each drains its own 128 x BN half) ----------------
         const int q = warp & 3;                          // TMEM lane quadrant this warp may read
         const int half = (warp - 2) >> 2;                // warps 2-5: columns [0, SPLIT), warps 6-9: the rest
-        const int c_begin = half ? C::SPLIT : 0, c_end = half ? BN : C::SPLIT;
+        // columns of a tile or piece that this half takes
+        int c_begin = 0, c_end = 0;
+        auto columns = [&](int width) {
+            const int split = width == BN ? C::SPLIT : BN / 4;
+            c_begin = half ? split : 0;
+            c_end = half ? width : split;
+        };
         constexpr int BLK_COLS = 128 / (int)sizeof(OutT);            // columns in one staged 128-byte row
         constexpr int CHUNKS_PER_BLK = BLK_COLS / 32;                // 32-column TMEM loads per staged block
         const int trow = q * 32 + lane;                  // row inside this CTA's half of the tile
@@ -229,8 +264,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // swizzled box per 32-column chunk (rows past M arrive as zeros)
         uint8_t* res_buf = smem + C::OFF_RES + (warp - 2) * C::RES_WARP_BYTES;
         RowTiles ahead_tiles = row_tiles;                // the walk of what is fetched a tile ahead
-        auto issue_res = [&](int tile) {
-            const int rm0 = ahead_tiles.at(tile / num_n) * (2 * BM) + (int)rank * BM + q * 32, rn0 = (tile % num_n) * BN;
+        auto issue_res = [&](int i) {
+            const auto wk = list.at(i);
+            const int rm0 = ahead_tiles.at(wk.row_tile) * (2 * BM) + (int)rank * BM + q * 32, rn0 = wk.n0;
+            columns(wk.width);
             mbar_expect_tx(&res_full[warp - 2], (uint32_t)((c_end - c_begin) / 32) * RES_BOX_BYTES);
             for (int c = c_begin; c < c_end; c += 32)
                 tma_load_2d(res_buf + ((c - c_begin) / 32) * RES_BOX_BYTES, &tmRes, &res_full[warp - 2], rn0 + c, rm0);
@@ -238,8 +275,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // The same boxes filled row by row through the row map: lane l looks up the source row of the
         // warp's row l; 16-byte asynchronous copies, a row's pieces by neighbouring lanes, land in the
         // layout the tensor map's 64-byte swizzle would give; rows past M are zero-filled.
-        auto issue_res_mapped = [&](int tile) {      // whole warp
-            const int rm0 = ahead_tiles.at(tile / num_n) * (2 * BM) + (int)rank * BM + q * 32, rn0 = (tile % num_n) * BN;
+        auto issue_res_mapped = [&](int i) {         // whole warp
+            const auto wk = list.at(i);
+            const int rm0 = ahead_tiles.at(wk.row_tile) * (2 * BM) + (int)rank * BM + q * 32, rn0 = wk.n0;
+            columns(wk.width);
             const int src_row = rm0 + lane < args.M ? __ldg(args.row_map + rm0 + lane) : -1;
             const int ppr = (c_end - c_begin) / 8, total = 32 * ppr;          // 16-byte pieces per row
             const __nv_bfloat16* base = reinterpret_cast<const __nv_bfloat16*>(args.residual) + rn0 + c_begin;
@@ -252,7 +291,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             }
             asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&res_full[warp - 2])) : "memory");
         };
-        if (C::RES_TMA && pair < tiles) {
+        if (C::RES_TMA && pair < works) {
             if (args.row_map) issue_res_mapped(pair);
             else if (lane == 0) issue_res(pair);
         }
@@ -262,16 +301,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // registers (up to kLnPre pairs; more are read on the spot), so their way from L2 is never waited for
         constexpr int kLnPre = EPI == EPI_BIAS_LN ? 16 : 1;
         float2 ln_pre[kLnPre];
-        auto ln_fetch = [&](int tile) {
-            const int frow = (tile < tiles ? ahead_tiles.at(tile / num_n) : 0) * (2 * BM) + (int)rank * BM + trow;
-            const bool ok = tile < tiles && frow < args.M && args.stats_parts <= kLnPre;
+        auto ln_fetch = [&](int i) {
+            const int frow = (i < works ? ahead_tiles.at(list.at(i).row_tile) : 0) * (2 * BM) + (int)rank * BM + trow;
+            const bool ok = i < works && frow < args.M && args.stats_parts <= kLnPre;
             const float2* sp = reinterpret_cast<const float2*>(args.stats_in) + (size_t)(ok ? frow : 0) * args.stats_parts;
 #pragma unroll
             for (int p = 0; p < kLnPre; ++p) ln_pre[p] = (ok && p < args.stats_parts) ? __ldg(sp + p) : make_float2(0.f, 0.f);
         };
         if (EPI == EPI_BIAS_LN) ln_fetch(pair);
-        for (int tile = pair; tile < tiles; tile += npairs, ++tl) {
-            const int m0 = row_tiles.at(tile / num_n) * (2 * BM) + (int)rank * BM, nt = tile % num_n, n0 = nt * BN;
+        const int slots = args.N / 64;                   // partial sums per row: one per 64 columns
+        for (int i = pair; i < works; i += npairs, ++tl) {
+            const auto wk = list.at(i);
+            const int m0 = row_tiles.at(wk.row_tile) * (2 * BM) + (int)rank * BM, n0 = wk.n0;
+            columns(wk.width);
             const uint32_t a = tl & 1u, aph = (tl >> 1) & 1u;
             const int row = m0 + trow;
             const bool valid = row < args.M;
@@ -297,7 +339,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 if (args.stats_parts <= kLnPre) {
 #pragma unroll
                     for (int p = 0; p < kLnPre; ++p) { s1 += ln_pre[p].x; s2 += ln_pre[p].y; }
-                    ln_fetch(tile + npairs);
+                    ln_fetch(i + npairs);
                 } else if (valid) {
                     const float2* sp = reinterpret_cast<const float2*>(args.stats_in) + (size_t)row * args.stats_parts;
                     for (int p = 0; p < args.stats_parts; ++p) {
@@ -465,24 +507,24 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     }
                     ++blk_ctr;
                 }
+                if ((c & 32) && (SCORE || (EPI == EPI_RESID && args.partials))) {      // 64 columns done: their sums
+                    const size_t pi = (size_t)row * slots + (col >> 6);
+                    if (valid) {
+                        if (EPI == EPI_SCORE_STATS) reinterpret_cast<float2*>(args.stats_out)[pi] = make_float2(st1, st2);
+                        if (args.dist == RS_DIST_COS) {
+                            args.partials[3 * pi] = sq; args.partials[3 * pi + 1] = sq1; args.partials[3 * pi + 2] = sq2;
+                        } else {
+                            args.partials[pi] = sq;
+                        }
+                    }
+                    st1 = st2 = sq = sq1 = sq2 = 0.f;
+                }
             }
             if (C::RES_TMA) {
                 __syncwarp();                            // every lane has read its residual rows
-                if (tile + npairs < tiles) {
-                    if (args.row_map) issue_res_mapped(tile + npairs);
-                    else if (lane == 0) issue_res(tile + npairs);
-                }
-            }
-            if (EPI == EPI_SCORE_STATS && valid) {
-                const size_t pi = (size_t)row * (2 * num_n) + 2 * nt + half;
-                reinterpret_cast<float2*>(args.stats_out)[pi] = make_float2(st1, st2);
-            }
-            if ((SCORE || (EPI == EPI_RESID && args.partials)) && valid) {
-                const size_t pi = (size_t)row * (2 * num_n) + 2 * nt + half;
-                if (args.dist == RS_DIST_COS) {
-                    args.partials[3 * pi] = sq; args.partials[3 * pi + 1] = sq1; args.partials[3 * pi + 2] = sq2;
-                } else {
-                    args.partials[pi] = sq;
+                if (i + npairs < works) {
+                    if (args.row_map) issue_res_mapped(i + npairs);
+                    else if (lane == 0) issue_res(i + npairs);
                 }
             }
         }
@@ -518,8 +560,8 @@ bool make_tmap_res(rs_ctx* ctx, CUtensorMap* out, const void* base, uint64_t row
 }
 
 template <int BN, int EPI, typename OutT>
-cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmOut, const CUtensorMap& tmRes,
-                       const GemmArgs& args, int sm_count, cudaStream_t st) {
+cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmBh, const CUtensorMap& tmOut,
+                       const CUtensorMap& tmRes, const GemmArgs& args, int sm_count, cudaStream_t st) {
     using C = Cfg<BN, EPI>;
     static PerDeviceOnce attr_once;   // per instantiation: the attribute is per function and per device
     int dev = -1;
@@ -530,7 +572,7 @@ cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUt
     });
     if (e != cudaSuccess) return e;
     const int tiles = ((args.M + 2 * BM - 1) / (2 * BM)) * (args.N / BN);
-    const int pairs = tiles < sm_count / 2 ? tiles : sm_count / 2;
+    const int most = BN == 256 ? 2 * tiles : tiles, pairs = most < sm_count / 2 ? most : sm_count / 2;     // (WorkList may cut tiles in two)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * pairs, 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
@@ -545,22 +587,20 @@ cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUt
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<BN, EPI, OutT>, tmA, tmB, tmOut, tmRes, args);
+    return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<BN, EPI, OutT>, tmA, tmB, tmBh, tmOut, tmRes, args);
 }
 
-// Tile width (256, 192 or 128 columns per pair): the one whose waves over the SM pairs cost
-// least, a wave of narrower tiles being charged a little more per column because it moves
-// more operand bytes per FLOP.
+// Tile width (256, 192 or 128 columns per pair): the one whose rounds over the SM pairs cost least (a round of 192- or
+// 128-wide tiles 0.83 or 0.58 of one of 256-wide ones, a last round of halves 0.65; see WorkList).
 int pick_bn(long long M, int N, int sm_count) {
     const long long pairs = sm_count / 2, mt = (M + 2 * BM - 1) / (2 * BM);
-    const int widths[3] = {256, 192, 128};
-    const int penalty[3] = {100, 110, 116};
+    const int widths[3] = {256, 192, 128}, round_cost[3] = {100, 83, 58};
     int best = 128;
     long long best_cost = -1;
     for (int i = 0; i < 3; ++i) {
         if (N % widths[i]) continue;
-        const long long waves = (mt * (N / widths[i]) + pairs - 1) / pairs;
-        const long long cost = waves * widths[i] * penalty[i];
+        const long long tiles = mt * (N / widths[i]), full = tiles / pairs, rest = tiles - full * pairs;
+        const long long cost = full * round_cost[i] + (rest == 0 ? 0 : widths[i] == 256 && rest * 2 <= pairs ? 65 : round_cost[i]);
         if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = widths[i]; }
     }
     return best;
@@ -630,9 +670,7 @@ bool gemm_tc_supported(long long M, int N, int K) {
     return M >= 1 && M < (1ll << 31) && N >= 128 && ((N % 128) == 0 || (N % 192) == 0) && K >= 64 && (K % 64) == 0;
 }
 
-int gemm_tc_score_parts(const rs_ctx* ctx, long long M, int N, int K) {
-    return 2 * (N / (gemm_small_plan(M, N, K, ctx->sm_count).use ? kSmallBN : pick_bn(M, N, ctx->sm_count)));
-}
+int gemm_tc_score_parts(int N) { return N / 64; }
 
 cudaError_t launch_gemm_tc(rs_ctx* ctx, int epi, const void* A, const void* W, const float* bias,
                            const void* residual, const void* residual2, const int32_t* row_map, void* out, rs_dtype out_dtype,
@@ -644,13 +682,15 @@ cudaError_t launch_gemm_tc(rs_ctx* ctx, int epi, const void* A, const void* W, c
     const SmallPlan small = gemm_small_plan(M, N, K, ctx->sm_count);
     const int bn = small.use ? kSmallBN : pick_bn(M, N, ctx->sm_count);
     const int out_bytes = (epi == EPI_RESID || (epi == EPI_SCORE && out_dtype == RS_F32)) ? 4 : 2;
-    if (epi == EPI_SCORE_STATS && ln->stats_parts_out) *ln->stats_parts_out = 2 * (N / bn);
-    CUtensorMap tmA, tmB, tmOut, tmRes;
+    if (epi == EPI_SCORE_STATS && ln->stats_parts_out) *ln->stats_parts_out = gemm_tc_score_parts(N);
+    CUtensorMap tmA, tmB, tmBh, tmOut, tmRes;
     if (epi == EPI_RESID && !row_map && !small.use && !make_tmap_res(ctx, &tmRes, residual, (uint64_t)M, (uint64_t)N)) return cudaErrorInvalidValue;
     if (!make_tmap_2d(ctx, &tmA, A, 2, (uint64_t)M, (uint64_t)K, BM) ||
         !make_tmap_2d(ctx, &tmB, W, 2, (uint64_t)N, (uint64_t)K, (uint32_t)(small.use ? bn : bn / 2)) ||
+        (bn == 256 && !make_tmap_2d(ctx, &tmBh, W, 2, (uint64_t)N, (uint64_t)K, 64)) ||
         (!small.use && !make_tmap_2d(ctx, &tmOut, out, out_bytes, (uint64_t)M, (uint64_t)N, 32)))
         return cudaErrorInvalidValue;
+    if (bn != 256) tmBh = tmB;                       // unused: only 256-wide tiles are cut
     if (epi != EPI_RESID || row_map) tmRes = tmOut;  // unused by the other epilogues and by the mapped residual
     GemmArgs args;
     args.M = (int)M; args.N = N; args.K = K; args.bias = bias; args.residual = residual;
@@ -666,9 +706,9 @@ cudaError_t launch_gemm_tc(rs_ctx* ctx, int epi, const void* A, const void* W, c
     if (small.use) return launch_gemm_small(epi, tmA, tmB, args, small.splits, out, out_dtype, weights_ready, st);
     const int sms = ctx->sm_count;
 #define RS_GEMM_CASE(E, T)                                                                       \
-    return bn == 256   ? launch_one<256, E, T>(tmA, tmB, tmOut, tmRes, args, sms, st)           \
-           : bn == 192 ? launch_one<192, E, T>(tmA, tmB, tmOut, tmRes, args, sms, st)           \
-                       : launch_one<128, E, T>(tmA, tmB, tmOut, tmRes, args, sms, st)
+    return bn == 256   ? launch_one<256, E, T>(tmA, tmB, tmBh, tmOut, tmRes, args, sms, st)           \
+           : bn == 192 ? launch_one<192, E, T>(tmA, tmB, tmBh, tmOut, tmRes, args, sms, st)           \
+                       : launch_one<128, E, T>(tmA, tmB, tmBh, tmOut, tmRes, args, sms, st)
     switch (epi) {
         case EPI_BIAS: RS_GEMM_CASE(EPI_BIAS, __nv_bfloat16);
         case EPI_BIAS_GELU: RS_GEMM_CASE(EPI_BIAS_GELU, __nv_bfloat16);

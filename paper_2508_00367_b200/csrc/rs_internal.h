@@ -138,7 +138,7 @@ void* tc_get_encode_fn();                       // cuTensorMapEncodeTiled via th
 bool tc_encode_cached(rs_ctx* ctx, CUtensorMap* out, const void* base, int rank, int dtype, const unsigned long long* dims,
                       const unsigned long long* strides, const unsigned int* box, int swizzle_bytes);
 bool gemm_tc_supported(long long M, int N, int K);
-int gemm_tc_score_parts(const rs_ctx* ctx, long long M, int N, int K);   // partial sums per row written by RS_EPI_SCORE / RS_EPI_RESID
+int gemm_tc_score_parts(int N);   // partial sums per row written by RS_EPI_SCORE / RS_EPI_RESID (one per 64 columns)
 // out[M, N] = epilogue(A[M, K] . W[N, K]^T); see rs_gemm_tc.cu for the epilogues.
 // row_map (optional, [M] int32): row t of the block input (the bf16 residual of RS_EPI_RESID, residual2
 // of RS_EPI_SCORE) is row row_map[t] of the given matrix -- the un-pruned output of the previous block.

@@ -18,8 +18,7 @@ namespace {
 // Score of one token from the partial sums the GEMM epilogues leave (fixed summation
 // order: run-to-run identical).  `enc` = number of partial sums | distance << 16.  L2: sqrt of the sum of
 // squares; L1: the sum; cosine: three sums per part (u.v, u.u, v.v) -> 1 - u.v / (|u||v|).
-// The number of parts is even (two column halves per tile) and the rows start on 8-byte boundaries; sixteen
-// parts are loaded before the first is added, so a token costs one round trip to L2 (adding as they came
+// Sixteen parts are loaded before the first is added, so a token costs one round trip to L2 (adding as they came
 // left two to four loads in flight and made the scores half of the selection's time).
 __device__ __forceinline__ float finish_score(const float* __restrict__ p, int enc) {
     const int nparts = enc & 0xffff, dist = enc >> 16;
@@ -28,16 +27,24 @@ __device__ __forceinline__ float finish_score(const float* __restrict__ p, int e
         for (int j = 0; j < nparts; ++j) { uv += p[3 * j]; uu += p[3 * j + 1]; vv += p[3 * j + 2]; }
         return 1.f - uv / fmaxf(sqrtf(uu) * sqrtf(vv), 1e-12f);
     }
-    const float2* p2 = reinterpret_cast<const float2*>(p);
     float acc = 0.f;
     for (int j0 = 0; j0 < nparts; j0 += 16) {
-        float2 v[8];
+        float v[16];
+        if ((nparts & 3) == 0) {             // rows start on 16-byte boundaries
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-            if (j0 + 2 * j < nparts) v[j] = __ldg(p2 + j0 / 2 + j);
+            for (int j = 0; j < 16; j += 4)
+                if (j0 + j < nparts) {
+                    const float4 t = __ldg(reinterpret_cast<const float4*>(p + j0 + j));
+                    v[j] = t.x; v[j + 1] = t.y; v[j + 2] = t.z; v[j + 3] = t.w;
+                }
+        } else {
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-            if (j0 + 2 * j < nparts) { acc += v[j].x; acc += v[j].y; }
+            for (int j = 0; j < 16; ++j)
+                if (j0 + j < nparts) v[j] = __ldg(p + j0 + j);
+        }
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+            if (j0 + j < nparts) acc += v[j];
     }
     return dist == RS_DIST_L1 ? acc : sqrtf(acc);
 }
