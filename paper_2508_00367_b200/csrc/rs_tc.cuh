@@ -284,9 +284,14 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t saddr, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
     return r;
 }
-// Arrive on an mbarrier given by a shared::cluster address (possibly in the peer CTA).
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+// Arrive on an mbarrier given by a shared::cluster address (possibly in the peer CTA), for what is ordered by other means:
+// no memory access of this thread is made visible by it.  The epilogues hand an accumulator back with it, whose reads
+// tcgen05.wait::ld has completed and tcgen05.fence::before_thread_sync has ordered.  The default, .release.cluster, also
+// waits for all earlier stores of the thread to be visible, staged and partial results among them: 2700 cycles a tile, half
+// of the plain epilogue's time and a quarter of the GELU one's.  Products of a block, with it / relaxed, us: QKV
+// 50432 x 576 x 192 23.5 / 17.8, projection 25216 x 768 x 768 40.2 / 35.6, FC1 25216 x 3072 x 768 87.2 / 79.0.
+__device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t cluster_addr) {
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // TMA load inside a CTA pair: the data lands in this CTA's shared memory, the completion
 // bytes are signalled on an mbarrier given by a shared::cluster address (the pair leader's).
