@@ -300,8 +300,34 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             if (args.row_map) issue_res_mapped(pair);
             else if (lane == 0) issue_res(pair);
         }
+        // The fp32 residual of the scoring epilogues: a warp fetches its 32 rows x 32 columns of the next chunk, the next
+        // tile's first one included, with neighbouring lanes on neighbouring 16-byte pieces of a row, into registers while
+        // it works on this one, and turns them over to one row per lane through the staging buffer that the results then
+        // replace.  A row read per lane from global memory touches 32 lines per load instruction: FC2 50432 x 192 x 768
+        // 34.2 -> 31.6 us, 25216 x 384 x 1536 40.8 -> 37.4, 25216 x 768 x 3072 98.6 -> 94.7, 16388 x 1024 x 4096 107.7 -> 105.
+        // (EPI_RESID's bf16 rows stay with TMA: this way 50432 x 192 x 192 took 22.6 us instead of 19.6.)
         constexpr bool SCORE = EPI == EPI_SCORE || EPI == EPI_SCORE_STATS;
-        constexpr int RES_VECS = EPI == EPI_RESID ? 4 : SCORE ? 8 : 1;   // 16-byte loads per 32 columns
+        constexpr int RES_VECS = EPI == EPI_RESID ? 4 : SCORE ? 8 : 1;   // 16-byte pieces per 32 columns of a row
+        uint4 res_next[RES_VECS];
+        auto load_res = [&](int m, int col) {            // rows past M: zeros
+            const char* base = reinterpret_cast<const char*>(args.residual) + (size_t)col * 4 + (lane & 7) * 16;
+#pragma unroll
+            for (int j = 0; j < RES_VECS; ++j) {
+                const int r = m + q * 32 + 4 * j + (lane >> 3);
+                res_next[j] = r < args.M ? __ldg(reinterpret_cast<const uint4*>(base + (size_t)r * args.N * 4)) : make_uint4(0u, 0u, 0u, 0u);
+            }
+        };
+        int m_next = 0, n_next = 0;                      // the next piece of work: its first row, this half's first column
+        auto look_ahead = [&](int i) {
+            if (!SCORE || i >= works) return;
+            const auto nw = list.at(i);
+            m_next = ahead_tiles.at(nw.row_tile) * (2 * BM) + (int)rank * BM;
+            n_next = nw.n0 + (half ? (nw.width == BN ? C::SPLIT : BN / 4) : 0);
+        };
+        if (SCORE && pair < works) {
+            look_ahead(pair);
+            load_res(m_next, n_next);
+        }
         // EPI_BIAS_LN: the partial row sums of this thread's row of the NEXT tile are fetched a tile ahead into
         // registers (up to kLnPre pairs; more are read on the spot), so their way from L2 is never waited for
         constexpr int kLnPre = EPI == EPI_BIAS_LN ? 16 : 1;
@@ -324,18 +350,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const bool valid = row < args.M;
             // row of the block input x (EPI_SCORE, whole-block shift), possibly through the row map
             const int xrow = (SCORE && args.score_kind == 2 && args.row_map && valid) ? __ldg(args.row_map + row) : row;
-            // Residual values of 32 columns of this thread's row (zeros for rows past M).  They are
-            // fetched one chunk ahead, the first chunk before the accumulator is even complete.
-            auto load_res = [&](int c, uint4* dst) {
-                if (SCORE) {
-                    const size_t off = (size_t)row * args.N + n0 + c;
-                    const uint4* rp = reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(args.residual) + off);
-#pragma unroll
-                    for (int j = 0; j < RES_VECS; ++j) dst[j] = valid ? __ldg(rp + j) : make_uint4(0u, 0u, 0u, 0u);
-                }
-            };
-            uint4 res_next[RES_VECS];
-            load_res(c_begin, res_next);
+            look_ahead(i + npairs);
             // EPI_BIAS_LN: mean and reciprocal standard deviation of this thread's row of A from the partial
             // sums its producer left (fetched while the accumulator is still being computed)
             float ln_mu = 0.f, ln_rstd = 0.f;
@@ -377,7 +392,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             for (int c = c_begin; c < c_end; c += 32) {
                 const int cb = (c / 32) % CHUNKS_PER_BLK;            // chunk inside the staged block
                 uint8_t* stg = smem + C::OFF_STG + ((warp - 2) * C::STG_PER_WARP + (C::STG_PER_WARP == 2 ? (blk_ctr & 1u) : 0u)) * STG_BYTES;
-                if (cb == 0) {
+                if (!SCORE && cb == 0) {
                     // the store that last read this buffer (two blocks ago, or the last one) must be done with it
                     if (lane == 0) tma_store_wait_read<C::STG_PER_WARP - 1>();
                     __syncwarp();
@@ -389,10 +404,25 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll
                     for (int j = 0; j < RES_VECS; ++j)
                         res[j] = *reinterpret_cast<const uint4*>(rrow + ((j ^ ((lane >> 1) & 3)) << 4));
-                } else {
+                } else if (SCORE) {
+                    // the residual passes through the buffer that takes the results, or, where two chunks share that
+                    // one (bf16 output), the second chunk's through the other, whose store must have been read by then
+                    constexpr bool SHARED = CHUNKS_PER_BLK == 2;
+                    uint8_t* tr = smem + C::OFF_STG + ((warp - 2) * 2 + ((blk_ctr + (uint32_t)cb) & 1u)) * STG_BYTES;
+                    if (!SHARED || cb) {
+                        if (lane == 0) tma_store_wait_read<SHARED ? 0 : 1>();
+                        __syncwarp();
+                    }
 #pragma unroll
-                    for (int j = 0; j < RES_VECS; ++j) res[j] = res_next[j];
-                    if (c + 32 < c_end) load_res(c + 32, res_next);
+                    for (int j = 0; j < RES_VECS; ++j) {
+                        const int rr = 4 * j + (lane >> 3);
+                        *reinterpret_cast<uint4*>(tr + rr * 128 + (((lane ^ rr) & 7) << 4)) = res_next[j];
+                    }
+                    __syncwarp();
+                    if (c + 32 < c_end) load_res(m0, n0 + c + 32);
+                    else if (i + npairs < works) load_res(m_next, n_next);
+#pragma unroll
+                    for (int j = 0; j < RES_VECS; ++j) res[j] = *reinterpret_cast<const uint4*>(tr + stg_row + ((j ^ r8) << 4));
                 }
                 uint32_t r[32];
                 __syncwarp();                            // tcgen05.ld is warp-collective
