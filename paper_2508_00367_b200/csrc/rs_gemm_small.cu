@@ -213,7 +213,7 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             v[e] = EPI == EPI_BIAS_LN ? fmaf(ln.y, fmaf(-ln.x, cv[e], v[e]), bv[e]) : v[e] + bv[e];
         if (EPI == EPI_BIAS_GELU) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) v[e] = gelu_erf(v[e]);
+            for (int e = 0; e < 4; e += 2) gelu_erf2(v[e], v[e + 1]);
         } else if (EPI == EPI_RESID) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) {

@@ -453,58 +453,59 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 }
                 if (EPI == EPI_BIAS_GELU) {
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] = gelu_erf(v[j]);
+                    for (int j = 0; j < 32; j += 2) gelu_erf2(v[j], v[j + 1]);
                 } else if (EPI == EPI_RESID) {
+                    float xs[32];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         const uint32_t w[4] = {res[j].x, res[j].y, res[j].z, res[j].w};
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
-                            const float x0 = __uint_as_float(w[e] << 16), x1 = __uint_as_float(w[e] & 0xffff0000u);
-                            if (args.partials) {                      // (u, v) = (SA(LN(x)), x)
-                                score_acc(args.dist, v[8 * j + 2 * e], x0, sq, sq1, sq2);
-                                score_acc(args.dist, v[8 * j + 2 * e + 1], x1, sq, sq1, sq2);
-                            }
-                            v[8 * j + 2 * e] += x0;
-                            v[8 * j + 2 * e + 1] += x1;
+                            xs[8 * j + 2 * e] = __uint_as_float(w[e] << 16);
+                            xs[8 * j + 2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
                         }
                     }
+                    if (args.partials)                                // (u, v) = (SA(LN(x)), x)
+                        with_dist(args.dist, [&](auto dist) {
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) score_acc(decltype(dist)::value, v[j], xs[j], sq, sq1, sq2);
+                        });
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) v[j] += xs[j];
                 } else if (SCORE) {
-                    if (args.score_kind == 2) {
-                        // whole-block shift: x^ - x, with the block input x read here (rows past M: zeros)
-                        const uint4* x0p = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(args.residual2) +
-                                                                          (size_t)xrow * args.N + col);
+                    float xs[32];
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const uint4 xv = valid ? __ldg(x0p + j) : make_uint4(0u, 0u, 0u, 0u);
-                            const uint32_t w[4] = {xv.x, xv.y, xv.z, xv.w};
-                            const float xp[8] = {__uint_as_float(res[2 * j].x), __uint_as_float(res[2 * j].y),
-                                                 __uint_as_float(res[2 * j].z), __uint_as_float(res[2 * j].w),
-                                                 __uint_as_float(res[2 * j + 1].x), __uint_as_float(res[2 * j + 1].y),
-                                                 __uint_as_float(res[2 * j + 1].z), __uint_as_float(res[2 * j + 1].w)};
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const float xa = __uint_as_float(w[e] << 16), xb = __uint_as_float(w[e] & 0xffff0000u);
-                                const float ya = v[8 * j + 2 * e] + xp[2 * e], yb = v[8 * j + 2 * e + 1] + xp[2 * e + 1];
-                                score_acc(args.dist, ya, xa, sq, sq1, sq2);
-                                score_acc(args.dist, yb, xb, sq, sq1, sq2);
-                                v[8 * j + 2 * e] = ya;
-                                v[8 * j + 2 * e + 1] = yb;
-                            }
-                        }
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const float xs[4] = {__uint_as_float(res[j].x), __uint_as_float(res[j].y),
-                                                 __uint_as_float(res[j].z), __uint_as_float(res[j].w)};
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const float m = v[4 * j + e], y = m + xs[e];
-                                score_acc(args.dist, args.score_kind ? y : m, xs[e], sq, sq1, sq2);
-                                v[4 * j + e] = y;
-                            }
-                        }
+                    for (int j = 0; j < 8; ++j) {
+                        xs[4 * j] = __uint_as_float(res[j].x); xs[4 * j + 1] = __uint_as_float(res[j].y);
+                        xs[4 * j + 2] = __uint_as_float(res[j].z); xs[4 * j + 3] = __uint_as_float(res[j].w);
                     }
+                    with_dist(args.dist, [&](auto dist) {
+                        if (args.score_kind == 2) {
+                            // whole-block shift: x^ - x, with the block input x read here (rows past M: zeros)
+                            const uint4* x0p = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(args.residual2) +
+                                                                              (size_t)xrow * args.N + col);
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const uint4 xv = valid ? __ldg(x0p + j) : make_uint4(0u, 0u, 0u, 0u);
+                                const uint32_t w[4] = {xv.x, xv.y, xv.z, xv.w};
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    float* y = v + 8 * j + 2 * e;
+                                    y[0] += xs[8 * j + 2 * e];
+                                    y[1] += xs[8 * j + 2 * e + 1];
+                                    score_acc(decltype(dist)::value, y[0], __uint_as_float(w[e] << 16), sq, sq1, sq2);
+                                    score_acc(decltype(dist)::value, y[1], __uint_as_float(w[e] & 0xffff0000u), sq, sq1, sq2);
+                                }
+                            }
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) {
+                                const float m = v[j];
+                                v[j] = m + xs[j];
+                                score_acc(decltype(dist)::value, args.score_kind ? v[j] : m, xs[j], sq, sq1, sq2);
+                            }
+                        }
+                    });
                 }
                 // stage the 32 values of this row: 16-byte pieces, XOR-swizzled like the TMA box
                 if (sizeof(OutT) == 2) {

@@ -1,0 +1,43 @@
+"""Epilogues of the tensor-core products: GELU over its range and at values that are not finite, and every score at row
+counts that stay with the pair-tile kernel (a last row tile of nine rows, output in both types)."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import parity
+from oracle import rs_oracle as orc
+from paper_2508_00367_b200 import synth
+from test_gpu_block import _np, _run_block, ctx   # noqa: F401  (the module's context fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M", [130, 16500])
+def test_gelu_range(ctx, M):   # noqa: F811
+    v = torch.linspace(-9.0, 9.0, M * 128).reshape(M, 128).bfloat16()
+    v[0, :8] = torch.tensor([0.0, -0.0, 30.0, -30.0, 1e4, -1e4, 3e38, -3e38]).bfloat16()
+    b = torch.zeros(128)
+    b[125], b[126], b[127] = math.inf, -math.inf, math.nan
+    got = ctx.linear_fwd(v.cuda(), torch.eye(128).bfloat16().cuda(), b.cuda(), "gelu").cpu().double()
+    want = orc.gelu(v.double().numpy())
+    # half a unit in the last place of a bf16 (8 significant bits: 2^-8 of the value at most), and 1e-6 of the polynomial
+    err = np.abs(got.numpy() - want)[:, :125] - 2.0 ** -8 * np.abs(want[:, :125])
+    assert err.max() < 1e-6, err.max()
+    assert (got[:, 125] == math.inf).all() and (got[:, 126] == 0).all() and got[:, 127].isnan().all()
+
+
+@pytest.mark.parametrize("out", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("mode,dist", [("mlp", "l2"), ("mlp", "cos"), ("mlp_delta", "l1"), ("attn", "l1"), ("attn", "cos"), ("block", "l2")])
+def test_block_pair_tiles_every_score(ctx, mode, dist, out):   # noqa: F811
+    B, N, D, H, r = 9, 257, 384, 6, 40
+    x, w = synth.make_tokens(B, N, D, "bf16", seed=11), synth.make_block_weights(D, 4 * D, "bf16", seed=12)
+    ref = orc.block_fwd(x.double().numpy(), _np(w), H, r, score_mode=mode, dist=dist)
+    res = _run_block(ctx, x, w, H, r, "bf16", out, score_mode=mode, dist=dist)
+    rounded = out == torch.bfloat16
+    parity.check_float(res["x_full"].double().numpy(), orc.round_to(ref["x_hat"], "bf16") if rounded else ref["x_hat"], "bf16", rounded)
+    # 5e-4 where the exact x' dominates the distance, else sums of bf16-operand products alone; |m| is a tenth of |x'|
+    tol = 5e-4 if (mode, dist) == ("mlp", "l2") else 3e-3 if mode == "mlp_delta" else 2e-3
+    rel = np.abs(res["scores"].double().numpy() - ref["scores"]) / np.abs(ref["scores"])
+    assert rel.max() < tol, rel.max()
