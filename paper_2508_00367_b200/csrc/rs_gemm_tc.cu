@@ -419,8 +419,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         *reinterpret_cast<uint4*>(tr + rr * 128 + (((lane ^ rr) & 7) << 4)) = res_next[j];
                     }
                     __syncwarp();
-                    if (c + 32 < c_end) load_res(m0, n0 + c + 32);
-                    else if (i + npairs < works) load_res(m_next, n_next);
 #pragma unroll
                     for (int j = 0; j < RES_VECS; ++j) res[j] = *reinterpret_cast<const uint4*>(tr + stg_row + ((j ^ r8) << 4));
                 }
@@ -432,6 +430,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive_cluster_relaxed(lead_tempty[a]);
+                }
+                if (SCORE) {
+                    if (c + 32 < c_end) load_res(m0, n0 + c + 32);
+                    else if (i + npairs < works) load_res(m_next, n_next);
                 }
                 const int col = n0 + c;
                 float v[32];
