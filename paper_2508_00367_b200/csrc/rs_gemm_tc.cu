@@ -83,19 +83,20 @@ template <int BN> struct WorkList {
 };
 
 // EPI_RESID brings the bf16 residual of a warp's rows in by TMA (a row per lane read straight from
-// global memory touches 32 lines per load instruction and cost a fifth of the projection's time):
-// one buffer per warp for a whole tile, loaded while the previous tile's main loop runs.  It pays
-// for the room with one staging buffer per warp instead of two and one operand stage less.
+// global memory touches 32 lines per load instruction and cost a fifth of the projection's time), two chunks of
+// 32 columns ahead, the next tile's first ones included.  It pays for the room with one operand stage less.  (A whole tile's boxes at a
+// time left room for one staging buffer per warp only, and a third of the epilogue waited for it: 50432 x 192 x 192
+// 19.5 -> 18.8 us, 25216 x 384 x 384 20.0 -> 19.2, 6924 x 1024 x 1024 21.5 -> 21.0.)
 template <int BN, int EPI> struct Cfg {
     static constexpr bool RES_TMA = EPI == EPI_RESID;
     static constexpr bool LN = EPI == EPI_BIAS_LN;                 // one staging buffer per warp, room for a second column vector
     static constexpr int B_BYTES = (BN / 2) * BK * 2;              // this CTA's half of the W tile
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-    static constexpr int STAGES = (BN == 128) ? 6 : RES_TMA ? 4 : 5;
+    static constexpr int STAGES = (BN == 128 ? 6 : 5) - (RES_TMA ? 1 : 0);
     static constexpr int TMEM_COLS = (BN == 128) ? 256 : 512;      // two accumulators, a power of two
     static constexpr int SPLIT = (BN == 128) ? 64 : 128;           // epilogue warps 2-5 take columns [0, SPLIT) of a whole tile
-    static constexpr int STG_PER_WARP = (RES_TMA || LN) ? 1 : 2;
-    static constexpr int RES_WARP_BYTES = RES_TMA ? (SPLIT / 32) * RES_BOX_BYTES : 0;   // the wider half's chunks
+    static constexpr int STG_PER_WARP = LN ? 1 : 2;
+    static constexpr int RES_WARP_BYTES = RES_TMA ? 2 * RES_BOX_BYTES : 0;
     static constexpr int OFF_STG = STAGES * STAGE_BYTES;
     static constexpr int OFF_RES = OFF_STG + kEpiWarps * STG_PER_WARP * STG_BYTES;
     static constexpr int OFF_BAR = OFF_RES + kEpiWarps * RES_WARP_BYTES;
@@ -128,7 +129,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * C::STAGES + 4);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile int* half_fail = reinterpret_cast<volatile int*>(tmem_slot + 2);   // [2]
-    uint64_t* res_full = bars + 2 * C::STAGES + 6;   // [kEpiWarps] the warp's residual of a tile landed (EPI_RESID)
+    uint64_t* res_full = bars + 2 * C::STAGES + 6;   // [kEpiWarps][2] a chunk of the warp's residual landed (EPI_RESID)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();     // 0 = leader of the pair
@@ -145,7 +146,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (C::RES_TMA) {
             prefetch_tmap(&tmRes);
             // one arrival by the lane that starts the TMA copies, or one by each lane's own indexed copies
-            for (int w = 0; w < kEpiWarps; ++w) mbar_init(&res_full[w], args.row_map ? 32 : 1);
+            for (int w = 0; w < 2 * kEpiWarps; ++w) mbar_init(&res_full[w], args.row_map ? 32 : 1);
         }
         *abort_flag = 0;
         half_fail[0] = 0;
@@ -265,41 +266,33 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // 16400 x 2304 x 768 40.9 / 39.4, 16156 x 3072 x 1024 67.8 / 65.7; with less K the epilogue is:
         // 25216 x 1536 x 512 31.5 / 32.3, x 1152 x 384 23.1 / 26.8.  The other epilogues pace themselves by their arithmetic and residuals.
         const bool paced = (EPI == EPI_BIAS || EPI == EPI_BIAS_LN) && kblocks >= 12;
-        // EPI_RESID: the residual of this warp's 32 rows x its half's columns of a tile, one 64-byte-
-        // swizzled box per 32-column chunk (rows past M arrive as zeros)
+        // EPI_RESID: the residual of this warp's 32 rows x 32 columns, two 64-byte-swizzled boxes in turn
+        // (rows past M arrive as zeros)
         uint8_t* res_buf = smem + C::OFF_RES + (warp - 2) * C::RES_WARP_BYTES;
+        uint64_t* res_bar = res_full + (warp - 2) * 2;
         RowTiles ahead_tiles = row_tiles;                // the walk of what is fetched a tile ahead
-        auto issue_res = [&](int i) {
-            const auto wk = list.at(i);
-            const int rm0 = ahead_tiles.at(wk.row_tile) * (2 * BM) + (int)rank * BM + q * 32, rn0 = wk.n0;
-            columns(wk.width);
-            mbar_expect_tx(&res_full[warp - 2], (uint32_t)((c_end - c_begin) / 32) * RES_BOX_BYTES);
-            for (int c = c_begin; c < c_end; c += 32)
-                tma_load_2d(res_buf + ((c - c_begin) / 32) * RES_BOX_BYTES, &tmRes, &res_full[warp - 2], rn0 + c, rm0);
-        };
-        // The same boxes filled row by row through the row map: lane l looks up the source row of the
-        // warp's row l; 16-byte asynchronous copies, a row's pieces by neighbouring lanes, land in the
-        // layout the tensor map's 64-byte swizzle would give; rows past M are zero-filled.
-        auto issue_res_mapped = [&](int i) {         // whole warp
-            const auto wk = list.at(i);
-            const int rm0 = ahead_tiles.at(wk.row_tile) * (2 * BM) + (int)rank * BM + q * 32, rn0 = wk.n0;
-            columns(wk.width);
-            const int src_row = rm0 + lane < args.M ? __ldg(args.row_map + rm0 + lane) : -1;
-            const int ppr = (c_end - c_begin) / 8, total = 32 * ppr;          // 16-byte pieces per row
-            const __nv_bfloat16* base = reinterpret_cast<const __nv_bfloat16*>(args.residual) + rn0 + c_begin;
-            for (int idx = lane; idx < total; idx += 32) {
-                const int r = idx / ppr, piece = idx - r * ppr;
-                const int sr = __shfl_sync(0xffffffffu, src_row, r);
-                const uint32_t dst = smem_u32(res_buf + (piece >> 2) * RES_BOX_BYTES + r * 64 + (((piece & 3) ^ ((r >> 1) & 3)) << 4));
-                const __nv_bfloat16* src = base + (size_t)(sr < 0 ? 0 : sr) * args.N + piece * 8;
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(sr < 0 ? 0 : 16) : "memory");
+        int m_next = 0, n_next = 0, map_cur = -1, map_next = -1;     // the next piece of work: its first row, this half's first column,
+                                                                     // and (row map) the source row of the warp's row `lane`
+        // With a row map the box is filled row by row: 16-byte asynchronous copies, a row's pieces by neighbouring
+        // lanes, land in the layout the tensor map's 64-byte swizzle would give; rows past M are zero-filled.
+        auto issue_res = [&](uint32_t buf, int m, int col, int map) {    // whole warp
+            uint8_t* box = res_buf + buf * RES_BOX_BYTES;
+            if (!args.row_map) {
+                if (lane == 0) {
+                    mbar_expect_tx(&res_bar[buf], RES_BOX_BYTES);
+                    tma_load_2d(box, &tmRes, &res_bar[buf], col, m + q * 32);
+                }
+                return;
             }
-            asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&res_full[warp - 2])) : "memory");
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int r = t * 8 + (lane >> 2), piece = lane & 3, sr = __shfl_sync(0xffffffffu, map, r);
+                const __nv_bfloat16* src = reinterpret_cast<const __nv_bfloat16*>(args.residual) + (size_t)(sr < 0 ? 0 : sr) * args.N + col + piece * 8;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(box + r * 64 + ((piece ^ ((r >> 1) & 3)) << 4))), "l"(src),
+                             "r"(sr < 0 ? 0 : 16) : "memory");
+            }
+            asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&res_bar[buf])) : "memory");
         };
-        if (C::RES_TMA && pair < works) {
-            if (args.row_map) issue_res_mapped(pair);
-            else if (lane == 0) issue_res(pair);
-        }
         // The fp32 residual of the scoring epilogues: a warp fetches its 32 rows x 32 columns of the next chunk, the next
         // tile's first one included, with neighbouring lanes on neighbouring 16-byte pieces of a row, into registers while
         // it works on this one, and turns them over to one row per lane through the staging buffer that the results then
@@ -317,17 +310,26 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 res_next[j] = r < args.M ? __ldg(reinterpret_cast<const uint4*>(base + (size_t)r * args.N * 4)) : make_uint4(0u, 0u, 0u, 0u);
             }
         };
-        int m_next = 0, n_next = 0;                      // the next piece of work: its first row, this half's first column
         auto look_ahead = [&](int i) {
-            if (!SCORE || i >= works) return;
+            if (!(SCORE || C::RES_TMA) || i >= works) return;
             const auto nw = list.at(i);
             m_next = ahead_tiles.at(nw.row_tile) * (2 * BM) + (int)rank * BM;
             n_next = nw.n0 + (half ? (nw.width == BN ? C::SPLIT : BN / 4) : 0);
+            if (C::RES_TMA && args.row_map) {
+                const int r = m_next + q * 32 + lane;
+                map_next = r < args.M ? __ldg(args.row_map + r) : -1;
+            }
         };
-        if (SCORE && pair < works) {
+        if ((SCORE || C::RES_TMA) && pair < works) {
             look_ahead(pair);
-            load_res(m_next, n_next);
+            if (SCORE) {
+                load_res(m_next, n_next);
+            } else {
+                issue_res(0, m_next, n_next, map_next);          // (a half has at least two chunks)
+                issue_res(1, m_next, n_next + 32, map_next);
+            }
         }
+        uint32_t res_ctr = 0;                            // chunks of the residual walked through
         // EPI_BIAS_LN: the partial row sums of this thread's row of the NEXT tile are fetched a tile ahead into
         // registers (up to kLnPre pairs; more are read on the spot), so their way from L2 is never waited for
         constexpr int kLnPre = EPI == EPI_BIAS_LN ? 16 : 1;
@@ -350,6 +352,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const bool valid = row < args.M;
             // row of the block input x (EPI_SCORE, whole-block shift), possibly through the row map
             const int xrow = (SCORE && args.score_kind == 2 && args.row_map && valid) ? __ldg(args.row_map + row) : row;
+            map_cur = map_next;
             look_ahead(i + npairs);
             // EPI_BIAS_LN: mean and reciprocal standard deviation of this thread's row of A from the partial
             // sums its producer left (fetched while the accumulator is still being computed)
@@ -382,7 +385,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             float* cs_s = reinterpret_cast<float*>(smem + C::OFF_COLSUM) + (tl & 1u) * 256 + half * 128;   // EPI_BIAS_LN only
             if (EPI == EPI_BIAS_LN && c_begin + t128 < c_end) cs_s[t128] = __ldg(args.colsum + n0 + c_begin + t128);
             if (!__all_sync(0xffffffffu, mbar_wait(&tfull[a], aph, abort_flag))) half_fail[half] = 1;
-            if (C::RES_TMA && !__all_sync(0xffffffffu, mbar_wait(&res_full[warp - 2], tl & 1u, abort_flag))) half_fail[half] = 1;
             named_barrier(1 + half, 128);
             if (half_fail[half]) break;
             tc_fence_after();
@@ -394,16 +396,27 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 uint8_t* stg = smem + C::OFF_STG + ((warp - 2) * C::STG_PER_WARP + (C::STG_PER_WARP == 2 ? (blk_ctr & 1u) : 0u)) * STG_BYTES;
                 if (!SCORE && cb == 0) {
                     // the store that last read this buffer (two blocks ago, or the last one) must be done with it
-                    if (lane == 0) tma_store_wait_read<C::STG_PER_WARP - 1>();
+                    if (lane == 0) {
+                        // (paced like the plain epilogues: 16156 x 1024 x 1024 34.0 us so, 35.2 with two stores in flight, as one before)
+                        if (EPI == EPI_RESID && kblocks >= 16) tma_store_wait_read<0>();
+                        else tma_store_wait_read<C::STG_PER_WARP - 1>();
+                    }
                     __syncwarp();
                 }
                 uint4 res[RES_VECS];
                 if (C::RES_TMA) {
-                    // this lane's row of the chunk's box: 64 bytes, 16-byte pieces XOR-ed with address bits 7-8
-                    const uint8_t* rrow = res_buf + ((c - c_begin) / 32) * RES_BOX_BYTES + lane * 64;
+                    // this lane's row of the chunk's box: 64 bytes, 16-byte pieces XOR-ed with address bits 7-8; then the
+                    // box two chunks on takes its place.  (On a time-out the values are void, and the next tile's wait ends the loop.)
+                    const uint32_t buf = res_ctr & 1u;
+                    mbar_wait(&res_bar[buf], (res_ctr >> 1) & 1u, abort_flag);
+                    const uint8_t* rrow = res_buf + buf * RES_BOX_BYTES + lane * 64;
 #pragma unroll
                     for (int j = 0; j < RES_VECS; ++j)
                         res[j] = *reinterpret_cast<const uint4*>(rrow + ((j ^ ((lane >> 1) & 3)) << 4));
+                    ++res_ctr;
+                    __syncwarp();
+                    if (c + 64 < c_end) issue_res(buf, m0, n0 + c + 64, map_cur);
+                    else if (i + npairs < works) issue_res(buf, m_next, n_next + (c + 64 - c_end), map_next);
                 } else if (SCORE) {
                     // the residual passes through the buffer that takes the results, or, where two chunks share that
                     // one (bf16 output), the second chunk's through the other, whose store must have been read by then
@@ -557,13 +570,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         }
                     }
                     st1 = st2 = sq = sq1 = sq2 = 0.f;
-                }
-            }
-            if (C::RES_TMA) {
-                __syncwarp();                            // every lane has read its residual rows
-                if (i + npairs < works) {
-                    if (args.row_map) issue_res_mapped(i + npairs);
-                    else if (lane == 0) issue_res(i + npairs);
                 }
             }
         }
