@@ -497,7 +497,8 @@ bool attn_tc_supported(const rs_attn_desc& d) {
 // This kernel or the one with three query tiles per CTA (rs_attn_tc3.cu)?  Both are paced by the longest
 // CTA: its items (in tenths) times the key tiles of an item, plus a cost per item; microseconds fitted to
 // CUDA-event times of thirteen shapes from N = 197 to 4097 (worst error 6 % and 9 %).  (Since the three-tile kernel
-// sends a part of its exponentials through the FMA pipes it runs 3 % under its line; the lines stay.)
+// sends a part of its exponentials through the FMA pipes it runs 3 % under its line, and up to 17 % under it where its items
+// run across heads; the lines stay.)
 AttnPlan attn_plan(long long BH, int N, int G) {
     const int nt = (N + BQ - 1) / BQ, per = (N + 2 * BQ - 1) / (2 * BQ);
     auto makespan = [&](long long hs) {

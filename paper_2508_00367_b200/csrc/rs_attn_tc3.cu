@@ -8,7 +8,7 @@
 // bounds the kernel, and what keeps that unit from saturating is the serial chain of each
 // softmax warp; three warps per scheduler instead of two fill more of its gaps.
 // An item is three consecutive 128-row query tiles of one (sample, head), which share the K/V
-// tiles streamed through the TMA ring.
+// tiles streamed through the TMA ring; or (ACROSS) of consecutive (sample, head)s.
 #include <math.h>
 
 #include "rs_internal.h"
@@ -43,42 +43,55 @@ constexpr size_t kSmem = (size_t)OFF_BAR + 512 + 1024 /*alignment slack*/;
 static_assert(kOCol + NG * DH <= kTmemCols, "tensor-memory columns");
 static_assert(kSmem <= 232448, "shared memory of one CTA");
 
-// Items: first the groups of three query tiles of every (sample, head) -- n3 of them, per3 to a head --
+// Items within heads: first the groups of three query tiles of every (sample, head) -- n3 of them, per3 to a head --
 // then, where the tile count is not a multiple of three, one item per head with the tail_ng tiles left
 // over (n_tail of them).  CTA c takes the groups c, c + G, ... and then tails: tail number
 // tail_pos + k * tail_stride for k = 0, 1, ..., where tail_pos = c - tail_first (CTAs before tail_first
 // take none, unless the tails wrap around: tail_wrap = 1, position (c - tail_first) mod G).
+// Items ACROSS heads: three tiles in a row whichever heads they belong to, so that the tails do not leave warpgroups
+// idle; an item that meets a head's end takes two K/V streams, a tile of each head in turn.  CTA c takes the items
+// c, c + G, ...; the tiles of the last round go one to an item where there are CTAs enough.
 struct Attn3Args {
     int N, H;
     int per3, n3, n_tail, tail_ng;
     int tail_first, tail_stride, tail_wrap;
+    int nt, tiles;           // ACROSS: query tiles per (sample, head), and in all
+    int full, rest, n_items; // ACROSS: items of three tiles that fill whole rounds, tiles per item after those, items in all
     float scale_log2;        // scale * log2(e)
     int* status;
 };
 
 struct Item3 {
-    int b, h, q0;            // sample, head, first query row of tile 0 (tile g starts at q0 + g * 128)
+    int bh, q;               // (sample, head) and query tile of tile 0
     int ng;                  // query tiles present: 1 .. 3
+    int split;               // tiles of the first (sample, head); the others, if any (ACROSS), belong to the next one
 };
-__device__ __forceinline__ Item3 decode_item3(const Attn3Args& a, int w) {
+template <bool ACROSS> __device__ __forceinline__ Item3 decode_item3(const Attn3Args& a, int w) {
     Item3 it;
-    int bh;
+    if (ACROSS) {
+        const int tile = w < a.full ? w * NG : a.full * NG + (w - a.full) * a.rest;
+        it.ng = min(w < a.full ? NG : a.rest, a.tiles - tile);
+        it.bh = tile / a.nt;
+        it.q = tile - it.bh * a.nt;
+        it.split = min(it.ng, a.nt - it.q);     // (nt >= 2: three tiles meet one boundary at most)
+        return it;
+    }
     if (w < a.n3) {
-        bh = w / a.per3;
-        it.q0 = (w - bh * a.per3) * NG * BQ;
+        it.bh = w / a.per3;
+        it.q = (w - it.bh * a.per3) * NG;
         it.ng = NG;
     } else {
-        bh = w - a.n3;
-        it.q0 = a.per3 * NG * BQ;
+        it.bh = w - a.n3;
+        it.q = a.per3 * NG;
         it.ng = a.tail_ng;
     }
-    it.b = bh / a.H;
-    it.h = bh - it.b * a.H;
+    it.split = it.ng;
     return it;
 }
 // The k-th item of this CTA, or -1 when it has none left.
-__device__ __forceinline__ int item_of(const Attn3Args& a, int k) {
+template <bool ACROSS> __device__ __forceinline__ int item_of(const Attn3Args& a, int k) {
     const int c = blockIdx.x, G = gridDim.x;
+    if (ACROSS) return c + k * G < a.n_items ? c + k * G : -1;
     const int mine3 = c < a.n3 ? (a.n3 - c + G - 1) / G : 0;
     if (k < mine3) return c + k * G;
     int pos = c - a.tail_first;
@@ -149,6 +162,7 @@ __device__ __forceinline__ float exp_pass64(uint32_t (&r)[BKV], float sl, float 
     return (a + b) + (c + d);
 }
 
+template <bool ACROSS>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO, const Attn3Args args) {
@@ -198,21 +212,27 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         if (elect_one()) {
             uint32_t kv_it = 0, item_n = 0;
             bool ok = true;
-            for (int w = item_of(args, 0); w >= 0 && ok; w = item_of(args, ++item_n)) {
-                const Item3 it = decode_item3(args, w);
+            for (int w = item_of<ACROSS>(args, 0); w >= 0 && ok; w = item_of<ACROSS>(args, ++item_n)) {
+                const Item3 it = decode_item3<ACROSS>(args, w);
                 const uint32_t qb = item_n & 1u;
                 if (!mbar_wait(&q_empty[qb], ((item_n >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
                 mbar_expect_tx(&q_full[qb], it.ng * Q_BYTES);
+                const int b0 = it.bh / args.H, h0 = it.bh - b0 * args.H;
+                const bool turn = h0 + 1 == args.H;               // the next (sample, head) is the next sample's first
+                const int b1 = turn ? b0 + 1 : b0, h1 = turn ? 0 : h0 + 1;
                 for (int g = 0; g < it.ng; ++g)
-                    tma_load_4d(smem + OFF_Q + (qb * NG + g) * Q_BYTES, &tmQ, &q_full[qb], 0, it.h, it.q0 + g * BQ, it.b);
-                for (int t = 0; t < nkv; ++t, ++kv_it) {
-                    const int s = kv_it % NS;
+                    tma_load_4d(smem + OFF_Q + (qb * NG + g) * Q_BYTES, &tmQ, &q_full[qb], 0, g < it.split ? h0 : h1,
+                                (g < it.split ? it.q + g : g - it.split) * BQ, g < it.split ? b0 : b1);
+                const bool two = ACROSS && it.split < it.ng;
+                for (int t = 0; t < (two ? 2 * nkv : nkv); ++t, ++kv_it) {
+                    const int s = kv_it % NS, row0 = (two ? t >> 1 : t) * BKV;
+                    const bool second = two && (t & 1);
                     if (!mbar_wait(&k_empty[s], ((kv_it / NS) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
                     mbar_expect_tx(&k_full[s], KV_BYTES);
-                    tma_load_4d(smem + OFF_K + s * KV_BYTES, &tmK, &k_full[s], 0, it.h, t * BKV, it.b);
+                    tma_load_4d(smem + OFF_K + s * KV_BYTES, &tmK, &k_full[s], 0, second ? h1 : h0, row0, second ? b1 : b0);
                     if (!mbar_wait(&v_empty[s], ((kv_it / NS) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
                     mbar_expect_tx(&v_full[s], KV_BYTES);
-                    tma_load_4d(smem + OFF_V + s * KV_BYTES, &tmV, &v_full[s], 0, it.h, t * BKV, it.b);
+                    tma_load_4d(smem + OFF_V + s * KV_BYTES, &tmV, &v_full[s], 0, second ? h1 : h0, row0, second ? b1 : b0);
                 }
             }
             // every copy started here must have landed before the CTA exits
@@ -234,18 +254,24 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             uint32_t ns[NG] = {0, 0, 0};                 // S tiles issued so far per query tile
             uint32_t item_n = 0, t = 0;
             bool ok = true;
-            for (int w = item_of(args, 0); w >= 0 && ok; w = item_of(args, ++item_n)) {
-                const int ng = decode_item3(args, w).ng;
+            for (int w = item_of<ACROSS>(args, 0); w >= 0 && ok; w = item_of<ACROSS>(args, ++item_n)) {
+                const Item3 it = decode_item3<ACROSS>(args, w);
                 const uint32_t qb = item_n & 1u;
                 if (!mbar_wait(&q_full[qb], (item_n >> 1) & 1u, abort_flag)) { ok = false; break; }
-                for (int j = 0; j < nkv && ok; ++j, ++t) {
-                    const int stage = t % NS, valid = min(BKV, args.N - j * BKV);
-                    if (!mbar_wait(&k_full[stage], (t / NS) & 1u, abort_flag)) { ok = false; break; }
+                for (int j = 0; j < nkv && ok; ++j) {
+                    const int valid = min(BKV, args.N - j * BKV);
                     const uint32_t idesc_s = valid == BKV ? idesc_s_full : idesc_bf16(BQ, (valid + 15) & ~15, 0, 0);
-                    const uint32_t dk = k_lo + (uint32_t)stage * kKV16;
+                    int stage = 0;
+                    uint32_t dk = 0;
 #pragma unroll
                     for (int g = 0; g < NG; ++g) {
-                        if (g >= ng || !ok) continue;
+                        if (g >= it.ng || !ok) continue;
+                        if (g == 0 || (ACROSS && g == it.split)) {   // a (sample, head)'s first tile: the next ring stage
+                            stage = t % NS;
+                            if (!mbar_wait(&k_full[stage], (t / NS) & 1u, abort_flag)) { ok = false; continue; }
+                            dk = k_lo + (uint32_t)stage * kKV16;
+                            ++t;
+                        }
                         if (ns[g] > 0 && !mbar_wait(&s_free[g], (ns[g] - 1) & 1u, abort_flag)) { ok = false; continue; }
                         tc_fence_after();
                         const uint32_t dq = q_lo + (qb * NG + g) * kQ16;
@@ -254,8 +280,9 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                             mma_ss_lh(tmem_base + kSCol + g * BKV, dq + 2u * k, dk + 2u * k, desc_hi, idesc_s, k != 0);
                         mma_commit(&s_full[g]);
                         ++ns[g];
+                        if (ACROSS && (g == it.ng - 1 || g == it.split - 1)) mma_commit(&k_empty[stage]);
                     }
-                    if (ok) mma_commit(&k_empty[stage]);
+                    if (!ACROSS && ok) mma_commit(&k_empty[stage]);
                 }
                 if (ok) mma_commit(&q_empty[qb]);
             }
@@ -272,16 +299,21 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             uint32_t np[NG] = {0, 0, 0};                 // P V products issued so far per query tile
             uint32_t t = 0, item_n = 0;
             bool ok = true;
-            for (int w = item_of(args, 0); w >= 0 && ok; w = item_of(args, ++item_n)) {
-                const int ng = decode_item3(args, w).ng;
-                for (int j = 0; j < nkv && ok; ++j, ++t) {
-                    const int stage = t % NS, valid = min(BKV, args.N - j * BKV);
-                    if (!mbar_wait(&v_full[stage], (t / NS) & 1u, abort_flag)) { ok = false; break; }
-                    const uint32_t dv = v_lo + (uint32_t)stage * kKV16;
-                    const int ksteps = (valid + 15) >> 4;
+            for (int w = item_of<ACROSS>(args, 0); w >= 0 && ok; w = item_of<ACROSS>(args, ++item_n)) {
+                const Item3 it = decode_item3<ACROSS>(args, w);
+                for (int j = 0; j < nkv && ok; ++j) {
+                    const int ksteps = (min(BKV, args.N - j * BKV) + 15) >> 4;
+                    int stage = 0;
+                    uint32_t dv = 0;
 #pragma unroll
                     for (int g = 0; g < NG; ++g) {
-                        if (g >= ng || !ok) continue;
+                        if (g >= it.ng || !ok) continue;
+                        if (g == 0 || (ACROSS && g == it.split)) {
+                            stage = t % NS;
+                            if (!mbar_wait(&v_full[stage], (t / NS) & 1u, abort_flag)) { ok = false; continue; }
+                            dv = v_lo + (uint32_t)stage * kKV16;
+                            ++t;
+                        }
                         if (!mbar_wait(&p_ready[g], np[g] & 1u, abort_flag)) { ok = false; continue; }
                         tc_fence_after();
                         const uint32_t o_col = tmem_base + kOCol + g * DH, p_col = tmem_base + kPCol + g * (BKV / 2);
@@ -289,8 +321,9 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                             mma_ts_lh(o_col, p_col + 8 * k, dv + 128u * k, desc_hi, idesc_o, !(j == 0 && k == 0));
                         mma_commit(&o_done[g]);
                         ++np[g];
+                        if (ACROSS && (g == it.ng - 1 || g == it.split - 1)) mma_commit(&v_empty[stage]);
                     }
-                    if (ok) mma_commit(&v_empty[stage]);
+                    if (!ACROSS && ok) mma_commit(&v_empty[stage]);
                 }
             }
         }
@@ -307,9 +340,10 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         uint32_t cnt = 0;                                // key tiles this warpgroup has walked through
         bool ok = true;
         uint32_t item_n = 0;
-        for (int w = item_of(args, 0); w >= 0 && ok; w = item_of(args, ++item_n)) {
-            const Item3 it = decode_item3(args, w);
+        for (int w = item_of<ACROSS>(args, 0); w >= 0 && ok; w = item_of<ACROSS>(args, ++item_n)) {
+            const Item3 it = decode_item3<ACROSS>(args, w);
             if (g >= it.ng) continue;
+            const int bh = it.bh + (g < it.split ? 0 : 1), row0 = (g < it.split ? it.q + g : g - it.split) * BQ + q * 32;
             float m_l2 = 0.f, l_run = 0.f;               // running maximum (times scale*log2 e) and sum
             for (int j = 0; j < nkv && ok; ++j, ++cnt) {
                 const int valid = min(BKV, args.N - j * BKV);
@@ -385,9 +419,9 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             }
             fence_async_smem();
             __syncwarp();
-            const int row0 = it.q0 + g * BQ + q * 32;
             if (lane == 0 && row0 < args.N) {
-                tma_store_4d(&tmO, smem + OFF_OST + (g * 4 + q) * 4096, 0, it.h, row0, it.b);
+                const int b = bh / args.H;
+                tma_store_4d(&tmO, smem + OFF_OST + (g * 4 + q) * 4096, 0, bh - b * args.H, row0, b);
                 tma_store_commit();
             }
         }
@@ -444,16 +478,24 @@ cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMa
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     e = (cudaError_t)attr_once.run(dev, [] {
-        return (int)cudaFuncSetAttribute(attn_tc3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+        cudaError_t a = cudaFuncSetAttribute(attn_tc3_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+        if (a == cudaSuccess) a = cudaFuncSetAttribute(attn_tc3_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+        return (int)a;
     });
     if (e != cudaSuccess) return e;
     Attn3Args args;
     args.N = d.N; args.H = d.H;
-    const int tiles = (d.N + BQ - 1) / BQ, G = ctx->sm_count;
+    const int G = ctx->sm_count;
     const long long BH = (long long)d.B * d.H;
-    args.per3 = tiles / NG;
-    args.tail_ng = tiles - args.per3 * NG;
-    if (BH * (args.per3 + 1) >= (1ll << 30)) return cudaErrorInvalidValue;
+    args.nt = (d.N + BQ - 1) / BQ;
+    const long long tiles = BH * args.nt, left = tiles % (NG * (long long)G);
+    if (tiles >= (1ll << 30)) return cudaErrorInvalidValue;
+    args.tiles = (int)tiles;
+    args.full = (int)((tiles - left) / NG);
+    args.rest = left <= G ? 1 : NG;
+    args.n_items = args.full + (int)((left + args.rest - 1) / args.rest);
+    args.per3 = args.nt / NG;
+    args.tail_ng = args.nt - args.per3 * NG;
     args.n3 = (int)(BH * args.per3);
     args.n_tail = args.tail_ng ? (int)BH : 0;
     const int r = args.n3 % G, idle = G - r;
@@ -461,12 +503,18 @@ cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMa
     args.tail_first = r;
     args.tail_stride = wrap ? G : idle;
     args.tail_wrap = wrap;
+    // Items run across heads where that shortens the longest CTA.  (Items with two K/V streams take a little longer:
+    // with the loads equal, 8 x 16 x 577 takes 29.7 us within heads and 31.9 across.)  Measured, within / across, us:
+    // 128 x 12 x 133 50.2 / 42.2, x 197 61.6 / 50.7, 28 x 16 x 577 88.7 / 78.1, 16 x 12 x 1569 190 / 183, 4 x 16 x 2305 142 / 135.
+    const long long load = args.full / G * 10 + (left == 0 ? 0 : left <= G ? 7 : 10);
+    const bool across = load < tc3_load(BH, d.N, G, wrap);
     const float scale = d.scale != 0.f ? d.scale : 0.125f;
     args.scale_log2 = scale * 1.4426950408889634f;
     args.status = ctx->d_status;
-    const long long all = (long long)args.n3 + args.n_tail;
+    const long long all = across ? args.n_items : (long long)args.n3 + args.n_tail;
     const int grid = all < G ? (int)all : G;
-    return launch_pdl(attn_tc3_kernel, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args);
+    if (across) return launch_pdl(attn_tc3_kernel<true>, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args);
+    return launch_pdl(attn_tc3_kernel<false>, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args);
 }
 
 }  // namespace rs

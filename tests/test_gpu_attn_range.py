@@ -26,3 +26,16 @@ def test_weights_over_the_range_of_exp2(pinned, kernel, gain):   # noqa: F811
     want = orc.attn(f[:, :, 0], f[:, :, 1], f[:, :, 2]).reshape(B, N, H * 64)
     # weights rounded to bf16 (2^-9 each, they sum to one), values up to |v|max; one rounding of the output
     assert np.abs(got - want).max() < (2.0 ** -8) * np.abs(f[:, :, 2]).max()
+
+
+@pytest.mark.parametrize("B,H,N", [(1, 2, 129), (3, 1, 200), (40, 20, 133), (25, 9, 256), (13, 12, 300), (30, 12, 500), (2, 3, 600), (11, 16, 577)])
+def test_query_tiles_across_heads(pinned, B, H, N):   # noqa: F811
+    """Three query tiles to an item, over the ends of heads and samples: two to five tiles per head, whole rounds of
+    items with tiles of the last round handed out singly or in threes."""
+    g = torch.Generator(device="cuda").manual_seed(N)
+    qkv = torch.randn(B, N, 3, H, 64, generator=g, device="cuda").bfloat16()
+    got = pinned[3].attn_fwd(qkv[:, :, 0], qkv[:, :, 1], qkv[:, :, 2]).double()
+    q, k, v = (qkv[:, :, i].transpose(1, 2).double() for i in range(3))
+    want = torch.softmax(q @ k.transpose(2, 3) / 8.0, -1) @ v
+    # weights rounded to bf16 (2^-9 each, they sum to one), values up to |v|max; one rounding of the output
+    assert (got - want.transpose(1, 2).reshape(B, N, H * 64)).abs().max() < 2.0 ** -8 * v.abs().max()
