@@ -8,7 +8,6 @@
 #include <type_traits>
 
 #include "rs.h"
-#include "rs_attn.cuh"
 
 namespace rs {
 namespace gemm {
@@ -43,38 +42,6 @@ struct GemmArgs {
 // weights, so they have to be finite.
 constexpr int kPadRows = 16;
 
-// Exact-erf GELU, v * Phi(v), to fp32 accuracy (max abs error 8e-7 over all v) without erff:
-// with q(t) = -log2(Phi(-t)) for t >= 0,  Phi(v) = 2^-q(|v|) for v < 0 and 1 - 2^-q(|v|) for
-// v >= 0.  q is smooth (about t^2/2 * log2(e) plus slow terms) and a degree-5 polynomial fitted
-// on [0, 7] with weight t * Phi(-t) reproduces GELU to that accuracy; its positive leading
-// coefficient keeps 2^-q -> 0 for large |v|.  Coefficients from csrc/fit_gelu.py.
-//
-// A pair at a time on packed FMAs, with n = -|v|: the polynomial in n gives -q, and GELU = max(v, 0) + n 2^-q for either
-// sign: 12 instructions a pair instead of 22, and the 2^x of the special-function unit (16 of its cycles a pair and warp) is
-// what is left.  FC1 50432 x 768 x 192 31.9 -> 30.9 us, 25216 x 3072 x 768 80.8 -> 78.3, 16400 x 3072 x 768 56.1 -> 54.2.
-// n stays finite, so an infinite v gives v or 0; max.NaN keeps a NaN.
-__device__ __forceinline__ float max_nan(float a, float b) {
-    float r;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void gelu_erf2(float& v0, float& v1) {
-    using attn::pack2; using attn::unpack2; using attn::ffma2;
-    const uint64_t n = pack2(max_nan(-fabsf(v0), -3.4e38f), max_nan(-fabsf(v1), -3.4e38f));
-    auto c = [](float x) { return pack2(x, x); };
-    uint64_t q = c(0.00047694556997157633f);
-    q = ffma2(q, n, c(0.00711308470266570f));
-    q = ffma2(q, n, c(0.05190887302160263f));
-    q = ffma2(q, n, c(-0.4598882496356964f));
-    q = ffma2(q, n, c(1.1508461236953735f));
-    q = ffma2(q, n, c(-1.0000265836715698f));
-    float q0, q1, e0, e1;
-    unpack2(q, q0, q1);
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(q0));
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(q1));
-    unpack2(ffma2(n, pack2(e0, e1), pack2(fmaxf(v0, 0.f), fmaxf(v1, 0.f))), v0, v1);
-}
-
 // Adds one element of the scored pair (u, v) to the running sums of the chosen distance (Sec. 3.3).  Called with a
 // constant distance in the pair-tile kernel (with_dist): the choice is made once per 32 columns there.
 __device__ __forceinline__ void score_acc(int dist, float u, float v, float& s0, float& s1, float& s2) {
@@ -96,11 +63,4 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 
 }  // namespace gemm
 
-// The kernel for few rows (rs_gemm_small.cu): whether a shape goes there, and the CTAs that share the K of a tile.
-// tmA: boxes of 128 rows; tmB: boxes of kSmallBN rows; both 64 columns, 128-byte swizzle.
-constexpr int kSmallBN = 64;
-struct SmallPlan { bool use; int splits; };
-SmallPlan gemm_small_plan(long long M, int N, int K, int sm_count);
-cudaError_t launch_gemm_small(int epi, const CUtensorMap& tmA, const CUtensorMap& tmB, const gemm::GemmArgs& args, int splits, void* out,
-                              rs_dtype out_dtype, bool weights_ready, cudaStream_t st);
 }  // namespace rs

@@ -1,4 +1,4 @@
-// bf16 GEMM for few rows on the tensor cores, with the epilogues of rs_gemm_tc.cu:
+// bf16 GEMM for few rows on the tensor cores, with the epilogues of rs_gemm_tc.cu (which includes this file):
 //     out[M, N] = epilogue(A[M, K] . W[N, K]^T)
 // With a few hundred rows the 256-row pair tiles of rs_gemm_tc.cu leave most SMs idle and each of the few busy
 // ones walks the whole of K: one image of 197 tokens has 6 pair tiles in its second MLP product, 48 dependent
@@ -10,6 +10,7 @@
 // Weights do not depend on the kernel before this one, so their first slabs are requested before the grid
 // dependency is waited for (args.weights_ready: the caller knows that nothing still running writes them).
 // Measured: see gemm_small_plan.
+#pragma once
 #include "rs_internal.h"
 #include "rs_gemm.cuh"
 #include "rs_device.cuh"
@@ -17,6 +18,11 @@
 #include "rs_tc.cuh"
 
 namespace rs {
+namespace few {
+
+// Whether a shape goes to this kernel, and the CTAs that share the K of a tile.
+constexpr int kSmallBN = 64;
+struct SmallPlan { bool use; int splits; };
 
 namespace {
 
@@ -213,7 +219,7 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             v[e] = EPI == EPI_BIAS_LN ? fmaf(ln.y, fmaf(-ln.x, cv[e], v[e]), bv[e]) : v[e] + bv[e];
         if (EPI == EPI_BIAS_GELU) {
 #pragma unroll
-            for (int e = 0; e < 4; e += 2) gelu_erf2(v[e], v[e + 1]);
+            for (int e = 0; e < 4; ++e) v[e] = gelu_erf(v[e]);
         } else if (EPI == EPI_RESID) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -321,6 +327,7 @@ SmallPlan gemm_small_plan(long long M, int N, int K, int sms) {
     return {tiles <= (K <= 256 ? 220 : 100), s};
 }
 
+// tmA: boxes of 128 rows; tmB: boxes of kSmallBN rows; both 64 columns, 128-byte swizzle.
 cudaError_t launch_gemm_small(int epi, const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmArgs& args, int splits, void* out,
                               rs_dtype out_dtype, bool weights_ready, cudaStream_t st) {
     switch (epi) {
@@ -336,4 +343,5 @@ cudaError_t launch_gemm_small(int epi, const CUtensorMap& tmA, const CUtensorMap
     return cudaErrorInvalidValue;
 }
 
+}  // namespace few
 }  // namespace rs
