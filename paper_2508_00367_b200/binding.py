@@ -176,12 +176,16 @@ def _torch_dt(code: int):
     return torch.bfloat16 if code == RS_BF16 else torch.float32
 
 
-def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
+    return None if t is None else t.data_ptr()
 
 
-def _stream(device) -> ctypes.c_void_p:
-    return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+# The current stream's handle without a Stream object around it (1 us of a call's 10 on the host).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
+def _stream(device) -> int:
+    return _raw_stream(torch.cuda.current_device() if device.index is None else device.index)
 
 
 class Context:
