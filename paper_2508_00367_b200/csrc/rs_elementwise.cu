@@ -1,6 +1,8 @@
 // HBM-bound row kernels: LayerNorm, the representation-shift score (Sec. 3.2)
 // and the residual-add epilogue with the score fused in.  One warp owns one
 // token row; rows move as 16-byte vectors, several in flight per lane.
+#include <type_traits>
+
 #include "rs_internal.h"
 #include "rs_device.cuh"
 #include "rs_gemm.cuh"
@@ -41,6 +43,76 @@ layernorm_kernel(const TI* __restrict__ x, const float* __restrict__ gamma,
         if (iv < nvec) raw[j] = ld_stream(xr + iv);
     }
     layernorm_row<TI, TO, MAXV>(raw, nvec, lane, gamma, beta, eps, D, out + row * D);
+}
+
+// The same for fp32 rows of at most 256 values, as LN2 reads them (x', D = 192): half a warp per row, VPL pieces per
+// lane, two rows of a half in flight.  A whole warp per row issues as many instructions for 48 pieces as for 64, two
+// reductions of five steps each among them, and was bound by that: after the projection of
+// 50432 x 192 rows 15.2 -> 10.0 us, 25216 x 128 7.4 -> 5.3, 25216 x 256 8.7 -> 8.4.
+constexpr int kNarrowRows = 4 * kWarpsPerCta;            // rows per CTA
+template <int VPL>
+__global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
+layernorm_narrow_kernel(const float* __restrict__ x, const float* __restrict__ gamma, const float* __restrict__ beta, float eps,
+                        long long T, int D, __nv_bfloat16* __restrict__ out, const int32_t* __restrict__ row_map, const int first,
+                        const int32_t* __restrict__ lens, unsigned seq_n) {
+    if (!first) grid_dep_launch();
+    grid_dep_wait();
+    if (first) grid_dep_launch();
+    const int l16 = threadIdx.x & 15, nvec = D / 4;
+    const long long row0 = (long long)blockIdx.x * kNarrowRows + (threadIdx.x >> 5) * 4 + ((threadIdx.x >> 4) & 1);
+    float4 v[2][VPL];
+    bool on[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const long long row = row0 + 2 * u;
+        on[u] = row < T;
+        if (on[u] && lens) {                     // padding that neither the products nor attention read
+            const unsigned b = (unsigned)row / seq_n, i = (unsigned)row - b * seq_n;
+            on[u] = (int)i < max(__ldg(lens + b), 1) + gemm::kPadRows;
+        }
+        const float* xr = x + (on[u] ? row_map ? (long long)row_map[row] : row : 0) * D;
+#pragma unroll
+        for (int j = 0; j < VPL; ++j) {
+            v[u][j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (on[u] && j * 16 + l16 < nvec) {
+                const uint4 t = ld_stream(reinterpret_cast<const uint4*>(xr) + j * 16 + l16);
+                v[u][j] = make_float4(__uint_as_float(t.x), __uint_as_float(t.y), __uint_as_float(t.z), __uint_as_float(t.w));
+            }
+        }
+    }
+    float mu[2], rstd[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        float sum = 0.f;
+#pragma unroll
+        for (int j = 0; j < VPL; ++j) sum += (v[u][j].x + v[u][j].y) + (v[u][j].z + v[u][j].w);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        mu[u] = sum / (float)D;
+        float sq = 0.f;
+#pragma unroll
+        for (int j = 0; j < VPL; ++j)
+            if (j * 16 + l16 < nvec) {
+                const float a = v[u][j].x - mu[u], b = v[u][j].y - mu[u], c = v[u][j].z - mu[u], d = v[u][j].w - mu[u];
+                sq += (a * a + b * b) + (c * c + d * d);
+            }
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        rstd[u] = rsqrtf(sq / (float)D + eps);
+    }
+#pragma unroll
+    for (int j = 0; j < VPL; ++j) {
+        const int iv = j * 16 + l16;
+        if (iv >= nvec) continue;
+        const float4 g = __ldg(reinterpret_cast<const float4*>(gamma) + iv), bt = __ldg(reinterpret_cast<const float4*>(beta) + iv);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if (!on[u]) continue;
+            const float y[4] = {(v[u][j].x - mu[u]) * rstd[u] * g.x + bt.x, (v[u][j].y - mu[u]) * rstd[u] * g.y + bt.y,
+                                (v[u][j].z - mu[u]) * rstd[u] * g.z + bt.z, (v[u][j].w - mu[u]) * rstd[u] * g.w + bt.w};
+            store_n<__nv_bfloat16, 4>(out + (row0 + 2 * u) * D + iv * 4, y);
+        }
+    }
 }
 
 // ---------------------------------------------------------------- shift score
@@ -204,6 +276,17 @@ cudaError_t ln_dispatch(const void* x, const float* g, const float* b, float eps
                         void* out, const int32_t* row_map, bool first, cudaStream_t st, const int32_t* lens, int seq_n) {
     const int nvec = D / Vec16<TI>::N;
     const dim3 grid(row_grid(T)), block(kWarpsPerCta * 32);
+    if constexpr (std::is_same<TI, float>::value && std::is_same<TO, __nv_bfloat16>::value) {
+        const dim3 narrow((unsigned)((T + kNarrowRows - 1) / kNarrowRows));
+#define RS_LN_CASE(VPL)                                                                                                    \
+    if (nvec <= 16 * VPL)                                                                                                  \
+        return launch_pdl(layernorm_narrow_kernel<VPL>, narrow, block, 0, st, (const float*)x, g, b, eps, T, D,            \
+                          (__nv_bfloat16*)out, row_map, (int)first, lens, (unsigned)seq_n)
+        RS_LN_CASE(2);
+        RS_LN_CASE(3);
+        RS_LN_CASE(4);
+#undef RS_LN_CASE
+    }
     if (nvec <= 32 * 4)
         return launch_pdl(layernorm_kernel<TI, TO, 4>, grid, block, 0, st, (const TI*)x, g, b, eps, T, D, (TO*)out, row_map, (int)first, lens, (unsigned)seq_n);
     else if (nvec <= 32 * 8)

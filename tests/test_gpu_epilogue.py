@@ -41,3 +41,13 @@ def test_block_pair_tiles_every_score(ctx, mode, dist, out):   # noqa: F811
     tol = 5e-4 if (mode, dist) == ("mlp", "l2") else 3e-3 if mode == "mlp_delta" else 2e-3
     rel = np.abs(res["scores"].double().numpy() - ref["scores"]) / np.abs(ref["scores"])
     assert rel.max() < tol, rel.max()
+
+
+@pytest.mark.parametrize("D", [128, 192, 256, 384])
+@pytest.mark.parametrize("B,N", [(1, 1), (1, 31), (3, 33), (5, 130)])
+def test_block_narrow_layernorm_rows(ctx, B, N, D):   # noqa: F811
+    """LN2 of rows of up to 256 values goes half a warp to a row, four rows to a warp: row counts around 4 and 32."""
+    x, w = synth.make_tokens(B, N, D, "bf16", seed=41), synth.make_block_weights(D, 4 * D, "bf16", seed=42)
+    ref = orc.block_fwd(x.double().numpy(), _np(w), D // 64, 0)
+    res = _run_block(ctx, x, w, D // 64, 0, "bf16", torch.float32)
+    parity.check_float(res["x_full"].double().numpy(), ref["x_hat"], "bf16", False)
