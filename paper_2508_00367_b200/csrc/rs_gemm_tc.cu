@@ -91,8 +91,7 @@ using namespace gemm;
 
 constexpr int BM = 128;                       // rows per CTA; the pair's tile has 2 * BM rows
 constexpr int BK = 64;
-constexpr int kThreads = 320;                 // warp 0: TMA, warp 1: MMA (leader CTA), warps 2-9: epilogue
-constexpr int kEpiWarps = 8;
+// warp 0: TMA, warp 1: MMA (leader CTA), the others: epilogue, in groups of four that take a range of columns each
 constexpr int A_BYTES = BM * BK * 2;          // 16 KB
 constexpr int STG_BYTES = 32 * 128;           // one staged output block of a warp: its 32 rows of 128 bytes
 constexpr int RES_BOX_BYTES = 32 * 64;         // residual of one 32-column chunk of a warp: 32 rows of 32 bf16
@@ -143,7 +142,10 @@ template <int BN> struct WorkList {
 // 32 columns ahead, the next tile's first ones included.  It pays for the room with one operand stage less.  (A whole tile's boxes at a
 // time left room for one staging buffer per warp only, and a third of the epilogue waited for it: 50432 x 192 x 192
 // 19.5 -> 18.8 us, 25216 x 384 x 384 20.0 -> 19.2, 6924 x 1024 x 1024 21.5 -> 21.0.)
-template <int BN, int EPI> struct Cfg {
+// WIDE: four (192 columns: three) groups of epilogue warps with 64 columns each instead of two with half a tile each, for
+// products whose K is so short that the epilogue is the longer part: four warps a scheduler instead of two cover
+// its latencies.  (Longer ones are slower that way, their stores then come in one burst: see wide_epilogue.)
+template <int BN, int EPI, bool WIDE> struct Cfg {
     static constexpr bool RES_TMA = EPI == EPI_RESID;
     static constexpr bool LN = EPI == EPI_BIAS_LN;                 // one staging buffer per warp, room for a second column vector
     static constexpr int B_BYTES = (BN / 2) * BK * 2;              // this CTA's half of the W tile
@@ -151,24 +153,25 @@ template <int BN, int EPI> struct Cfg {
     static constexpr int STAGES = (BN == 128 ? 6 : 5) - (RES_TMA ? 1 : 0);
     static constexpr int TMEM_COLS = (BN == 128) ? 256 : 512;      // two accumulators, a power of two
     static constexpr int SPLIT = (BN == 128) ? 64 : 128;           // epilogue warps 2-5 take columns [0, SPLIT) of a whole tile
-    static constexpr int STG_PER_WARP = LN ? 1 : 2;
+    static constexpr int GROUPS = WIDE ? BN / 64 : 2, EPI_WARPS = 4 * GROUPS, THREADS = 64 + 32 * EPI_WARPS;
+    static constexpr int STG_PER_WARP = LN || WIDE ? 1 : 2;
     static constexpr int RES_WARP_BYTES = RES_TMA ? 2 * RES_BOX_BYTES : 0;
     static constexpr int OFF_STG = STAGES * STAGE_BYTES;
-    static constexpr int OFF_RES = OFF_STG + kEpiWarps * STG_PER_WARP * STG_BYTES;
-    static constexpr int OFF_BAR = OFF_RES + kEpiWarps * RES_WARP_BYTES;
-    static constexpr int OFF_BIAS = OFF_BAR + 256;                 // float [2 tile parities][2 halves][128]: bias slices
-    static constexpr int OFF_COLSUM = OFF_BIAS + 2048;             // EPI_BIAS_LN: float [2][2][128] like the bias slices
+    static constexpr int OFF_RES = OFF_STG + EPI_WARPS * STG_PER_WARP * STG_BYTES;
+    static constexpr int OFF_BAR = OFF_RES + EPI_WARPS * RES_WARP_BYTES;
+    static constexpr int OFF_BIAS = OFF_BAR + 256;                 // float [2 tile parities][256]: bias of the tile's columns
+    static constexpr int OFF_COLSUM = OFF_BIAS + 2048;             // EPI_BIAS_LN: float [2][256] like the bias
     static constexpr int OFF_MASK = OFF_BIAS + (LN ? 4096 : 2048);  // one bit per row tile (batches with a count per sample)
     static constexpr size_t SMEM = (size_t)OFF_MASK + kMaskWords * 4;   // the window itself must be 1024-byte aligned
     static_assert(SMEM <= 227 * 1024, "shared memory of one CTA");
 };
 
-template <int BN, int EPI, typename OutT>
-__global__ void __launch_bounds__(kThreads, 1)
+template <int BN, int EPI, typename OutT, bool WIDE>
+__global__ void __launch_bounds__((Cfg<BN, EPI, WIDE>::THREADS), 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ CUtensorMap tmOut,
                const __grid_constant__ CUtensorMap tmRes, const GemmArgs args) {
-    using C = Cfg<BN, EPI>;
+    using C = Cfg<BN, EPI, WIDE>;
     // The 128-byte swizzle wants 1024-byte aligned stage and staging buffers, and the layout leaves no
     // room to round the base up: a window that is not aligned is reported, and nothing else is done.
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -184,8 +187,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint64_t* tempty = bars + 2 * C::STAGES + 2; // [2] leader's: both CTAs' epilogues drained it
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * C::STAGES + 4);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    volatile int* half_fail = reinterpret_cast<volatile int*>(tmem_slot + 2);   // [2]
-    uint64_t* res_full = bars + 2 * C::STAGES + 6;   // [kEpiWarps][2] a chunk of the warp's residual landed (EPI_RESID)
+    volatile int* group_fail = reinterpret_cast<volatile int*>(tmem_slot + 2);   // [GROUPS]
+    uint64_t* res_full = bars + 2 * C::STAGES + 6;   // [EPI_WARPS][2] a chunk of the warp's residual landed (EPI_RESID)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();     // 0 = leader of the pair
@@ -198,15 +201,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         prefetch_tmap(&tmB);
         prefetch_tmap(&tmOut);
         for (int s = 0; s < C::STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        for (int a = 0; a < 2; ++a) { mbar_init(&tfull[a], 1); mbar_init(&tempty[a], 2 * kEpiWarps); }
+        for (int a = 0; a < 2; ++a) { mbar_init(&tfull[a], 1); mbar_init(&tempty[a], 2 * C::EPI_WARPS); }
         if (C::RES_TMA) {
             prefetch_tmap(&tmRes);
             // one arrival by the lane that starts the TMA copies, or one by each lane's own indexed copies
-            for (int w = 0; w < 2 * kEpiWarps; ++w) mbar_init(&res_full[w], args.row_map ? 32 : 1);
+            for (int w = 0; w < 2 * C::EPI_WARPS; ++w) mbar_init(&res_full[w], args.row_map ? 32 : 1);
         }
         *abort_flag = 0;
-        half_fail[0] = 0;
-        half_fail[1] = 0;
+        for (int g = 0; g < C::GROUPS; ++g) group_fail[g] = 0;
         mbar_fence_init();
     }
     if (warp == 1) {
@@ -225,7 +227,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     int tiles = num_m * num_n;
     uint32_t* mask = args.lens ? reinterpret_cast<uint32_t*>(smem + C::OFF_MASK) : nullptr;
     if (mask) {                                  // which row tiles hold rows in use (num_m <= kMaskTiles)
-        for (int t0 = warp * 32; t0 < kMaskTiles; t0 += kThreads) {
+        for (int t0 = warp * 32; t0 < kMaskTiles; t0 += C::THREADS) {
             const int r0 = (t0 + lane) * 2 * BM, r1 = min(r0 + 2 * BM, args.M);
             bool used = false;
             for (int b = r0 / args.seq_n; r0 < args.M && b * args.seq_n < r1 && !used; ++b)
@@ -301,20 +303,25 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     } else {
         // ---------------- epilogue (both CTAs; each drains its own 128 x BN half) ----------------
         const int q = warp & 3;                          // TMEM lane quadrant this warp may read
-        const int half = (warp - 2) >> 2;                // warps 2-5: columns [0, SPLIT), warps 6-9: the rest
-        // columns of a tile or piece that this half takes
+        const int group = (warp - 2) >> 2;
+        // columns of a tile or piece that this group takes: half of it, or (WIDE) 64 (none of a piece that is narrower)
         int c_begin = 0, c_end = 0;
         auto columns = [&](int width) {
+            if (WIDE) {
+                c_begin = min(group * 64, width);
+                c_end = min(group * 64 + 64, width);
+                return;
+            }
             const int split = width == BN ? C::SPLIT : BN / 4;
-            c_begin = half ? split : 0;
-            c_end = half ? width : split;
+            c_begin = group ? split : 0;
+            c_end = group ? width : split;
         };
         constexpr int BLK_COLS = 128 / (int)sizeof(OutT);            // columns in one staged 128-byte row
         constexpr int CHUNKS_PER_BLK = BLK_COLS / 32;                // 32-column TMEM loads per staged block
         const int trow = q * 32 + lane;                  // row inside this CTA's half of the tile
         const uint32_t stg_row = (uint32_t)(lane >> 3) * 1024u + (uint32_t)(lane & 7) * 128u;   // inside the warp's 32-row slab
         const int r8 = lane & 7;
-        const int t128 = ((warp - 2) & 3) * 32 + lane;   // this thread's index among the 128 of its half
+        const int t128 = ((warp - 2) & 3) * 32 + lane;   // this thread's index among the 128 of its group
         const uint32_t lead_tempty[2] = {map_to_cta(smem_u32(&tempty[0]), 0), map_to_cta(smem_u32(&tempty[1]), 0)};
         uint32_t tl = 0, blk_ctr = 0;
         // Where the main loop is the longer part, the plain epilogues wait for a block to be written before they go on to
@@ -327,7 +334,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         uint8_t* res_buf = smem + C::OFF_RES + (warp - 2) * C::RES_WARP_BYTES;
         uint64_t* res_bar = res_full + (warp - 2) * 2;
         RowTiles ahead_tiles = row_tiles;                // the walk of what is fetched a tile ahead
-        int m_next = 0, n_next = 0, map_cur = -1, map_next = -1;     // the next piece of work: its first row, this half's first column,
+        int m_next = 0, n_next = 0, map_cur = -1, map_next = -1;     // the next piece of work: its first row, this group's first column,
                                                                      // and (row map) the source row of the warp's row `lane`
         // With a row map the box is filled row by row: 16-byte asynchronous copies, a row's pieces by neighbouring
         // lanes, land in the layout the tensor map's 64-byte swizzle would give; rows past M are zero-filled.
@@ -370,7 +377,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             if (!(SCORE || C::RES_TMA) || i >= works) return;
             const auto nw = list.at(i);
             m_next = ahead_tiles.at(nw.row_tile) * (2 * BM) + (int)rank * BM;
-            n_next = nw.n0 + (half ? (nw.width == BN ? C::SPLIT : BN / 4) : 0);
+            n_next = nw.n0 + (group ? (nw.width == BN ? C::SPLIT : BN / 4) : 0);
             if (C::RES_TMA && args.row_map) {
                 const int r = m_next + q * 32 + lane;
                 map_next = r < args.M ? __ldg(args.row_map + r) : -1;
@@ -431,21 +438,29 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 ln_rstd = rsqrtf(fmaxf(s2 * inv_d - ln_mu * ln_mu, 0.f) + args.ln_eps);
             }
             float st1 = 0.f, st2 = 0.f;                  // EPI_SCORE_STATS: sums over this thread's columns
-            // The four warps of a column half decide together whether to go on: the named
+            // The four warps of a group decide together whether to go on: the named
             // barriers below have no time limit, so no warp may leave the loop alone.
-            // this half's slice of the bias goes to shared memory while the accumulator is still being
+            // this group's slice of the bias goes to shared memory while the accumulator is still being
             // computed (the barrier below publishes it): the chunk loop then has no global read on its chain.
             // Two copies, by tile parity: a warp may still be reading the last tile's slice.
-            float* bias_s = reinterpret_cast<float*>(smem + C::OFF_BIAS) + (tl & 1u) * 256 + half * 128;
-            if (c_begin + t128 < c_end) bias_s[t128] = args.bias ? __ldg(args.bias + n0 + c_begin + t128) : 0.f;
-            float* cs_s = reinterpret_cast<float*>(smem + C::OFF_COLSUM) + (tl & 1u) * 256 + half * 128;   // EPI_BIAS_LN only
-            if (EPI == EPI_BIAS_LN && c_begin + t128 < c_end) cs_s[t128] = __ldg(args.colsum + n0 + c_begin + t128);
-            if (!__all_sync(0xffffffffu, mbar_wait(&tfull[a], aph, abort_flag))) half_fail[half] = 1;
-            named_barrier(1 + half, 128);
-            if (half_fail[half]) break;
+            float* bias_s = reinterpret_cast<float*>(smem + C::OFF_BIAS) + (tl & 1u) * 256;
+            float* cs_s = reinterpret_cast<float*>(smem + C::OFF_COLSUM) + (tl & 1u) * 256;   // EPI_BIAS_LN only
+            if (c_begin + t128 < c_end) {
+                bias_s[c_begin + t128] = args.bias ? __ldg(args.bias + n0 + c_begin + t128) : 0.f;
+                if (EPI == EPI_BIAS_LN) cs_s[c_begin + t128] = __ldg(args.colsum + n0 + c_begin + t128);
+            }
+            if (!__all_sync(0xffffffffu, mbar_wait(&tfull[a], aph, abort_flag))) group_fail[group] = 1;
+            named_barrier(1 + group, 128);
+            if (group_fail[group]) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + a * BN;
             float sq = 0.f, sq1 = 0.f, sq2 = 0.f;
+            auto hand_back = [&]() {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster_relaxed(lead_tempty[a]);
+            };
+            if (WIDE && c_begin == c_end) hand_back();
 #pragma unroll 1
             for (int c = c_begin; c < c_end; c += 32) {
                 const int cb = (c / 32) % CHUNKS_PER_BLK;            // chunk inside the staged block
@@ -495,11 +510,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 __syncwarp();                            // tcgen05.ld is warp-collective
                 tmem_ld_32x32(taddr + c, r);
                 tmem_wait_ld();
-                if (c + 32 >= c_end) {                   // accumulator fully read by this warp
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive_cluster_relaxed(lead_tempty[a]);
-                }
+                if (c + 32 >= c_end) hand_back();        // accumulator fully read by this warp
                 if (SCORE) {
                     if (c + 32 < c_end) load_res(m0, n0 + c + 32);
                     else if (i + npairs < works) load_res(m_next, n_next);
@@ -508,9 +519,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 float v[32];
 #pragma unroll
                 for (int j = 0; j < 32; j += 4) {
-                    const float4 b = *reinterpret_cast<const float4*>(bias_s + (c - c_begin) + j);
+                    const float4 b = *reinterpret_cast<const float4*>(bias_s + c + j);
                     if (EPI == EPI_BIAS_LN) {
-                        const float4 cc = *reinterpret_cast<const float4*>(cs_s + (c - c_begin) + j);
+                        const float4 cc = *reinterpret_cast<const float4*>(cs_s + c + j);
                         v[j] = fmaf(ln_rstd, fmaf(-ln_mu, cc.x, __uint_as_float(r[j])), b.x);
                         v[j + 1] = fmaf(ln_rstd, fmaf(-ln_mu, cc.y, __uint_as_float(r[j + 1])), b.y);
                         v[j + 2] = fmaf(ln_rstd, fmaf(-ln_mu, cc.z, __uint_as_float(r[j + 2])), b.z);
@@ -660,23 +671,23 @@ bool make_tmap_res(rs_ctx* ctx, CUtensorMap* out, const void* base, uint64_t row
     return tc_encode_cached(ctx, out, base, 2, 0, dims, strides, box, 64);
 }
 
-template <int BN, int EPI, typename OutT>
+template <int BN, int EPI, typename OutT, bool WIDE = false>
 cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmBh, const CUtensorMap& tmOut,
                        const CUtensorMap& tmRes, const GemmArgs& args, int sm_count, cudaStream_t st) {
-    using C = Cfg<BN, EPI>;
+    using C = Cfg<BN, EPI, WIDE>;
     static PerDeviceOnce attr_once;   // per instantiation: the attribute is per function and per device
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     e = (cudaError_t)attr_once.run(dev, [] {
-        return (int)cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI, OutT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+        return (int)cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI, OutT, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     });
     if (e != cudaSuccess) return e;
     const int tiles = ((args.M + 2 * BM - 1) / (2 * BM)) * (args.N / BN);
     const int most = BN == 256 ? 2 * tiles : tiles, pairs = most < sm_count / 2 ? most : sm_count / 2;     // (WorkList may cut tiles in two)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * pairs, 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.blockDim = dim3(C::THREADS, 1, 1);
     cfg.dynamicSmemBytes = C::SMEM;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -688,7 +699,17 @@ cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUt
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<BN, EPI, OutT>, tmA, tmB, tmBh, tmOut, tmRes, args);
+    return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<BN, EPI, OutT, WIDE>, tmA, tmB, tmBh, tmOut, tmRes, args);
+}
+
+// Where 64 columns to a group of epilogue warps is the faster split (see Cfg): the plain epilogues up to K = 256, GELU, whose
+// arithmetic is longer, up to 384.  Halves / 64 columns each, us: QKV 50432 x 576 x 192 18.5 / 17.1, FC1 x 768 x 192 31.3 / 28.6,
+// 25216 x 1024 x 256 23.8 / 22.9, x 1536 x 384 35.7 / 33.0; but QKV 25216 x 1152 x 384 22.9 / 23.5, x 2304 x 768 59.9 / 64.5,
+// FC1 x 3072 x 768 78 / 84.
+// (192 columns with a folded LayerNorm: the two column vectors of 256 do not fit beside sixteen staging buffers.)
+bool wide_epilogue(int epi, int bn, int K) {
+    if (epi == EPI_BIAS_LN) return bn == 192 && K <= 256;
+    return bn >= 192 && ((epi == EPI_BIAS && K <= 256) || (epi == EPI_BIAS_GELU && K <= 384));
 }
 
 // Tile width (256, 192 or 128 columns per pair): the one whose rounds over the SM pairs cost least (a round of 192- or
@@ -806,6 +827,14 @@ cudaError_t launch_gemm_tc(rs_ctx* ctx, int epi, const void* A, const void* W, c
     args.seq_n = skips ? rows->seq_n : 0;
     if (small.use) return few::launch_gemm_small(epi, tmA, tmB, args, small.splits, out, out_dtype, weights_ready, st);
     const int sms = ctx->sm_count;
+    if (wide_epilogue(epi, bn, K)) {
+        if (epi == EPI_BIAS_LN) return launch_one<192, EPI_BIAS_LN, __nv_bfloat16, true>(tmA, tmB, tmBh, tmOut, tmRes, args, sms, st);
+        if (epi == EPI_BIAS_GELU)
+            return bn == 256 ? launch_one<256, EPI_BIAS_GELU, __nv_bfloat16, true>(tmA, tmB, tmBh, tmOut, tmRes, args, sms, st)
+                             : launch_one<192, EPI_BIAS_GELU, __nv_bfloat16, true>(tmA, tmB, tmBh, tmOut, tmRes, args, sms, st);
+        return bn == 256 ? launch_one<256, EPI_BIAS, __nv_bfloat16, true>(tmA, tmB, tmBh, tmOut, tmRes, args, sms, st)
+                         : launch_one<192, EPI_BIAS, __nv_bfloat16, true>(tmA, tmB, tmBh, tmOut, tmRes, args, sms, st);
+    }
 #define RS_GEMM_CASE(E, T)                                                                       \
     return bn == 256   ? launch_one<256, E, T>(tmA, tmB, tmBh, tmOut, tmRes, args, sms, st)           \
            : bn == 192 ? launch_one<192, E, T>(tmA, tmB, tmBh, tmOut, tmRes, args, sms, st)           \

@@ -51,3 +51,15 @@ def test_block_narrow_layernorm_rows(ctx, B, N, D):   # noqa: F811
     ref = orc.block_fwd(x.double().numpy(), _np(w), D // 64, 0)
     res = _run_block(ctx, x, w, D // 64, 0, "bf16", torch.float32)
     parity.check_float(res["x_full"].double().numpy(), ref["x_hat"], "bf16", False)
+
+
+@pytest.mark.parametrize("epilogue", ["bias", "gelu"])
+@pytest.mark.parametrize("M,N,K", [(2500, 768, 192), (2500, 768, 384), (9473, 768, 256), (9473, 576, 192), (12700, 576, 64)])
+def test_linear_short_k(ctx, M, N, K, epilogue):   # noqa: F811
+    """Four (three) groups of epilogue warps: whole tiles, tiles cut in two (two groups idle), a last row tile of a few rows."""
+    g = torch.Generator().manual_seed(M + N + K)
+    a, w = torch.randn(M, K, generator=g).bfloat16(), (0.1 * torch.randn(N, K, generator=g)).bfloat16()
+    b = 0.1 * torch.randn(N, generator=g)
+    got = ctx.linear_fwd(a.cuda(), w.cuda(), b.cuda(), epilogue).cpu().double().numpy()
+    want = orc.linear(a.double().numpy(), w.double().numpy(), b.double().numpy())
+    parity.check_float(got, orc.round_to(orc.gelu(want) if epilogue == "gelu" else want, "bf16"), "bf16", rounded_output=True)
