@@ -497,8 +497,11 @@ bool attn_tc_supported(const rs_attn_desc& d) {
 // This kernel or the one with three query tiles per CTA (rs_attn_tc3.cu)?  Both are paced by the longest
 // CTA: its items (in tenths) times the key tiles of an item, plus a cost per item; microseconds fitted to
 // CUDA-event times of thirteen shapes from N = 197 to 4097 (worst error 6 % and 9 %).  (Since the three-tile kernel
-// sends a part of its exponentials through the FMA pipes it runs 3 % under its line, and up to 17 % under it where its items
-// run across heads; the lines stay.)
+// sends a part of its exponentials through the FMA pipes it runs 3 % under its line; the lines stay.)
+// With its items across heads the three-tile kernel has a line of its own: the same one at the lower load, the steps a
+// little longer by the share of items with two K/V streams (two in as many items as a head has tiles): 41.3 expected at
+// 128 x 12 x 133, 41.5 us measured, 50.2 / 50.0 at x 197, 80.7 / 77.5 at 28 x 16 x 577.  It is chosen where that is
+// 8 % better, about the errors of the fits: 28 x 16 x 577 91.2 -> 77.5 us, 128 x 12 x 197 55.5 -> 50.0.
 AttnPlan attn_plan(long long BH, int N, int G) {
     const int nt = (N + BQ - 1) / BQ, per = (N + 2 * BQ - 1) / (2 * BQ);
     auto makespan = [&](long long hs) {
@@ -531,7 +534,9 @@ AttnPlan attn_plan(long long BH, int N, int G) {
         const long long u3 = attn_tc3_plan(BH, N, G, &wrap3);
         const double t2 = best / 10.0 * (((N + BKV - 1) / BKV) * 1.505 + 2.51) + 2.32;
         const double t3 = u3 / 10.0 * (((N + 63) / 64) * 1.136 + 1.00) + 6.71;
-        plan.three = t3 < t2;
+        const double two_streams = 1.0 + 0.12 * (nt % 3 ? 2.0 / nt : 0.0);
+        const double t3a = attn_tc3_across_load(BH, N, G) / 10.0 * (((N + 63) / 64) * 1.136 + 1.00) * two_streams + 6.71;
+        plan.three = t3 < t2 || t3a < 0.92 * t2;
         plan.wrap3 = wrap3;
     }
     memo[key] = plan;

@@ -469,6 +469,13 @@ long long attn_tc3_plan(long long BH, int N, int G, int* wrap) {
     return *wrap ? b : a;
 }
 
+// The same load with items across heads: whole rounds of three tiles, then the tiles of the last round one to an item
+// where there are CTAs enough.
+long long attn_tc3_across_load(long long BH, int N, int G) {
+    const long long tiles = BH * ((N + BQ - 1) / BQ), left = tiles % (NG * (long long)G);
+    return (tiles - left) / (NG * (long long)G) * 10 + (left == 0 ? 0 : left <= G ? 7 : 10);
+}
+
 // tmK, tmV: boxes of 64 rows; tmQ: 128 rows; tmO: 32 rows.
 cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMap& tmQ, const CUtensorMap& tmK,
                             const CUtensorMap& tmV, const CUtensorMap& tmO, int wrap, cudaStream_t st) {
@@ -506,8 +513,7 @@ cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMa
     // Items run across heads where that shortens the longest CTA.  (Items with two K/V streams take a little longer:
     // with the loads equal, 8 x 16 x 577 takes 29.7 us within heads and 31.9 across.)  Measured, within / across, us:
     // 128 x 12 x 133 50.2 / 42.2, x 197 61.6 / 50.7, 28 x 16 x 577 88.7 / 78.1, 16 x 12 x 1569 190 / 183, 4 x 16 x 2305 142 / 135.
-    const long long load = args.full / G * 10 + (left == 0 ? 0 : left <= G ? 7 : 10);
-    const bool across = load < tc3_load(BH, d.N, G, wrap);
+    const bool across = attn_tc3_across_load(BH, d.N, G) < tc3_load(BH, d.N, G, wrap);
     const float scale = d.scale != 0.f ? d.scale : 0.125f;
     args.scale_log2 = scale * 1.4426950408889634f;
     args.status = ctx->d_status;

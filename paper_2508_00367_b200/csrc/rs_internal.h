@@ -174,6 +174,7 @@ struct AttnPlan { long long best_hs; int three, wrap3; };
 AttnPlan attn_plan(long long BH, int N, int G);
 // Three query tiles per CTA (rs_attn_tc3.cu), N > 128: the longest CTA's load under its item list, and the launch.
 long long attn_tc3_plan(long long BH, int N, int G, int* wrap);
+long long attn_tc3_across_load(long long BH, int N, int G);
 cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMap& tmQ, const CUtensorMap& tmK,
                             const CUtensorMap& tmV, const CUtensorMap& tmO, int wrap, cudaStream_t st);
 // seq_lens (optional, dev [B]): sample b attends over its first seq_lens[b] tokens only.
