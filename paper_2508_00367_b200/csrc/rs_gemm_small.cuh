@@ -274,7 +274,7 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             }
         }
     }
-    if (splits > 1) cluster_sync(); else __syncthreads();                // no CTA leaves while a peer reads its partial tile
+    if (splits > 1) cluster_leave(); else __syncthreads();               // no CTA leaves while a peer reads its partial tile
     if (*abort_flag && tid == 0) atomicExch(args.status, RS_DEV_TIMEOUT);
     if (warp == 1) {
         tc_fence_after();

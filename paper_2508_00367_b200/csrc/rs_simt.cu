@@ -203,7 +203,7 @@ gemm_simt_kernel(const SimtArgs args) {
         if (args.out_bf16) store_n<__nv_bfloat16, 4>((__nv_bfloat16*)args.out + at, o);
         else store_n<float, 4>((float*)args.out + at, o);
     }
-    if (args.splits > 1) tc::cluster_sync();                             // no CTA leaves while a peer reads its patches
+    if (args.splits > 1) tc::cluster_leave();                            // no CTA leaves while a peer reads its patches
 }
 
 template <typename T, int WM, int WN, int WK, int NJ>
