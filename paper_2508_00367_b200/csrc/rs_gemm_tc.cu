@@ -646,7 +646,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     tc_fence_before();
     __syncthreads();
     if (*abort_flag && threadIdx.x == 0) atomicExch(args.status, RS_DEV_TIMEOUT);
-    cluster_sync();                                      // neither CTA of the pair leaves while the other may signal it
+    cluster_leave();                                     // neither CTA of the pair leaves while the other may signal it
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
