@@ -31,7 +31,7 @@ layernorm_kernel(const TI* __restrict__ x, const float* __restrict__ gamma,
     if (row >= T) return;
     if (lens) {                                  // padding that neither the products nor attention read
         const unsigned b = (unsigned)row / seq_n, i = (unsigned)row - b * seq_n;
-        if ((int)i >= max(__ldg(lens + b), 1) + gemm::kPadRows) return;
+        if ((int)i >= gemm::rows_needed(lens, b, seq_n)) return;
     }
     const int nvec = D / VN;
     const long long src = row_map ? (long long)row_map[row] : row;
@@ -68,7 +68,7 @@ layernorm_narrow_kernel(const float* __restrict__ x, const float* __restrict__ g
         on[u] = row < T;
         if (on[u] && lens) {                     // padding that neither the products nor attention read
             const unsigned b = (unsigned)row / seq_n, i = (unsigned)row - b * seq_n;
-            on[u] = (int)i < max(__ldg(lens + b), 1) + gemm::kPadRows;
+            on[u] = (int)i < gemm::rows_needed(lens, b, seq_n);
         }
         const float* xr = x + (on[u] ? row_map ? (long long)row_map[row] : row : 0) * D;
 #pragma unroll

@@ -41,6 +41,11 @@ struct GemmArgs {
 // Rows behind a sample's own that are computed all the same: attention multiplies values of up to 15 of them by zero
 // weights, so they have to be finite.
 constexpr int kPadRows = 16;
+// Rows of sample b (of seq_n) that have to be computed.  A count is whatever the caller's array holds: it is clamped before
+// kPadRows is added (INT_MAX for "the whole sample" would wrap around).
+__device__ __forceinline__ int rows_needed(const int* __restrict__ lens, int b, int seq_n) {
+    return min(min(max(__ldg(lens + b), 1), seq_n) + kPadRows, seq_n);
+}
 
 // Adds one element of the scored pair (u, v) to the running sums of the chosen distance (Sec. 3.3).  Called with a
 // constant distance in the pair-tile kernel (with_dist): the choice is made once per 32 columns there.

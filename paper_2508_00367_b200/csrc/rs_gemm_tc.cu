@@ -231,7 +231,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const int r0 = (t0 + lane) * 2 * BM, r1 = min(r0 + 2 * BM, args.M);
             bool used = false;
             for (int b = r0 / args.seq_n; r0 < args.M && b * args.seq_n < r1 && !used; ++b)
-                used = b * args.seq_n + min(min(max(__ldg(args.lens + b), 1), args.seq_n) + kPadRows, args.seq_n) > r0;
+                used = b * args.seq_n + rows_needed(args.lens, b, args.seq_n) > r0;
             const uint32_t w = __ballot_sync(0xffffffffu, used);
             if (lane == 0) mask[t0 / 32] = w;
         }

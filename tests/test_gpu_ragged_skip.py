@@ -51,3 +51,26 @@ def test_block_over_poisoned_buffers(ctx, lens, N, D):   # noqa: F811
     torch.cuda.synchronize()
     assert torch.equal(full["x_out"].cpu(), res["x_out"])
     ctx.async_status()
+
+
+@pytest.mark.parametrize("D", [256, 384])                             # both LayerNorm kernels in LN2
+@pytest.mark.parametrize("counts", [[2147483647, 2147483640, 1300, 40], [0, -5, -2147483648, 300]])
+def test_counts_outside_the_sample_are_clamped(ctx, counts, D):   # noqa: F811
+    """seq_lens holds any int: it stands for its value clamped to [1, N], in every kernel, over poisoned buffers too."""
+    import paper_2508_00367_b200 as rs
+    N, B = 300, 4
+    x = synth.make_tokens(B, N, D, "bf16", seed=5).bfloat16().cuda()
+    dw = rs.DeviceBlockWeights(synth.make_block_weights(D, 4 * D, "bf16", seed=6), torch.bfloat16, ctx.device)
+    drops = torch.tensor([0, 30, 0, 7], dtype=torch.int32, device="cuda")
+    got = []
+    for c in (counts, [min(max(n, 1), N) for n in counts]):
+        dl = torch.tensor(c, dtype=torch.int32, device="cuda")
+        torch.cuda.empty_cache()
+        _poison()
+        res = ctx.block_fwd_ragged(x, dw, D // 64, dl, drops, N)
+        torch.cuda.synchronize()
+        got.append({k: v.cpu() for k, v in res.items()})
+    assert torch.isfinite(got[0]["scores"]).all() and torch.isfinite(got[0]["x_out"].float()).all()
+    for k in got[0]:
+        assert torch.equal(got[0][k], got[1][k]), k
+    ctx.async_status()
