@@ -43,27 +43,34 @@ __device__ __forceinline__ uint64_t fadd2(uint64_t a, uint64_t b) {
     return r;
 }
 
+// The larger of the two; NaN if either is (fmaxf drops a NaN).
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
 
 // 2^x for a pair on the FMA pipes instead of the special-function unit: round to nearest by adding 1.5 * 2^23 (whose
-// low mantissa bits then hold the integer), a degree-5 polynomial on [-1/2, 1/2] (least maximum relative error by
-// iterated weighted least squares, 2.1e-7 in fp32 arithmetic -- ex2.approx has 2 ulp), and the integer added to the
-// exponent.  x up to about 120; below -125 the result is 2^-125.
+// low mantissa bits then hold the integer n), a degree-5 polynomial for 2^(x - n) on [-1/2, 1/2] (csrc/fit_ex2.py: relative
+// error 2.2e-7 in fp32 arithmetic -- ex2.approx has 2 ulp), and a product with 2^n.  x up to about 120.  Values that are
+// not finite come out as ex2.approx gives them: NaN stays NaN (max.NaN keeps it, and 2^n is multiplied in, not added to the
+// exponent bits, which would make a number of it), and x below -126.5 gives 0.
 __device__ __forceinline__ void ex2_pair_fma(uint64_t x2, float& p0, float& p1) {
     float x0, x1;
     unpack2(x2, x0, x1);
-    x2 = pack2(fmaxf(x0, -125.f), fmaxf(x1, -125.f));
+    x2 = pack2(max_nan(x0, -127.f), max_nan(x1, -127.f));
     const uint64_t t = fadd2(x2, pack2(12582912.f, 12582912.f));
     const uint64_t f = ffma2(fadd2(t, pack2(-12582912.f, -12582912.f)), pack2(-1.f, -1.f), x2);
-    uint64_t q = ffma2(f, pack2(0.001327647129073739f, 0.001327647129073739f), pack2(0.009675541892647743f, 0.009675541892647743f));
-    q = ffma2(f, q, pack2(0.05550713092088699f, 0.05550713092088699f));
+    uint64_t q = ffma2(f, pack2(0.001327644451521337f, 0.001327644451521337f), pack2(0.00967553723603487f, 0.00967553723603487f));
+    q = ffma2(f, q, pack2(0.05550713464617729f, 0.05550713464617729f));
     q = ffma2(f, q, pack2(0.24022120237350464f, 0.24022120237350464f));
     q = ffma2(f, q, pack2(0.6931469440460205f, 0.6931469440460205f));
     q = ffma2(f, q, pack2(1.0000001192092896f, 1.0000001192092896f));
-    float q0, q1, t0, t1;
-    unpack2(q, q0, q1);
+    float t0, t1;
     unpack2(t, t0, t1);
-    p0 = __uint_as_float(__float_as_uint(q0) + (__float_as_uint(t0) << 23));
-    p1 = __uint_as_float(__float_as_uint(q1) + (__float_as_uint(t1) << 23));
+    const uint64_t scale = pack2(__uint_as_float((__float_as_uint(t0) << 23) + 0x3f800000u),     // 2^n; n = -127: 0
+                                 __uint_as_float((__float_as_uint(t1) << 23) + 0x3f800000u));
+    unpack2(ffma2(q, scale, 0ull), p0, p1);
 }
 
 }  // namespace attn

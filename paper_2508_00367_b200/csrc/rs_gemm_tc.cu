@@ -37,11 +37,7 @@ namespace gemm {
 // coefficient keeps 2^-q -> 0 for large |v|.  Coefficients from csrc/fit_gelu.py.
 // A value stays above -infinity, so that -infinity gives 0; max.NaN keeps a NaN.
 constexpr float kLowest = -3.4e38f;
-__device__ __forceinline__ float max_nan(float a, float b) {
-    float r;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
+using attn::max_nan;
 __device__ __forceinline__ float ex2_ftz(float x) {
     float e;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x));

@@ -219,6 +219,28 @@ def test_gelu_polynomial_matches_exact_erf_gelu():
     assert fg.max_error_fp32(in_kernel) < 1e-6
 
 
+def test_ex2_polynomial_and_its_ends():
+    """The attention kernel's 2^x on the FMA pipes comes from csrc/fit_ex2.py: refit and check the bound that the kernel's
+    comment states, for the coefficients that are compiled in too, and the values that are not finite."""
+    import importlib.util
+    import re
+    import numpy as np
+    csrc = os.path.join(ROOT, "paper_2508_00367_b200", "csrc")
+    spec = importlib.util.spec_from_file_location("fit_ex2", os.path.join(csrc, "fit_ex2.py"))
+    fe = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(fe)
+    assert fe.max_rel_error_fp32(fe.fit()) < 2.2e-7
+    body = open(os.path.join(csrc, "rs_attn.cuh")).read()
+    body = body[body.index("uint64_t q = ffma2(f"):]
+    body = body[:body.index("float t0")]
+    consts = [float(m) for m in re.findall(r"(-?\d+\.\d+(?:e-?\d+)?)f", body)]
+    assert len(consts) == 12 and consts[::2] == consts[1::2]      # both halves of each pair, highest degree first
+    in_kernel = np.array(consts[::-2])
+    assert fe.max_rel_error_fp32(in_kernel) < 2.2e-7
+    ends = fe.ex2_fp32(np.array([-127.0, -1e30, -np.inf, np.nan], dtype=np.float32), in_kernel)
+    assert (ends[:3] == 0).all() and np.isnan(ends[3])
+
+
 def test_attention_kernel_choice_follows_the_measured_winners():
     """The cost model that picks between the two attention kernels (two or three query tiles per thread
     block) against the kernel that was the faster one when both were timed on a B200 of 148 SMs (CUDA
