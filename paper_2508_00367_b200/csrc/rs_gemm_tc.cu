@@ -295,6 +295,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 }
                 if (ok) mma_commit_pair(&tfull[a], 3);  // accumulator complete in both CTAs
             }
+            // The peer's epilogue hands accumulators back by arrivals on this CTA's barriers that nothing else orders: the last
+            // one of either accumulator must have landed before this shared memory can be given to another CTA.  (They
+            // come long before the epilogues' last stores, which this CTA waits for anyway.)
+            for (uint32_t t = tl > 2 ? tl - 2 : 0; t < tl && ok; ++t)
+                ok = mbar_wait(&tempty[t & 1u], (t >> 1) & 1u, abort_flag);
         }
     } else {
         // ---------------- epilogue (both CTAs; each drains its own 128 x BN half) ----------------
@@ -642,7 +647,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     tc_fence_before();
     __syncthreads();
     if (*abort_flag && threadIdx.x == 0) atomicExch(args.status, RS_DEV_TIMEOUT);
-    cluster_leave();                                     // neither CTA of the pair leaves while the other may signal it
+    cluster_leave();                                     // (each CTA has seen everything that its peer signals to it: see the roles' ends)
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();

@@ -279,7 +279,9 @@ __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // The last meeting of a cluster's CTAs, before one of them leaves whose shared memory the others have read: every value read
-// has been used by then, and nothing is handed over, so the arrival need not wait for the thread's stores to global memory.  (The
+// has been used by then, and nothing is handed over, so the arrival need not wait for the thread's stores to global memory.
+// It orders nothing: remote arrivals on a CTA's barriers have to be waited for by that CTA before it comes here (the
+// pair-tile products do that where each role ends).  (The
 // products for few rows of one image of 197 tokens: 0.2 to 0.3 us each of 5 to 8, 503.7 -> 489.7 us for the pass; the pair-tile products 0.3 to 0.6 us: 12608 x 192 x 192 8.2 -> 7.5.)
 __device__ __forceinline__ void cluster_leave() {
     __syncwarp();

@@ -63,3 +63,20 @@ def test_linear_short_k(ctx, M, N, K, epilogue):   # noqa: F811
     got = ctx.linear_fwd(a.cuda(), w.cuda(), b.cuda(), epilogue).cpu().double().numpy()
     want = orc.linear(a.double().numpy(), w.double().numpy(), b.double().numpy())
     parity.check_float(got, orc.round_to(orc.gelu(want) if epilogue == "gelu" else want, "bf16"), "bf16", rounded_output=True)
+
+
+@pytest.mark.parametrize("epilogue", ["bias", "gelu", "residual"])
+def test_pair_products_back_to_back(ctx, epilogue):   # noqa: F811
+    """Pairs with one, two, three and more pieces of work, launch after launch without a pause between them (a CTA's
+    shared memory goes to the next launch at once): the same bits every time, and no wait that ran out."""
+    g = torch.Generator(device="cuda").manual_seed(9)
+    jobs = []
+    for M, N, K in [(3000, 768, 320), (9473, 768, 320), (12700, 576, 192), (19200, 768, 320)]:
+        a, w = torch.randn(M, K, generator=g, device="cuda").bfloat16(), (0.1 * torch.randn(N, K, generator=g, device="cuda")).bfloat16()
+        res = torch.randn(M, N, generator=g, device="cuda").bfloat16() if epilogue == "residual" else None
+        jobs.append((a, w, res))
+    rounds = [[ctx.linear_fwd(a, w, None, epilogue, res) for a, w, res in jobs] for _ in range(25)]
+    ctx.async_status()
+    for outs in rounds[1:]:
+        for first, again in zip(rounds[0], outs):
+            assert torch.equal(first, again)
