@@ -453,7 +453,10 @@ static rs_status block_fwd_impl(rs_ctx* ctx, const rs_block_desc* d, const rs_bl
         } else {
             RS_CHECK_LAUNCH(ctx, RS_K_GEMM, st, rs::launch_gemm_tc(ctx, rs::RS_EPI_BIAS, x_ln, w->w_qkv, w->b_qkv, nullptr, nullptr, nullptr, qkv, RS_BF16, nullptr, 0, 0, T, 3 * D, D, st, nullptr, true, &in_use), "QKV");
         }
-        RS_CHECK_LAUNCH(ctx, RS_K_ATTN, st, rs::launch_attn_tc(ctx, ad, qkv, kp, vp, o, hk ? hk->seq_lens : nullptr, st), "attention");
+        // Blocks that only the 192-column tiles take had fp32 attention weights on the fp32-FMA kernels: bf16 weights raised the
+        // error of their attention score against 64 bits to 1.19x (4 x 50 tokens, D = 192; 1.08x at 32 x 197), two bf16 parts keep it.
+        const bool split_weights = (D % 128) != 0 || (Dm % 128) != 0;
+        RS_CHECK_LAUNCH(ctx, RS_K_ATTN, st, rs::launch_attn_tc(ctx, ad, qkv, kp, vp, o, hk ? hk->seq_lens : nullptr, st, split_weights), "attention");
         // shift through attention (operation choice (i)): partial sums of (SA(LN(x)) - x)^2 from this epilogue
         const bool attn_score = d->score_mode == RS_SCORE_ATTN;
         nparts = rs::gemm_tc_score_parts(D);

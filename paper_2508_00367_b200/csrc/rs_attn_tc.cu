@@ -544,7 +544,7 @@ AttnPlan attn_plan(long long BH, int N, int G) {
 }
 
 cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, const void* k, const void* v,
-                           void* out, const int32_t* seq_lens, cudaStream_t st) {
+                           void* out, const int32_t* seq_lens, cudaStream_t st, bool split_weights) {
     if (!ctx->encode_tiled) return cudaErrorNotSupported;
     static PerDeviceOnce attr_once;   // the attribute belongs to the device current at the call
     int dev = -1;
@@ -571,18 +571,20 @@ cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, co
     long long items = (long long)args.per * (args.dual ? d.B : (long long)d.B * d.H);
     if (items >= (1ll << 30)) return cudaErrorInvalidValue;
     args.n_pair_items = (int)items; args.first_single_bh = d.B * d.H; args.tile_count = (d.N + BQ - 1) / BQ;
+    auto three_tiles = [&](int wrap, bool split) {
+        CUtensorMap tmK3, tmV3;
+        if (!make_tmap_qkv(ctx, &tmK3, k, d.B, d.N, d.H, d.k_batch_stride, d.k_row_stride, d.k_head_stride, 64) ||
+            !make_tmap_qkv(ctx, &tmV3, v, d.B, d.N, d.H, d.v_batch_stride, d.v_row_stride, d.v_head_stride, 64))
+            return cudaErrorInvalidValue;
+        return launch_attn_tc3(ctx, d, tmQ, tmK3, tmV3, tmO, wrap, split, st);
+    };
+    if (split_weights && !seq_lens) return three_tiles(0, true);
     if (!args.dual) {
         const long long BH = (long long)d.B * d.H;
         const int nt = args.tile_count, per = args.per;
         const AttnPlan plan = attn_plan(BH, d.N, ctx->sm_count);
         const int force = ctx->attn_kernel;                    // RS_ATTN_KERNEL=2 / 3: one kernel for every shape it takes
-        if (!seq_lens && (force == 3 || (force != 2 && plan.three))) {
-            CUtensorMap tmK3, tmV3;
-            if (!make_tmap_qkv(ctx, &tmK3, k, d.B, d.N, d.H, d.k_batch_stride, d.k_row_stride, d.k_head_stride, 64) ||
-                !make_tmap_qkv(ctx, &tmV3, v, d.B, d.N, d.H, d.v_batch_stride, d.v_row_stride, d.v_head_stride, 64))
-                return cudaErrorInvalidValue;
-            return launch_attn_tc3(ctx, d, tmQ, tmK3, tmV3, tmO, plan.wrap3, st);
-        }
+        if (!seq_lens && (force == 3 || (force != 2 && plan.three))) return three_tiles(plan.wrap3, false);
         const long long best_hs = plan.best_hs;
         args.n_pair_items = (int)((BH - best_hs) * per);
         args.first_single_bh = (int)(BH - best_hs);

@@ -9,6 +9,9 @@
 // softmax warp; three warps per scheduler instead of two fill more of its gaps.
 // An item is three consecutive 128-row query tiles of one (sample, head), which share the K/V
 // tiles streamed through the TMA ring; or (ACROSS) of consecutive (sample, head)s.
+// SPLIT: the weights go to the second product as a bf16 and the bf16 of what that left over, one after the other
+// through the same tensor-memory columns: 16 bits of mantissa instead of 8, for the blocks that used to have fp32
+// weights (see rs_block_fwd).
 #include <math.h>
 
 #include "rs_internal.h"
@@ -65,6 +68,11 @@ struct Item3 {
     int bh, q;               // (sample, head) and query tile of tile 0
     int ng;                  // query tiles present: 1 .. 3
     int split;               // tiles of the first (sample, head); the others, if any (ACROSS), belong to the next one
+                             // (SPLIT with one query tile per (sample, head): each tile to its own)
+    // which of the item's (sample, head)s tile g belongs to, and whether it is the first or the last tile of one
+    template <bool SPLIT> __device__ __forceinline__ int stream(const Attn3Args& a, int g) const { return SPLIT && a.nt == 1 ? g : g >= split; }
+    template <bool SPLIT> __device__ __forceinline__ bool starts(const Attn3Args& a, int g) const { return g == 0 || g == split || (SPLIT && a.nt == 1); }
+    template <bool SPLIT> __device__ __forceinline__ bool ends(const Attn3Args& a, int g) const { return g == ng - 1 || g == split - 1 || (SPLIT && a.nt == 1); }
 };
 template <bool ACROSS> __device__ __forceinline__ Item3 decode_item3(const Attn3Args& a, int w) {
     Item3 it;
@@ -73,7 +81,7 @@ template <bool ACROSS> __device__ __forceinline__ Item3 decode_item3(const Attn3
         it.ng = min(w < a.full ? NG : a.rest, a.tiles - tile);
         it.bh = tile / a.nt;
         it.q = tile - it.bh * a.nt;
-        it.split = min(it.ng, a.nt - it.q);     // (nt >= 2: three tiles meet one boundary at most)
+        it.split = min(it.ng, a.nt - it.q);     // (nt >= 2: three tiles meet one boundary at most; nt = 1: see stream())
         return it;
     }
     if (w < a.n3) {
@@ -131,8 +139,10 @@ __device__ __forceinline__ float row_max64(const uint32_t (&r)[BKV], int valid) 
 // 4097: 380 us with none, 379 / 371 / 368 / 371 / 382 with 2 / 5 / 6 / 8 / 11 pairs, 435 with all second pairs of four
 // elements; 16 x 12 x 1569 195 -> 190, 32 x 16 x 577 94.3 -> 91.4.  (In the two-tile kernel any share is slower: its two
 // warps per scheduler have no issue slots to spare for it.)
-template <bool MASKED>
-__device__ __forceinline__ float exp_pass64(uint32_t (&r)[BKV], float sl, float mneg, int valid) {
+// SPLIT: lo gets what the bf16s in r leave of the p_i, as bf16 pairs (and the exponentials all go to the special-function
+// unit, which is not the busiest pipe there).
+template <bool MASKED, bool SPLIT>
+__device__ __forceinline__ float exp_pass64(uint32_t (&r)[BKV], uint32_t (&lo)[SPLIT ? BKV / 2 : 1], float sl, float mneg, int valid) {
     const uint64_t sl2 = pack2(sl, sl), mneg2 = pack2(mneg, mneg);
     uint64_t l01 = pack2(0.f, 0.f), l23 = l01;
 #pragma unroll
@@ -149,12 +159,17 @@ __device__ __forceinline__ float exp_pass64(uint32_t (&r)[BKV], float sl, float 
         const float p0 = ex2(x0), p1 = ex2(x1);   // ex2(-inf) = 0
         float p2, p3;
         constexpr int kByFma = 0x52;                     // which of eight consecutive groups of four send their second pair there
-        if (!MASKED && ((kByFma >> ((i / 4) % 8)) & 1)) ex2_pair_fma(pack2(x2, x3), p2, p3);
+        if (!MASKED && !SPLIT && ((kByFma >> ((i / 4) % 8)) & 1)) ex2_pair_fma(pack2(x2, x3), p2, p3);
         else { p2 = ex2(x2); p3 = ex2(x3); }
         l01 = fadd2(l01, pack2(p0, p1));
         l23 = fadd2(l23, pack2(p2, p3));
-        r[i >> 1] = pack_bf16(p0, p1);
-        r[(i >> 1) + 1] = pack_bf16(p2, p3);
+        const uint32_t h01 = pack_bf16(p0, p1), h23 = pack_bf16(p2, p3);
+        if constexpr (SPLIT) {
+            lo[i >> 1] = pack_bf16(p0 - __uint_as_float(h01 << 16), p1 - __uint_as_float(h01 & 0xffff0000u));
+            lo[(i >> 1) + 1] = pack_bf16(p2 - __uint_as_float(h23 << 16), p3 - __uint_as_float(h23 & 0xffff0000u));
+        }
+        r[i >> 1] = h01;
+        r[(i >> 1) + 1] = h23;
     }
     float a, b, c, d;
     unpack2(l01, a, b);
@@ -162,10 +177,12 @@ __device__ __forceinline__ float exp_pass64(uint32_t (&r)[BKV], float sl, float 
     return (a + b) + (c + d);
 }
 
-template <bool ACROSS>
+template <bool ACROSS, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO, const Attn3Args args) {
+    static_assert(ACROSS || !SPLIT, "the split weights come with items across heads only");
+    constexpr int PARTS = SPLIT ? 2 : 1;     // products P V per key tile
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + OFF_BAR);
@@ -218,22 +235,22 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 if (!mbar_wait(&q_empty[qb], ((item_n >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
                 mbar_expect_tx(&q_full[qb], it.ng * Q_BYTES);
                 const int b0 = it.bh / args.H, h0 = it.bh - b0 * args.H;
-                const bool turn = h0 + 1 == args.H;               // the next (sample, head) is the next sample's first
-                const int b1 = turn ? b0 + 1 : b0, h1 = turn ? 0 : h0 + 1;
-                for (int g = 0; g < it.ng; ++g)
-                    tma_load_4d(smem + OFF_Q + (qb * NG + g) * Q_BYTES, &tmQ, &q_full[qb], 0, g < it.split ? h0 : h1,
-                                (g < it.split ? it.q + g : g - it.split) * BQ, g < it.split ? b0 : b1);
-                const bool two = ACROSS && it.split < it.ng;
-                for (int t = 0; t < (two ? 2 * nkv : nkv); ++t, ++kv_it) {
-                    const int s = kv_it % NS, row0 = (two ? t >> 1 : t) * BKV;
-                    const bool second = two && (t & 1);
-                    if (!mbar_wait(&k_empty[s], ((kv_it / NS) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
-                    mbar_expect_tx(&k_full[s], KV_BYTES);
-                    tma_load_4d(smem + OFF_K + s * KV_BYTES, &tmK, &k_full[s], 0, second ? h1 : h0, row0, second ? b1 : b0);
-                    if (!mbar_wait(&v_empty[s], ((kv_it / NS) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
-                    mbar_expect_tx(&v_full[s], KV_BYTES);
-                    tma_load_4d(smem + OFF_V + s * KV_BYTES, &tmV, &v_full[s], 0, second ? h1 : h0, row0, second ? b1 : b0);
+                auto next = [&](int& b, int& h) { if (++h == args.H) { h = 0; ++b; } };      // the next (sample, head)
+                for (int g = 0, b = b0, h = h0; g < it.ng; ++g) {
+                    if (ACROSS && g && it.starts<SPLIT>(args, g)) next(b, h);
+                    tma_load_4d(smem + OFF_Q + (qb * NG + g) * Q_BYTES, &tmQ, &q_full[qb], 0, h, (it.q + g - it.stream<SPLIT>(args, g) * args.nt) * BQ, b);
                 }
+                const int streams = ACROSS ? it.stream<SPLIT>(args, it.ng - 1) + 1 : 1;
+                for (int t = 0; t < nkv && ok; ++t)
+                    for (int sm = 0, b = b0, h = h0; sm < streams; ++sm, ++kv_it, next(b, h)) {
+                        const int s = kv_it % NS;
+                        if (!mbar_wait(&k_empty[s], ((kv_it / NS) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+                        mbar_expect_tx(&k_full[s], KV_BYTES);
+                        tma_load_4d(smem + OFF_K + s * KV_BYTES, &tmK, &k_full[s], 0, h, t * BKV, b);
+                        if (!mbar_wait(&v_empty[s], ((kv_it / NS) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+                        mbar_expect_tx(&v_full[s], KV_BYTES);
+                        tma_load_4d(smem + OFF_V + s * KV_BYTES, &tmV, &v_full[s], 0, h, t * BKV, b);
+                    }
             }
             // every copy started here must have landed before the CTA exits
             for (uint32_t n = item_n > 2 ? item_n - 2 : 0; n < item_n && ok; ++n)
@@ -266,7 +283,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 #pragma unroll
                     for (int g = 0; g < NG; ++g) {
                         if (g >= it.ng || !ok) continue;
-                        if (g == 0 || (ACROSS && g == it.split)) {   // a (sample, head)'s first tile: the next ring stage
+                        if (ACROSS ? it.starts<SPLIT>(args, g) : g == 0) {   // a (sample, head)'s first tile: the next ring stage
                             stage = t % NS;
                             if (!mbar_wait(&k_full[stage], (t / NS) & 1u, abort_flag)) { ok = false; continue; }
                             dk = k_lo + (uint32_t)stage * kKV16;
@@ -280,7 +297,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                             mma_ss_lh(tmem_base + kSCol + g * BKV, dq + 2u * k, dk + 2u * k, desc_hi, idesc_s, k != 0);
                         mma_commit(&s_full[g]);
                         ++ns[g];
-                        if (ACROSS && (g == it.ng - 1 || g == it.split - 1)) mma_commit(&k_empty[stage]);
+                        if (ACROSS && it.ends<SPLIT>(args, g)) mma_commit(&k_empty[stage]);
                     }
                     if (!ACROSS && ok) mma_commit(&k_empty[stage]);
                 }
@@ -305,23 +322,31 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                     const int ksteps = (min(BKV, args.N - j * BKV) + 15) >> 4;
                     int stage = 0;
                     uint32_t dv = 0;
+                    int stage_of[NG];                    // SPLIT: kept for the second part
 #pragma unroll
-                    for (int g = 0; g < NG; ++g) {
-                        if (g >= it.ng || !ok) continue;
-                        if (g == 0 || (ACROSS && g == it.split)) {
-                            stage = t % NS;
-                            if (!mbar_wait(&v_full[stage], (t / NS) & 1u, abort_flag)) { ok = false; continue; }
-                            dv = v_lo + (uint32_t)stage * kKV16;
-                            ++t;
+                    for (int part = 0; part < PARTS; ++part) {
+#pragma unroll
+                        for (int g = 0; g < NG; ++g) {
+                            if (g >= it.ng || !ok) continue;
+                            if (part == 0 && (ACROSS ? it.starts<SPLIT>(args, g) : g == 0)) {
+                                stage = t % NS;
+                                if (!mbar_wait(&v_full[stage], (t / NS) & 1u, abort_flag)) { ok = false; continue; }
+                                dv = v_lo + (uint32_t)stage * kKV16;
+                                ++t;
+                            }
+                            if (SPLIT) {
+                                if (part == 0) stage_of[g] = stage;
+                                else { stage = stage_of[g]; dv = v_lo + (uint32_t)stage * kKV16; }
+                            }
+                            if (!mbar_wait(&p_ready[g], np[g] & 1u, abort_flag)) { ok = false; continue; }
+                            tc_fence_after();
+                            const uint32_t o_col = tmem_base + kOCol + g * DH, p_col = tmem_base + kPCol + g * (BKV / 2);
+                            for (int k = 0; k < ksteps; ++k)
+                                mma_ts_lh(o_col, p_col + 8 * k, dv + 128u * k, desc_hi, idesc_o, !(j == 0 && part == 0 && k == 0));
+                            mma_commit(&o_done[g]);
+                            ++np[g];
+                            if (ACROSS && part == PARTS - 1 && it.ends<SPLIT>(args, g)) mma_commit(&v_empty[stage]);
                         }
-                        if (!mbar_wait(&p_ready[g], np[g] & 1u, abort_flag)) { ok = false; continue; }
-                        tc_fence_after();
-                        const uint32_t o_col = tmem_base + kOCol + g * DH, p_col = tmem_base + kPCol + g * (BKV / 2);
-                        for (int k = 0; k < ksteps; ++k)
-                            mma_ts_lh(o_col, p_col + 8 * k, dv + 128u * k, desc_hi, idesc_o, !(j == 0 && k == 0));
-                        mma_commit(&o_done[g]);
-                        ++np[g];
-                        if (ACROSS && (g == it.ng - 1 || g == it.split - 1)) mma_commit(&v_empty[stage]);
                     }
                     if (!ACROSS && ok) mma_commit(&v_empty[stage]);
                 }
@@ -343,7 +368,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         for (int w = item_of<ACROSS>(args, 0); w >= 0 && ok; w = item_of<ACROSS>(args, ++item_n)) {
             const Item3 it = decode_item3<ACROSS>(args, w);
             if (g >= it.ng) continue;
-            const int bh = it.bh + (g < it.split ? 0 : 1), row0 = (g < it.split ? it.q + g : g - it.split) * BQ + q * 32;
+            const int sm = it.stream<SPLIT>(args, g), bh = it.bh + sm, row0 = (it.q + g - sm * args.nt) * BQ + q * 32;
             float m_l2 = 0.f, l_run = 0.f;               // running maximum (times scale*log2 e) and sum
             for (int j = 0; j < nkv && ok; ++j, ++cnt) {
                 const int valid = min(BKV, args.N - j * BKV);
@@ -366,7 +391,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                     m_l2 = mx_l2;
                 } else if (__any_sync(0xffffffffu, mx_l2 > m_l2 + kRescaleGap)) {
                     // rare: rescale O and the sum; O += P V of the previous key tile must have retired
-                    if (!__all_sync(0xffffffffu, mbar_wait(&o_done[g], (cnt - 1) & 1u, abort_flag))) { ok = false; break; }
+                    if (!__all_sync(0xffffffffu, mbar_wait(&o_done[g], (cnt * PARTS - 1) & 1u, abort_flag))) { ok = false; break; }
                     tc_fence_after();
                     const bool raise = mx_l2 > m_l2 + kRescaleGap;
                     const float alpha = raise ? ex2(m_l2 - mx_l2) : 1.f;
@@ -383,10 +408,11 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                     }
                     tmem_wait_st();
                 }
-                l_run += valid == BKV ? exp_pass64<false>(r, sl, -m_l2, valid) : exp_pass64<true>(r, sl, -m_l2, valid);
+                uint32_t lo[SPLIT ? BKV / 2 : 1];
+                l_run += valid == BKV ? exp_pass64<false, SPLIT>(r, lo, sl, -m_l2, valid) : exp_pass64<true, SPLIT>(r, lo, sl, -m_l2, valid);
                 if (cnt > 0) {
                     // P V of the previous key tile reads the P columns: it must have retired
-                    if (!__all_sync(0xffffffffu, mbar_wait(&o_done[g], (cnt - 1) & 1u, abort_flag))) { ok = false; break; }
+                    if (!__all_sync(0xffffffffu, mbar_wait(&o_done[g], (cnt * PARTS - 1) & 1u, abort_flag))) { ok = false; break; }
                     tc_fence_after();
                 }
                 tmem_st_32x32(p_addr, r);
@@ -394,9 +420,18 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&p_ready[g]);
+                if constexpr (SPLIT) {                   // the rest of the weights, when the product with the first part is done
+                    if (!__all_sync(0xffffffffu, mbar_wait(&o_done[g], 0, abort_flag))) { ok = false; break; }
+                    tc_fence_after();
+                    tmem_st_32x32(p_addr, lo);
+                    tmem_wait_st();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&p_ready[g]);
+                }
             }
             // epilogue of the item: O / l -> bf16 -> global
-            if (!ok || !__all_sync(0xffffffffu, mbar_wait(&o_done[g], (cnt - 1) & 1u, abort_flag))) { ok = false; break; }
+            if (!ok || !__all_sync(0xffffffffu, mbar_wait(&o_done[g], (cnt * PARTS - 1) & 1u, abort_flag))) { ok = false; break; }
             tc_fence_after();
             const float inv = 1.f / l_run;
             uint32_t o[64];
@@ -478,15 +513,16 @@ long long attn_tc3_across_load(long long BH, int N, int G) {
 
 // tmK, tmV: boxes of 64 rows; tmQ: 128 rows; tmO: 32 rows.
 cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMap& tmQ, const CUtensorMap& tmK,
-                            const CUtensorMap& tmV, const CUtensorMap& tmO, int wrap, cudaStream_t st) {
-    if (d.N <= BQ) return cudaErrorInvalidValue;          // one query tile: the two-heads-per-item kernel's
+                            const CUtensorMap& tmV, const CUtensorMap& tmO, int wrap, bool split, cudaStream_t st) {
+    if (d.N <= BQ && !split) return cudaErrorInvalidValue;          // one query tile: the two-heads-per-item kernel's
     static PerDeviceOnce attr_once;   // the attribute belongs to the device current at the call
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     e = (cudaError_t)attr_once.run(dev, [] {
-        cudaError_t a = cudaFuncSetAttribute(attn_tc3_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-        if (a == cudaSuccess) a = cudaFuncSetAttribute(attn_tc3_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+        cudaError_t a = cudaFuncSetAttribute(attn_tc3_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+        if (a == cudaSuccess) a = cudaFuncSetAttribute(attn_tc3_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+        if (a == cudaSuccess) a = cudaFuncSetAttribute(attn_tc3_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
         return (int)a;
     });
     if (e != cudaSuccess) return e;
@@ -513,14 +549,15 @@ cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMa
     // Items run across heads where that shortens the longest CTA.  (Items with two K/V streams take a little longer:
     // with the loads equal, 8 x 16 x 577 takes 29.7 us within heads and 31.9 across.)  Measured, within / across, us:
     // 128 x 12 x 133 50.2 / 42.2, x 197 61.6 / 50.7, 28 x 16 x 577 88.7 / 78.1, 16 x 12 x 1569 190 / 183, 4 x 16 x 2305 142 / 135.
-    const bool across = attn_tc3_across_load(BH, d.N, G) < tc3_load(BH, d.N, G, wrap);
+    const bool across = split || attn_tc3_across_load(BH, d.N, G) < tc3_load(BH, d.N, G, wrap);
     const float scale = d.scale != 0.f ? d.scale : 0.125f;
     args.scale_log2 = scale * 1.4426950408889634f;
     args.status = ctx->d_status;
     const long long all = across ? args.n_items : (long long)args.n3 + args.n_tail;
     const int grid = all < G ? (int)all : G;
-    if (across) return launch_pdl(attn_tc3_kernel<true>, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args);
-    return launch_pdl(attn_tc3_kernel<false>, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args);
+    if (split) return launch_pdl(attn_tc3_kernel<true, true>, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args);
+    if (across) return launch_pdl(attn_tc3_kernel<true, false>, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args);
+    return launch_pdl(attn_tc3_kernel<false, false>, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args);
 }
 
 }  // namespace rs

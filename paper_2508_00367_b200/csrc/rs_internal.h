@@ -176,9 +176,10 @@ AttnPlan attn_plan(long long BH, int N, int G);
 long long attn_tc3_plan(long long BH, int N, int G, int* wrap);
 long long attn_tc3_across_load(long long BH, int N, int G);
 cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMap& tmQ, const CUtensorMap& tmK,
-                            const CUtensorMap& tmV, const CUtensorMap& tmO, int wrap, cudaStream_t st);
+                            const CUtensorMap& tmV, const CUtensorMap& tmO, int wrap, bool split, cudaStream_t st);
 // seq_lens (optional, dev [B]): sample b attends over its first seq_lens[b] tokens only.
+// split_weights: the softmax weights are multiplied with V as two bf16 parts (16 bits of mantissa); without seq_lens only.
 cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, const void* k, const void* v,
-                           void* out, const int32_t* seq_lens, cudaStream_t st);
+                           void* out, const int32_t* seq_lens, cudaStream_t st, bool split_weights = false);
 
 }  // namespace rs

@@ -56,3 +56,31 @@ def test_layer_loop_of_three_heads_with_folded_ln1(ctx):   # noqa: F811
             parity.check_float(o["x_out"].double().cpu().numpy(), orc.round_to(ref["x_out"], "bf16"), "bf16", True)
         cur = o["x_out"]
     ctx.async_status()
+
+
+@pytest.mark.parametrize("B,N,D", [(4, 50, 192), (3, 1, 192), (2, 64, 192), (31, 100, 192), (60, 128, 192), (2, 129, 192), (32, 197, 192), (1, 65, 576),
+                                   (3, 320, 576), (2, 513, 960), (1, 1201, 192)])
+def test_attention_weights_of_these_widths(ctx, B, N, D, monkeypatch):   # noqa: F811
+    """These blocks ran on the fp32-FMA kernels with fp32 attention weights: the error of what attention adds, against 64
+    bits, stays what those kernels make of the same roundings (bf16 weights: 1.04 to 1.19 times as much)."""
+    import paper_2508_00367_b200 as rs
+    monkeypatch.setenv("RS_DISABLE_TC", "1")
+    fma = rs.Context(0)
+    monkeypatch.delenv("RS_DISABLE_TC")
+    x, w = synth.make_tokens(B, N, D, "bf16", seed=N), synth.make_block_weights(D, 4 * D, "bf16", seed=D)
+    # values well above the other terms' roundings: attention's output counts
+    w["w_qkv"][2 * D:] *= 8
+    wd = {k: v.double().cuda() for k, v in w.items()}
+    xd = x.double().cuda()
+    u = torch.nn.functional.layer_norm(xd, (D,), wd["ln1_g"], wd["ln1_b"], 1e-6)
+    q, k, v = (u @ wd["w_qkv"].T + wd["b_qkv"]).view(B, N, 3, D // 64, 64).permute(2, 0, 3, 1, 4)
+    att = (torch.softmax(q @ k.transpose(2, 3) / 8.0, -1) @ v).transpose(1, 2).reshape(B, N, D)
+    want = (att @ wd["w_o"].T + wd["b_o"]).norm(dim=-1)
+    err = []
+    for c in (ctx, fma):
+        dw = rs.DeviceBlockWeights(w, torch.bfloat16, c.device)
+        res = c.block_fwd(x.bfloat16().cuda(), dw, D // 64, 0, out_dtype=torch.float32, score_mode="attn")
+        c.async_status()
+        err.append((res["scores"].double() - ((att @ wd["w_o"].T + wd["b_o"]) - xd).norm(dim=-1)).norm().item())
+    assert want.min() > 0 and err[0] <= 1.02 * err[1], err
+    fma.close()
