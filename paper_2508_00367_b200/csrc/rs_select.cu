@@ -508,6 +508,17 @@ cudaError_t launch_copy(const void* x, const Src& src, long long rows, int row_v
     return launch_pdl(gather_kernel<4, void, Src>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, (const uint4*)x, src, (unsigned)rows, row_vecs, (uint4*)x_out, ln);
 }
 
+// launch(first sample, rows) over whole samples of `per_sample` rows: the kernels count the rows of a launch in 32 bits, so a
+// batch of 2^31 rows or more goes in several launches.
+template <typename F> cudaError_t by_samples(int B, int per_sample, F launch) {
+    const long long most = ((1ll << 31) - 1) / per_sample;
+    for (long long b0 = 0; b0 < B; b0 += most) {
+        const cudaError_t e = launch(b0, (B - b0 < most ? B - b0 : most) * per_sample);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 }  // namespace
 
 cudaError_t launch_select(const float* scores, int nparts, float* scores_out, int B, int N, int K, int has_cls,
@@ -538,19 +549,24 @@ bool ln_fusable(rs_dtype dtype, int D) { return (size_t)D * dtype_size(dtype) / 
 
 cudaError_t launch_gather(rs_dtype dtype, const void* x, const int32_t* keep_idx, int B, int N, int K,
                           int D, void* x_out, const LnFuse* ln, cudaStream_t st) {
-    const long long rows = (long long)B * K;
-    if (rows == 0) return cudaSuccess;
-    if (rows >= (1ll << 31)) return cudaErrorInvalidValue;
+    if (B == 0 || K == 0) return cudaSuccess;
     const int row_vecs = (int)((size_t)D * dtype_size(dtype) / 16);
     const bool norm = ln && ln->gamma;               // else ln, if given, only asks for the row sums of the copy
     if ((norm && !ln_fusable(dtype, D)) || (!x_out && !norm)) return cudaErrorInvalidValue;
     const LnFuse none = {nullptr, nullptr, 0.f, nullptr, nullptr};
-    const TokenRows src = {keep_idx, (unsigned)K, N};
-    if (!norm) return launch_copy(x, src, rows, row_vecs, x_out, ln ? *ln : none, st);
-    const dim3 grid((unsigned)((rows + 7) / 8));
-    if (dtype == RS_BF16)
-        return launch_pdl(gather_kernel<4, __nv_bfloat16, TokenRows>, grid, dim3(256), 0, st, (const uint4*)x, src, (unsigned)rows, row_vecs, (uint4*)x_out, *ln);
-    return launch_pdl(gather_kernel<4, float, TokenRows>, grid, dim3(256), 0, st, (const uint4*)x, src, (unsigned)rows, row_vecs, (uint4*)x_out, *ln);
+    return by_samples(B, K, [&](long long b0, long long rows) {
+        const uint4* xb = (const uint4*)x + b0 * N * row_vecs;
+        uint4* ob = x_out ? (uint4*)x_out + b0 * K * row_vecs : nullptr;
+        LnFuse lb = ln ? *ln : none;
+        if (norm) lb.out = (char*)ln->out + (size_t)b0 * K * D * dtype_size(dtype);
+        if (lb.stats) lb.stats += 2 * b0 * K;
+        const TokenRows src = {keep_idx + b0 * K, (unsigned)K, N};
+        if (!norm) return launch_copy(xb, src, rows, row_vecs, ob, lb, st);
+        const dim3 grid((unsigned)((rows + 7) / 8));
+        if (dtype == RS_BF16)
+            return launch_pdl(gather_kernel<4, __nv_bfloat16, TokenRows>, grid, dim3(256), 0, st, xb, src, (unsigned)rows, row_vecs, ob, lb);
+        return launch_pdl(gather_kernel<4, float, TokenRows>, grid, dim3(256), 0, st, xb, src, (unsigned)rows, row_vecs, ob, lb);
+    });
 }
 
 int linewise_max_lines() { return kLineMax; }
@@ -563,12 +579,13 @@ cudaError_t launch_line_select(const float* scores, int B, int H, int W, int Hk,
 
 cudaError_t launch_line_gather(rs_dtype dtype, const void* x, const int32_t* keep_rows, const int32_t* keep_cols, int B, int H,
                                int W, int Hk, int Wk, int D, void* x_out, cudaStream_t st) {
-    const long long rows = (long long)B * Hk * Wk;
-    if (rows == 0) return cudaSuccess;
-    if (rows >= (1ll << 31)) return cudaErrorInvalidValue;
-    const GridRows src = {keep_rows, keep_cols, (unsigned)Hk, (unsigned)Wk, H, W};
+    if (B == 0) return cudaSuccess;
+    const int row_vecs = (int)((size_t)D * dtype_size(dtype) / 16);
     const LnFuse none = {nullptr, nullptr, 0.f, nullptr, nullptr};
-    return launch_copy(x, src, rows, (int)((size_t)D * dtype_size(dtype) / 16), x_out, none, st);
+    return by_samples(B, Hk * Wk, [&](long long b0, long long rows) {
+        const GridRows src = {keep_rows + b0 * Hk, keep_cols + b0 * Wk, (unsigned)Hk, (unsigned)Wk, H, W};
+        return launch_copy((const uint4*)x + b0 * H * W * row_vecs, src, rows, row_vecs, (uint4*)x_out + b0 * Hk * Wk * row_vecs, none, st);
+    });
 }
 
 }  // namespace rs

@@ -63,3 +63,48 @@ def test_grid_rows_of_every_width_class(ctx, pieces, H, W, dr, dc):   # noqa: F8
     np.testing.assert_array_equal(kc.cpu().numpy(), want_c)
     for b in range(2):
         assert torch.equal(xo[b].cpu(), x[b][torch.from_numpy(want_r[b]).long()][:, torch.from_numpy(want_c[b]).long()])
+
+
+def _needs_memory(nbytes):
+    torch.cuda.empty_cache()
+    if torch.cuda.mem_get_info()[0] < nbytes:
+        pytest.skip("not enough free device memory")
+
+
+def test_more_kept_rows_than_a_launch_counts(ctx):   # noqa: F811
+    """2^31 kept rows and more: the samples around the place where the second launch begins, the first and the last."""
+    N, r, D = 32768, 1, 8
+    K = N - r
+    cut = (2 ** 31 - 1) // K                                         # samples of the first launch
+    B = cut + 3
+    _needs_memory(100 << 30)
+    x, s = torch.empty(B, N, D, dtype=torch.bfloat16, device="cuda"), torch.zeros(B, N, device="cuda")
+    look = [0, 1, cut - 1, cut, cut + 1, B - 1]
+    x[look] = torch.randn(len(look), N, D, device="cuda").bfloat16()
+    for i, b in enumerate(look):
+        s[b, 5 + i] = -1.0                                           # the token that goes
+    x_out, keep = ctx.topk_compact(s, x, r)
+    for i, b in enumerate(look):
+        want = [t for t in range(N) if t != 5 + i]
+        assert keep[b].tolist() == want and torch.equal(x_out[b], x[b, want])
+    del x, s, x_out, keep
+    torch.cuda.empty_cache()
+
+
+def test_more_kept_positions_than_a_launch_counts(ctx):   # noqa: F811
+    H = W = 256
+    D, dr, dc = 8, 1, 0
+    cut = (2 ** 31 - 1) // ((H - dr) * (W - dc))
+    B = cut + 2
+    _needs_memory(100 << 30)
+    x, s = torch.empty(B, H, W, D, dtype=torch.bfloat16, device="cuda"), torch.ones(B, H, W, device="cuda")
+    look = [0, cut - 1, cut, B - 1]
+    x[look] = torch.randn(len(look), H, W, D, device="cuda").bfloat16()
+    for i, b in enumerate(look):
+        s[b, 7 + i] = 0.0                                            # the line that goes
+    x_out, rows, cols = ctx.linewise_compact(s, x, dr, dc)
+    for i, b in enumerate(look):
+        want = [t for t in range(H) if t != 7 + i]
+        assert rows[b].tolist() == want and cols[b].tolist() == list(range(W)) and torch.equal(x_out[b], x[b, want])
+    del x, s, x_out, rows, cols
+    torch.cuda.empty_cache()
