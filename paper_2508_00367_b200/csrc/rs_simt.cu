@@ -86,9 +86,10 @@ gemm_simt_kernel(const SimtArgs args) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int wk = warp / (WM * WN), wm = (warp % (WM * WN)) / WN, wn = warp % WN;
     const int ty = lane >> 3, tx = lane & 7;
-    const int rank = blockIdx.x;                                         // the cluster spans grid dimension x
-    const long long m0 = (long long)blockIdx.z * C::TM;
-    const int n0 = blockIdx.y * C::TN;
+    // grid dimension x: the clusters of `splits` (a power of two) along N -- x alone has room for every N --, y: along M
+    const int rank = blockIdx.x & (args.splits - 1);
+    const long long m0 = (long long)blockIdx.y * C::TM;
+    const int n0 = (blockIdx.x >> (__ffs(args.splits) - 1)) * C::TN;
     const T* A = reinterpret_cast<const T*>(args.A);
     const T* W = reinterpret_cast<const T*>(args.W);
     const int K = args.K, slabs = (K + C::BK - 1) / C::BK;
@@ -220,7 +221,7 @@ cudaError_t launch_simt(const SimtArgs& args, cudaStream_t st) {
     const long long mt = (args.M + C::TM - 1) / C::TM;
     if (mt > 65535) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)args.splits, (unsigned)((args.N + C::TN - 1) / C::TN), (unsigned)mt);
+    cfg.gridDim = dim3((unsigned)args.splits * (unsigned)(((long long)args.N + C::TN - 1) / C::TN), (unsigned)mt, 1);
     cfg.blockDim = dim3(C::THREADS, 1, 1);
     cfg.dynamicSmemBytes = C::SMEM;
     cfg.stream = st;

@@ -28,6 +28,15 @@ def test_linear_fp32_edges(ctx, M, N, K, epilogue):   # noqa: F811
     assert (np.abs(got[rows] - want) <= bound).all()
 
 
+def test_linear_fp32_of_many_columns(ctx):   # noqa: F811
+    """More than 65535 tiles of 32 columns."""
+    M, N, K = 3, 2_200_008, 40
+    g = torch.Generator(device="cuda").manual_seed(3)
+    a, w = torch.randn(M, K, generator=g, device="cuda"), torch.randn(N, K, generator=g, device="cuda")
+    got, want = ctx.linear_fwd(a, w), a.double() @ w.double().T
+    assert ((got.double() - want).norm() / want.norm()).item() < 1e-6      # fp32 sums of 40 products
+
+
 @pytest.mark.parametrize("M,N,K", [(1, 72, 72), (70, 200, 328), (400, 1000, 64)])       # widths the tensor cores do not take
 def test_linear_bf16_on_fma_kernels(ctx, M, N, K):   # noqa: F811
     g = torch.Generator().manual_seed(M + N + K)
