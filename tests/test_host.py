@@ -257,3 +257,8 @@ def test_attention_kernel_choice_follows_the_measured_winners():
         assert rs.attn_kernel_choice(148, 64, 12, N) == 2        # one query tile per head: two heads per item
     assert rs.attn_kernel_choice(0, 1, 1, 1) == 0
 
+
+def test_a_layer_loop_of_no_blocks_can_be_made():
+    import torch
+    import paper_2508_00367_b200 as rs
+    assert rs.PrunedViT(None, [], 6, [], torch.bfloat16).drops == []
