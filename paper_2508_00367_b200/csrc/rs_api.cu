@@ -272,7 +272,7 @@ rs_status rs_shift_score(rs_ctx* ctx, rs_dtype dtype, rs_dist dist, int B, int N
     if (!after || !before || !scores) return fail(ctx, RS_ERR_INVALID_ARG, "rs_shift_score: null pointer");
     if (!aligned16(after) || !aligned16(before) || (reinterpret_cast<uintptr_t>(scores) & 3u))
         return fail(ctx, RS_ERR_INVALID_ARG, "rs_shift_score: misaligned pointer");
-    RS_CHECK_LAUNCH(ctx, RS_K_SCORE, (cudaStream_t)stream, rs::launch_shift_score(dtype, dist, (long long)B * N, D, after, before, scores, (cudaStream_t)stream),
+    RS_CHECK_LAUNCH(ctx, RS_K_SCORE, (cudaStream_t)stream, rs::launch_shift_score(dtype, dist, (long long)B * N, D, after, before, scores, ctx->sm_count, (cudaStream_t)stream),
                     "shift score launch");
     return RS_OK;
 }

@@ -119,8 +119,9 @@ layernorm_narrow_kernel(const float* __restrict__ x, const float* __restrict__ g
 // s = D(F(x), x) per token (Sec. 3.2); DIST 0: L2, 1: L1, 2: cosine distance.
 // Bound by HBM.  The 16-byte pieces stay packed in registers until they are reduced, so that eight loads per
 // lane are in flight at about 48 registers per thread and enough warps fit an SM to cover the HBM latency.
-// `before` is read with an evict-first hint: what the L2 can keep of the two is then `after`, whose kept rows
-// the compaction reads next.
+// With HINT `before` is read with an evict-first hint: what the L2 can keep of the two is then `after`, whose kept rows
+// the compaction reads next.  Inputs that the L2 holds anyway go without it: 5000 x 256 bf16 2.3 us with, 1.9 without,
+// 20000 x 768 7.0 / 6.45 (the cosine's three sums are scheduled better with it, 2.5 / 2.9: always on there).
 template <typename T, int DIST> struct ShiftSums {
     float acc = 0.f, aa = 0.f, bb = 0.f;
     __device__ __forceinline__ void add(const uint4& ra, const uint4& rb) {
@@ -153,7 +154,7 @@ template <typename T, int DIST> struct ShiftSums {
 };
 
 // One warp per token.
-template <typename T, int DIST>
+template <typename T, int DIST, bool HINT>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, 5)
 shift_score_kernel(const T* __restrict__ after, const T* __restrict__ before, long long rows, int D,
                    float* __restrict__ scores) {
@@ -173,7 +174,7 @@ shift_score_kernel(const T* __restrict__ after, const T* __restrict__ before, lo
 #pragma unroll
         for (int u = 0; u < UNROLL; ++u) {
             const int iv = base + u * 32 + lane;
-            if (iv < nvec) { ra[u] = ld_stream(a + iv); rb[u] = ld_stream(b + iv, once); }
+            if (iv < nvec) { ra[u] = ld_stream(a + iv); rb[u] = HINT ? ld_stream(b + iv, once) : ld_stream(b + iv); }
         }
 #pragma unroll
         for (int u = 0; u < UNROLL; ++u)
@@ -183,10 +184,10 @@ shift_score_kernel(const T* __restrict__ after, const T* __restrict__ before, lo
     if (lane == 0) scores[row] = d;
 }
 
-// Tokens of at most 32 * VPR pieces (VPR 1 or 2): 4 / VPR groups of 32 >> lsh tokens side by side per warp, 1 << lsh
+// Tokens of at most 32 * VPR pieces (VPR 1 or 2), many of them (launch_shift_score): 4 / VPR groups of 32 >> lsh tokens side by side per warp, 1 << lsh
 // lanes per token, so that a lane has eight loads in flight here too (a warp per token of 256 bf16 had two:
 // 64 x 56 x 56 positions took 56 us = 3.7 TB/s; this takes 36 = 5.7 TB/s).
-template <typename T, int DIST, int VPR>
+template <typename T, int DIST, int VPR, bool HINT>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, 5)
 shift_score_short_kernel(const T* __restrict__ after, const T* __restrict__ before, long long rows, int D, int lsh,
                          float* __restrict__ scores) {
@@ -208,7 +209,8 @@ shift_score_short_kernel(const T* __restrict__ after, const T* __restrict__ befo
             ra[u][j] = rb[u][j] = make_uint4(0u, 0u, 0u, 0u);
             if (row < rows && iv < nvec) {
                 ra[u][j] = ld_stream(reinterpret_cast<const uint4*>(after + row * D) + iv);
-                rb[u][j] = ld_stream(reinterpret_cast<const uint4*>(before + row * D) + iv, once);
+                const uint4* p = reinterpret_cast<const uint4*>(before + row * D) + iv;
+                rb[u][j] = HINT ? ld_stream(p, once) : ld_stream(p);
             }
         }
     }
@@ -307,17 +309,29 @@ cudaError_t launch_layernorm(rs_dtype in_dtype, rs_dtype out_dtype, const void* 
 }
 
 cudaError_t launch_shift_score(rs_dtype dtype, rs_dist dist, long long T, int D, const void* after,
-                               const void* before, float* scores, cudaStream_t st) {
+                               const void* before, float* scores, int sm_count, cudaStream_t st) {
     if (T == 0) return cudaSuccess;
     const int nvec = (int)((size_t)D * dtype_size(dtype) / 16);
     int lsh = 0;
     while (lsh < 5 && (1 << lsh) < nvec) ++lsh;
-    const long long per_cta = kWarpsPerCta * (nvec <= 32 ? 4 * (32 >> lsh) : nvec <= 64 ? 2 : 1);
+    // Tokens of up to 32 pieces go several to a warp once a warp per token would take more than one round of the 40 warps
+    // that an SM holds (two and a half for 17 to 32 pieces, of which a warp takes four one after the other, half of one for one
+    // or two pieces); fewer tokens are done sooner with a warp each.  Several to a warp / a warp each, us, L2 of bf16: 1000 x 256 2.3 / 1.8, 6000 x 128 2.5 / 2.7,
+    // 6000 x 256 3.1 / 2.7, 12000 x 256 4.1 / 3.9, 16000 x 256 4.3 / 4.7, 40000 x 256 6.6 / 9.4.
+    // Of 33 to 64 pieces two go to a warp from ten tokens per SM on (the cosine of 100 x 384 1.8 / 1.6, 2000 x 384 2.1 / 2.3).
+    const bool several = nvec <= 32 && 2 * T > 40ll * sm_count * (lsh <= 1 ? 1 : lsh < 5 ? 2 : 5), two = nvec > 32 && nvec <= 64 && T > 10ll * sm_count;
+    const long long per_cta = kWarpsPerCta * (several ? 4 * (32 >> lsh) : two ? 2 : 1);
+    const bool hint = dist == RS_DIST_COS || 2 * T * D * (long long)dtype_size(dtype) > (64ll << 20);      // half of the L2
     const dim3 grid((unsigned)((T + per_cta - 1) / per_cta)), block(kWarpsPerCta * 32);
-#define RS_SCORE_CASE(TT, DD)                                                                                                        \
-    return nvec <= 32   ? launch_pdl(shift_score_short_kernel<TT, DD, 1>, grid, block, 0, st, (const TT*)after, (const TT*)before, T, D, lsh, scores) \
-           : nvec <= 64 ? launch_pdl(shift_score_short_kernel<TT, DD, 2>, grid, block, 0, st, (const TT*)after, (const TT*)before, T, D, lsh, scores) \
-                        : launch_pdl(shift_score_kernel<TT, DD>, grid, block, 0, st, (const TT*)after, (const TT*)before, T, D, scores)
+#define RS_SCORE_HINT(TT, DD, HH)                                                                                                       \
+    return several ? launch_pdl(shift_score_short_kernel<TT, DD, 1, HH>, grid, block, 0, st, (const TT*)after, (const TT*)before, T, D, lsh, scores) \
+           : two   ? launch_pdl(shift_score_short_kernel<TT, DD, 2, HH>, grid, block, 0, st, (const TT*)after, (const TT*)before, T, D, lsh, scores) \
+                   : launch_pdl(shift_score_kernel<TT, DD, HH>, grid, block, 0, st, (const TT*)after, (const TT*)before, T, D, scores)
+#define RS_SCORE_CASE(TT, DD)                                \
+    do {                                                     \
+        if (hint) RS_SCORE_HINT(TT, DD, true);               \
+        RS_SCORE_HINT(TT, DD, (DD == 2));                    \
+    } while (0)
     if (dtype == RS_BF16) {
         if (dist == RS_DIST_L2) RS_SCORE_CASE(__nv_bfloat16, 0);
         else if (dist == RS_DIST_L1) RS_SCORE_CASE(__nv_bfloat16, 1);
@@ -328,6 +342,7 @@ cudaError_t launch_shift_score(rs_dtype dtype, rs_dist dist, long long T, int D,
         else RS_SCORE_CASE(float, 2);
     }
 #undef RS_SCORE_CASE
+#undef RS_SCORE_HINT
     return cudaGetLastError();
 }
 

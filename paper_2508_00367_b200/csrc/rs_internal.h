@@ -85,7 +85,7 @@ cudaError_t launch_layernorm(rs_dtype in_dtype, rs_dtype out_dtype, const void* 
                              const int32_t* row_map, bool first, cudaStream_t st, const int32_t* lens = nullptr, int seq_n = 0);
 // s[t] = D(after[t,:], before[t,:]).
 cudaError_t launch_shift_score(rs_dtype dtype, rs_dist dist, long long T, int D, const void* after,
-                               const void* before, float* scores, cudaStream_t st);
+                               const void* before, float* scores, int sm_count, cudaStream_t st);
 // Residual-add epilogue with the score fused in: x_hat = m + x_prime (out_dtype);
 // s = |m - x_prime| (MLP), |m| (MLP_DELTA), |x_prime - 2 x| = |SA(LN(x)) - x| (ATTN) or
 // |x_hat - x| (BLOCK).  m, x_prime fp32; x (the block input, x_dtype) only for ATTN and BLOCK.

@@ -65,6 +65,20 @@ def test_grid_rows_of_every_width_class(ctx, pieces, H, W, dr, dc):   # noqa: F8
         assert torch.equal(xo[b].cpu(), x[b][torch.from_numpy(want_r[b]).long()][:, torch.from_numpy(want_c[b]).long()])
 
 
+@pytest.mark.parametrize("dist", ["l2", "l1", "cos"])
+@pytest.mark.parametrize("D,edge", [(8, 2960), (24, 5920), (128, 5920), (136, 14800), (256, 14800), (264, 1480), (512, 1480)])
+def test_scores_where_several_tokens_share_a_warp(ctx, D, edge, dist):   # noqa: F811
+    """The token counts (on 148 SMs) from which tokens of up to 64 pieces go several to a warp, one and a warp's worth more."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for T in (edge * sms // 148, edge * sms // 148 + 1, edge * sms // 148 + 129):
+        g = torch.Generator(device="cuda").manual_seed(T)
+        a, b = (torch.randn(1, T, D, generator=g, device="cuda").bfloat16() for _ in range(2))
+        got, u, v = ctx.shift_score(a, b, dist=dist).double(), a.double(), b.double()
+        want = (u - v).norm(dim=-1) if dist == "l2" else (u - v).abs().sum(-1) if dist == "l1" else 1 - (u * v).sum(-1) / (u.norm(dim=-1) * v.norm(dim=-1))
+        # sums of at most 512 terms in fp32; the cosine is a difference of numbers near one
+        assert (got - want).abs().max() <= (2e-6 if dist == "cos" else 2e-6 * want.max())
+
+
 def _needs_memory(nbytes):
     torch.cuda.empty_cache()
     if torch.cuda.mem_get_info()[0] < nbytes:
