@@ -113,14 +113,14 @@ bool ln_fusable(rs_dtype dtype, int D);   // the row fits the registers of one w
 // x_out may be null when ln is given: only the normalised rows are written (no dense copy).  Rows with index -1
 // become zeros.
 cudaError_t launch_gather(rs_dtype dtype, const void* x, const int32_t* keep_idx, int B, int N, int K,
-                          int D, void* x_out, const LnFuse* ln /*null: none*/, cudaStream_t st);
+                          int D, void* x_out, const LnFuse* ln /*null: none*/, int sm_count, cudaStream_t st);
 // Line-wise pruning of a 2-D token grid: keep_rows [B, Hk], keep_cols [B, Wk] and, when x is given,
 // x_out[b, i, j, :] = x[b, keep_rows[b, i], keep_cols[b, j], :].  H, W <= linewise_max_lines().
 int linewise_max_lines();
 cudaError_t launch_line_select(const float* scores, int B, int H, int W, int Hk, int Wk, int32_t* keep_rows,
                                int32_t* keep_cols, cudaStream_t st);
 cudaError_t launch_line_gather(rs_dtype dtype, const void* x, const int32_t* keep_rows, const int32_t* keep_cols, int B, int H,
-                               int W, int Hk, int Wk, int D, void* x_out, cudaStream_t st);
+                               int W, int Hk, int Wk, int D, void* x_out, int sm_count, cudaStream_t st);
 
 // ---- SIMT contraction path (rs_simt.cu): fp32 FMA, used for RS_F32 and as a cross-check ----
 // out[M, N] = act(A[M, K] * W[N, K]^T + bias) + residual.

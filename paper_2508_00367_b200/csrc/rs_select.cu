@@ -493,11 +493,13 @@ line_select_kernel(const float* __restrict__ scores, int H, int W, int Hk, int W
     (kind ? keep_cols + (long long)b * Wk : keep_rows + (long long)b * Hk)[pos] = l;
 }
 
-// Launch of the copy: several narrow rows per warp, else a warp per row.
+// Launch of the copy: several narrow rows per warp, else a warp per row.  Few narrow rows are done sooner with a warp each,
+// too: several / one to a warp, us with the selection kernel before it, 200 x 192 bf16 3.1 / 2.5, 6000 x 192 3.7 / 3.3,
+// 8000 x 192 3.7 / 3.9, 40000 x 192 6.2 / 8.9; two / one to a warp 200 x 384 2.7 / 2.5, 4000 x 384 3.2 / 3.4.
 template <typename Src>
-cudaError_t launch_copy(const void* x, const Src& src, long long rows, int row_vecs, void* x_out, const LnFuse& ln, cudaStream_t st) {
-    if (row_vecs <= 64) {
-        const int vpr = row_vecs <= 32 ? 1 : 2;
+cudaError_t launch_copy(const void* x, const Src& src, long long rows, int row_vecs, void* x_out, const LnFuse& ln, int sm_count, cudaStream_t st) {
+    const int vpr = row_vecs <= 32 ? 1 : 2;
+    if (row_vecs <= 64 && rows > (vpr == 1 ? 48ll : 20ll) * sm_count) {
         int lsh = 0;
         while (lsh < 5 && (1 << lsh) < row_vecs) ++lsh;
         const unsigned per_cta = vpr == 1 ? 8 * 4 * (32u >> lsh) : 16;
@@ -548,7 +550,7 @@ cudaError_t launch_select(const float* scores, int nparts, float* scores_out, in
 bool ln_fusable(rs_dtype dtype, int D) { return (size_t)D * dtype_size(dtype) / 16 <= 32 * 4; }
 
 cudaError_t launch_gather(rs_dtype dtype, const void* x, const int32_t* keep_idx, int B, int N, int K,
-                          int D, void* x_out, const LnFuse* ln, cudaStream_t st) {
+                          int D, void* x_out, const LnFuse* ln, int sm_count, cudaStream_t st) {
     if (B == 0 || K == 0) return cudaSuccess;
     const int row_vecs = (int)((size_t)D * dtype_size(dtype) / 16);
     const bool norm = ln && ln->gamma;               // else ln, if given, only asks for the row sums of the copy
@@ -561,7 +563,7 @@ cudaError_t launch_gather(rs_dtype dtype, const void* x, const int32_t* keep_idx
         if (norm) lb.out = (char*)ln->out + (size_t)b0 * K * D * dtype_size(dtype);
         if (lb.stats) lb.stats += 2 * b0 * K;
         const TokenRows src = {keep_idx + b0 * K, (unsigned)K, N};
-        if (!norm) return launch_copy(xb, src, rows, row_vecs, ob, lb, st);
+        if (!norm) return launch_copy(xb, src, rows, row_vecs, ob, lb, sm_count, st);
         const dim3 grid((unsigned)((rows + 7) / 8));
         if (dtype == RS_BF16)
             return launch_pdl(gather_kernel<4, __nv_bfloat16, TokenRows>, grid, dim3(256), 0, st, xb, src, (unsigned)rows, row_vecs, ob, lb);
@@ -578,13 +580,13 @@ cudaError_t launch_line_select(const float* scores, int B, int H, int W, int Hk,
 }
 
 cudaError_t launch_line_gather(rs_dtype dtype, const void* x, const int32_t* keep_rows, const int32_t* keep_cols, int B, int H,
-                               int W, int Hk, int Wk, int D, void* x_out, cudaStream_t st) {
+                               int W, int Hk, int Wk, int D, void* x_out, int sm_count, cudaStream_t st) {
     if (B == 0) return cudaSuccess;
     const int row_vecs = (int)((size_t)D * dtype_size(dtype) / 16);
     const LnFuse none = {nullptr, nullptr, 0.f, nullptr, nullptr};
     return by_samples(B, Hk * Wk, [&](long long b0, long long rows) {
         const GridRows src = {keep_rows + b0 * Hk, keep_cols + b0 * Wk, (unsigned)Hk, (unsigned)Wk, H, W};
-        return launch_copy((const uint4*)x + b0 * H * W * row_vecs, src, rows, row_vecs, (uint4*)x_out + b0 * Hk * Wk * row_vecs, none, st);
+        return launch_copy((const uint4*)x + b0 * H * W * row_vecs, src, rows, row_vecs, (uint4*)x_out + b0 * Hk * Wk * row_vecs, none, sm_count, st);
     });
 }
 

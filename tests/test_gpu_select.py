@@ -21,7 +21,7 @@ def test_selection_at_the_keys_per_thread_edges(ctx, kind, N):   # noqa: F811
 
 
 @pytest.mark.parametrize("pieces", [1, 31, 32, 33, 63, 64, 65, 300])
-@pytest.mark.parametrize("B,N,r", [(1, 3, 1), (3, 50, 7)])       # row counts that leave a warp partly filled
+@pytest.mark.parametrize("B,N,r", [(1, 3, 1), (3, 50, 7), (62, 130, 7)])       # row counts that leave a warp partly filled; the last: several to a warp
 def test_rows_of_every_width_class(ctx, pieces, B, N, r):   # noqa: F811
     D = 8 * pieces
     s = _scores(B, N, "normal", pieces)
@@ -52,7 +52,7 @@ def test_score_of_every_width_class(ctx, pieces, dist):   # noqa: F811
 
 
 @pytest.mark.parametrize("pieces", [2, 3, 32, 33, 64, 65])
-@pytest.mark.parametrize("H,W,dr,dc", [(7, 5, 2, 1), (90, 91, 30, 40), (91, 91, 1, 90)])   # staged scores up to 8192
+@pytest.mark.parametrize("H,W,dr,dc", [(7, 5, 2, 1), (90, 91, 30, 40), (91, 91, 1, 90), (91, 90, 1, 3)])   # staged scores up to 8192; the last: several to a warp
 def test_grid_rows_of_every_width_class(ctx, pieces, H, W, dr, dc):   # noqa: F811
     D = 8 * pieces
     s = _scores(2, H * W, "normal", pieces).reshape(2, H, W)
