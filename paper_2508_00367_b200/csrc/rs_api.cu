@@ -298,7 +298,7 @@ rs_status rs_topk_compact(rs_ctx* ctx, rs_dtype dtype, int B, int N, int D, int 
         const size_t xbytes = (size_t)B * N * D * sz, obytes = (size_t)B * K * D * sz;
         if (xa < xo + obytes && xo < xa + xbytes) return fail(ctx, RS_ERR_INVALID_ARG, "rs_topk_compact: x_out overlaps x");
     }
-    RS_CHECK_LAUNCH(ctx, RS_K_SELECT, st, rs::launch_select(scores, 0, nullptr, B, N, K, has_cls ? 1 : 0, keep_idx, nullptr, st), "select launch");
+    RS_CHECK_LAUNCH(ctx, RS_K_SELECT, st, rs::launch_select(scores, 0, nullptr, B, N, K, has_cls ? 1 : 0, keep_idx, nullptr, ctx->sm_count, st), "select launch");
     if (x) RS_CHECK_LAUNCH(ctx, RS_K_GATHER, st, rs::launch_gather(dtype, x, keep_idx, B, N, K, D, x_out, nullptr, ctx->sm_count, st), "gather launch");
     return RS_OK;
 }
@@ -505,13 +505,13 @@ static rs_status block_fwd_impl(rs_ctx* ctx, const rs_block_desc* d, const rs_bl
     const int cls = d->has_cls ? 1 : 0;
     if (ragged) {
         // per-sample counts: sample b keeps lens[b] - drops[b] of its first lens[b] tokens; K is the row stride
-        RS_CHECK_LAUNCH(ctx, RS_K_SELECT, st, rs::launch_select(sel_in, sel_enc, sel_out, d->B, d->N, K, cls, keep, nullptr, st, hk->seq_lens, hk->drops, hk->lens_out), "select (per-sample counts)");
+        RS_CHECK_LAUNCH(ctx, RS_K_SELECT, st, rs::launch_select(sel_in, sel_enc, sel_out, d->B, d->N, K, cls, keep, nullptr, ctx->sm_count, st, hk->seq_lens, hk->drops, hk->lens_out), "select (per-sample counts)");
         RS_CHECK_LAUNCH(ctx, RS_K_GATHER, st, rs::launch_gather(d->out_dtype, x_hat, keep, d->B, d->N, K, D, x_out, nullptr, ctx->sm_count, st), "gather (per-sample counts)");
         return RS_OK;
     }
     // nothing dropped and neither the scores nor the (identity) index list asked for: nothing left to do
     if (!moves && hk && !scores && !keep_idx) return RS_OK;
-    RS_CHECK_LAUNCH(ctx, RS_K_SELECT, st, rs::launch_select(sel_in, sel_enc, sel_out, d->B, d->N, K, cls, keep, out_map, st), "select");
+    RS_CHECK_LAUNCH(ctx, RS_K_SELECT, st, rs::launch_select(sel_in, sel_enc, sel_out, d->B, d->N, K, cls, keep, out_map, ctx->sm_count, st), "select");
     if (moves && (dense || ln))
         RS_CHECK_LAUNCH(ctx, RS_K_GATHER, st, rs::launch_gather(d->out_dtype, x_hat, keep, d->B, d->N, K, D, dense, ln, ctx->sm_count, st), "gather");
     return RS_OK;
@@ -568,7 +568,7 @@ rs_status rs_topk_compact_ragged(rs_ctx* ctx, rs_dtype dtype, int B, int N, int 
         if (xa < xo + obytes && xo < xa + xbytes) return fail(ctx, RS_ERR_INVALID_ARG, "rs_topk_compact_ragged: x_out overlaps x");
     }
     cudaStream_t st = (cudaStream_t)stream;
-    RS_CHECK_LAUNCH(ctx, RS_K_SELECT, st, rs::launch_select(scores, 0, nullptr, B, N, K_pad, has_cls ? 1 : 0, keep_idx, nullptr, st, seq_lens, drops, lens_out), "select launch (per-sample counts)");
+    RS_CHECK_LAUNCH(ctx, RS_K_SELECT, st, rs::launch_select(scores, 0, nullptr, B, N, K_pad, has_cls ? 1 : 0, keep_idx, nullptr, ctx->sm_count, st, seq_lens, drops, lens_out), "select launch (per-sample counts)");
     if (x) RS_CHECK_LAUNCH(ctx, RS_K_GATHER, st, rs::launch_gather(dtype, x, keep_idx, B, N, K_pad, D, x_out, nullptr, ctx->sm_count, st), "gather launch (per-sample counts)");
     return RS_OK;
 }

@@ -102,7 +102,7 @@ cudaError_t launch_residual_score(const float* m, const float* x_prime, const vo
 // seq_lens, drops (optional, dev [B]): per-sample token counts (rs_topk_compact_ragged); index -1 past a sample's
 // count; lens_out (optional, dev [B]) receives the kept counts.
 cudaError_t launch_select(const float* scores, int nparts, float* scores_out, int B, int N, int K, int has_cls,
-                          int32_t* keep_idx, int32_t* row_map, cudaStream_t st, const int32_t* seq_lens = nullptr,
+                          int32_t* keep_idx, int32_t* row_map, int sm_count, cudaStream_t st, const int32_t* seq_lens = nullptr,
                           const int32_t* drops = nullptr, int32_t* lens_out = nullptr);
 // The compaction kernels can also write LN(x_out) for the block that follows (its LN1 of Eq. att):
 // the warp that copies a kept row has it in registers.  out: [B, K, D] of the rows' dtype.

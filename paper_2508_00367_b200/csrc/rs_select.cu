@@ -524,7 +524,7 @@ template <typename F> cudaError_t by_samples(int B, int per_sample, F launch) {
 }  // namespace
 
 cudaError_t launch_select(const float* scores, int nparts, float* scores_out, int B, int N, int K, int has_cls,
-                          int32_t* keep_idx, int32_t* row_map, cudaStream_t st, const int32_t* seq_lens,
+                          int32_t* keep_idx, int32_t* row_map, int sm_count, cudaStream_t st, const int32_t* seq_lens,
                           const int32_t* drops, int32_t* lens_out) {
     if (B == 0) return cudaSuccess;
     if (K == N && !seq_lens) {
@@ -533,14 +533,18 @@ cudaError_t launch_select(const float* scores, int nparts, float* scores_out, in
     }
     const Ragged rg = {seq_lens, drops, lens_out};
     // keys per thread: the fewest that leave at most 1024 threads (latency is what counts: more threads per
-    // sample mean fewer keys to compare per step), whole warps
+    // sample mean fewer keys to compare per step), whole warps.  With samples for two rounds and more it is samples at a time
+    // that count: more than 512 threads of the kernel's 64 registers leave room for one CTA on an SM, so that 2561 to 5120
+    // tokens take sixteen keys a thread there.  Five / sixteen, us: 256 x 4097 18.2 / 20.1, 512 x 2561 25.8 / 20.1, 512 x 4097
+    // 32.2 / 27.6, 2048 x 4097 111 / 81.
+    const bool many = B >= 2 * sm_count && N > 2560;
 #define RS_SEL_CASE(KPT)                                                                                            \
     if (N <= KPT * kSelMaxThreads)                                                                                  \
         return launch_pdl(select_kernel<KPT>, dim3(B), dim3(((N + KPT - 1) / KPT + 31) / 32 * 32), 0, st, scores,   \
                           nparts, scores_out, N, K, has_cls, keep_idx, row_map, rg)
     RS_SEL_CASE(1);
     RS_SEL_CASE(2);
-    RS_SEL_CASE(5);
+    if (!many) RS_SEL_CASE(5);
     RS_SEL_CASE(16);
     RS_SEL_CASE(32);
 #undef RS_SEL_CASE

@@ -20,6 +20,16 @@ def test_selection_at_the_keys_per_thread_edges(ctx, kind, N):   # noqa: F811
             np.testing.assert_array_equal(keep.cpu().numpy(), orc.topk(s.astype(np.float64), r, has_cls), err_msg=f"r={r} cls={has_cls}")
 
 
+@pytest.mark.parametrize("kind", ["normal", "ties"])
+@pytest.mark.parametrize("N", [2560, 2561, 5120])
+def test_selection_of_many_samples(ctx, kind, N):   # noqa: F811
+    """Two samples to an SM and more: sixteen keys per thread from 2561 tokens on."""
+    B = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    s = _scores(B, N, kind, N)
+    _, keep = ctx.topk_compact(torch.from_numpy(s).cuda(), None, N // 3, True)
+    np.testing.assert_array_equal(keep.cpu().numpy(), orc.topk(s.astype(np.float64), N // 3, True))
+
+
 @pytest.mark.parametrize("pieces", [1, 31, 32, 33, 63, 64, 65, 300])
 @pytest.mark.parametrize("B,N,r", [(1, 3, 1), (3, 50, 7), (62, 130, 7)])       # row counts that leave a warp partly filled; the last: several to a warp
 def test_rows_of_every_width_class(ctx, pieces, B, N, r):   # noqa: F811
