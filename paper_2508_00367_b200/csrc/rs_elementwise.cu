@@ -53,11 +53,9 @@ constexpr int kNarrowRows = 4 * kWarpsPerCta;            // rows per CTA
 template <int VPL>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
 layernorm_narrow_kernel(const float* __restrict__ x, const float* __restrict__ gamma, const float* __restrict__ beta, float eps,
-                        long long T, int D, __nv_bfloat16* __restrict__ out, const int32_t* __restrict__ row_map, const int first,
-                        const int32_t* __restrict__ lens, unsigned seq_n) {
-    if (!first) grid_dep_launch();
+                        long long T, int D, __nv_bfloat16* __restrict__ out, const int32_t* __restrict__ lens, unsigned seq_n) {
+    grid_dep_launch();
     grid_dep_wait();
-    if (first) grid_dep_launch();
     const int l16 = threadIdx.x & 15, nvec = D / 4;
     const long long row0 = (long long)blockIdx.x * kNarrowRows + (threadIdx.x >> 5) * 4 + ((threadIdx.x >> 4) & 1);
     float4 v[2][VPL];
@@ -70,7 +68,7 @@ layernorm_narrow_kernel(const float* __restrict__ x, const float* __restrict__ g
             const unsigned b = (unsigned)row / seq_n, i = (unsigned)row - b * seq_n;
             on[u] = (int)i < gemm::rows_needed(lens, b, seq_n);
         }
-        const float* xr = x + (on[u] ? row_map ? (long long)row_map[row] : row : 0) * D;
+        const float* xr = x + (on[u] ? row : 0) * D;
 #pragma unroll
         for (int j = 0; j < VPL; ++j) {
             v[u][j] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -281,9 +279,9 @@ cudaError_t ln_dispatch(const void* x, const float* g, const float* b, float eps
     if constexpr (std::is_same<TI, float>::value && std::is_same<TO, __nv_bfloat16>::value) {
         const dim3 narrow((unsigned)((T + kNarrowRows - 1) / kNarrowRows));
 #define RS_LN_CASE(VPL)                                                                                                    \
-    if (nvec <= 16 * VPL)                                                                                                  \
+    if (!row_map && !first && nvec <= 16 * VPL)                                                                            \
         return launch_pdl(layernorm_narrow_kernel<VPL>, narrow, block, 0, st, (const float*)x, g, b, eps, T, D,            \
-                          (__nv_bfloat16*)out, row_map, (int)first, lens, (unsigned)seq_n)
+                          (__nv_bfloat16*)out, lens, (unsigned)seq_n)
         RS_LN_CASE(2);
         RS_LN_CASE(3);
         RS_LN_CASE(4);

@@ -39,11 +39,6 @@ constexpr size_t kSmem = (size_t)OFF_ROWS + BM * 8 + 1024 /*alignment slack*/;
 static_assert(BM * RED_LD * 4 <= STAGES * STAGE_BYTES, "partial tile");
 static_assert(2 * (kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
 
-__device__ __forceinline__ float4 ld_cluster(uint32_t addr) {
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
-}
 __device__ __forceinline__ void unpack4(const uint2& t, float (&v)[4]) {
     v[0] = __uint_as_float(t.x << 16); v[1] = __uint_as_float(t.x & 0xffff0000u);
     v[2] = __uint_as_float(t.y << 16); v[3] = __uint_as_float(t.y & 0xffff0000u);

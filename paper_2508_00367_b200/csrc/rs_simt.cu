@@ -44,11 +44,6 @@ __device__ __forceinline__ float pair_sum(uint64_t v) {
     unpack2(v, a, b);
     return a + b;
 }
-__device__ __forceinline__ float4 ld_cluster(uint32_t addr) {
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
-}
 
 // ---------------------------------------------------------------- GEMM
 // out[M, N] = act(A[M, K] . W[N, K]^T + bias) + residual.  A warp owns a 32 x 8 NJ patch of the output (8 x NJ
@@ -178,7 +173,7 @@ gemm_simt_kernel(const SimtArgs args) {
 #pragma unroll
             for (int w = 0; w < WK; ++w) {
                 const float* p = red + (w * C::TM + r) * C::RED_LD + c;
-                const float4 t = args.splits > 1 ? ld_cluster(tc::map_to_cta(tc::smem_u32(p), s)) : *reinterpret_cast<const float4*>(p);
+                const float4 t = args.splits > 1 ? tc::ld_cluster(tc::map_to_cta(tc::smem_u32(p), s)) : *reinterpret_cast<const float4*>(p);
                 v.x += t.x; v.y += t.y; v.z += t.z; v.w += t.w;
             }
         if (args.bias) {

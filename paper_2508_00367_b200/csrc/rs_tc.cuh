@@ -293,6 +293,12 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t saddr, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
     return r;
 }
+// Four floats at a shared::cluster address.
+__device__ __forceinline__ float4 ld_cluster(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
+}
 // Arrive on an mbarrier given by a shared::cluster address (possibly in the peer CTA), for what is ordered by other means:
 // no memory access of this thread is made visible by it.  The epilogues hand an accumulator back with it, whose reads
 // tcgen05.wait::ld has completed and tcgen05.fence::before_thread_sync has ordered.  The default, .release.cluster, also
