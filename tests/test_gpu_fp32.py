@@ -23,9 +23,16 @@ def test_linear_fp32_edges(ctx, M, N, K, epilogue):   # noqa: F811
         want = orc.gelu(want)
     if epilogue == "residual":
         want = want + res.double().numpy()[rows]
-    # K products of size ~0.05, summed in fp32 in at most K steps: |error| <= K * 2^-24 * sum |a w| (a loose bound)
-    bound = 2.0 ** -23 + K * 2.0 ** -24 * (np.abs(a.double().numpy()[rows]) @ np.abs(w.double().numpy()).T + 5.0)
+    # K fp32 roundings of partial sums of at most sum |a w|, of random sign: sqrt(K) of them, four deviations; and the
+    # epilogue's few roundings of the result
+    size = np.abs(a.double().numpy()[rows]) @ np.abs(w.double().numpy()).T
+    bound = 2.0 ** -23 + 4 * np.sqrt(K) * 2.0 ** -24 * size + 2.0 ** -22 * np.abs(want)
     assert (np.abs(got[rows] - want) <= bound).all()
+    # the bound tells fp32 products from TF32 ones (operands of 11 bits)
+    if epilogue == "bias":
+        tf32 = lambda t: ((t.numpy().view(np.int32) + 0x1000) & ~0x1fff).view(np.float32).astype(np.float64)   # noqa: E731
+        rough = orc.linear(tf32(a)[rows], tf32(w), b.double().numpy())
+        assert not (np.abs(rough - want) <= bound).all()
 
 
 def test_linear_fp32_of_many_columns(ctx):   # noqa: F811
