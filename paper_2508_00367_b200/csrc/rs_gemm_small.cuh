@@ -312,14 +312,16 @@ cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const Gem
 // forwards of 12 blocks (20 % dropped three times), all products on pair tiles / line at 60 / 100 / 150 / 220
 // tiles, us: 1 x 197 x 768 633 / 496 / 492 / 496 / 493; 4 x 197 x 768 651 / 554 / 552 / 561 / 561; 8 x 197 x 768
 // 659 / 659 / 648 / 668 / 676; 1 x 577 x 1024 738 / 671 / 653 / 650 / 645; 3 x 577 x 1024 857 / 857 / 857 / 938 / 972;
-// 2 x 69 x 1024 709 / 511 / 489 / 486 / 486; 8 x 197 x 192 510 / 446 / 433 / 426 / 424.
+// 2 x 69 x 1024 709 / 511 / 489 / 486 / 486; 8 x 197 x 192 510 / 446 / 433 / 426 / 424.  The residual epilogue stays at 100 for
+// every K: its fp32 rows cost more here than the short prologue gains (few rows / pair tiles, us: 5000 x 256 x 256 7.1 / 5.6,
+// 9000 x 192 x 192 7.0 / 6.4, 1576 x 1024 x 64 6.3 / 5.1; six blocks of 47 x 197 x 192 303 / 301, of 25 x 197 x 256 268 / 264).
 // Splits: as many as leave three slabs of K to a CTA and 4 / 3 CTAs to an SM (the second MLP product of one image of
 // 197 tokens: 20 us unsplit, 12.6 by two, 8.7 by four, 7.3 by eight; 17.4 on pair tiles).
-SmallPlan gemm_small_plan(long long M, int N, int K, int sms) {
+SmallPlan gemm_small_plan(int epi, long long M, int N, int K, int sms) {
     const long long tiles = ((M + BM - 1) / BM) * (N / BN);
     int s = 1;
     while (s < 8 && tiles * (s + 1) <= sms + sms / 3 && K / BK >= 3 * (s + 1)) ++s;
-    return {tiles <= (K <= 256 ? 220 : 100), s};
+    return {tiles <= (K <= 256 && epi != EPI_RESID ? 220 : 100), s};
 }
 
 // tmA: boxes of 128 rows; tmB: boxes of kSmallBN rows; both 64 columns, 128-byte swizzle.

@@ -802,7 +802,7 @@ cudaError_t launch_gemm_tc(rs_ctx* ctx, int epi, const void* A, const void* W, c
     if (!ctx->encode_tiled) return cudaErrorNotSupported;
     if (ln && epi == EPI_SCORE && ln->stats_out && out_dtype == RS_BF16) epi = EPI_SCORE_STATS;
     if (ln && epi == EPI_BIAS && ln->stats_in) epi = EPI_BIAS_LN;
-    const few::SmallPlan small = few::gemm_small_plan(M, N, K, ctx->sm_count);
+    const few::SmallPlan small = few::gemm_small_plan(epi, M, N, K, ctx->sm_count);
     const int bn = small.use ? few::kSmallBN : pick_bn(M, N, ctx->sm_count);
     const int out_bytes = (epi == EPI_RESID || (epi == EPI_SCORE && out_dtype == RS_F32)) ? 4 : 2;
     if (epi == EPI_SCORE_STATS && ln->stats_parts_out) *ln->stats_parts_out = gemm_tc_score_parts(N);

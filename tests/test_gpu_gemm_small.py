@@ -29,6 +29,23 @@ def test_linear_few_rows(ctx, M, N, K, epilogue):   # noqa: F811
         parity.check_float(got, orc.round_to(want, "bf16"), "bf16", rounded_output=True)
 
 
+@pytest.mark.parametrize("epilogue", ["bias", "gelu", "residual"])
+@pytest.mark.parametrize("M,N,K", [(3200, 256, 256), (3201, 256, 256), (6400, 128, 64), (6401, 128, 64), (7040, 256, 128), (7041, 256, 128)])
+def test_linear_at_the_lines_of_the_few_row_kernel(ctx, M, N, K, epilogue):   # noqa: F811
+    """100 and 220 tiles of 128 x 64: the residual epilogue goes to the pair tiles after the first, the others after the second."""
+    g = torch.Generator(device="cuda").manual_seed(M + K)
+    a, w = torch.randn(M, K, generator=g, device="cuda").bfloat16(), (0.05 * torch.randn(N, K, generator=g, device="cuda")).bfloat16()
+    b, res = 0.1 * torch.randn(N, generator=g, device="cuda"), torch.randn(M, N, generator=g, device="cuda").bfloat16() if epilogue == "residual" else None
+    got = ctx.linear_fwd(a, w, b, epilogue, res).cpu().double().numpy()
+    want = (a.double() @ w.double().T + b.double()).cpu().numpy()
+    if epilogue == "gelu":
+        want = orc.gelu(want)
+    if epilogue == "residual":
+        parity.check_float(got, want + res.cpu().double().numpy(), "bf16", rounded_output=False)
+    else:
+        parity.check_float(got, orc.round_to(want, "bf16"), "bf16", rounded_output=True)
+
+
 @pytest.mark.parametrize("mode,dist", [("mlp", "l2"), ("mlp", "cos"), ("mlp_delta", "l1"), ("attn", "l1"), ("attn", "cos"), ("block", "l2")])
 def test_block_few_rows_every_score(ctx, mode, dist):   # noqa: F811
     B, N, D, H, r = 1, 130, 384, 6, 40
