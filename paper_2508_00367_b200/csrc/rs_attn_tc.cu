@@ -496,12 +496,14 @@ bool attn_tc_supported(const rs_attn_desc& d) {
 // (a query tile alone runs faster than next to another, but not twice as fast: measured).
 // This kernel or the one with three query tiles per CTA (rs_attn_tc3.cu)?  Both are paced by the longest
 // CTA: its items (in tenths) times the key tiles of an item, plus a cost per item; microseconds fitted to
-// CUDA-event times of thirteen shapes from N = 197 to 4097 (worst error 6 % and 9 %).  (Since the three-tile kernel
-// sends a part of its exponentials through the FMA pipes it runs 3 % under its line; the lines stay.)
+// CUDA-event times of thirteen shapes from N = 197 to 4097 (worst error 6 % and 9 %).  The lines are those of earlier kernels:
+// since the three-tile kernel sends a part of its exponentials through the FMA pipes and takes items across heads it runs under
+// its lines.  At the workloads' shapes the choice is the faster kernel (32 x 16 x 577 82.9 us, two tiles 101; 16 x 12 x 1569 182 /
+// 208; 64 x 12 x 181 26.3 / 29.5) but for 4 x 16 x 2305 (two tiles 151, three would take 134), x 1729 (92.1 / 90.2),
+// 64 x 12 x 197 (31.8 / 30.5), 16 x 12 x 539 (38.8 / 36.7) and 32 x 16 x 457 (59.8 / 59.2).
 // With its items across heads the three-tile kernel has a line of its own: the same one at the lower load, the steps a
-// little longer by the share of items with two K/V streams (two in as many items as a head has tiles): 41.3 expected at
-// 128 x 12 x 133, 41.5 us measured, 50.2 / 50.0 at x 197, 80.7 / 77.5 at 28 x 16 x 577.  It is chosen where that is
-// 8 % better, about the errors of the fits: 28 x 16 x 577 91.2 -> 77.5 us, 128 x 12 x 197 55.5 -> 50.0.
+// little longer by the share of items with two K/V streams (two in as many items as a head has tiles).  It is chosen where
+// that is 8 % better, about the errors of the fits.
 AttnPlan attn_plan(long long BH, int N, int G) {
     const int nt = (N + BQ - 1) / BQ, per = (N + 2 * BQ - 1) / (2 * BQ);
     auto makespan = [&](long long hs) {

@@ -182,8 +182,8 @@ shift_score_kernel(const T* __restrict__ after, const T* __restrict__ before, lo
     if (lane == 0) scores[row] = d;
 }
 
-// Tokens of at most 32 * VPR pieces (VPR 1 or 2), many of them (launch_shift_score): 4 / VPR groups of 32 >> lsh tokens side by side per warp, 1 << lsh
-// lanes per token, so that a lane has eight loads in flight here too (a warp per token of 256 bf16 had two:
+// Tokens of at most 32 * VPR pieces (VPR 1 or 2), many of them (launch_shift_score): 4 / VPR groups of 32 >> lsh tokens
+// side by side per warp, 1 << lsh lanes per token, so that a lane has eight loads in flight here too (a warp per token of 256 bf16 had two:
 // 64 x 56 x 56 positions took 56 us = 3.7 TB/s; this takes 36 = 5.7 TB/s).
 template <typename T, int DIST, int VPR, bool HINT>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, 5)
@@ -314,8 +314,9 @@ cudaError_t launch_shift_score(rs_dtype dtype, rs_dist dist, long long T, int D,
     while (lsh < 5 && (1 << lsh) < nvec) ++lsh;
     // Tokens of up to 32 pieces go several to a warp once a warp per token would take more than one round of the 40 warps
     // that an SM holds (two and a half for 17 to 32 pieces, of which a warp takes four one after the other, half of one for one
-    // or two pieces); fewer tokens are done sooner with a warp each.  Several to a warp / a warp each, us, L2 of bf16: 1000 x 256 2.3 / 1.8, 6000 x 128 2.5 / 2.7,
-    // 6000 x 256 3.1 / 2.7, 12000 x 256 4.1 / 3.9, 16000 x 256 4.3 / 4.7, 40000 x 256 6.6 / 9.4.
+    // or two pieces); fewer tokens are done sooner with a warp each.  Several to a warp / a warp each, us, L2 of bf16:
+    // 1000 x 256 2.3 / 1.8, 6000 x 128 2.5 / 2.7, 6000 x 256 3.1 / 2.7, 12000 x 256 4.1 / 3.9, 16000 x 256 4.3 / 4.7,
+    // 40000 x 256 6.6 / 9.4.
     // Of 33 to 64 pieces two go to a warp from ten tokens per SM on (the cosine of 100 x 384 1.8 / 1.6, 2000 x 384 2.1 / 2.3).
     const bool several = nvec <= 32 && 2 * T > 40ll * sm_count * (lsh <= 1 ? 1 : lsh < 5 ? 2 : 5), two = nvec > 32 && nvec <= 64 && T > 10ll * sm_count;
     const long long per_cta = kWarpsPerCta * (several ? 4 * (32 >> lsh) : two ? 2 : 1);
