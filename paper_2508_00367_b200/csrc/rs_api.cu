@@ -445,6 +445,8 @@ static rs_status block_fwd_impl(rs_ctx* ctx, const rs_block_desc* d, const rs_bl
         RS_CHECK_LAUNCH(ctx, RS_K_LAYERNORM, st, rs::launch_layernorm(d->dtype, d->dtype, x, w->ln1_g, w->ln1_b, eps, T, D, u, in_map, true, st, in_use.lens, in_use.seq_n), "LN1");
         x_ln = u;
     }
+    const bool attn_score = d->score_mode == RS_SCORE_ATTN;
+    const bool one_tail = tc && rs::tail_tc_use(T, D, Dm);      // projection and MLP in one kernel
     if (tc) {
         if (fold_ln1) {
             // LN1 applied in the epilogue: the product reads the block input itself
@@ -457,30 +459,36 @@ static rs_status block_fwd_impl(rs_ctx* ctx, const rs_block_desc* d, const rs_bl
         // error of their attention score against 64 bits to 1.19x (4 x 50 tokens, D = 192; 1.08x at 32 x 197), two bf16 parts keep it.
         const bool split_weights = (D % 128) != 0 || (Dm % 128) != 0;
         RS_CHECK_LAUNCH(ctx, RS_K_ATTN, st, rs::launch_attn_tc(ctx, ad, qkv, kp, vp, o, hk ? hk->seq_lens : nullptr, st, split_weights), "attention");
+        nparts = one_tail ? rs::tail_tc_parts() : rs::gemm_tc_score_parts(D);
         // shift through attention (operation choice (i)): partial sums of (SA(LN(x)) - x)^2 from this epilogue
-        const bool attn_score = d->score_mode == RS_SCORE_ATTN;
-        nparts = rs::gemm_tc_score_parts(D);
-        float* attn_parts = attn_score ? m : nullptr;
-        RS_CHECK_LAUNCH(ctx, RS_K_GEMM, st, rs::launch_gemm_tc(ctx, rs::RS_EPI_RESID, o, w->w_o, w->b_o, x, nullptr, in_map, x_prime, RS_F32, attn_parts, 0, (int)d->dist, T, D, D, st, nullptr, true, &in_use), "proj");
+        if (!one_tail)
+            RS_CHECK_LAUNCH(ctx, RS_K_GEMM, st, rs::launch_gemm_tc(ctx, rs::RS_EPI_RESID, o, w->w_o, w->b_o, x, nullptr, in_map, x_prime, RS_F32, attn_score ? m : nullptr, 0, (int)d->dist, T, D, D, st, nullptr, true, &in_use), "proj");
     } else {
         RS_CHECK_LAUNCH(ctx, RS_K_GEMM, st, rs::launch_gemm_simt(d->dtype, x_ln, w->w_qkv, w->b_qkv, 0, nullptr, RS_F32, qkv, d->dtype, T, 3 * D, D, ctx->sm_count, st), "QKV");
         RS_CHECK_LAUNCH(ctx, RS_K_ATTN, st, rs::launch_attn_simt(ad, qkv, kp, vp, o, ctx->sm_count, st), "attention");
         RS_CHECK_LAUNCH(ctx, RS_K_GEMM, st, rs::launch_gemm_simt(d->dtype, o, w->w_o, w->b_o, 0, x, d->dtype, x_prime, RS_F32, T, D, D, ctx->sm_count, st), "proj");
     }
     // x^ = MLP(LN(x')) + x',  s = |MLP(LN(x')) - x'|                      (Eq. MLP, Sec. 3.2)
-    RS_CHECK_LAUNCH(ctx, RS_K_LAYERNORM, st, rs::launch_layernorm(RS_F32, d->dtype, x_prime, w->ln2_g, w->ln2_b, eps, T, D, u, nullptr, false, st, in_use.lens, in_use.seq_n), "LN2");
+    if (!one_tail)
+        RS_CHECK_LAUNCH(ctx, RS_K_LAYERNORM, st, rs::launch_layernorm(RS_F32, d->dtype, x_prime, w->ln2_g, w->ln2_b, eps, T, D, u, nullptr, false, st, in_use.lens, in_use.seq_n), "LN2");
     if (tc) {
         // The FC2 epilogue adds the residual and leaves per-tile partial sums of squares of the
         // shift in `m`; the selection kernel adds them up in a fixed order.
         // (when the score came from the projection, this epilogue's partial sums go to a second array)
-        float* fc2_parts = d->score_mode == RS_SCORE_ATTN ? m + (size_t)T * nparts * 3 : m;
+        float* fc2_parts = attn_score ? m + (size_t)T * nparts * 3 : m;
         const int kind = d->score_mode == RS_SCORE_MLP_DELTA ? 1 : d->score_mode == RS_SCORE_BLOCK ? 2 : 0;
-        RS_CHECK_LAUNCH(ctx, RS_K_GEMM, st, rs::launch_gemm_tc(ctx, rs::RS_EPI_BIAS_GELU, u, w->w_fc1, w->b_fc1, nullptr, nullptr, nullptr, h, RS_BF16, nullptr, 0, 0, T, Dm, D, st, nullptr, true, &in_use), "FC1");
         // row sums for a LayerNorm folded into the next block's QKV: from this epilogue when the block's output is
         // the next block's input as it stands, else from the kernel that moves the kept rows (below)
         const bool fc2_stats = hk && hk->stats_out && x_hat == x_out;
         const rs::GemmLn lnout = {fc2_stats ? hk->stats_out : nullptr, fc2_stats ? hk->parts_out : nullptr, nullptr, 0, nullptr, 0.f};
-        RS_CHECK_LAUNCH(ctx, RS_K_GEMM, st, rs::launch_gemm_tc(ctx, rs::RS_EPI_SCORE, h, w->w_fc2, w->b_fc2, x_prime, x, in_map, x_hat, d->out_dtype, fc2_parts, kind, (int)d->dist, T, D, Dm, st, fc2_stats ? &lnout : nullptr, true, &in_use), "FC2+residual+score");
+        if (one_tail) {
+            const rs::TailCall tail = {T, Dm, o, x, in_map, w->w_o, w->w_fc1, w->w_fc2, w->b_o, w->b_fc1, w->b_fc2, w->ln2_g, w->ln2_b, eps, x_hat, d->out_dtype,
+                                       attn_score ? m : nullptr, attn_score ? nullptr : m, kind, (int)d->dist, lnout.stats_out, lnout.stats_parts_out, true, &in_use};
+            RS_CHECK_LAUNCH(ctx, RS_K_GEMM, st, rs::launch_tail_tc(ctx, tail, st), "proj+LN2+FC1+FC2+residual+score");
+        } else {
+            RS_CHECK_LAUNCH(ctx, RS_K_GEMM, st, rs::launch_gemm_tc(ctx, rs::RS_EPI_BIAS_GELU, u, w->w_fc1, w->b_fc1, nullptr, nullptr, nullptr, h, RS_BF16, nullptr, 0, 0, T, Dm, D, st, nullptr, true, &in_use), "FC1");
+            RS_CHECK_LAUNCH(ctx, RS_K_GEMM, st, rs::launch_gemm_tc(ctx, rs::RS_EPI_SCORE, h, w->w_fc2, w->b_fc2, x_prime, x, in_map, x_hat, d->out_dtype, fc2_parts, kind, (int)d->dist, T, D, Dm, st, fc2_stats ? &lnout : nullptr, true, &in_use), "FC2+residual+score");
+        }
     } else {
         RS_CHECK_LAUNCH(ctx, RS_K_GEMM, st, rs::launch_gemm_simt(d->dtype, u, w->w_fc1, w->b_fc1, 1, nullptr, RS_F32, h, d->dtype, T, Dm, D, ctx->sm_count, st), "FC1");
         RS_CHECK_LAUNCH(ctx, RS_K_GEMM, st, rs::launch_gemm_simt(d->dtype, h, w->w_fc2, w->b_fc2, 0, nullptr, RS_F32, m, RS_F32, T, D, Dm, ctx->sm_count, st), "FC2");

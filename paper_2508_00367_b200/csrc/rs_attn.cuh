@@ -43,6 +43,12 @@ __device__ __forceinline__ uint64_t fadd2(uint64_t a, uint64_t b) {
     return r;
 }
 
+__device__ __forceinline__ uint64_t fmul2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
 // The larger of the two; NaN if either is (fmaxf drops a NaN).
 __device__ __forceinline__ float max_nan(float a, float b) {
     float r;

@@ -47,6 +47,37 @@ __device__ __forceinline__ int rows_needed(const int* __restrict__ lens, int b, 
     return min(min(max(__ldg(lens + b), 1), seq_n) + kPadRows, seq_n);
 }
 
+// Batches with a count per sample: row tiles that hold padding alone are left out.  Up to this many row tiles of 256.
+constexpr int kMaskWords = 32, kMaskTiles = 32 * kMaskWords;
+// The k-th row tile in use, for a caller whose k never decreases.
+struct RowTiles {
+    const uint32_t* mask;    // null: all
+    int word = 0, before = 0;
+    __device__ __forceinline__ int at(int k) {
+        if (!mask) return k;
+        while (word < kMaskWords - 1 && before + __popc(mask[word]) <= k) before += __popc(mask[word++]);
+        uint32_t m = mask[word];
+        for (int i = before; i < k; ++i) m &= m - 1;
+        return word * 32 + __ffs(m) - 1;
+    }
+};
+
+// Which row tiles of 256 rows hold rows in use (at most kMaskTiles), written to shared memory by the whole CTA of `threads`;
+// returns how many do.
+__device__ __forceinline__ int mark_row_tiles(uint32_t* mask, const int* __restrict__ lens, int seq_n, int M, int warp, int lane, int threads) {
+    for (int t0 = warp * 32; t0 < kMaskTiles; t0 += threads) {
+        const int r0 = (t0 + lane) * 256, r1 = min(r0 + 256, M);
+        bool used = false;
+        for (int b = r0 / seq_n; r0 < M && b * seq_n < r1 && !used; ++b) used = b * seq_n + rows_needed(lens, b, seq_n) > r0;
+        const uint32_t w = __ballot_sync(0xffffffffu, used);
+        if (lane == 0) mask[t0 / 32] = w;
+    }
+    __syncthreads();
+    int tiles = 0;
+    for (int w = 0; w < kMaskWords; ++w) tiles += __popc(mask[w]);
+    return tiles;
+}
+
 // Adds one element of the scored pair (u, v) to the running sums of the chosen distance (Sec. 3.3).  Called with a
 // constant distance in the pair-tile kernel (with_dist): the choice is made once per 32 columns there.
 __device__ __forceinline__ void score_acc(int dist, float u, float v, float& s0, float& s1, float& s2) {

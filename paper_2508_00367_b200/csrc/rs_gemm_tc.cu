@@ -77,6 +77,7 @@ __device__ __forceinline__ void gelu_erf2(float& v0, float& v1) {
 }  // namespace rs
 
 #include "rs_gemm_small.cuh"
+#include "rs_tail.cuh"
 
 namespace rs {
 
@@ -91,21 +92,6 @@ constexpr int BK = 64;
 constexpr int A_BYTES = BM * BK * 2;          // 16 KB
 constexpr int STG_BYTES = 32 * 128;           // one staged output block of a warp: its 32 rows of 128 bytes
 constexpr int RES_BOX_BYTES = 32 * 64;         // residual of one 32-column chunk of a warp: 32 rows of 32 bf16
-
-// Batches with a count per sample: row tiles that hold padding alone are left out.  Up to this many row tiles of 256.
-constexpr int kMaskWords = 32, kMaskTiles = 32 * kMaskWords;
-// The k-th row tile in use, for a caller whose k never decreases.
-struct RowTiles {
-    const uint32_t* mask;    // null: all
-    int word = 0, before = 0;
-    __device__ __forceinline__ int at(int k) {
-        if (!mask) return k;
-        while (word < kMaskWords - 1 && before + __popc(mask[word]) <= k) before += __popc(mask[word++]);
-        uint32_t m = mask[word];
-        for (int i = before; i < k; ++i) m &= m - 1;
-        return word * 32 + __ffs(m) - 1;
-    }
-};
 
 // The list of work of a launch.  Whole tiles go to the pairs round robin; 256-wide tiles left for a last round that
 // half of the pairs or fewer would work on are cut in two, so that the round takes a part of a tile's time.  A
@@ -222,20 +208,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 
     int tiles = num_m * num_n;
     uint32_t* mask = args.lens ? reinterpret_cast<uint32_t*>(smem + C::OFF_MASK) : nullptr;
-    if (mask) {                                  // which row tiles hold rows in use (num_m <= kMaskTiles)
-        for (int t0 = warp * 32; t0 < kMaskTiles; t0 += C::THREADS) {
-            const int r0 = (t0 + lane) * 2 * BM, r1 = min(r0 + 2 * BM, args.M);
-            bool used = false;
-            for (int b = r0 / args.seq_n; r0 < args.M && b * args.seq_n < r1 && !used; ++b)
-                used = b * args.seq_n + rows_needed(args.lens, b, args.seq_n) > r0;
-            const uint32_t w = __ballot_sync(0xffffffffu, used);
-            if (lane == 0) mask[t0 / 32] = w;
-        }
-        __syncthreads();
-        tiles = 0;
-        for (int w = 0; w < kMaskWords; ++w) tiles += __popc(mask[w]);
-        tiles *= num_n;
-    }
+    if (mask) tiles = num_n * mark_row_tiles(mask, args.lens, args.seq_n, args.M, warp, lane, C::THREADS);
     RowTiles row_tiles = {mask};                 // (each role walks its own copy)
     const WorkList<BN> list(tiles, num_n, npairs);
     const int works = list.count();
@@ -852,6 +825,42 @@ cudaError_t launch_gemm_tc(rs_ctx* ctx, int epi, const void* A, const void* W, c
     }
 #undef RS_GEMM_CASE
     return cudaErrorInvalidValue;
+}
+
+// Which blocks take their projection and MLP as one kernel: those of 192 columns with more than two tiles' rows.  Fewer rows
+// are done sooner by the four kernels for few rows, which spread a tile's columns over the SMs.  Whole pruned forwards of 12
+// blocks (20 % dropped three times), four kernels / one, us: 1 x 197 388 / 399, 2 x 197 393 / 404, 4 x 197 418 / 410, 8 x 197
+// 443 / 413, 16 x 197 479 / 436, 32 x 197 542 / 467, 1 x 2353 735 / 708, 256 x 197 1294 / 1059.  A tile takes some 28000 cycles of
+// which the tensor pipe needs 12700: a chunk's chain (product, GELU, product and the three hand-overs, 1500 cycles for 960 of
+// products; two chunks are under way, tensor memory holds no third) and the row phases before and after it, 10000, bound it.
+bool tail_tc_use(long long T, int D, int Dm) {
+    return T > 512 && D == tail::D && Dm >= 2 * tail::C && Dm % tail::C == 0 && Dm <= tail::kMaxHidden && T < (1ll << 31);
+}
+int tail_tc_parts() { return tail::kParts; }
+
+cudaError_t launch_tail_tc(rs_ctx* ctx, const TailCall& c, cudaStream_t st) {
+    if (!ctx->encode_tiled) return cudaErrorNotSupported;
+    CUtensorMap tmO, tmX, tmWo, tmW1, tmW2, tmOut;
+    constexpr int D = tail::D;
+    if (!make_tmap_2d(ctx, &tmO, c.o, 2, (uint64_t)c.T, D, 128) || !make_tmap_2d(ctx, &tmWo, c.wo, 2, D, D, D / 2) ||
+        !make_tmap_2d(ctx, &tmW1, c.w1, 2, (uint64_t)c.Dm, D, tail::C / 2) || !make_tmap_2d(ctx, &tmW2, c.w2, 2, D, (uint64_t)c.Dm, D / 2) ||
+        !make_tmap_2d(ctx, &tmOut, c.out, c.out_dtype == RS_F32 ? 4 : 2, (uint64_t)c.T, D, 32) ||
+        (!c.row_map && !make_tmap_2d(ctx, &tmX, c.x, 2, (uint64_t)c.T, D, 128)))
+        return cudaErrorInvalidValue;
+    if (c.row_map) tmX = tmO;                        // unused: x is read through the map
+    tail::TailArgs a;
+    a.T = (int)c.T; a.Dm = c.Dm; a.bo = c.bo; a.ln_g = c.ln_g; a.ln_b = c.ln_b; a.b1 = c.b1; a.b2 = c.b2; a.ln_eps = c.ln_eps;
+    a.x = reinterpret_cast<const __nv_bfloat16*>(c.x); a.row_map = c.row_map;
+    a.attn_partials = c.attn_partials; a.partials = c.partials; a.score_kind = c.score_kind; a.dist = c.dist;
+    a.stats_out = c.out_dtype == RS_BF16 ? c.stats_out : nullptr;
+    if (a.stats_out && c.stats_parts_out) *c.stats_parts_out = tail::kParts;
+    a.weights_ready = c.weights_ready ? 1 : 0;
+    const bool skips = c.rows && c.rows->lens && (c.T + 255) / 256 <= kMaskTiles;
+    a.lens = skips ? c.rows->lens : nullptr;
+    a.seq_n = skips ? c.rows->seq_n : 0;
+    a.status = ctx->d_status;
+    return c.out_dtype == RS_F32 ? tail::launch<float>(tmO, tmX, tmWo, tmW1, tmW2, tmOut, a, ctx->sm_count, st)
+                                 : tail::launch<__nv_bfloat16>(tmO, tmX, tmWo, tmW1, tmW2, tmOut, a, ctx->sm_count, st);
 }
 
 }  // namespace rs

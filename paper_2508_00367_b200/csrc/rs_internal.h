@@ -166,6 +166,31 @@ cudaError_t launch_gemm_tc(rs_ctx* ctx, int epi, const void* A, const void* W, c
                            rs_dtype out_dtype, float* partials, int score_kind, int dist, long long M, int N, int K,
                            cudaStream_t st, const GemmLn* ln = nullptr, bool weights_ready = false, const GemmRows* rows = nullptr);
 
+// Projection and MLP of a block of 192 columns in one kernel (rs_tail.cuh): x' = o Wo^T + bo + x,
+// out = m + x', m = GELU(LN(x') W1^T + b1) W2^T + b2, with tail_tc_parts() partial sums of the scored pair per row (and, for bf16
+// outputs, as many pairs of the output's row sums).
+struct TailCall {
+    long long T;
+    int Dm;
+    const void *o, *x;                      // bf16 [T, D]: attention's output, block input (through row_map if that is given)
+    const int32_t* row_map;
+    const void *wo, *w1, *w2;               // [D, D], [Dm, D], [D, Dm]
+    const float *bo, *b1, *b2;              // or null
+    const float *ln_g, *ln_b;
+    float ln_eps;
+    void* out;
+    rs_dtype out_dtype;
+    float *attn_partials, *partials;        // of the pair (SA(LN(x)), x), of the pair that score_kind names; or null
+    int score_kind, dist;
+    float* stats_out;                       // or null
+    int* stats_parts_out;
+    bool weights_ready;                     // as for launch_gemm_tc
+    const GemmRows* rows;
+};
+bool tail_tc_use(long long T, int D, int Dm);
+int tail_tc_parts();
+cudaError_t launch_tail_tc(rs_ctx* ctx, const TailCall& c, cudaStream_t st);
+
 // ---- tcgen05 attention (rs_attn_tc.cu): bf16, head dimension 64 ----
 bool attn_tc_supported(const rs_attn_desc& d);
 // Which attention kernel runs a shape of BH (sample, head)s and N > 128 tokens on G SMs, and how: best_hs heads handed

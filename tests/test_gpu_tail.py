@@ -1,0 +1,113 @@
+"""Blocks of 192 columns with more than 512 rows: projection and MLP as one kernel (rs_tail.cuh).  Row counts at the edges of its
+tiles of 256 rows and of its rounds, every scored pair and distance, both output types, hidden widths with an odd count of chunks,
+the residual through a row map, batches with a count per sample."""
+import numpy as np
+import pytest
+import torch
+
+import parity
+from oracle import rs_oracle as orc
+from paper_2508_00367_b200 import synth
+from test_gpu_block import _check_block, _np, _run_block, ctx   # noqa: F401  (the module's context fixture)
+
+pytestmark = pytest.mark.gpu
+D, H = 192, 3
+
+
+def _launches(ctx, B, N, Dm=4 * D):
+    """Kernels of one block call."""
+    import paper_2508_00367_b200 as rs
+    dw = rs.DeviceBlockWeights(synth.make_block_weights(D, Dm, "bf16", seed=1), torch.bfloat16, ctx.device)
+    n = ctx.launch_count()
+    ctx.block_fwd(torch.zeros(B, N, D, device="cuda", dtype=torch.bfloat16), dw, H, 1)
+    return ctx.launch_count() - n
+
+
+def test_which_blocks(ctx):   # noqa: F811
+    assert _launches(ctx, 2, 256) == 9 and _launches(ctx, 1, 513) == 6 and _launches(ctx, 3, 197) == 6
+    assert _launches(ctx, 3, 197, 576) == 6 and _launches(ctx, 3, 197, 1536) == 9
+
+
+@pytest.mark.parametrize("out_dtype", [None, torch.float32])
+@pytest.mark.parametrize("B,N,Dm", [(1, 513, 768), (2, 320, 576), (3, 256, 128), (1, 769, 768), (5, 127, 768)])
+def test_row_counts(ctx, B, N, Dm, out_dtype):   # noqa: F811
+    x, w = synth.make_tokens(B, N, D, "bf16", seed=N), synth.make_block_weights(D, Dm, "bf16", seed=Dm)
+    res = _run_block(ctx, x, w, H, N // 5, "bf16", out_dtype)
+    _check_block(res, orc.block_fwd(x.double().numpy(), _np(w), H, N // 5), "bf16", out_dtype)
+
+
+@pytest.mark.parametrize("out_dtype", [None, torch.float32])
+def test_several_tiles_a_pair(ctx, out_dtype):   # noqa: F811
+    """2 x 74 tiles and one row more: a second and a third round; the first and the last samples against the oracle."""
+    B, N = (2 * 74 * 256 + 1) // 257 + 1, 257
+    x, w = synth.make_tokens(B, N, D, "bf16", seed=7), synth.make_block_weights(D, 4 * D, "bf16", seed=8)
+    res = _run_block(ctx, x, w, H, 50, "bf16", out_dtype)
+    again = _run_block(ctx, x, w, H, 50, "bf16", out_dtype)
+    for k in res:
+        assert torch.equal(res[k], again[k]), k
+    for b in (0, B // 2, B - 1):
+        ref = orc.block_fwd(x[b:b + 1].double().numpy(), _np(w), H, 50)
+        _check_block({k: v[b:b + 1] for k, v in res.items()}, ref, "bf16", out_dtype)
+
+
+@pytest.mark.parametrize("mode,dist", [("mlp", "l1"), ("mlp", "cos"), ("mlp_delta", "l2"), ("attn", "l2"), ("attn", "cos"), ("block", "l2"), ("block", "l1")])
+def test_scores(ctx, mode, dist):   # noqa: F811
+    """Bounds as where these scores come from the epilogues of the single products (bf16 operands in full)."""
+    B, N = 3, 190
+    x, w = synth.make_tokens(B, N, D, "bf16", seed=51), synth.make_block_weights(D, 4 * D, "bf16", seed=52)
+    ref = orc.block_fwd(x.double().numpy(), _np(w), H, 9, score_mode=mode, dist=dist)
+    res = _run_block(ctx, x, w, H, 9, "bf16", torch.float32, score_mode=mode, dist=dist)
+    parity.check_float(res["x_full"].double().numpy(), ref["x_hat"], "bf16", False)
+    err = np.abs(res["scores"].double().numpy() - ref["scores"])
+    assert (err if dist == "cos" else err / ref["scores"]).max() < (3e-3 if mode == "mlp_delta" else 2e-3)
+
+
+@pytest.mark.parametrize("mode", ["mlp", "block"])
+def test_rows_through_the_map(ctx, mode):   # noqa: F811
+    """The layer loop without dense copies reads the block input through the row map: the bits of chained block calls."""
+    import paper_2508_00367_b200 as rs
+    B, N, drops = 4, 197, [39, 0, 20, 0]
+    x = synth.make_tokens(B, N, D, "bf16", seed=3).bfloat16().cuda()
+    blocks = [synth.make_block_weights(D, 4 * D, "bf16", seed=4 + l) for l in range(4)]
+    got = rs.PrunedViT(ctx, blocks, H, drops, torch.bfloat16, tap_blocks=(), score_mode=mode).forward(x)[-1]["x_out"]
+    cur = x
+    for w, d in zip(blocks, drops):
+        cur = ctx.block_fwd(cur, rs.DeviceBlockWeights(w, torch.bfloat16, ctx.device), H, d, score_mode=mode)["x_out"]
+    assert torch.equal(got, cur)
+    ctx.async_status()
+
+
+def test_row_sums_for_a_folded_layernorm(ctx):   # noqa: F811
+    """Every block of the folded loop against the oracle fed this loop's own input."""
+    import paper_2508_00367_b200 as rs
+    B, N, drops = 4, 197, [0, 30, 0, 5]
+    x = synth.make_tokens(B, N, D, "bf16", seed=13).bfloat16().cuda()
+    blocks = [synth.make_block_weights(D, 4 * D, "bf16", seed=14 + l) for l in range(4)]
+    outs, cur = rs.PrunedViT(ctx, blocks, H, drops, torch.bfloat16, fold_ln1=True).forward(x), x
+    torch.cuda.synchronize()
+    for l, o in enumerate(outs):
+        ref = orc.block_fwd(cur.double().cpu().numpy(), _np(blocks[l]), H, drops[l])
+        s = o["scores"].double().cpu().numpy()
+        assert (np.abs(s - ref["scores"]) / ref["scores"]).max() < 5e-4
+        if parity.check_keep(ref["scores"], ref["keep_idx"], o["keep_idx"].cpu().numpy()) == 0:
+            parity.check_float(o["x_out"].double().cpu().numpy(), orc.round_to(ref["x_out"], "bf16"), "bf16", True)
+        cur = o["x_out"]
+    ctx.async_status()
+
+
+def test_counts_per_sample(ctx):   # noqa: F811
+    import paper_2508_00367_b200 as rs
+    N, lens = 300, [300, 17, 1, 2, 128, 250, 40]
+    drops = [n // 4 for n in lens]
+    x = synth.make_tokens(len(lens), N, D, "bf16", seed=11)
+    w = synth.make_block_weights(D, 4 * D, "bf16", seed=12)
+    dw = rs.DeviceBlockWeights(w, torch.bfloat16, ctx.device)
+    dl, dd = (torch.tensor(v, dtype=torch.int32, device="cuda") for v in (lens, drops))
+    res = {k: v.cpu() for k, v in ctx.block_fwd_ragged(x.bfloat16().cuda(), dw, H, dl, dd, N).items()}
+    for b, n in enumerate(lens):
+        ref = orc.block_fwd(x[b:b + 1, :n].double().numpy(), _np(w), H, drops[b])
+        s = res["scores"][b, :n].double().numpy()
+        assert (np.abs(s - ref["scores"][0]) / ref["scores"][0]).max() < 5e-4
+        if parity.check_keep(ref["scores"], ref["keep_idx"], res["keep_idx"][b:b + 1, :n - drops[b]].numpy()) == 0:
+            parity.check_float(res["x_out"][b, :n - drops[b]].double().numpy(), orc.round_to(ref["x_out"][0], "bf16"), "bf16", True)
+    ctx.async_status()
