@@ -829,28 +829,29 @@ cudaError_t launch_gemm_tc(rs_ctx* ctx, int epi, const void* A, const void* W, c
 
 // Which blocks take their projection and MLP as one kernel: those of 192 columns with more than two tiles' rows.  Fewer rows
 // are done sooner by the four kernels for few rows, which spread a tile's columns over the SMs.  Whole pruned forwards of 12
-// blocks (20 % dropped three times), four kernels / one, us: 1 x 197 388 / 399, 2 x 197 393 / 404, 4 x 197 418 / 410, 8 x 197
-// 443 / 413, 16 x 197 479 / 436, 32 x 197 542 / 467, 1 x 2353 735 / 708, 256 x 197 1294 / 1059.  A tile takes some 28000 cycles of
-// which the tensor pipe needs 12700: a chunk's chain (product, GELU, product and the three hand-overs, 1500 cycles for 960 of
-// products; two chunks are under way, tensor memory holds no third) and the row phases before and after it, 10000, bound it.
+// blocks (20 % dropped three times), four kernels / one, us: 1 x 197 388 / 399, 2 x 197 393 / 404, 4 x 197 418 / 416, 8 x 197
+// 443 / 399, 16 x 197 479 / 424, 32 x 197 542 / 457, 1 x 1569 622 / 585, 256 x 197 1292 / 1044.  A tile takes some 27000 cycles, of
+// which the tensor pipe needs 10400: six chunks of 2150 (GELU: sixteen warps keep the special-function unit, the FMA and the ALU
+// pipes half busy each, and its hand-overs are waits), x' and LN(x') 5000, x of the next tile and the output 8000.  With x'
+// in tensor memory and chunks of 64 columns, two of them under way, a chunk's chain took 1500 cycles for half the columns
+// and 256 x 197 1059 us.
 bool tail_tc_use(long long T, int D, int Dm) {
-    return T > 512 && D == tail::D && Dm >= 2 * tail::C && Dm % tail::C == 0 && Dm <= tail::kMaxHidden && T < (1ll << 31);
+    return T > 512 && D == tail::D && Dm >= tail::C && Dm % tail::C == 0 && Dm <= tail::kMaxHidden && T < (1ll << 31);
 }
 int tail_tc_parts() { return tail::kParts; }
 
 cudaError_t launch_tail_tc(rs_ctx* ctx, const TailCall& c, cudaStream_t st) {
     if (!ctx->encode_tiled) return cudaErrorNotSupported;
-    CUtensorMap tmO, tmX, tmWo, tmW1, tmW2, tmOut;
+    CUtensorMap tmO, tmX, tmWo, tmW1, tmW2;
     constexpr int D = tail::D;
     if (!make_tmap_2d(ctx, &tmO, c.o, 2, (uint64_t)c.T, D, 128) || !make_tmap_2d(ctx, &tmWo, c.wo, 2, D, D, D / 2) ||
         !make_tmap_2d(ctx, &tmW1, c.w1, 2, (uint64_t)c.Dm, D, tail::C / 2) || !make_tmap_2d(ctx, &tmW2, c.w2, 2, D, (uint64_t)c.Dm, D / 2) ||
-        !make_tmap_2d(ctx, &tmOut, c.out, c.out_dtype == RS_F32 ? 4 : 2, (uint64_t)c.T, D, 32) ||
         (!c.row_map && !make_tmap_2d(ctx, &tmX, c.x, 2, (uint64_t)c.T, D, 128)))
         return cudaErrorInvalidValue;
     if (c.row_map) tmX = tmO;                        // unused: x is read through the map
     tail::TailArgs a;
     a.T = (int)c.T; a.Dm = c.Dm; a.bo = c.bo; a.ln_g = c.ln_g; a.ln_b = c.ln_b; a.b1 = c.b1; a.b2 = c.b2; a.ln_eps = c.ln_eps;
-    a.x = reinterpret_cast<const __nv_bfloat16*>(c.x); a.row_map = c.row_map;
+    a.x = reinterpret_cast<const __nv_bfloat16*>(c.x); a.row_map = c.row_map; a.out = c.out;
     a.attn_partials = c.attn_partials; a.partials = c.partials; a.score_kind = c.score_kind; a.dist = c.dist;
     a.stats_out = c.out_dtype == RS_BF16 ? c.stats_out : nullptr;
     if (a.stats_out && c.stats_parts_out) *c.stats_parts_out = tail::kParts;
@@ -859,8 +860,8 @@ cudaError_t launch_tail_tc(rs_ctx* ctx, const TailCall& c, cudaStream_t st) {
     a.lens = skips ? c.rows->lens : nullptr;
     a.seq_n = skips ? c.rows->seq_n : 0;
     a.status = ctx->d_status;
-    return c.out_dtype == RS_F32 ? tail::launch<float>(tmO, tmX, tmWo, tmW1, tmW2, tmOut, a, ctx->sm_count, st)
-                                 : tail::launch<__nv_bfloat16>(tmO, tmX, tmWo, tmW1, tmW2, tmOut, a, ctx->sm_count, st);
+    return c.out_dtype == RS_F32 ? tail::launch<float>(tmO, tmX, tmWo, tmW1, tmW2, a, ctx->sm_count, st)
+                                 : tail::launch<__nv_bfloat16>(tmO, tmX, tmWo, tmW1, tmW2, a, ctx->sm_count, st);
 }
 
 }  // namespace rs

@@ -2,17 +2,15 @@
 //     x' = o Wo^T + bo + x,   m = GELU(LN(x') W1^T + b1) W2^T + b2,   out = m + x',   the scored pair's partial sums, row sums
 // As four kernels such a block moves x' (fp32) three times, LN(x') twice and the hidden layer, four times as wide as the
 // tokens, twice through memory, and with K of three slabs the products are bound by their epilogues.  A tile of 192 columns
-// holds whole rows, and tensor memory holds x', the output's accumulator and two chunks of the hidden layer of 128 rows, so
-// here a pair of CTAs takes 256 rows from o to out:
-//   * P = o Wo^T; sixteen warps (four to a row quadrant, 48 columns each) add bias and residual, put x' back where P was and
-//     write LN(x') as a K-major operand in shared memory;
-//   * the hidden layer goes by in chunks of 64 columns: S = LN(x') W1c^T; the sixteen warps read it (sixteen columns each),
-//     apply bias and GELU and write it back, rounded to bf16, over the columns they have read, as the tensor-memory A operand
-//     of O += h W2c^T;
-//   * they take O and x' out through the LN(x') buffer.
-// The weights stream through a TMA ring, each CTA of the pair loading its half of every slab (no multicast); o and x of the
-// next tile are fetched while this one is computed.  LN(x') and the hidden layer are rounded to bf16, and x' is fp32, as where
-// they go through memory.
+// holds whole rows, and a pair of CTAs has room for all that 256 rows need from o to out:
+//   * P = o Wo^T in tensor memory; sixteen warps (four to a row quadrant, 48 columns each) add bias and residual, keep x' in
+//     shared memory and write LN(x') where o was, as a K-major operand;
+//   * the hidden layer goes by in chunks of 128 columns: S = LN(x') W1c^T (two buffers in turn); the sixteen warps read it (32
+//     columns each), apply bias and GELU and write it, rounded to bf16, as the tensor-memory A operand of O += h W2c^T, where
+//     P was;
+//   * they take O and x' out.
+// The weights stream through a TMA ring, each CTA of the pair loading its half of every piece (no multicast).  LN(x') and the
+// hidden layer are rounded to bf16, and x' is fp32, as where they go through memory.
 // What bounds it: see tail_tc_use.
 #pragma once
 #include "rs_internal.h"
@@ -24,7 +22,7 @@
 namespace rs {
 namespace tail {
 
-constexpr int D = 192, C = 64;                           // columns of a token; hidden columns per chunk
+constexpr int D = 192, C = 128;                          // columns of a token; hidden columns per chunk
 constexpr int kMaxHidden = 768;                          // b1 is held in shared memory
 constexpr int kParts = 4, kPartCols = D / kParts;        // partial sums per row, one per 48 columns
 
@@ -37,6 +35,7 @@ struct TailArgs {
     float* attn_partials;                                // sums of the pair (SA(LN(x)), x), or null
     float* partials;                                     // sums of the pair score_kind names, or null
     float* stats_out;                                    // [T, kParts][2] or null
+    void* out;                                           // [T, D]
     int score_kind, dist;
     int weights_ready;
     const int* lens;
@@ -54,17 +53,19 @@ constexpr int BM = 128, BK = 64;                         // rows per CTA, column
 constexpr int kRow0 = 4, kRowWarps = 16, kThreads = 32 * (kRow0 + kRowWarps);
 constexpr int TILE_BYTES = BM * D * 2;                   // 48 KB: three slabs of 128 rows x 128 bytes, 128-byte swizzle
 constexpr int SLAB_BYTES = BM * 128;
-constexpr int STAGE_BYTES = C * D;                       // 12 KB: this CTA's half of a [64, 192] or [192, 64] piece of a weight
-constexpr int STAGES = 6;
-constexpr int OFF_O = 0, OFF_U = TILE_BYTES, OFF_X = 2 * TILE_BYTES, OFF_STAGE = 3 * TILE_BYTES;
+constexpr int STAGE_BYTES = C * D;                       // 24 KB: this CTA's half of a [128, 192] or [192, 128] piece of a weight
+constexpr int STAGES = 3;
+// o and then LN(x') | x (three slabs) and then x' (six slabs of 32 columns of fp32) and then out in its place | weights
+constexpr int OFF_O = 0, OFF_U = 0, OFF_X = TILE_BYTES, OFF_STAGE = OFF_X + 2 * TILE_BYTES;
 constexpr int OFF_BAR = OFF_STAGE + STAGES * STAGE_BYTES;
 constexpr int OFF_VEC = OFF_BAR + 256;                   // float bo, ln_g, ln_b, b2 [D] each, b1 [kMaxHidden]
 constexpr int OFF_RED = OFF_VEC + (4 * D + kMaxHidden) * 4;      // float [2][kParts][BM]: sums of a row's quarters
 constexpr int OFF_MASK = OFF_RED + 2 * kParts * BM * 4;
 constexpr size_t SMEM = (size_t)OFF_MASK + kMaskWords * 4;       // the window itself must be 1024-byte aligned
 static_assert(SMEM <= 227 * 1024, "shared memory of one CTA");
-constexpr int P_COL = 0, O_COL = D, S_COL = 2 * D;       // tensor memory: P and then x' | O | two chunks
-static_assert(S_COL + 2 * C <= 512, "tensor memory");
+static_assert(D == 3 * BK && C == 2 * BK, "boxes of the weights");
+constexpr int P_COL = 0, O_COL = 0, S_COL = D, H_COL = D + 2 * C;    // tensor memory: P and then O | two chunks | a chunk after GELU
+static_assert(H_COL + C / 2 <= 512, "tensor memory");
 
 // Sixteen columns as packed pairs.
 using attn::pack2; using attn::unpack2; using attn::ffma2; using attn::fadd2; using attn::fmul2;
@@ -118,8 +119,7 @@ __device__ __forceinline__ void score16(int dist, const uint64_t (&u)[8], const 
 template <typename OutT>
 __global__ void __launch_bounds__(kThreads, 1)
 tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmWo,
-            const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmOut,
-            const TailArgs args) {
+            const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2, OutT* __restrict__ out, const TailArgs args) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = smem_raw;
     if (smem_u32(smem) & 1023u) {
@@ -133,12 +133,14 @@ tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUt
     uint64_t* p_full = a_full + 1;               // per CTA: P complete (and o read)
     uint64_t* u_full = p_full + 1;               // leader's: LN(x') written (one arrival per row warp of either CTA)
     uint64_t* s_full = u_full + 1;               // [2] per CTA: S of a chunk complete
-    uint64_t* h_ready = s_full + 2;              // [2] leader's: the hidden chunk written (one arrival per row warp of either CTA)
-    uint64_t* h_free = h_ready + 2;              // [2] leader's: the product reading it retired, S may be overwritten
-    uint64_t* o_full = h_free + 2;               // per CTA: O of the tile complete (and LN(x') read)
-    uint64_t* o_empty = o_full + 1;              // leader's: O and x' read by all row warps of both CTAs
+    uint64_t* s_free = s_full + 2;               // [2] leader's: S read (one arrival per row warp of either CTA)
+    uint64_t* h_ready = s_free + 2;              // leader's: the chunk after GELU written (likewise)
+    uint64_t* h_free = h_ready + 1;              // per CTA: the product reading it retired
+    uint64_t* u_free = h_free + 1;               // per CTA: the first layer's products of the tile retired
+    uint64_t* o_full = u_free + 1;               // per CTA: O of the tile complete
+    uint64_t* o_empty = o_full + 1;              // leader's: O read by all row warps of both CTAs
     uint64_t* x_full = o_empty + 1;              // per CTA: x of the tile landed
-    uint64_t* x_empty = x_full + 1;              // per CTA: x read
+    uint64_t* x_empty = x_full + 1;              // per CTA: the output that replaced x' has been taken out
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(x_empty + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     float* vec = reinterpret_cast<float*>(smem + OFF_VEC);
@@ -150,16 +152,18 @@ tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUt
     const int num_m = (args.T + 2 * BM - 1) / (2 * BM), NC = args.Dm / C;
 
     if (threadIdx.x == 0) {
-        prefetch_tmap(&tmO); prefetch_tmap(&tmX); prefetch_tmap(&tmWo); prefetch_tmap(&tmW1); prefetch_tmap(&tmW2); prefetch_tmap(&tmOut);
+        prefetch_tmap(&tmO); prefetch_tmap(&tmX); prefetch_tmap(&tmWo); prefetch_tmap(&tmW1); prefetch_tmap(&tmW2);
         for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         mbar_init(a_full, 1);
         mbar_init(p_full, 1);
         mbar_init(u_full, 2 * kRowWarps);
         for (int b = 0; b < 2; ++b) {
             mbar_init(&s_full[b], 1);
-            mbar_init(&h_ready[b], 2 * kRowWarps);
-            mbar_init(&h_free[b], 1);
+            mbar_init(&s_free[b], 2 * kRowWarps);
         }
+        mbar_init(h_ready, 2 * kRowWarps);
+        mbar_init(h_free, 1);
+        mbar_init(u_free, 1);
         mbar_init(o_full, 1);
         mbar_init(o_empty, 2 * kRowWarps);
         mbar_init(x_full, args.row_map ? 32 : 1);        // by the lane that starts the TMA copies, or by each lane's own copies
@@ -207,8 +211,8 @@ tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUt
         if (elect_one()) {
             uint32_t it = 0;
             bool ok = true, waited = !early;
-            auto load_o = [&](int t) {           // the P product of the tile before has read the buffer
-                if (t > 0) ok = ok && mbar_wait(p_full, (t - 1) & 1u, abort_flag);
+            auto load_o = [&](int t) {           // the first layer has read LN(x') of the tile before
+                if (t > 0) ok = ok && mbar_wait(u_free, (t - 1) & 1u, abort_flag);
                 if (!ok) return;
                 const uint32_t lead = map_to_cta(smem_u32(a_full), 0);
                 const int m = row0(t);
@@ -216,8 +220,8 @@ tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUt
 #pragma unroll
                 for (int kb = 0; kb < D / BK; ++kb) tma_load_2d_pair(smem + OFF_O + kb * SLAB_BYTES, &tmO, lead, kb * BK, m);
             };
-            // kind 0: slab i of Wo, 1: chunk i of W1, 2: chunk i of W2
-            auto slab = [&](int kind, int i) {
+            // kind 0: slabs 2 i and 2 i + 1 of Wo, 1: chunk i of W1, 2: chunk i of W2
+            auto piece = [&](int kind, int i) {
                 if (!waited && it == STAGES) {   // the ring is full: now o of the first tile
                     grid_dep_wait();
                     waited = true;
@@ -228,25 +232,24 @@ tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUt
                 if (!ok) return;
                 uint8_t* dst = smem + OFF_STAGE + s * STAGE_BYTES;
                 const uint32_t lead_full = map_to_cta(smem_u32(&full[s]), 0);
-                if (rank == 0) mbar_expect_tx(&full[s], 2 * STAGE_BYTES);
-                if (kind == 1) {
-#pragma unroll
-                    for (int kb = 0; kb < D / BK; ++kb) tma_load_2d_pair(dst + kb * (C / 2) * 128, &tmW1, lead_full, kb * BK, i * C + (int)rank * (C / 2));
-                } else {
-                    tma_load_2d_pair(dst, kind == 0 ? &tmWo : &tmW2, lead_full, i * BK, (int)rank * (D / 2));
+                const int boxes = kind == 1 ? D / BK : kind == 0 && i == 1 ? 1 : 2, box_bytes = kind == 1 ? (C / 2) * 128 : (D / 2) * 128;
+                if (rank == 0) mbar_expect_tx(&full[s], 2 * boxes * box_bytes);
+                for (int k = 0; k < boxes; ++k) {
+                    if (kind == 1) tma_load_2d_pair(dst + k * box_bytes, &tmW1, lead_full, k * BK, i * C + (int)rank * (C / 2));
+                    else tma_load_2d_pair(dst + k * box_bytes, kind == 0 ? &tmWo : &tmW2, lead_full, (2 * i + k) * BK, (int)rank * (D / 2));
                 }
                 ++it;
             };
             if (waited && mine > 0) load_o(0);
             for (int t = 0; t < mine && ok; ++t) {
-                for (int kb = 0; kb < D / BK; ++kb) slab(0, kb);
-                slab(1, 0);
+                piece(0, 0);
+                piece(0, 1);
+                piece(1, 0);
                 for (int c = 0; c < NC && ok; ++c) {
-                    if (c + 1 < NC) slab(1, c + 1);
-                    slab(2, c);
-                    // (the ring holds six slabs: P of this tile, the first three of thirteen and more, is under way)
-                    if (c == (NC > 2 ? 2 : NC - 1) && t + 1 < mine) load_o(t + 1);
+                    if (c + 1 < NC) piece(1, c + 1);
+                    piece(2, c);
                 }
+                if (t + 1 < mine) load_o(t + 1);
             }
             if (!waited) grid_dep_wait();
             // every stage filled here has been read (and its copies have landed) before the CTA may exit
@@ -270,10 +273,10 @@ tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUt
                 db = smem_desc_sw128(smem_u32(smem + OFF_STAGE + s * STAGE_BYTES), 16, 1024);
                 return &empty[s];
             };
-            const uint64_t da_o = smem_desc_sw128(smem_u32(smem + OFF_O), 16, 1024), da_u = smem_desc_sw128(smem_u32(smem + OFF_U), 16, 1024);
-            auto first = [&](int g) {            // S = LN(x') W1c^T
+            const uint64_t da_u = smem_desc_sw128(smem_u32(smem + OFF_U), 16, 1024);         // (o and LN(x') in turn)
+            auto first = [&](int g, bool last) { // S = LN(x') W1c^T
                 const int b = g & 1;
-                if (g >= 2) ok = ok && mbar_wait(&h_free[b], ((g >> 1) - 1) & 1u, abort_flag);
+                if (g >= 2) ok = ok && mbar_wait(&s_free[b], ((g >> 1) - 1) & 1u, abort_flag);
                 uint64_t db;
                 uint64_t* done = next_stage(db);
                 if (!ok) return;
@@ -282,47 +285,50 @@ tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUt
                     mma_ss_pair(tmem_base + S_COL + b * C, da_u + (k / 4) * (SLAB_BYTES >> 4) + 2 * (k % 4), db + (k / 4) * ((C / 2) * 128 >> 4) + 2 * (k % 4), idesc_c, k != 0);
                 mma_commit_pair(done, 3);
                 mma_commit_pair(&s_full[b], 3);
+                if (last) mma_commit_pair(u_free, 3);
             };
             for (int t = 0, g = 0; t < mine && ok; ++t) {
                 // P = o Wo^T, over what the warps have read of the tile before
                 ok = mbar_wait(a_full, t & 1u, abort_flag) && (t == 0 || mbar_wait(o_empty, (t - 1) & 1u, abort_flag));
-                for (int kb = 0; kb < D / BK && ok; ++kb) {
+                for (int i = 0; i < 2 && ok; ++i) {
                     uint64_t db;
                     uint64_t* done = next_stage(db);
                     if (!ok) break;
+                    for (int kb = 2 * i; kb < D / BK && kb < 2 * i + 2; ++kb)
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        mma_ss_pair(tmem_base + P_COL, da_o + kb * (SLAB_BYTES >> 4) + 2 * k, db + 2 * k, idesc_d, (kb | k) != 0);
+                        for (int k = 0; k < 4; ++k)
+                            mma_ss_pair(tmem_base + P_COL, da_u + kb * (SLAB_BYTES >> 4) + 2 * k, db + (kb - 2 * i) * ((D / 2) * 128 >> 4) + 2 * k, idesc_d, (kb | k) != 0);
                     mma_commit_pair(done, 3);
                 }
                 if (!ok) break;
                 mma_commit_pair(p_full, 3);
                 ok = mbar_wait(u_full, t & 1u, abort_flag);
-                if (ok) first(g);
+                if (ok) first(g, NC == 1);
                 for (int c = 0; c < NC && ok; ++c, ++g) {
-                    if (c + 1 < NC) first(g + 1);
-                    const int b = g & 1;
-                    ok = ok && mbar_wait(&h_ready[b], (g >> 1) & 1u, abort_flag);
+                    if (c + 1 < NC) first(g + 1, c + 2 == NC);
+                    ok = ok && mbar_wait(h_ready, g & 1u, abort_flag);
                     uint64_t db;
                     uint64_t* done = next_stage(db);
                     if (!ok) break;
 #pragma unroll
-                    for (int k = 0; k < C / 16; ++k)     // O (+)= h W2c^T (sixteen columns of the chunk lie where they were read from)
-                        mma_ts_pair(tmem_base + O_COL, tmem_base + S_COL + b * C + 16 * k, db + 2 * k, idesc_d, (c | k) != 0);
+                    for (int k = 0; k < C / 16; ++k)     // O (+)= h W2c^T
+                        mma_ts_pair(tmem_base + O_COL, tmem_base + H_COL + 8 * k, db + (k / 4) * ((D / 2) * 128 >> 4) + 2 * (k % 4), idesc_d, (c | k) != 0);
                     mma_commit_pair(done, 3);
-                    mma_commit_pair(&h_free[b], 1);
+                    mma_commit_pair(h_free, 3);
                     if (c == NC - 1) mma_commit_pair(o_full, 3);
                 }
             }
             // arrivals on this CTA's barriers that nothing above waited for
             const int chunks = mine * NC;
-            for (int g = chunks > 2 ? chunks - 2 : 0; g < chunks && ok; ++g) ok = mbar_wait(&h_free[g & 1], (g >> 1) & 1u, abort_flag);
+            for (int g = chunks > 2 ? chunks - 2 : 0; g < chunks && ok; ++g) ok = mbar_wait(&s_free[g & 1], (g >> 1) & 1u, abort_flag);
             if (mine > 0 && ok) mbar_wait(o_empty, (mine - 1) & 1u, abort_flag);
         }
     } else if (warp == 2) {
         // ---------------- x of the tiles, a tile ahead ----------------
         for (int t = 0; t < mine; ++t) {
             const int m = row0(t);
+            if (t > 0 && !args.row_map && lane == 0)     // (x lands when x' of the tile before has been used, and should come from the L2 then)
+                for (int kb = 0; kb < D / BK; ++kb) tma_prefetch_2d(&tmX, kb * BK, m);
             if (t > 0 && !__all_sync(0xffffffffu, mbar_wait(x_empty, (t - 1) & 1u, abort_flag))) break;
             if (!args.row_map) {
                 if (lane == 0) {
@@ -350,15 +356,17 @@ tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUt
         // ---------------- rows: bias, residual, LayerNorm; GELU; output ----------------
         // A wait that ran out is not acted on here: the values are void, the status says so, and all sixteen warps still come to
         // the same barriers.
-        const int q = warp & 3, grp = (warp - kRow0) >> 2;           // rows of the tile; columns 48 grp .. + 47, or 16 grp .. + 15 of a chunk
+        const int q = warp & 3, grp = (warp - kRow0) >> 2;           // rows of the tile; columns 48 grp .. + 47, or 32 grp .. + 31 of a chunk
         const int r = q * 32 + lane, c0 = grp * kPartCols, swz = r & 7;
         const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
-        const uint32_t s_addr = lane_addr + S_COL + grp * 16;
+        const uint32_t s_addr = lane_addr + S_COL + grp * 32, h_addr = lane_addr + H_COL + grp * 16;
         const uint32_t lead_u = map_to_cta(smem_u32(u_full), 0), lead_oe = map_to_cta(smem_u32(o_empty), 0);
-        const uint32_t lead_h[2] = {map_to_cta(smem_u32(&h_ready[0]), 0), map_to_cta(smem_u32(&h_ready[1]), 0)};
+        const uint32_t lead_h = map_to_cta(smem_u32(h_ready), 0), lead_s[2] = {map_to_cta(smem_u32(&s_free[0]), 0), map_to_cta(smem_u32(&s_free[1]), 0)};
         float* red = reinterpret_cast<float*>(smem + OFF_RED);
         // 16-byte piece i of this thread's 48 columns in a tile of bf16
         auto piece = [&](int base, int i) { const int p = grp * (kPartCols / 8) + i; return smem + base + (p >> 3) * SLAB_BYTES + r * 128 + (((p & 7) ^ swz) << 4); };
+        // piece i of four fp32 columns from column col on, of row rr, in the tile of x'
+        auto piece32 = [&](int rr, int col, int i) { return smem + OFF_X + (col >> 5) * SLAB_BYTES + rr * 128 + (((((col & 31) >> 2) + i) ^ (rr & 7)) << 4); };
         // the row's total from its four quarters, in one order (named barrier of the row quadrant's 128 threads)
         auto row_sum = [&](int which, float s) {
             red[(which * kParts + grp) * BM + r] = s;
@@ -413,11 +421,8 @@ tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUt
                 unpairs(y, v);
                 tmem_st_32x16(lane_addr + P_COL + c0 + i, v);
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(x_empty);
             if (args.attn_partials && valid) put_sums(args.attn_partials, row, sq, sq1, sq2);
             // LN(x') -> the operand of the first layer
-            if (grp == 0 && lane == 0) tma_store_wait_read<0>();         // the tile before has left through this buffer
             const float mu = row_sum(0, both(sum2)) / (float)D;
             const uint64_t mneg2 = pack2(-mu, -mu);
             tmem_wait_st();
@@ -442,6 +447,9 @@ tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUt
                 uint32_t v[16];
                 tmem_ld_32x16(lane_addr + P_COL + c0 + i, v);
                 tmem_wait_ld();
+                // (x' takes the place of x, which all of the row's threads have read before the sums)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) *reinterpret_cast<uint4*>(piece32(r, c0 + i, j)) = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
                 uint64_t y[8];
                 pairs(v, y);
 #pragma unroll
@@ -461,15 +469,18 @@ tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUt
 #pragma unroll 1
             for (int c = 0; c < NC; ++c, ++g) {
                 const int b = g & 1;
-                const float* bias = b1_s + c * C + grp * 16;
+                const float* bias = b1_s + c * C + grp * 32;
                 mbar_wait(&s_full[b], (g >> 1) & 1u, abort_flag);
                 __syncwarp();
                 tc_fence_after();
-                uint32_t v[16], h[8];
-                tmem_ld_32x16(s_addr + b * C, v);
+                uint32_t v[32], h[16];
+                tmem_ld_32x32(s_addr + b * C, v);
                 tmem_wait_ld();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster_relaxed(lead_s[b]);       // the product of the chunk after next may overwrite S
 #pragma unroll
-                for (int j = 0; j < 16; j += 4) {
+                for (int j = 0; j < 32; j += 4) {
                     const float4 bb = *reinterpret_cast<const float4*>(bias + j);
                     float y0 = __uint_as_float(v[j]) + bb.x, y1 = __uint_as_float(v[j + 1]) + bb.y;
                     float y2 = __uint_as_float(v[j + 2]) + bb.z, y3 = __uint_as_float(v[j + 3]) + bb.w;
@@ -478,11 +489,16 @@ tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUt
                     h[j / 2] = pack_bf16(y0, y1);
                     h[j / 2 + 1] = pack_bf16(y2, y3);
                 }
-                tmem_st_32x8(s_addr + b * C, h);         // over columns read above
+                if (g > 0) {                             // the product with the chunk before has read its place
+                    mbar_wait(h_free, (g - 1) & 1u, abort_flag);
+                    __syncwarp();
+                    tc_fence_after();
+                }
+                tmem_st_32x16(h_addr, h);
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive_cluster_relaxed(lead_h[b]);
+                if (lane == 0) mbar_arrive_cluster_relaxed(lead_h);
             }
 
             // out = O + b2 + x', score, row sums
@@ -492,79 +508,93 @@ tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUt
             tc_fence_after();
             sq = sq1 = sq2 = 0.f;
             uint64_t st1 = pack2(0.f, 0.f), st2 = st1;
-            const int steps = sizeof(OutT) == 2 ? 1 : 2; // fp32: 96 columns at a time, those of groups 0 and 1, then those of 2 and 3
-            for (int turn = 0; turn < steps; ++turn) {
-                if (sizeof(OutT) == 2 || (grp >> 1) == turn) {
 #pragma unroll 1
-                    for (int i = 0; i < kPartCols; i += 16) {
-                        uint32_t v[16], w[16];
-                        tmem_ld_32x16(lane_addr + O_COL + c0 + i, v);
-                        tmem_ld_32x16(lane_addr + P_COL + c0 + i, w);
-                        tmem_wait_ld();
-                        if (i + 16 == kPartCols) {       // O and x' fully read by this warp
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive_cluster_relaxed(lead_oe);
-                        }
-                        uint64_t y[8], xp[8];
-                        pairs(v, y);
-                        pairs(w, xp);
-                        add_vec(y, b2_s + c0 + i);
-                        float u[16];
-                        if (args.score_kind == 2) {
-                            // whole-block shift: x^ - x, with the block input x read here (rows past T: zeros)
-                            const uint4* x0p = reinterpret_cast<const uint4*>(args.x + (size_t)xrow * D + c0 + i);
-                            unpack16<__nv_bfloat16>(valid ? __ldg(x0p) : make_uint4(0u, 0u, 0u, 0u), *reinterpret_cast<float(*)[8]>(u));
-                            unpack16<__nv_bfloat16>(valid ? __ldg(x0p + 1) : make_uint4(0u, 0u, 0u, 0u), *reinterpret_cast<float(*)[8]>(u + 8));
-                        } else {
+            for (int i = 0; i < kPartCols; i += 16) {
+                uint32_t v[16];
+                tmem_ld_32x16(lane_addr + O_COL + c0 + i, v);
+                float w[16], u[16];
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) u[j] = __uint_as_float(w[j]);
-                        }
-                        if (args.partials && args.score_kind == 0) score16(args.dist, y, u, sq, sq1, sq2);
+                for (int j = 0; j < 4; ++j) {
+                    const float4 x4 = *reinterpret_cast<const float4*>(piece32(r, c0 + i, j));
+                    w[4 * j] = x4.x; w[4 * j + 1] = x4.y; w[4 * j + 2] = x4.z; w[4 * j + 3] = x4.w;
+                }
+                tmem_wait_ld();
+                if (i + 16 == kPartCols) {               // O fully read by this warp
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_cluster_relaxed(lead_oe);
+                }
+                uint64_t y[8];
+                pairs(v, y);
+                add_vec(y, b2_s + c0 + i);
+                if (args.score_kind == 2) {
+                    // whole-block shift: x^ - x, with the block input x read here (rows past T: zeros)
+                    const uint4* x0p = reinterpret_cast<const uint4*>(args.x + (size_t)xrow * D + c0 + i);
+                    unpack16<__nv_bfloat16>(valid ? __ldg(x0p) : make_uint4(0u, 0u, 0u, 0u), *reinterpret_cast<float(*)[8]>(u));
+                    unpack16<__nv_bfloat16>(valid ? __ldg(x0p + 1) : make_uint4(0u, 0u, 0u, 0u), *reinterpret_cast<float(*)[8]>(u + 8));
+                } else {
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) y[j] = fadd2(y[j], xp[j]);
-                        if (args.partials && args.score_kind != 0) score16(args.dist, y, u, sq, sq1, sq2);
-                        // the rows leave through the LN(x') buffer, whose products have retired
-                        if constexpr (sizeof(OutT) == 2) {
-                            put_bf16(y, OFF_U, i / 8);
-                            if (args.stats_out) {        // sums of the values as stored: the next block reads these bf16 numbers
+                    for (int j = 0; j < 16; ++j) u[j] = w[j];
+                }
+                if (args.partials && args.score_kind == 0) score16(args.dist, y, u, sq, sq1, sq2);
 #pragma unroll
-                                for (int j = 0; j < 8; ++j) {
-                                    float a, b;
-                                    unpack2(y[j], a, b);
-                                    const uint32_t pk = pack_bf16(a, b);
-                                    const uint64_t z = pack2(__uint_as_float(pk << 16), __uint_as_float(pk & 0xffff0000u));
-                                    st1 = fadd2(st1, z);
-                                    st2 = ffma2(z, z, st2);
-                                }
-                            }
-                        } else {
+                for (int j = 0; j < 8; ++j) y[j] = fadd2(y[j], pack2(w[2 * j], w[2 * j + 1]));
+                if (args.partials && args.score_kind != 0) score16(args.dist, y, u, sq, sq1, sq2);
+                // a lane's results take the place of its x'
+                if constexpr (sizeof(OutT) == 2) {
+                    uint32_t pk[8];
 #pragma unroll
-                            for (int j = 0; j < 8; j += 2) {
-                                const int p = ((grp & 1) * kPartCols + i) / 4 + j / 2;       // 16-byte piece of the 96 columns
-                                float4 o4;
-                                unpack2(y[j], o4.x, o4.y);
-                                unpack2(y[j + 1], o4.z, o4.w);
-                                *reinterpret_cast<float4*>(smem + OFF_U + (p >> 3) * SLAB_BYTES + r * 128 + (((p & 7) ^ swz) << 4)) = o4;
-                            }
+                    for (int j = 0; j < 8; ++j) {
+                        float a, b;
+                        unpack2(y[j], a, b);
+                        pk[j] = pack_bf16(a, b);
+                        if (args.stats_out) {            // sums of the values as stored: the next block reads these bf16 numbers
+                            const uint64_t z = pack2(__uint_as_float(pk[j] << 16), __uint_as_float(pk[j] & 0xffff0000u));
+                            st1 = fadd2(st1, z);
+                            st2 = ffma2(z, z, st2);
                         }
                     }
-                    fence_async_smem();
+                    *reinterpret_cast<uint4*>(piece32(r, c0 + i, 0)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                    *reinterpret_cast<uint4*>(piece32(r, c0 + i, 1)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 8; j += 2) {
+                        float4 o4;
+                        unpack2(y[j], o4.x, o4.y);
+                        unpack2(y[j + 1], o4.z, o4.w);
+                        *reinterpret_cast<float4*>(piece32(r, c0 + i, j / 2)) = o4;
+                    }
                 }
-                named_barrier(1 + q, 128);
-                if (grp == 0 && lane == 0) {             // boxes of 32 rows x 128 bytes
-                    if (m0 + q * 32 < args.T)
-                        for (int kb = 0; kb < 3; ++kb)
-                            tma_store_2d(&tmOut, smem + OFF_U + kb * SLAB_BYTES + q * 4096, turn * 96 + kb * (128 / (int)sizeof(OutT)), m0 + q * 32);
-                    tma_store_commit();
-                    if (turn + 1 < steps) tma_store_wait_read<0>();
+            }
+            __syncwarp();
+            // the warp's 32 rows x 48 columns leave with neighbouring lanes on neighbouring 16-byte pieces of a row: LPR lanes to the
+            // sixteen columns of a row, and rows to a quarter of a warp whose pieces lie in different banks
+            constexpr int LPR = sizeof(OutT) == 2 ? 2 : 4, ROWS = 32 / LPR, ID = LPR == 2 ? 1 : 2;
+            const int sub = lane & (LPR - 1), idx = lane >> ID;
+            const int rsub = LPR == 2 ? (idx >> 3) * 8 + (idx & 3) * 2 + ((idx >> 2) & 1) : (idx & 1) * 4 + (idx >> 1);
+#pragma unroll
+            for (int rb = 0; rb < 32; rb += ROWS) {
+                const int rr = q * 32 + rb + rsub;
+                uint4 t4[3];
+#pragma unroll
+                for (int i = 0; i < 3; ++i) t4[i] = *reinterpret_cast<const uint4*>(piece32(rr, c0 + 16 * i, sub));
+                char* to = reinterpret_cast<char*>(out + (size_t)(m0 + rr) * D + c0) + sub * 16;
+                if (m0 + rr < args.T) {
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) *reinterpret_cast<uint4*>(to + i * 16 * sizeof(OutT)) = t4[i];
                 }
-                if (turn + 1 < steps) named_barrier(1 + q, 128);
             }
             if (args.partials && valid) put_sums(args.partials, row, sq, sq1, sq2);
             if (args.stats_out && valid) reinterpret_cast<float2*>(args.stats_out)[(size_t)row * kParts + grp] = make_float2(both(st1), both(st2));
+            fence_async_smem();                          // (the next x lands over what was written here)
+            __syncwarp();
+            if (lane == 0) mbar_arrive(x_empty);
         }
-        if (grp == 0 && lane == 0) tma_store_wait<0>();  // all output written before the CTA exits
+        // the last signals on this CTA's barriers that nothing above waited for
+        if (mine > 0) {
+            mbar_wait(h_free, (mine * NC - 1) & 1u, abort_flag);
+            mbar_wait(u_free, (mine - 1) & 1u, abort_flag);
+        }
     }
 
     tc_fence_before();
@@ -580,7 +610,7 @@ tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUt
 
 template <typename OutT>
 cudaError_t launch(const CUtensorMap& tmO, const CUtensorMap& tmX, const CUtensorMap& tmWo, const CUtensorMap& tmW1, const CUtensorMap& tmW2,
-                   const CUtensorMap& tmOut, const TailArgs& args, int sm_count, cudaStream_t st) {
+                   const TailArgs& args, int sm_count, cudaStream_t st) {
     static PerDeviceOnce attr_once;
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
@@ -602,7 +632,7 @@ cudaError_t launch(const CUtensorMap& tmO, const CUtensorMap& tmX, const CUtenso
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, tail_kernel<OutT>, tmO, tmX, tmWo, tmW1, tmW2, tmOut, args);
+    return cudaLaunchKernelEx(&cfg, tail_kernel<OutT>, tmO, tmX, tmWo, tmW1, tmW2, (OutT*)args.out, args);
 }
 
 }  // namespace
