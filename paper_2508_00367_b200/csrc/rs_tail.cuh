@@ -302,7 +302,7 @@ tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUt
                 }
                 if (!ok) break;
                 mma_commit_pair(p_full, 3);
-                ok = mbar_wait(u_full, t & 1u, abort_flag);
+                ok = mbar_wait<true>(u_full, t & 1u, abort_flag);    // LN(x') of the peer's rows too
                 if (ok) first(g, NC == 1);
                 for (int c = 0; c < NC && ok; ++c, ++g) {
                     if (c + 1 < NC) first(g + 1, c + 2 == NC);

@@ -45,17 +45,31 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// kCluster: the wait acquires at cluster scope, for what threads of the peer CTA wrote to their shared memory before
+// mbar_arrive_cluster_release.  The default acquires at CTA scope.
+template <bool kCluster = false>
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
-    asm volatile(
-        "{\n"
-        ".reg .pred p;\n"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        "selp.u32 %0, 1, 0, p;\n"
-        "}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
+    if constexpr (kCluster)
+        asm volatile(
+            "{\n"
+            ".reg .pred p;\n"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+            "selp.u32 %0, 1, 0, p;\n"
+            "}\n"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
+    else
+        asm volatile(
+            "{\n"
+            ".reg .pred p;\n"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+            "selp.u32 %0, 1, 0, p;\n"
+            "}\n"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
     return ok != 0;
 }
 
@@ -63,12 +77,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // already given up), so a lost arrival ends the kernel with a status instead of a hang.
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 
+template <bool kCluster = false>
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_try_wait<kCluster>(bar, parity)) return true;
     const uint64_t t0 = globaltimer_ns();
     uint32_t spins = 0;
     while (true) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (mbar_try_wait<kCluster>(bar, parity)) return true;
         if ((++spins & 255u) == 0) {
             if (*abort_flag) return false;
             if (globaltimer_ns() - t0 > kWaitLimitNs) {
@@ -307,16 +322,17 @@ __device__ __forceinline__ float4 ld_cluster(uint32_t addr) {
 }
 // Arrive on an mbarrier given by a shared::cluster address (possibly in the peer CTA), for what is ordered by other means:
 // no memory access of this thread is made visible by it.  The epilogues hand an accumulator back with it, whose reads
-// tcgen05.wait::ld has completed and tcgen05.fence::before_thread_sync has ordered.  The default, .release.cluster, also
+// tcgen05.wait::ld has completed and tcgen05.fence::before_thread_sync has ordered.  A .release.cluster there also
 // waits for all earlier stores of the thread to be visible, staged and partial results among them: 2700 cycles a tile, half
 // of the plain epilogue's time and a quarter of the GELU one's.  Products of a block, with it / relaxed, us: QKV
 // 50432 x 576 x 192 23.5 / 17.8, projection 25216 x 768 x 768 40.2 / 35.6, FC1 25216 x 3072 x 768 87.2 / 79.0.
 __device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
-// The same after writes to this CTA's shared memory that fence.proxy.async has made visible to the tensor core.
+// Arrive on such an mbarrier for ordinary writes to this CTA's shared memory (after fence.proxy.async, where the tensor core
+// reads them).  The thread that waits may be the peer's, so both sides work at cluster scope: mbar_wait<true> there.
 __device__ __forceinline__ void mbar_arrive_cluster_release(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // TMA load inside a CTA pair: the data lands in this CTA's shared memory, the completion
 // bytes are signalled on an mbarrier given by a shared::cluster address (the pair leader's).

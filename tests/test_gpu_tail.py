@@ -50,6 +50,30 @@ def test_several_tiles_a_pair(ctx, out_dtype):   # noqa: F811
         _check_block({k: v[b:b + 1] for k, v in res.items()}, ref, "bf16", out_dtype)
 
 
+def _past_rounds(ctx, rounds):   # noqa: F811
+    """(B, N) of the fewest rows above that many whole rounds of 256-row tiles, of samples whose length divides them."""
+    first = rounds * (torch.cuda.get_device_properties(ctx.device).multi_processor_count // 2) * 256
+    return next((T // N, N) for T in range(first + 1, first + 256) for N in range(128, 63, -1) if T % N == 0)
+
+
+@pytest.mark.parametrize("mode,dist,out_dtype", [("mlp", "l2", torch.bfloat16), ("attn", "cos", torch.float32), ("block", "l1", torch.bfloat16)])
+def test_rows_of_later_rounds(ctx, mode, dist, out_dtype):   # noqa: F811
+    """Two whole rounds and a tile of a few rows: bit for bit what the samples give in calls of one round (an eighth of them
+    each), where no buffer, barrier or part of tensor memory is used for a second tile."""
+    import paper_2508_00367_b200 as rs
+    B, N = _past_rounds(ctx, 2)
+    x = synth.make_tokens(B, N, D, "bf16", seed=21).bfloat16().cuda()
+    dw = rs.DeviceBlockWeights(synth.make_block_weights(D, 4 * D, "bf16", seed=22), torch.bfloat16, ctx.device)
+    run = lambda t: ctx.block_fwd(t, dw, H, N // 5, out_dtype=out_dtype, score_mode=mode, dist=dist, want_full=True)   # noqa: E731
+    whole, step = run(x), (B + 7) // 8
+    assert step * N > 3200                               # (with fewer rows QKV is summed in another order)
+    for b in [*range(0, B - step, step), B - step]:
+        part = run(x[b:b + step].contiguous())
+        for k in part:
+            assert torch.equal(whole[k][b:b + step], part[k]), (k, b)
+    ctx.async_status()
+
+
 @pytest.mark.parametrize("mode,dist", [("mlp", "l1"), ("mlp", "cos"), ("mlp_delta", "l2"), ("attn", "l2"), ("attn", "cos"), ("block", "l2"), ("block", "l1")])
 def test_scores(ctx, mode, dist):   # noqa: F811
     """Bounds as where these scores come from the epilogues of the single products (bf16 operands in full)."""
