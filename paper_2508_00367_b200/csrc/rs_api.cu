@@ -483,7 +483,7 @@ static rs_status block_fwd_impl(rs_ctx* ctx, const rs_block_desc* d, const rs_bl
         const rs::GemmLn lnout = {fc2_stats ? hk->stats_out : nullptr, fc2_stats ? hk->parts_out : nullptr, nullptr, 0, nullptr, 0.f};
         if (one_tail) {
             const rs::TailCall tail = {T, Dm, o, x, in_map, w->w_o, w->w_fc1, w->w_fc2, w->b_o, w->b_fc1, w->b_fc2, w->ln2_g, w->ln2_b, eps, x_hat, d->out_dtype,
-                                       attn_score ? m : nullptr, attn_score ? nullptr : m, kind, (int)d->dist, lnout.stats_out, lnout.stats_parts_out, true, &in_use};
+                                       attn_score ? m : nullptr, attn_score ? nullptr : m, kind, (int)d->dist, lnout.stats_out, lnout.stats_parts_out, &in_use};
             RS_CHECK_LAUNCH(ctx, RS_K_GEMM, st, rs::launch_tail_tc(ctx, tail, st), "proj+LN2+FC1+FC2+residual+score");
         } else {
             RS_CHECK_LAUNCH(ctx, RS_K_GEMM, st, rs::launch_gemm_tc(ctx, rs::RS_EPI_BIAS_GELU, u, w->w_fc1, w->b_fc1, nullptr, nullptr, nullptr, h, RS_BF16, nullptr, 0, 0, T, Dm, D, st, nullptr, true, &in_use), "FC1");

@@ -855,7 +855,6 @@ cudaError_t launch_tail_tc(rs_ctx* ctx, const TailCall& c, cudaStream_t st) {
     a.attn_partials = c.attn_partials; a.partials = c.partials; a.score_kind = c.score_kind; a.dist = c.dist;
     a.stats_out = c.out_dtype == RS_BF16 ? c.stats_out : nullptr;
     if (a.stats_out && c.stats_parts_out) *c.stats_parts_out = tail::kParts;
-    a.weights_ready = c.weights_ready ? 1 : 0;
     const bool skips = c.rows && c.rows->lens && (c.T + 255) / 256 <= kMaskTiles;
     a.lens = skips ? c.rows->lens : nullptr;
     a.seq_n = skips ? c.rows->seq_n : 0;

@@ -168,7 +168,8 @@ cudaError_t launch_gemm_tc(rs_ctx* ctx, int epi, const void* A, const void* W, c
 
 // Projection and MLP of a block of 192 columns in one kernel (rs_tail.cuh): x' = o Wo^T + bo + x,
 // out = m + x', m = GELU(LN(x') W1^T + b1) W2^T + b2, with tail_tc_parts() partial sums of the scored pair per row (and, for bf16
-// outputs, as many pairs of the output's row sums).
+// outputs, as many pairs of the output's row sums).  Weights and vectors are read before the kernel waits for its predecessor: as for
+// weights_ready above, every earlier kernel that could write them has completed.
 struct TailCall {
     long long T;
     int Dm;
@@ -184,7 +185,6 @@ struct TailCall {
     int score_kind, dist;
     float* stats_out;                       // or null
     int* stats_parts_out;
-    bool weights_ready;                     // as for launch_gemm_tc
     const GemmRows* rows;
 };
 bool tail_tc_use(long long T, int D, int Dm);

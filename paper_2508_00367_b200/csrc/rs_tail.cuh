@@ -37,7 +37,6 @@ struct TailArgs {
     float* stats_out;                                    // [T, kParts][2] or null
     void* out;                                           // [T, D]
     int score_kind, dist;
-    int weights_ready;
     const int* lens;
     int seq_n;
     int* status;
@@ -175,32 +174,26 @@ tail_kernel(const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUt
         tmem_alloc_pair(tmem_slot, 512);
         tmem_relinquish_pair();
     }
-    auto load_vectors = [&]() {
-        for (int i = threadIdx.x; i < D; i += kThreads) {
-            bo_s[i] = args.bo ? __ldg(args.bo + i) : 0.f;
-            g_s[i] = __ldg(args.ln_g + i);
-            be_s[i] = __ldg(args.ln_b + i);
-            b2_s[i] = args.b2 ? __ldg(args.b2 + i) : 0.f;
-        }
-        for (int i = threadIdx.x; i < args.Dm; i += kThreads) b1_s[i] = args.b1 ? __ldg(args.b1 + i) : 0.f;
-    };
-    if (args.weights_ready) load_vectors();
+    for (int i = threadIdx.x; i < D; i += kThreads) {
+        bo_s[i] = args.bo ? __ldg(args.bo + i) : 0.f;
+        g_s[i] = __ldg(args.ln_g + i);
+        be_s[i] = __ldg(args.ln_b + i);
+        b2_s[i] = args.b2 ? __ldg(args.b2 + i) : 0.f;
+    }
+    for (int i = threadIdx.x; i < args.Dm; i += kThreads) b1_s[i] = args.b1 ? __ldg(args.b1 + i) : 0.f;
     tc_fence_before();
     __syncthreads();
     cluster_sync();                              // the peer's barriers exist before anything signals them
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     grid_dep_launch();
-    // Weights do not depend on the kernel before this one: the producer fills the ring first (below).
-    const bool early = args.weights_ready && !args.lens;
+    // Weights do not depend on the kernel before this one (TailCall): the producer fills the ring first (below), unless a mask of row
+    // tiles has to be made with the whole CTA.
+    const bool early = !args.lens;
     if (!(warp == 0 && early)) grid_dep_wait();
 
     int tiles = num_m;
     uint32_t* mask = args.lens ? reinterpret_cast<uint32_t*>(smem + OFF_MASK) : nullptr;
-    if (!args.weights_ready) {
-        load_vectors();
-        __syncthreads();
-    }
     if (mask) tiles = mark_row_tiles(mask, args.lens, args.seq_n, args.T, warp, lane, kThreads);
     const int mine = tiles > pair ? (tiles - pair + npairs - 1) / npairs : 0;      // tiles pair, pair + npairs, ...
     RowTiles row_tiles = {mask};                 // (each role walks its own copy)
