@@ -19,7 +19,7 @@ def _poison(nbytes=1 << 28):
 
 
 @pytest.mark.parametrize("lens", [[300, 1, 17, 128, 250, 2, 40, 129, 113], [300, 300, 1, 1, 1, 1, 1, 1, 300], [3] * 8 + [300]])
-@pytest.mark.parametrize("N,D", [(300, 384), (1100, 256)])
+@pytest.mark.parametrize("N,D", [(300, 384), (1100, 256), (1100, 192)])
 def test_block_over_poisoned_buffers(ctx, lens, N, D):   # noqa: F811
     import paper_2508_00367_b200 as rs
     B, H = 9, D // 64
@@ -53,7 +53,7 @@ def test_block_over_poisoned_buffers(ctx, lens, N, D):   # noqa: F811
     ctx.async_status()
 
 
-@pytest.mark.parametrize("D", [256, 384])                             # both LayerNorm kernels in LN2
+@pytest.mark.parametrize("D", [192, 256, 384])                        # LN2 in the kernel for 192 columns, both LayerNorm kernels
 @pytest.mark.parametrize("counts", [[2147483647, 2147483640, 1300, 40], [0, -5, -2147483648, 300]])
 def test_counts_outside_the_sample_are_clamped(ctx, counts, D):   # noqa: F811
     """seq_lens holds any int: it stands for its value clamped to [1, N], in every kernel, over poisoned buffers too."""
