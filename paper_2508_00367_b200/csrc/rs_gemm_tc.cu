@@ -829,12 +829,18 @@ cudaError_t launch_gemm_tc(rs_ctx* ctx, int epi, const void* A, const void* W, c
 
 // Which blocks take their projection and MLP as one kernel: those of 192 columns with more than two tiles' rows.  Fewer rows
 // are done sooner by the four kernels for few rows, which spread a tile's columns over the SMs.  Whole pruned forwards of 12
-// blocks (20 % dropped three times), four kernels / one, us: 1 x 197 388 / 399, 2 x 197 393 / 404, 4 x 197 418 / 416, 8 x 197
-// 443 / 399, 16 x 197 479 / 424, 32 x 197 542 / 457, 1 x 1569 622 / 585, 256 x 197 1292 / 1044.  A tile takes some 27000 cycles, of
-// which the tensor pipe needs 10400: six chunks of 2150 (GELU: sixteen warps keep the special-function unit, the FMA and the ALU
-// pipes half busy each, and its hand-overs are waits), x' and LN(x') 5000, x of the next tile and the output 8000.  With x'
-// in tensor memory and chunks of 64 columns, two of them under way, a chunk's chain took 1500 cycles for half the columns
-// and 256 x 197 1059 us.
+// blocks (hidden width 768, 20 % dropped three times, captured in a graph below 2500 rows), four kernels / one, us: 1 x 197 388 / 399 and 2 x 197
+// 393 / 404 with the line left out; 3 x 173 398 / 395, 5 x 128 400 / 406, 4 x 197 420 / 417, 1 x 785 494 / 497, 6 x 160 405 / 403, 8 x 197 444 / 403,
+// 16 x 197 478 / 427, 32 x 197 544 / 458, 1 x 1569 622 / 589, 256 x 197 1301 / 1056.  Without pruning 3 x 173 385 / 385, 1 x 700 482 / 493, 4 x 197
+// 435 / 400.  One block a call, hidden width 768: 4 x 197 43.2 / 42.8, 8 x 197 44.1 / 43.5, 16 x 197 50.2 / 44.7; captured in a graph, where a
+// launch costs less, up to 2000 rows are the slower for it: 3 x 190 39.0 / 39.3, 4 x 197 39.5 / 40.8, 8 x 197 40.6 / 41.6, 16 x 197 46.0 / 42.1.
+// Narrower hidden layers leave less to do in the chunks and gain at all of these: 128 3 x 190 40.7 / 33.6, 4 x 197 42.2 / 34.9; 512 39.9 / 36.8,
+// 41.5 / 38.2 (640 at 8 x 197 39.6 / 40.5).
+// A tile in mid-launch takes 28000 to 30000 cycles, of which the tensor pipe needs 10400: waiting for x 1300 to 2400, x' and LN(x') 4900, its
+// hand-over 1000, the first chunk 3600, five more 2100 each (GELU and its hand-overs), the wait for O 1450, the output 5000 to
+// 5800; the first tile of a launch 41000.  Over 197 tiles the schedulers issue in 39 % of the cycles, with the ALU 23, the special-function unit 18 and
+// the FMA pipe 17 % busy.  With x' in tensor memory and chunks of 64 columns, two of them under way, a chunk's chain took
+// 1500 cycles for half the columns and 256 x 197 1059 us where this form took 1044 (before its hand-over at cluster scope).
 bool tail_tc_use(long long T, int D, int Dm) {
     return T > 512 && D == tail::D && Dm >= tail::C && Dm % tail::C == 0 && Dm <= tail::kMaxHidden && T < (1ll << 31);
 }
