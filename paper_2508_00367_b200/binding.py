@@ -160,7 +160,7 @@ def load_library() -> ctypes.CDLL:
 
 
 def attn_kernel_choice(sm_count: int, B: int, H: int, N: int) -> int:
-    """rs_attn_kernel_choice: 2 or 3, the attention kernel rs_attn_fwd picks for the shape (host arithmetic only)."""
+    """rs_attn_kernel_choice: 2 or 3, what a cost model of earlier attention kernels picks for the shape (host arithmetic only)."""
     return int(load_library().rs_attn_kernel_choice(sm_count, B, H, N))
 
 

@@ -1,5 +1,6 @@
 // Fused attention on the tensor cores (Eq. sa): out = Softmax(Q K^T * scale) V per
 // (sample, head), head dimension 64, without ever writing the N x N matrix.
+// This kernel serves batches of very many samples with a count each, and as the other kernel's cross-check (see launch_attn_tc).
 //
 // Persistent kernel, one CTA per SM, looping over work items.  An item is two 128-row query
 // tiles A and B: for N > 128 two consecutive query tiles of one (sample, head), which share
@@ -488,22 +489,44 @@ bool attn_tc_supported(const rs_attn_desc& d) {
     return true;
 }
 
-// How a shape with more than one query tile per head is run (host side, remembered per shape).
-// Two query tiles per CTA (this file): items go to the CTAs round robin, and a pair of query tiles costs
+// The load of the longest CTA, in tenths of three query tiles of one head, when the kernel with three tiles per CTA takes its items
+// within heads: the one or two tiles left over per head (two cost as much as three, one 7) follow the groups, on the CTAs that
+// the last round of groups left out, up to two each (wrap = 0; -1: too many), or round robin over all (wrap = 1).
+static long long three_tile_load(long long BH, int N, int G, int wrap) {
+    constexpr int NG = 3;
+    const int tiles = (N + BQ - 1) / BQ, per3 = tiles / NG, tail_ng = tiles - per3 * NG;
+    const long long n3 = BH * per3, n_tail = tail_ng ? BH : 0;
+    const int r = (int)(n3 % G), idle = G - r;
+    if (!wrap && n_tail > 2ll * idle) return -1;
+    const int stride = wrap ? G : idle, tail_cost = tail_ng == 1 ? 7 : 10;
+    long long worst = 0;
+    for (int c = 0; c < G; ++c) {
+        long long load = c < n3 ? 10 * ((n3 - c + G - 1) / G) : 0;
+        int pos = c - r;
+        if (pos < 0) {
+            if (!wrap) { worst = load > worst ? load : worst; continue; }
+            pos += G;
+        }
+        if (pos < n_tail) load += tail_cost * ((n_tail - pos + stride - 1) / stride);
+        worst = load > worst ? load : worst;
+    }
+    return worst;
+}
+// The same with items across heads.
+static long long three_tile_across_load(long long BH, int N, int G) {
+    const long long tiles = BH * ((N + BQ - 1) / BQ), left = tiles % (3ll * G);
+    return (tiles - left) / (3ll * G) * 10 + (left == 0 ? 0 : left <= G ? 7 : 10);
+}
+
+// How this kernel cuts a shape with more than one query tile per head (host side, remembered per shape).  Items go to the CTAs
+// round robin, and a pair of query tiles costs
 // twice a single one, so a last round with few pairs left keeps most SMs idle for a whole pair's time.
 // The tiles of the last few (sample, head)s are therefore handed out one by one where that shortens the
 // longest CTA: best_hs is the count with the smallest makespan under the cost model pair = 10, single = 7
 // (a query tile alone runs faster than next to another, but not twice as fast: measured).
-// This kernel or the one with three query tiles per CTA (rs_attn_tc3.cu)?  Both are paced by the longest
-// CTA: its items (in tenths) times the key tiles of an item, plus a cost per item; microseconds fitted to
-// CUDA-event times of thirteen shapes from N = 197 to 4097 (worst error 6 % and 9 %).  The lines are those of earlier kernels:
-// since the three-tile kernel sends a part of its exponentials through the FMA pipes and takes items across heads it runs under
-// its lines.  At the workloads' shapes the choice is the faster kernel (32 x 16 x 577 82.9 us, two tiles 101; 16 x 12 x 1569 182 /
-// 208; 64 x 12 x 181 26.3 / 29.5) but for 4 x 16 x 2305 (two tiles 151, three would take 134), x 1729 (92.1 / 90.2),
-// 64 x 12 x 197 (31.8 / 30.5), 16 x 12 x 539 (38.8 / 36.7) and 32 x 16 x 457 (59.8 / 59.2).
-// With its items across heads the three-tile kernel has a line of its own: the same one at the lower load, the steps a
-// little longer by the share of items with two K/V streams (two in as many items as a head has tiles).  It is chosen where
-// that is 8 % better, about the errors of the fits.
+// `three` is what a cost model of two earlier kernels says of this one against the one with three tiles per CTA: both paced by
+// the longest CTA, its items (in tenths) times the key tiles of an item plus a cost per item, microseconds fitted to thirteen
+// shapes from N = 197 to 4097.  rs_attn_kernel_choice reports it; the dispatch does not follow it any more (see launch_attn_tc).
 AttnPlan attn_plan(long long BH, int N, int G) {
     const int nt = (N + BQ - 1) / BQ, per = (N + 2 * BQ - 1) / (2 * BQ);
     auto makespan = [&](long long hs) {
@@ -519,7 +542,7 @@ AttnPlan attn_plan(long long BH, int N, int G) {
     };
     static std::mutex memo_mu;
     static std::map<std::tuple<long long, int, int>, AttnPlan> memo;
-    AttnPlan plan = {0, 0, 0};
+    AttnPlan plan = {0, 0};
     const auto key = std::make_tuple(BH, N, G);
     std::lock_guard<std::mutex> lock(memo_mu);
     const auto hit = memo.find(key);
@@ -532,14 +555,12 @@ AttnPlan attn_plan(long long BH, int N, int G) {
             const long long m = makespan(hs);
             if (best < 0 || m < best) { best = m; plan.best_hs = hs; }
         }
-        int wrap3 = 0;
-        const long long u3 = attn_tc3_plan(BH, N, G, &wrap3);
+        const long long u_in = three_tile_load(BH, N, G, 0), u_wrap = three_tile_load(BH, N, G, 1), u3 = u_in < 0 || u_wrap < u_in ? u_wrap : u_in;
         const double t2 = best / 10.0 * (((N + BKV - 1) / BKV) * 1.505 + 2.51) + 2.32;
         const double t3 = u3 / 10.0 * (((N + 63) / 64) * 1.136 + 1.00) + 6.71;
         const double two_streams = 1.0 + 0.12 * (nt % 3 ? 2.0 / nt : 0.0);
-        const double t3a = attn_tc3_across_load(BH, N, G) / 10.0 * (((N + 63) / 64) * 1.136 + 1.00) * two_streams + 6.71;
+        const double t3a = three_tile_across_load(BH, N, G) / 10.0 * (((N + 63) / 64) * 1.136 + 1.00) * two_streams + 6.71;
         plan.three = t3 < t2 || t3a < 0.92 * t2;
-        plan.wrap3 = wrap3;
     }
     memo[key] = plan;
     return plan;
@@ -573,20 +594,21 @@ cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, co
     long long items = (long long)args.per * (args.dual ? d.B : (long long)d.B * d.H);
     if (items >= (1ll << 30)) return cudaErrorInvalidValue;
     args.n_pair_items = (int)items; args.first_single_bh = d.B * d.H; args.tile_count = (d.N + BQ - 1) / BQ;
-    auto three_tiles = [&](int wrap, bool split) {
+    // The kernel with three query tiles per CTA takes every shape but batches of very many samples with a count each: two tiles /
+    // three, us, 4 x 16 x 4097 404 / 335, x 2305 151 / 122, 16 x 12 x 1569 207 / 165, 32 x 16 x 577 101 / 72, 64 x 12 x 197 31.8 / 26.1, x 101 14.1 / 11.6,
+    // x 17 9.4 / 7.4, 1 x 12 x 197 6.3 / 6.0.  RS_ATTN_KERNEL=2 keeps this file's for all (tests compare each with the oracle).
+    const bool split = split_weights && !seq_lens;          // (this file's kernel has no such weights)
+    if (split || (ctx->attn_kernel != 2 && (!seq_lens || d.B <= attn_tc3_max_samples()))) {
         CUtensorMap tmK3, tmV3;
         if (!make_tmap_qkv(ctx, &tmK3, k, d.B, d.N, d.H, d.k_batch_stride, d.k_row_stride, d.k_head_stride, 64) ||
             !make_tmap_qkv(ctx, &tmV3, v, d.B, d.N, d.H, d.v_batch_stride, d.v_row_stride, d.v_head_stride, 64))
             return cudaErrorInvalidValue;
-        return launch_attn_tc3(ctx, d, tmQ, tmK3, tmV3, tmO, wrap, split, st);
-    };
-    if (split_weights && !seq_lens) return three_tiles(0, true);
+        return launch_attn_tc3(ctx, d, tmQ, tmK3, tmV3, tmO, seq_lens, split, st);
+    }
     if (!args.dual) {
         const long long BH = (long long)d.B * d.H;
         const int nt = args.tile_count, per = args.per;
         const AttnPlan plan = attn_plan(BH, d.N, ctx->sm_count);
-        const int force = ctx->attn_kernel;                    // RS_ATTN_KERNEL=2 / 3: one kernel for every shape it takes
-        if (!seq_lens && (force == 3 || (force != 2 && plan.three))) return three_tiles(plan.wrap3, false);
         const long long best_hs = plan.best_hs;
         args.n_pair_items = (int)((BH - best_hs) * per);
         args.first_single_bh = (int)(BH - best_hs);

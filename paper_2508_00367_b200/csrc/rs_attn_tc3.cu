@@ -1,4 +1,4 @@
-// Fused attention on the tensor cores (Eq. sa) for long sequences: three query tiles per CTA.
+// Fused attention on the tensor cores (Eq. sa): three query tiles per CTA.
 //
 // Same scheme as rs_attn_tc.cu -- S = Q K^T by tcgen05.mma into tensor memory, a softmax warpgroup
 // per query tile with a row per thread, P as the tensor-memory A operand of O += P V, lazy
@@ -7,8 +7,13 @@
 // columns for three tiles.  With head dimension 64 the special-function unit (the exponentials)
 // bounds the kernel, and what keeps that unit from saturating is the serial chain of each
 // softmax warp; three warps per scheduler instead of two fill more of its gaps.
+// The softmax warps' loop over whole key tiles carries nothing else: no masks, no rescaling of O, no second form of the
+// exponentials.  A tile that needs any of these goes through a second, short piece of code (16 columns at a time from tensor
+// memory).  What a loop that long also carries is paid for at every tile and in instruction fetches (32 KB at full rate,
+// then a third of it): with masked and rescaling forms in the loop a key tile of three query tiles took 2000 to 2200 cycles, so 1750 to
+// 1850, of which 1250 are exponentials; 4 x 16 x 4097 369 -> 337 us, 16 x 12 x 1569 181 -> 160, 32 x 16 x 577 82.8 -> 72.3, 64 x 12 x 197 30.5 -> 24.1.
 // An item is three consecutive 128-row query tiles of one (sample, head), which share the K/V
-// tiles streamed through the TMA ring; or (ACROSS) of consecutive (sample, head)s.
+// tiles streamed through the TMA ring, or of consecutive (sample, head)s.
 // SPLIT: the weights go to the second product as a bf16 and the bf16 of what that left over, one after the other
 // through the same tensor-memory columns: 16 bits of mantissa instead of 8, for the blocks that used to have fp32
 // weights (see rs_block_fwd).
@@ -37,129 +42,135 @@ constexpr int kLaunchRegs = 128, kSoftmaxRegs = 152, kOtherRegs = 56;
 static_assert(384 * kSoftmaxRegs + 128 * kOtherRegs <= kThreads * kLaunchRegs, "register pool of the CTA");
 constexpr int kSCol = 0, kPCol = NG * BKV, kOCol = kPCol + NG * (BKV / 2);   // S 0..191, P 192..287, O 288..479
 constexpr int kTmemCols = 512;
+constexpr float kLowest = -3.0e38f;              // stands for a maximum of -infinity: such scores are weights of 0
 constexpr float kRescaleGap = 8.f;              // log2 units the tile maximum may exceed the running one
 // shared memory: Q[2 buffers][NG] | K[NS] | V[NS] | output staging | barriers
 constexpr int OFF_Q = 0, OFF_K = 2 * NG * Q_BYTES, OFF_V = OFF_K + NS * KV_BYTES;
 constexpr int OFF_OST = OFF_V + NS * KV_BYTES;  // output staging: 12 softmax warps x 32 rows x 128 bytes
 constexpr int OFF_BAR = OFF_OST + 4 * NG * 4096;
-constexpr size_t kSmem = (size_t)OFF_BAR + 512 + 1024 /*alignment slack*/;
+constexpr int kMaxSamples = 256;                 // of a launch with a count per sample
+constexpr int OFF_SAMPLES = OFF_BAR + 512;      // what those launches keep of the counts
+constexpr size_t kSmem = (size_t)OFF_SAMPLES + 4 * (kMaxSamples + 2) + kMaxSamples + 1024 /*alignment slack*/;
 static_assert(kOCol + NG * DH <= kTmemCols, "tensor-memory columns");
 static_assert(kSmem <= 232448, "shared memory of one CTA");
 
-// Items within heads: first the groups of three query tiles of every (sample, head) -- n3 of them, per3 to a head --
-// then, where the tile count is not a multiple of three, one item per head with the tail_ng tiles left
-// over (n_tail of them).  CTA c takes the groups c, c + G, ... and then tails: tail number
-// tail_pos + k * tail_stride for k = 0, 1, ..., where tail_pos = c - tail_first (CTAs before tail_first
-// take none, unless the tails wrap around: tail_wrap = 1, position (c - tail_first) mod G).
-// Items ACROSS heads: three tiles in a row whichever heads they belong to, so that the tails do not leave warpgroups
-// idle; an item that meets a head's end takes two K/V streams, a tile of each head in turn.  CTA c takes the items
-// c, c + G, ...; the tiles of the last round go one to an item where there are CTAs enough.
+// The work: the query tiles of all (sample, head)s in a row, three to an item, whichever heads they belong to; an item that
+// meets a head's end takes two K/V streams, a tile of each in turn (with one query tile per head, three).  CTA c takes
+// the items c, c + G, ...  The tiles of the last round are spread over the CTAs, `rest` to an item.  Where the plan says so the
+// last `cut` query tiles of every head come after all others, one to an item with the keys cut in three: each warpgroup
+// takes a third of them for the same queries, and the first merges the three results, which lie in the same tensor-memory
+// lanes.  (Always the same tiles of every head: a sample's result does not depend on its place in the batch.)
+// RAGGED: items of one sample after the other, the longest first (`order`, `first_item`), each with its own count of tokens.
 struct Attn3Args {
-    int N, H;
-    int per3, n3, n_tail, tail_ng;
-    int tail_first, tail_stride, tail_wrap;
-    int nt, tiles;           // ACROSS: query tiles per (sample, head), and in all
-    int full, rest, n_items; // ACROSS: items of three tiles that fill whole rounds, tiles per item after those, items in all
+    int N, H, B;
+    int nt, tiles;           // query tiles per (sample, head) that see all keys at once, and in all
+    int cut;                 // and those with the keys cut in three
+    uint32_t by_nt, by_h, by_cut;    // 2^32 over nt, H and cut, rounded down: see divide()
+    int full, rest;          // items of three tiles that fill whole rounds, tiles per item after those
+    int n_whole, n_items;    // items before those with the keys cut, and in all
+    const int* lens;         // RAGGED: [B], sample b attends over its first lens[b] tokens only (clamped to 1 .. N)
     float scale_log2;        // scale * log2(e)
     int* status;
 };
 
-struct Item3 {
-    int bh, q;               // (sample, head) and query tile of tile 0
-    int ng;                  // query tiles present: 1 .. 3
-    int split;               // tiles of the first (sample, head); the others, if any (ACROSS), belong to the next one
-                             // (SPLIT with one query tile per (sample, head): each tile to its own)
-    // which of the item's (sample, head)s tile g belongs to, and whether it is the first or the last tile of one
-    template <bool SPLIT> __device__ __forceinline__ int stream(const Attn3Args& a, int g) const { return SPLIT && a.nt == 1 ? g : g >= split; }
-    template <bool SPLIT> __device__ __forceinline__ bool starts(const Attn3Args& a, int g) const { return g == 0 || g == split || (SPLIT && a.nt == 1); }
-    template <bool SPLIT> __device__ __forceinline__ bool ends(const Attn3Args& a, int g) const { return g == ng - 1 || g == split - 1 || (SPLIT && a.nt == 1); }
-};
-template <bool ACROSS> __device__ __forceinline__ Item3 decode_item3(const Attn3Args& a, int w) {
-    Item3 it;
-    if (ACROSS) {
-        const int tile = w < a.full ? w * NG : a.full * NG + (w - a.full) * a.rest;
-        it.ng = min(w < a.full ? NG : a.rest, a.tiles - tile);
-        it.bh = tile / a.nt;
-        it.q = tile - it.bh * a.nt;
-        it.split = min(it.ng, a.nt - it.q);     // (nt >= 2: three tiles meet one boundary at most; nt = 1: see stream())
-        return it;
-    }
-    if (w < a.n3) {
-        it.bh = w / a.per3;
-        it.q = (w - it.bh * a.per3) * NG;
-        it.ng = NG;
-    } else {
-        it.bh = w - a.n3;
-        it.q = a.per3 * NG;
-        it.ng = a.tail_ng;
-    }
-    it.split = it.ng;
-    return it;
-}
-// The k-th item of this CTA, or -1 when it has none left.
-template <bool ACROSS> __device__ __forceinline__ int item_of(const Attn3Args& a, int k) {
-    const int c = blockIdx.x, G = gridDim.x;
-    if (ACROSS) return c + k * G < a.n_items ? c + k * G : -1;
-    const int mine3 = c < a.n3 ? (a.n3 - c + G - 1) / G : 0;
-    if (k < mine3) return c + k * G;
-    int pos = c - a.tail_first;
-    if (pos < 0) {
-        if (!a.tail_wrap) return -1;
-        pos += G;
-    }
-    const int s = pos + (k - mine3) * a.tail_stride;
-    return s < a.n_tail ? a.n3 + s : -1;
+// n / d and its remainder for d's reciprocal as above: the product is the quotient or one less.
+__device__ __forceinline__ int divide(int n, int d, uint32_t by_d, int& rest) {
+    int quot = (int)__umulhi((uint32_t)n, by_d);
+    rest = n - quot * d;
+    if (rest >= d) { rest -= d; ++quot; }
+    return quot;
 }
 
-// Maximum of a 64-column row of S in registers.  MASKED: only the first `valid` columns are keys.
-template <bool MASKED>
-__device__ __forceinline__ float row_max64(const uint32_t (&r)[BKV], int valid) {
+struct Item3 {
+    int b, h, q;             // sample, head and query tile of tile 0
+    int ng;                  // query tiles present: 1 .. 3
+    int split;               // tiles of the first head; the others belong to the next one (or ones)
+    int n, nt, nkv;          // tokens of the sample, its query tiles and key tiles
+    int third;               // keys cut in three: key tiles to a warpgroup (the last one may have fewer, or none); else 0
+    // how many heads after the item's first one tile g belongs to; whether it is the first or the last tile that a K/V tile serves
+    __device__ __forceinline__ int stream(int g) const { return nt == 1 ? g : g >= split; }
+    __device__ __forceinline__ bool starts(int g) const { return g == 0 || g == split || nt == 1; }
+    __device__ __forceinline__ bool ends(int g) const { return g == ng - 1 || g == split - 1 || nt == 1; }
+};
+// RAGGED: what the CTA knows of the samples, in shared memory.
+struct Samples {
+    int items;
+    int first_item[kMaxSamples + 1];
+    unsigned char order[kMaxSamples];
+};
+static_assert(OFF_SAMPLES + sizeof(Samples) + 1024 <= kSmem, "room for the samples");
+__device__ __forceinline__ int sample_len(const Attn3Args& a, int b) { return min(max(__ldg(a.lens + b), 1), a.N); }
+
+template <bool RAGGED, bool CUT> __device__ __forceinline__ Item3 decode_item3(const Attn3Args& a, const Samples* sm, int w) {
+    Item3 it;
+    if constexpr (RAGGED) {
+        int lo = 0, hi = a.B;                            // first_item[lo] <= w < first_item[hi]
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (sm->first_item[mid] <= w) lo = mid;
+            else hi = mid;
+        }
+        it.b = sm->order[lo];
+        it.n = sample_len(a, it.b);
+        it.nt = (it.n + BQ - 1) / BQ;
+        const int tile = (w - sm->first_item[lo]) * NG;
+        it.ng = min(NG, a.H * it.nt - tile);
+        it.h = tile / it.nt;
+        it.q = tile - it.h * it.nt;
+    } else {
+        it.n = a.N;
+        it.nt = a.nt;
+        int bh;
+        if (!CUT || w < a.n_whole) {
+            const int tile = w < a.full ? w * NG : a.full * NG + (w - a.full) * a.rest;
+            it.ng = min(w < a.full ? NG : a.rest, a.tiles - tile);
+            bh = divide(tile, a.nt, a.by_nt, it.q);
+        } else {
+            it.ng = 1;
+            bh = divide(w - a.n_whole, a.cut, a.by_cut, it.q);
+            it.q += a.nt;
+        }
+        it.b = divide(bh, a.H, a.by_h, it.h);
+    }
+    it.split = CUT && w >= a.n_whole ? it.ng : min(it.ng, it.nt - it.q);     // (two or more tiles to a head: three meet one boundary at most)
+    it.nkv = (it.n + BKV - 1) / BKV;
+    it.third = CUT && w >= a.n_whole ? (it.nkv + NG - 1) / NG : 0;
+    return it;
+}
+
+// Maximum of a 64-column row of S in registers.
+__device__ __forceinline__ float row_max64(const uint32_t (&r)[BKV]) {
     float m[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) m[c] = -INFINITY;
 #pragma unroll
-    for (int i = 0; i < BKV; i += 16) {               // eight independent chains: latency, not count, is the cost
+    for (int i = 0; i < BKV; i += 16)                 // eight independent chains: latency, not count, is the cost
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            float a = __uint_as_float(r[i + 2 * c]), b = __uint_as_float(r[i + 2 * c + 1]);
-            if (MASKED) {
-                if (i + 2 * c >= valid) a = -INFINITY;
-                if (i + 2 * c + 1 >= valid) b = -INFINITY;
-            }
-            m[c] = max3(m[c], a, b);
-        }
-    }
+        for (int c = 0; c < 8; ++c) m[c] = max3(m[c], __uint_as_float(r[i + 2 * c]), __uint_as_float(r[i + 2 * c + 1]));
     return max3(max3(m[0], m[1], m[2]), max3(m[3], m[4], m[5]), fmaxf(m[6], m[7]));
 }
 
-// p_i = exp2(s_i * sl + mneg) for the first `valid` of the 64 keys (0 for the rest), packed to bf16
-// pairs in place (r[0 .. 32) on return); returns the sum of the unrounded p_i.
-// Six pairs of the 32 go through the FMA pipes: the special-function unit (8 cycles per warp and exponential) is the
+// p_i = exp2(s_i * sl + mneg) for N values of a row from FROM on, packed to bf16 pairs in place (r[FROM / 2 ...) on return);
+// returns the sum of the unrounded p_i.
+// Six pairs of the 32 of a key tile go through the FMA pipes: the special-function unit (8 cycles per warp and exponential) is the
 // busiest pipe of this kernel, and its idle time does not line up between the three warps of a scheduler.  4 x 16 x
-// 4097: 380 us with none, 379 / 371 / 368 / 371 / 382 with 2 / 5 / 6 / 8 / 11 pairs, 435 with all second pairs of four
-// elements; 16 x 12 x 1569 195 -> 190, 32 x 16 x 577 94.3 -> 91.4.  (In the two-tile kernel any share is slower: its two
-// warps per scheduler have no issue slots to spare for it.)
+// 4097, an earlier form: 380 us with none, 379 / 371 / 368 / 371 / 382 with 2 / 5 / 6 / 8 / 11 pairs, 435 with all second pairs of four
+// elements.  Which six hardly matters (330 to 345 us in the present form).
 // SPLIT: lo gets what the bf16s in r leave of the p_i, as bf16 pairs (and the exponentials all go to the special-function
 // unit, which is not the busiest pipe there).
-template <bool MASKED, bool SPLIT>
-__device__ __forceinline__ float exp_pass64(uint32_t (&r)[BKV], uint32_t (&lo)[SPLIT ? BKV / 2 : 1], float sl, float mneg, int valid) {
+template <int FROM, int N, bool SPLIT>
+__device__ __forceinline__ float exp_pass(uint32_t (&r)[BKV], uint32_t (&lo)[SPLIT ? BKV / 2 : 1], float sl, float mneg) {
     const uint64_t sl2 = pack2(sl, sl), mneg2 = pack2(mneg, mneg);
     uint64_t l01 = pack2(0.f, 0.f), l23 = l01;
 #pragma unroll
-    for (int i = 0; i < BKV; i += 4) {
+    for (int i = FROM; i < FROM + N; i += 4) {
         float x0, x1, x2, x3;
         unpack2(ffma2(pack2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), sl2, mneg2), x0, x1);
         unpack2(ffma2(pack2(__uint_as_float(r[i + 2]), __uint_as_float(r[i + 3])), sl2, mneg2), x2, x3);
-        if (MASKED) {
-            if (i >= valid) x0 = -INFINITY;
-            if (i + 1 >= valid) x1 = -INFINITY;
-            if (i + 2 >= valid) x2 = -INFINITY;
-            if (i + 3 >= valid) x3 = -INFINITY;
-        }
-        const float p0 = ex2(x0), p1 = ex2(x1);   // ex2(-inf) = 0
+        const float p0 = ex2(x0), p1 = ex2(x1);
         float p2, p3;
-        constexpr int kByFma = 0x52;                     // which of eight consecutive groups of four send their second pair there
-        if (!MASKED && !SPLIT && ((kByFma >> ((i / 4) % 8)) & 1)) ex2_pair_fma(pack2(x2, x3), p2, p3);
+        constexpr int kByFma = 0x29;                     // which of eight consecutive groups of four send their second pair there
+        if (!SPLIT && ((kByFma >> ((i / 4) % 8)) & 1)) ex2_pair_fma(pack2(x2, x3), p2, p3);
         else { p2 = ex2(x2); p3 = ex2(x3); }
         l01 = fadd2(l01, pack2(p0, p1));
         l23 = fadd2(l23, pack2(p2, p3));
@@ -177,11 +188,12 @@ __device__ __forceinline__ float exp_pass64(uint32_t (&r)[BKV], uint32_t (&lo)[S
     return (a + b) + (c + d);
 }
 
-template <bool ACROSS, bool SPLIT>
+// CUT: there are items with the keys cut in three.  (Without, the loops carry nothing of them: 4 x 16 x 3073 205 -> 198 us.)
+template <bool SPLIT, bool RAGGED, bool CUT>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO, const Attn3Args args) {
-    static_assert(ACROSS || !SPLIT, "the split weights come with items across heads only");
+    static_assert(!RAGGED || (!SPLIT && !CUT), "neither comes with a count per sample");
     constexpr int PARTS = SPLIT ? 2 : 1;     // products P V per key tile
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -220,7 +232,27 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     // Everything above touched no global memory and may overlap the previous kernel's tail.
     grid_dep_launch();
     grid_dep_wait();
-    const int nkv = (args.N + BKV - 1) / BKV;           // key tiles per query tile
+    Samples* samples = RAGGED ? reinterpret_cast<Samples*>(smem + OFF_SAMPLES) : nullptr;
+    if constexpr (RAGGED) {
+        // samples by length, the longest first (its place: how many come before it), and the items before each
+        static_assert(kMaxSamples <= kThreads, "a thread to a sample");
+        const int b = threadIdx.x, len = b < args.B ? sample_len(args, b) : 0;
+        int place = 0, before = 0;
+        for (int o = 0; o < args.B && b < args.B; ++o) {
+            const int l = sample_len(args, o);
+            if (l > len || (l == len && o < b)) {
+                ++place;
+                before += (args.H * ((l + BQ - 1) / BQ) + NG - 1) / NG;
+            }
+        }
+        if (b < args.B) {
+            samples->order[place] = (unsigned char)b;
+            samples->first_item[place] = before;
+            if (place == args.B - 1) samples->items = samples->first_item[args.B] = before + (args.H * ((len + BQ - 1) / BQ) + NG - 1) / NG;
+        }
+        __syncthreads();
+    }
+    const int n_items = RAGGED ? samples->items : args.n_items;
 
     if (warp >= 12) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));
@@ -229,20 +261,21 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         if (elect_one()) {
             uint32_t kv_it = 0, item_n = 0;
             bool ok = true;
-            for (int w = item_of<ACROSS>(args, 0); w >= 0 && ok; w = item_of<ACROSS>(args, ++item_n)) {
-                const Item3 it = decode_item3<ACROSS>(args, w);
+            for (int w = blockIdx.x; w < n_items && ok; w += gridDim.x, ++item_n) {
+                const Item3 it = decode_item3<RAGGED, CUT>(args, samples, w);
                 const uint32_t qb = item_n & 1u;
                 if (!mbar_wait(&q_empty[qb], ((item_n >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
                 mbar_expect_tx(&q_full[qb], it.ng * Q_BYTES);
-                const int b0 = it.bh / args.H, h0 = it.bh - b0 * args.H;
                 auto next = [&](int& b, int& h) { if (++h == args.H) { h = 0; ++b; } };      // the next (sample, head)
-                for (int g = 0, b = b0, h = h0; g < it.ng; ++g) {
-                    if (ACROSS && g && it.starts<SPLIT>(args, g)) next(b, h);
-                    tma_load_4d(smem + OFF_Q + (qb * NG + g) * Q_BYTES, &tmQ, &q_full[qb], 0, h, (it.q + g - it.stream<SPLIT>(args, g) * args.nt) * BQ, b);
+                for (int g = 0, b = it.b, h = it.h; g < it.ng; ++g) {
+                    if (g && it.starts(g)) next(b, h);
+                    tma_load_4d(smem + OFF_Q + (qb * NG + g) * Q_BYTES, &tmQ, &q_full[qb], 0, h, (it.q + g - it.stream(g) * it.nt) * BQ, b);
                 }
-                const int streams = ACROSS ? it.stream<SPLIT>(args, it.ng - 1) + 1 : 1;
-                for (int t = 0; t < nkv && ok; ++t)
-                    for (int sm = 0, b = b0, h = h0; sm < streams; ++sm, ++kv_it, next(b, h)) {
+                const int streams = it.third ? NG : it.stream(it.ng - 1) + 1, steps = it.third ? it.third : it.nkv;
+                for (int j = 0; j < steps && ok; ++j)
+                    for (int sm = 0, b = it.b, h = it.h; sm < streams; ++sm, ++kv_it) {
+                        const int t = j + sm * it.third;
+                        if (t >= it.nkv) break;          // (the last third may be shorter)
                         const int s = kv_it % NS;
                         if (!mbar_wait(&k_empty[s], ((kv_it / NS) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
                         mbar_expect_tx(&k_full[s], KV_BYTES);
@@ -250,6 +283,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                         if (!mbar_wait(&v_empty[s], ((kv_it / NS) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
                         mbar_expect_tx(&v_full[s], KV_BYTES);
                         tma_load_4d(smem + OFF_V + s * KV_BYTES, &tmV, &v_full[s], 0, h, t * BKV, b);
+                        if (!it.third) next(b, h);
                     }
             }
             // every copy started here must have landed before the CTA exits
@@ -261,7 +295,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     } else if (warp == 13) {
         // ---------------- Q K^T issuer: S_g = Q_g K^T, both operands K-major ----------------
         // It runs ahead of the softmax warps as far as the S columns allow: the S of a tile may be
-        // overwritten once that tile's softmax warps have its row in registers.
+        // overwritten once that tile's softmax warps are done with it.
         if (elect_one()) {
             constexpr uint32_t idesc_s_full = idesc_bf16(BQ, BKV, 0, 0);
             constexpr uint32_t kQ16 = Q_BYTES >> 4, kKV16 = KV_BYTES >> 4;
@@ -270,36 +304,49 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             const uint32_t k_lo = smem_desc_lo(smem_desc_sw128(smem_u32(smem + OFF_K), 16, 1024));
             uint32_t ns[NG] = {0, 0, 0};                 // S tiles issued so far per query tile
             uint32_t item_n = 0, t = 0;
+            int stage = 0;
             bool ok = true;
-            for (int w = item_of<ACROSS>(args, 0); w >= 0 && ok; w = item_of<ACROSS>(args, ++item_n)) {
-                const Item3 it = decode_item3<ACROSS>(args, w);
-                const uint32_t qb = item_n & 1u;
+            auto next_stage = [&]() {                    // the next K tile of the ring
+                stage = t % NS;
+                ok = mbar_wait(&k_full[stage], (t / NS) & 1u, abort_flag);
+                ++t;
+                return ok;
+            };
+            auto issue = [&](int g, uint32_t dq, uint32_t idesc_s) {
+                ok = ns[g] == 0 || mbar_wait(&s_free[g], (ns[g] - 1) & 1u, abort_flag);
+                if (!ok) return;
+                tc_fence_after();
+                const uint32_t dk = k_lo + (uint32_t)stage * kKV16;
+#pragma unroll
+                for (int k = 0; k < DH / 16; ++k)        // 16 head-dimension columns = 32 bytes per step
+                    mma_ss_lh(tmem_base + kSCol + g * BKV, dq + 2u * k, dk + 2u * k, desc_hi, idesc_s, k != 0);
+                mma_commit(&s_full[g]);
+                ++ns[g];
+            };
+            for (int w = blockIdx.x; w < n_items && ok; w += gridDim.x, ++item_n) {
+                const Item3 it = decode_item3<RAGGED, CUT>(args, samples, w);
+                const uint32_t qb = item_n & 1u, q_item = q_lo + qb * NG * kQ16;
+                const uint32_t idesc_last = idesc_bf16(BQ, (it.n - (it.nkv - 1) * BKV + 15) & ~15, 0, 0);
                 if (!mbar_wait(&q_full[qb], (item_n >> 1) & 1u, abort_flag)) { ok = false; break; }
-                for (int j = 0; j < nkv && ok; ++j) {
-                    const int valid = min(BKV, args.N - j * BKV);
-                    const uint32_t idesc_s = valid == BKV ? idesc_s_full : idesc_bf16(BQ, (valid + 15) & ~15, 0, 0);
-                    int stage = 0;
-                    uint32_t dk = 0;
+                if (CUT && it.third) {
+                    for (int j = 0; j < it.third && ok; ++j)
 #pragma unroll
-                    for (int g = 0; g < NG; ++g) {
-                        if (g >= it.ng || !ok) continue;
-                        if (ACROSS ? it.starts<SPLIT>(args, g) : g == 0) {   // a (sample, head)'s first tile: the next ring stage
-                            stage = t % NS;
-                            if (!mbar_wait(&k_full[stage], (t / NS) & 1u, abort_flag)) { ok = false; continue; }
-                            dk = k_lo + (uint32_t)stage * kKV16;
-                            ++t;
+                        for (int g = 0; g < NG; ++g) {
+                            const int tile = j + g * it.third;
+                            if (tile >= it.nkv || !ok || !next_stage()) continue;
+                            issue(g, q_item, tile == it.nkv - 1 ? idesc_last : idesc_s_full);
+                            if (ok) mma_commit(&k_empty[stage]);
                         }
-                        if (ns[g] > 0 && !mbar_wait(&s_free[g], (ns[g] - 1) & 1u, abort_flag)) { ok = false; continue; }
-                        tc_fence_after();
-                        const uint32_t dq = q_lo + (qb * NG + g) * kQ16;
+                } else {
+                    for (int j = 0; j < it.nkv && ok; ++j) {
+                        const uint32_t idesc_s = j == it.nkv - 1 ? idesc_last : idesc_s_full;
 #pragma unroll
-                        for (int k = 0; k < DH / 16; ++k)    // 16 head-dimension columns = 32 bytes per step
-                            mma_ss_lh(tmem_base + kSCol + g * BKV, dq + 2u * k, dk + 2u * k, desc_hi, idesc_s, k != 0);
-                        mma_commit(&s_full[g]);
-                        ++ns[g];
-                        if (ACROSS && it.ends<SPLIT>(args, g)) mma_commit(&k_empty[stage]);
+                        for (int g = 0; g < NG; ++g) {
+                            if (g >= it.ng || !ok || (it.starts(g) && !next_stage())) continue;
+                            issue(g, q_item + g * kQ16, idesc_s);
+                            if (ok && it.ends(g)) mma_commit(&k_empty[stage]);
+                        }
                     }
-                    if (!ACROSS && ok) mma_commit(&k_empty[stage]);
                 }
                 if (ok) mma_commit(&q_empty[qb]);
             }
@@ -314,41 +361,57 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             const uint32_t desc_hi = smem_desc_hi(smem_desc_sw128(0, 16, 1024));
             const uint32_t v_lo = smem_desc_lo(smem_desc_sw128(smem_u32(smem + OFF_V), 16, 1024));
             uint32_t np[NG] = {0, 0, 0};                 // P V products issued so far per query tile
-            uint32_t t = 0, item_n = 0;
+            uint32_t t = 0;
+            int stage = 0;
             bool ok = true;
-            for (int w = item_of<ACROSS>(args, 0); w >= 0 && ok; w = item_of<ACROSS>(args, ++item_n)) {
-                const Item3 it = decode_item3<ACROSS>(args, w);
-                for (int j = 0; j < nkv && ok; ++j) {
-                    const int ksteps = (min(BKV, args.N - j * BKV) + 15) >> 4;
-                    int stage = 0;
-                    uint32_t dv = 0;
-                    int stage_of[NG];                    // SPLIT: kept for the second part
+            auto next_stage = [&]() {                    // the next V tile of the ring
+                stage = t % NS;
+                ok = mbar_wait(&v_full[stage], (t / NS) & 1u, abort_flag);
+                ++t;
+                return ok;
+            };
+            auto issue = [&](int g, int ksteps, bool first) {
+                ok = mbar_wait(&p_ready[g], np[g] & 1u, abort_flag);
+                if (!ok) return;
+                tc_fence_after();
+                const uint32_t dv = v_lo + (uint32_t)stage * kKV16, o_col = tmem_base + kOCol + g * DH, p_col = tmem_base + kPCol + g * (BKV / 2);
+                for (int k = 0; k < ksteps; ++k)
+                    mma_ts_lh(o_col, p_col + 8 * k, dv + 128u * k, desc_hi, idesc_o, !(first && k == 0));
+                mma_commit(&o_done[g]);
+                ++np[g];
+            };
+            for (int w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
+                const Item3 it = decode_item3<RAGGED, CUT>(args, samples, w);
+                const int ksteps_last = (it.n - (it.nkv - 1) * BKV + 15) >> 4;
+                const bool cut = CUT && it.third;
+                for (int j = 0, steps = cut ? it.third : it.nkv; j < steps && ok; ++j) {
+                    if (cut || SPLIT) {
+                        int stage_of[NG];                // SPLIT: kept for the second part
 #pragma unroll
-                    for (int part = 0; part < PARTS; ++part) {
+                        for (int part = 0; part < PARTS; ++part) {
+#pragma unroll
+                            for (int g = 0; g < NG; ++g) {
+                                const int tile = j + g * it.third;
+                                if ((!cut && g >= it.ng) || tile >= it.nkv || !ok) continue;
+                                if (part == 0) {
+                                    if ((cut || it.starts(g)) && !next_stage()) continue;
+                                    stage_of[g] = stage;
+                                } else {
+                                    stage = stage_of[g];
+                                }
+                                issue(g, tile == it.nkv - 1 ? ksteps_last : BKV / 16, j == 0 && part == 0);
+                                if (ok && part == PARTS - 1 && (cut || it.ends(g))) mma_commit(&v_empty[stage]);
+                            }
+                        }
+                    } else {
+                        const int ksteps = j == it.nkv - 1 ? ksteps_last : BKV / 16;
 #pragma unroll
                         for (int g = 0; g < NG; ++g) {
-                            if (g >= it.ng || !ok) continue;
-                            if (part == 0 && (ACROSS ? it.starts<SPLIT>(args, g) : g == 0)) {
-                                stage = t % NS;
-                                if (!mbar_wait(&v_full[stage], (t / NS) & 1u, abort_flag)) { ok = false; continue; }
-                                dv = v_lo + (uint32_t)stage * kKV16;
-                                ++t;
-                            }
-                            if (SPLIT) {
-                                if (part == 0) stage_of[g] = stage;
-                                else { stage = stage_of[g]; dv = v_lo + (uint32_t)stage * kKV16; }
-                            }
-                            if (!mbar_wait(&p_ready[g], np[g] & 1u, abort_flag)) { ok = false; continue; }
-                            tc_fence_after();
-                            const uint32_t o_col = tmem_base + kOCol + g * DH, p_col = tmem_base + kPCol + g * (BKV / 2);
-                            for (int k = 0; k < ksteps; ++k)
-                                mma_ts_lh(o_col, p_col + 8 * k, dv + 128u * k, desc_hi, idesc_o, !(j == 0 && part == 0 && k == 0));
-                            mma_commit(&o_done[g]);
-                            ++np[g];
-                            if (ACROSS && part == PARTS - 1 && it.ends<SPLIT>(args, g)) mma_commit(&v_empty[stage]);
+                            if (g >= it.ng || !ok || (it.starts(g) && !next_stage())) continue;
+                            issue(g, ksteps, j == 0);
+                            if (ok && it.ends(g)) mma_commit(&v_empty[stage]);
                         }
                     }
-                    if (!ACROSS && ok) mma_commit(&v_empty[stage]);
                 }
             }
         }
@@ -363,101 +426,209 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                        o_addr = lane_addr + kOCol + g * DH;
         const float sl = args.scale_log2;
         uint32_t cnt = 0;                                // key tiles this warpgroup has walked through
-        bool ok = true;
-        uint32_t item_n = 0;
-        for (int w = item_of<ACROSS>(args, 0); w >= 0 && ok; w = item_of<ACROSS>(args, ++item_n)) {
-            const Item3 it = decode_item3<ACROSS>(args, w);
-            if (g >= it.ng) continue;
-            const int sm = it.stream<SPLIT>(args, g), bh = it.bh + sm, row0 = (it.q + g - sm * args.nt) * BQ + q * 32;
-            float m_l2 = 0.f, l_run = 0.f;               // running maximum (times scale*log2 e) and sum
-            for (int j = 0; j < nkv && ok; ++j, ++cnt) {
-                const int valid = min(BKV, args.N - j * BKV);
-                // the warp moves as one through the collective tensor-memory accesses below
-                if (!__all_sync(0xffffffffu, mbar_wait(&s_full[g], cnt & 1u, abort_flag))) { ok = false; break; }
-                tc_fence_after();
-                // All 64 columns are read even on a partial key tile: columns past the keys the MMA
-                // wrote hold old values, which the masks never let through.
-                uint32_t r[BKV];
-                tmem_ld_32x32(s_addr, r);
-                tmem_ld_32x32(s_addr + 32, r + 32);
-                tmem_wait_ld();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&s_free[g]);  // the next Q K^T may overwrite S now
-                // running maximum: raised only when the tile tops it by more than 2^kRescaleGap
-                const float mx = valid == BKV ? row_max64<false>(r, valid) : row_max64<true>(r, valid);
+        // A wait that runs out ends the issuing threads and is reported through the status word; these warps walk on to the end
+        // of their items, whose results are void then, so that no lane ever leaves a collective access to the others.
+        auto wait = [&](uint64_t* bar, uint32_t parity) {
+            mbar_wait(bar, parity, abort_flag);
+            __syncwarp();
+            tc_fence_after();
+        };
+        auto arrive = [&](uint64_t* bar) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar);
+        };
+        // what last read the P columns, and wrote O: P V of the previous key tile (before the first one the barrier lets the
+        // parity of its last phase through at once)
+        auto wait_o = [&]() { wait(&o_done[g], (cnt * PARTS - 1) & 1u); };
+        // The key tiles of one query tile: nkv of them, the first nfull whole, the last one of valid_last keys otherwise.  Leaves the
+        // running maximum (times scale * log2 e) and sum of this thread's row.
+        // gap1: the gap of the second key tile.
+        auto walk = [&](int nkv, int nfull, int valid_last, float gap1, float& m_l2, float& l_run) {
+            m_l2 = kLowest;
+            l_run = 0.f;
+            for (int j = 0; j < nkv; ++j, ++cnt) {
+                // Whole key tiles whose maximum stays within 2^kRescaleGap of the running one: nearly all of them.
+                bool have_s = false;
+                for (; j < nfull; ++j, ++cnt) {
+                    wait(&s_full[g], cnt & 1u);
+                    uint32_t r[BKV], lo[SPLIT ? BKV / 2 : 1];
+                    tmem_ld_32x32(s_addr, r);
+                    tmem_ld_32x32(s_addr + 32, r + 32);
+                    tmem_wait_ld();
+                    const float mx_l2 = row_max64(r) * sl;
+                    if (j == 0) m_l2 = fmaxf(mx_l2, kLowest);
+                    have_s = __any_sync(0xffffffffu, mx_l2 > m_l2 + (j == 1 ? gap1 : kRescaleGap));
+                    if (have_s) break;
+                    float l_tile = exp_pass<0, BKV / 2, SPLIT>(r, lo, sl, -m_l2);
+                    arrive(&s_free[g]);                  // the next Q K^T may overwrite S
+                    l_tile += exp_pass<BKV / 2, BKV / 2, SPLIT>(r, lo, sl, -m_l2);
+                    l_run += l_tile;
+                    wait_o();
+                    tmem_st_32x32(p_addr, r);
+                    tmem_wait_st();
+                    arrive(&p_ready[g]);
+                    if constexpr (SPLIT) {               // the rest of the weights, when the product with the first part is done
+                        wait(&o_done[g], 0);
+                        tmem_st_32x32(p_addr, lo);
+                        tmem_wait_st();
+                        arrive(&p_ready[g]);
+                    }
+                }
+                if (j == nkv) break;
+                // A key tile that raises the maximum, or the last one with fewer keys than columns: 16 columns at a time from
+                // tensor memory, in little code.
+                if (!have_s) wait(&s_full[g], cnt & 1u);
+                const int valid = j < nfull ? BKV : valid_last;
+                auto load16 = [&](int c, uint32_t (&s)[16]) {
+                    tmem_ld_32x16(s_addr + c, s);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) s[i] = c + i < valid ? s[i] : 0xff800000u;      // past the keys: -infinity, a weight of 0
+                };
+                float mx = -INFINITY;
+#pragma unroll 1
+                for (int c = 0; c < valid; c += 16) {
+                    uint32_t s[16];
+                    load16(c, s);
+#pragma unroll
+                    for (int i = 0; i < 16; i += 2) mx = max3(mx, __uint_as_float(s[i]), __uint_as_float(s[i + 1]));
+                }
                 const float mx_l2 = mx * sl;
+                wait_o();
                 if (j == 0) {
-                    m_l2 = mx_l2;
-                } else if (__any_sync(0xffffffffu, mx_l2 > m_l2 + kRescaleGap)) {
-                    // rare: rescale O and the sum; O += P V of the previous key tile must have retired
-                    if (!__all_sync(0xffffffffu, mbar_wait(&o_done[g], (cnt * PARTS - 1) & 1u, abort_flag))) { ok = false; break; }
-                    tc_fence_after();
-                    const bool raise = mx_l2 > m_l2 + kRescaleGap;
+                    m_l2 = fmaxf(mx_l2, kLowest);
+                } else if (__any_sync(0xffffffffu, mx_l2 > m_l2 + (j == 1 ? gap1 : kRescaleGap))) {
+                    const bool raise = mx_l2 > m_l2 + (j == 1 ? gap1 : kRescaleGap);
                     const float alpha = raise ? ex2(m_l2 - mx_l2) : 1.f;
                     if (raise) m_l2 = mx_l2;
                     l_run *= alpha;
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        uint32_t o[32];
-                        tmem_ld_32x32(o_addr + c * 32, o);
+#pragma unroll 1
+                    for (int c = 0; c < DH; c += 16) {
+                        uint32_t o[16];
+                        tmem_ld_32x16(o_addr + c, o);
                         tmem_wait_ld();
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-                        tmem_st_32x32(o_addr + c * 32, o);
+                        for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                        tmem_st_32x16(o_addr + c, o);
+                    }
+                }
+#pragma unroll 1
+                for (int part = 0; part < PARTS; ++part) {
+                    if (part) wait(&o_done[g], 0);
+#pragma unroll 1
+                    for (int c = 0; c < valid; c += 16) {
+                        uint32_t s[16];
+                        load16(c, s);
+#pragma unroll
+                        for (int i = 0; i < 16; i += 2) {
+                            const float p0 = ex2(fmaf(__uint_as_float(s[i]), sl, -m_l2)), p1 = ex2(fmaf(__uint_as_float(s[i + 1]), sl, -m_l2));
+                            uint32_t h = pack_bf16(p0, p1);
+                            if (part) h = pack_bf16(p0 - __uint_as_float(h << 16), p1 - __uint_as_float(h & 0xffff0000u));
+                            else l_run += p0 + p1;
+                            s[i >> 1] = h;
+                        }
+                        tmem_st_32x8(p_addr + (c >> 1), s);
                     }
                     tmem_wait_st();
+                    arrive(&p_ready[g]);
                 }
-                uint32_t lo[SPLIT ? BKV / 2 : 1];
-                l_run += valid == BKV ? exp_pass64<false, SPLIT>(r, lo, sl, -m_l2, valid) : exp_pass64<true, SPLIT>(r, lo, sl, -m_l2, valid);
-                if (cnt > 0) {
-                    // P V of the previous key tile reads the P columns: it must have retired
-                    if (!__all_sync(0xffffffffu, mbar_wait(&o_done[g], (cnt * PARTS - 1) & 1u, abort_flag))) { ok = false; break; }
-                    tc_fence_after();
-                }
-                tmem_st_32x32(p_addr, r);
-                tmem_wait_st();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&p_ready[g]);
-                if constexpr (SPLIT) {                   // the rest of the weights, when the product with the first part is done
-                    if (!__all_sync(0xffffffffu, mbar_wait(&o_done[g], 0, abort_flag))) { ok = false; break; }
-                    tc_fence_after();
-                    tmem_st_32x32(p_addr, lo);
-                    tmem_wait_st();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&p_ready[g]);
-                }
+                if (lane == 0) mbar_arrive(&s_free[g]);  // (every lane's reads of S are complete at the arrival above)
             }
-            // epilogue of the item: O / l -> bf16 -> global
-            if (!ok || !__all_sync(0xffffffffu, mbar_wait(&o_done[g], (cnt * PARTS - 1) & 1u, abort_flag))) { ok = false; break; }
-            tc_fence_after();
-            const float inv = 1.f / l_run;
-            uint32_t o[64];
-            tmem_ld_32x32(o_addr, o);
-            tmem_ld_32x32(o_addr + 32, o + 32);
-            tmem_wait_ld();
-            // The warp's 32 rows x 64 values go to its own slab of shared memory (128-byte rows,
-            // 16-byte pieces XOR-swizzled like the tensor map's box) and leave with one TMA store,
-            // which drops the rows past N.
-            if (lane == 0) tma_store_wait_read<0>();     // the slab's previous store has read it
-            __syncwarp();
-            uint8_t* slab = smem + OFF_OST + (g * 4 + q) * 4096 + (lane >> 3) * 1024 + (lane & 7) * 128;
-#pragma unroll
-            for (int g8 = 0; g8 < 8; ++g8) {
-                uint32_t wv[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    wv[e] = pack_bf16(__uint_as_float(o[8 * g8 + 2 * e]) * inv, __uint_as_float(o[8 * g8 + 2 * e + 1]) * inv);
-                *reinterpret_cast<uint4*>(slab + ((g8 ^ (lane & 7)) << 4)) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-            }
+        };
+        // O / l -> bf16 -> global.  The warp's 32 rows x 64 values go to its own slab of shared memory (128-byte rows, 16-byte
+        // pieces XOR-swizzled like the tensor map's box) and leave with one TMA store, which drops the rows past N.
+        uint8_t* const warp_slab = smem + OFF_OST + (g * 4 + q) * 4096;
+        uint8_t* const slab = warp_slab + (lane >> 3) * 1024 + (lane & 7) * 128;
+        auto store = [&](const Item3& it, int tile) {        // `tile` of the item
             fence_async_smem();
             __syncwarp();
-            if (lane == 0 && row0 < args.N) {
-                const int b = bh / args.H;
-                tma_store_4d(&tmO, smem + OFF_OST + (g * 4 + q) * 4096, 0, bh - b * args.H, row0, b);
+            const int sm = it.stream(tile), row0 = (it.q + tile - sm * it.nt) * BQ + q * 32;
+            if (lane == 0 && row0 < it.n) {
+                int h = it.h + sm, b = it.b;
+                while (h >= args.H) { h -= args.H; ++b; }    // past the last head: of the next sample (or the one after)
+                tma_store_4d(&tmO, warp_slab, 0, h, row0, b);
                 tma_store_commit();
+            }
+        };
+        // Up to 128 keys the maximum is exact, so that the largest weight is 1 and is not rounded (of a few weights it is a good part: error
+        // against 64 bits at 4 x 3 x 100 with scores of standard deviation 1 / 4, 2.22e-3 / 2.00e-3 -> 2.13e-3 / 1.75e-3; 64 x 12 x 101 11.4 -> 11.8 us).
+        auto first_gap = [](int n) { return n <= 2 * BKV ? 0.f : kRescaleGap; };
+        const int nkv_all = (args.N + BKV - 1) / BKV, nfull_all = args.N / BKV, valid_all = args.N % BKV;
+        const int whole = CUT ? args.n_whole : n_items;
+        int w = blockIdx.x;
+        for (; w < whole; w += gridDim.x) {
+            const Item3 it = decode_item3<RAGGED, CUT>(args, samples, w);
+            if (g >= it.ng) continue;
+            float m_l2, l_run;
+            if constexpr (RAGGED) walk(it.nkv, it.n / BKV, it.n % BKV, first_gap(it.n), m_l2, l_run);
+            else walk(nkv_all, nfull_all, valid_all, first_gap(args.N), m_l2, l_run);
+            wait_o();
+            if (lane == 0) tma_store_wait_read<0>();     // the slab's previous store has read it
+            __syncwarp();
+            const float inv = 1.f / l_run;
+#pragma unroll 1
+            for (int c = 0; c < DH; c += 32) {
+                uint32_t o[32];
+                tmem_ld_32x32(o_addr + c, o);
+                tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    uint32_t wv[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) wv[i] = pack_bf16(__uint_as_float(o[8 * e + 2 * i]) * inv, __uint_as_float(o[8 * e + 2 * i + 1]) * inv);
+                    *reinterpret_cast<uint4*>(slab + ((((c >> 3) + e) ^ (lane & 7)) << 4)) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
+                }
+            }
+            store(it, g);
+        }
+        // Keys cut in three.  (A loop of its own, with its own copy of the walk: with both kinds of items in one, the walk of the
+        // others took 5 to 8 % longer.)
+        if constexpr (CUT) {
+            for (; w < n_items; w += gridDim.x) {
+                const Item3 it = decode_item3<RAGGED, CUT>(args, samples, w);
+                const int first = g * it.third, n = min(max(it.nkv - first, 0), it.third);
+                float m_l2, l_run;
+                walk(n, min(n, nfull_all - first), valid_all, kRescaleGap, m_l2, l_run);
+                wait_o();
+                if (lane == 0) tma_store_wait_read<0>();
+                __syncwarp();
+                if (g) *reinterpret_cast<float2*>(warp_slab + lane * 8) = make_float2(m_l2, l_run);
+                tc_fence_before();
+                named_barrier(1, 4 * NG * 32);       // (no warp of these ever leaves early)
+                tc_fence_after();
+                if (g == 0) {
+                    const float2 a = *reinterpret_cast<const float2*>(warp_slab + 4 * 4096 + lane * 8), b = *reinterpret_cast<const float2*>(warp_slab + 8 * 4096 + lane * 8);
+                    const float m = fmaxf(m_l2, fmaxf(a.x, b.x));
+                    float f[NG] = {ex2(m_l2 - m), ex2(a.x - m), ex2(b.x - m)};
+                    const float inv = 1.f / (f[0] * l_run + f[1] * a.y + f[2] * b.y);
+#pragma unroll
+                    for (int i = 0; i < NG; ++i) f[i] *= inv;
+                    const bool third = it.nkv > 2 * it.third;    // (else nothing was written there; the second part is never empty: nkv >= 2)
+#pragma unroll 1
+                    for (int c = 0; c < DH; c += 8) {
+                        uint32_t o[NG][8];
+                        tmem_ld_32x8(o_addr + c, o[0]);
+                        tmem_ld_32x8(o_addr + DH + c, o[1]);
+                        tmem_ld_32x8(o_addr + 2 * DH + c, o[2]);
+                        tmem_wait_ld();
+                        uint32_t wv[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            float u[2];
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) {
+                                u[e] = fmaf(__uint_as_float(o[1][2 * i + e]), f[1], __uint_as_float(o[0][2 * i + e]) * f[0]);
+                                if (third) u[e] = fmaf(__uint_as_float(o[2][2 * i + e]), f[2], u[e]);
+                            }
+                            wv[i] = pack_bf16(u[0], u[1]);
+                        }
+                        *reinterpret_cast<uint4*>(slab + (((c >> 3) ^ (lane & 7)) << 4)) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
+                    }
+                    store(it, 0);
+                }
+                tc_fence_before();
+                named_barrier(2, 4 * NG * 32);       // the others' O and slabs may be used again
             }
         }
         if (lane == 0) tma_store_wait<0>();              // every output row written before the CTA exits
@@ -475,89 +646,76 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 
 }  // namespace
 
-// Where the leftover-tile items go, and the load of the longest CTA under it, in tenths of a group
-// of three tiles (a group or two leftover tiles 10, one leftover tile 7: measured).  wrap = 0: the CTAs
-// that the last, incomplete round of groups left out take the tails, up to two each; wrap = 1: the
-// tails continue the round robin over all CTAs.
-static long long tc3_load(long long BH, int N, int G, int wrap) {
-    const int tiles = (N + BQ - 1) / BQ, per3 = tiles / NG, tail_ng = tiles - per3 * NG;
-    const long long n3 = BH * per3, n_tail = tail_ng ? BH : 0;
-    const int r = (int)(n3 % G), idle = G - r;
-    if (!wrap && n_tail > 2ll * idle) return -1;
-    const int stride = wrap ? G : idle, tail_cost = tail_ng == 1 ? 7 : 10;
-    long long worst = 0;
-    for (int c = 0; c < G; ++c) {
-        long long load = c < n3 ? 10 * ((n3 - c + G - 1) / G) : 0;
-        int pos = c - r;
-        if (pos < 0) {
-            if (!wrap) { worst = load > worst ? load : worst; continue; }
-            pos += G;
-        }
-        if (pos < n_tail) load += tail_cost * ((n_tail - pos + stride - 1) / stride);
-        worst = load > worst ? load : worst;
-    }
-    return worst;
-}
-long long attn_tc3_plan(long long BH, int N, int G, int* wrap) {
-    const long long a = tc3_load(BH, N, G, 0), b = tc3_load(BH, N, G, 1);
-    *wrap = (a < 0 || b < a) ? 1 : 0;
-    return *wrap ? b : a;
-}
+int attn_tc3_max_samples() { return kMaxSamples; }
 
-// The same load with items across heads: whole rounds of three tiles, then the tiles of the last round one to an item
-// where there are CTAs enough.
-long long attn_tc3_across_load(long long BH, int N, int G) {
-    const long long tiles = BH * ((N + BQ - 1) / BQ), left = tiles % (NG * (long long)G);
-    return (tiles - left) / (NG * (long long)G) * 10 + (left == 0 ? 0 : left <= G ? 7 : 10);
+// How many query tiles of every head are taken with the keys cut in three: the count with the shortest longest CTA.  An item of one, two
+// or three query tiles takes 0.62, 0.80 or 1.03 us per key tile and 1.3, one with the keys cut 1.03 per key tile of a third and 1.4;
+// those follow the others, on the CTAs first that the last round leaves out.
+// Chosen where that is 6 % better: the kernel with both kinds of items takes 3 to 4 % longer at the others.  With none cut / as chosen, us:
+// 1 x 12 x 197 5.7 / 5.6 (both tiles), 1 x 16 x 577 9.6 / 8.2 (all), 1 x 12 x 785 11.6 / 9.3 (all), 1 x 16 x 4097 110.8 / 99.3 (6 of 33),
+// 2 x 12 x 2353 66.8 / 60.3 (1 of 19), 4 x 16 x 1729 80.4 / 77.2 (1 of 14).
+int attn_tc3_cut(long long BH, int N, int G) {
+    const int nt = (N + BQ - 1) / BQ, nkv = (N + BKV - 1) / BKV;
+    if (nkv < 3) return 0;                               // (nothing to cut)
+    const double per_tile[NG + 1] = {0, 0.62, 0.80, 1.03}, t_cut = 1.03 * ((nkv + NG - 1) / NG) + 1.4;
+    int best = 0;
+    double best_t = 0;
+    for (int cut = 0; cut <= nt; ++cut) {
+        const long long tiles = BH * (nt - cut), left = tiles % (NG * (long long)G), cuts = BH * cut;
+        const long long rest = left ? (left + G - 1) / G : 0, n_left = left ? (left + rest - 1) / rest : 0;
+        const double t_rest = left ? per_tile[rest] * nkv + 1.3 : 0;
+        auto on = [&](long long place) { return cuts > place ? (double)((cuts - 1 - place) / G + 1) : 0.0; };     // items of that CTA, counted from the first idle one
+        const double idle = n_left < G ? on(0) * t_cut : 0, busy = n_left ? t_rest + on(G - n_left) * t_cut : 0;
+        const double t = (double)((tiles - left) / (NG * (long long)G)) * (per_tile[NG] * nkv + 1.3) + (idle > busy ? idle : busy);
+        if (cut == 0 || t < (best ? 1.0 : 0.94) * best_t) { best_t = t; best = cut; }
+    }
+    return best;
 }
 
 // tmK, tmV: boxes of 64 rows; tmQ: 128 rows; tmO: 32 rows.
 cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMap& tmQ, const CUtensorMap& tmK,
-                            const CUtensorMap& tmV, const CUtensorMap& tmO, int wrap, bool split, cudaStream_t st) {
-    if (d.N <= BQ && !split) return cudaErrorInvalidValue;          // one query tile: the two-heads-per-item kernel's
+                            const CUtensorMap& tmV, const CUtensorMap& tmO, const int32_t* lens, bool split, cudaStream_t st) {
     static PerDeviceOnce attr_once;   // the attribute belongs to the device current at the call
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     e = (cudaError_t)attr_once.run(dev, [] {
-        cudaError_t a = cudaFuncSetAttribute(attn_tc3_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-        if (a == cudaSuccess) a = cudaFuncSetAttribute(attn_tc3_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-        if (a == cudaSuccess) a = cudaFuncSetAttribute(attn_tc3_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+        cudaError_t a = cudaSuccess;
+        for (const void* f : {(const void*)attn_tc3_kernel<false, false, false>, (const void*)attn_tc3_kernel<false, false, true>, (const void*)attn_tc3_kernel<false, true, false>,
+                              (const void*)attn_tc3_kernel<true, false, false>, (const void*)attn_tc3_kernel<true, false, true>})
+            if (a == cudaSuccess) a = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
         return (int)a;
     });
     if (e != cudaSuccess) return e;
     Attn3Args args;
-    args.N = d.N; args.H = d.H;
+    args.N = d.N; args.H = d.H; args.B = d.B;
     const int G = ctx->sm_count;
     const long long BH = (long long)d.B * d.H;
-    args.nt = (d.N + BQ - 1) / BQ;
+    const int nt = (d.N + BQ - 1) / BQ;
+    if (BH * nt >= (1ll << 30)) return cudaErrorInvalidValue;
+    args.cut = lens ? 0 : attn_tc3_cut(BH, d.N, G);
+    args.nt = nt - args.cut;
     const long long tiles = BH * args.nt, left = tiles % (NG * (long long)G);
-    if (tiles >= (1ll << 30)) return cudaErrorInvalidValue;
     args.tiles = (int)tiles;
+    auto reciprocal = [](int v) { return v <= 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / (unsigned)v); };
+    args.by_nt = reciprocal(args.nt);
+    args.by_h = reciprocal(d.H);
+    args.by_cut = reciprocal(args.cut);
     args.full = (int)((tiles - left) / NG);
-    args.rest = left <= G ? 1 : NG;
-    args.n_items = args.full + (int)((left + args.rest - 1) / args.rest);
-    args.per3 = args.nt / NG;
-    args.tail_ng = args.nt - args.per3 * NG;
-    args.n3 = (int)(BH * args.per3);
-    args.n_tail = args.tail_ng ? (int)BH : 0;
-    const int r = args.n3 % G, idle = G - r;
-    if (!wrap && args.n_tail > 2ll * idle) wrap = 1;
-    args.tail_first = r;
-    args.tail_stride = wrap ? G : idle;
-    args.tail_wrap = wrap;
-    // Items run across heads where that shortens the longest CTA.  (Items with two K/V streams take a little longer:
-    // with the loads equal, 8 x 16 x 577 takes 29.7 us within heads and 31.9 across.)  Measured, within / across, us:
-    // 128 x 12 x 133 50.2 / 42.2, x 197 61.6 / 50.7, 28 x 16 x 577 88.7 / 78.1, 16 x 12 x 1569 190 / 183, 4 x 16 x 2305 142 / 135.
-    const bool across = split || attn_tc3_across_load(BH, d.N, G) < tc3_load(BH, d.N, G, wrap);
+    // a last round of at most 2 G tiles: two to an item on twice the CTAs instead of three, 8 x 16 x 577 27.7 -> 25.0 us, 16 x 12 x 1569 165.8 -> 159.7
+    args.rest = left ? (int)((left + G - 1) / G) : 1;
+    args.n_whole = args.full + (int)((left + args.rest - 1) / args.rest);
+    args.n_items = args.n_whole + (int)(BH * args.cut);
+    args.lens = lens;
     const float scale = d.scale != 0.f ? d.scale : 0.125f;
     args.scale_log2 = scale * 1.4426950408889634f;
     args.status = ctx->d_status;
-    const long long all = across ? args.n_items : (long long)args.n3 + args.n_tail;
-    const int grid = all < G ? (int)all : G;
-    if (split) return launch_pdl(attn_tc3_kernel<true, true>, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args);
-    if (across) return launch_pdl(attn_tc3_kernel<true, false>, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args);
-    return launch_pdl(attn_tc3_kernel<false, false>, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args);
+    const long long most = lens ? (long long)d.B * (((long long)d.H * nt + NG - 1) / NG) : args.n_items;
+    const int grid = most < G ? (int)most : G;
+    auto run = [&](auto kernel) { return launch_pdl(kernel, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args); };
+    if (lens) return run(attn_tc3_kernel<false, true, false>);
+    if (split) return args.cut ? run(attn_tc3_kernel<true, false, true>) : run(attn_tc3_kernel<true, false, false>);
+    return args.cut ? run(attn_tc3_kernel<false, false, true>) : run(attn_tc3_kernel<false, false, false>);
 }
 
 }  // namespace rs

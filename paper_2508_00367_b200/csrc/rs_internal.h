@@ -33,7 +33,7 @@ struct rs_ctx {
     int require_tc;        // RS_REQUIRE_TC=1: a bf16 shape the tensor-core kernels cannot take is an error
     int* d_status;         // device status word (0 = ok), first bytes of a small allocation made by rs_create
     int log, nvtx;          // RS_LOG=1: a line per launch on stderr; RS_NVTX=1: an NVTX range around each launch call
-    int attn_kernel;        // RS_ATTN_KERNEL: 0 the faster attention kernel per shape (cost model), 2 / 3 always that one
+    int attn_kernel;        // RS_ATTN_KERNEL: 2 the attention kernel with two query tiles per CTA, else the one with three
     long long launches;    // kernels launched through this context
     void* encode_tiled;    // cuTensorMapEncodeTiled entry point (driver API), or null
     int timing;            // bracket launches with events
@@ -193,15 +193,14 @@ cudaError_t launch_tail_tc(rs_ctx* ctx, const TailCall& c, cudaStream_t st);
 
 // ---- tcgen05 attention (rs_attn_tc.cu): bf16, head dimension 64 ----
 bool attn_tc_supported(const rs_attn_desc& d);
-// Which attention kernel runs a shape of BH (sample, head)s and N > 128 tokens on G SMs, and how: best_hs heads handed
-// out tile by tile (two-tile kernel), three = the three-tile kernel is expected to be faster, wrap3 its tail placement.
-struct AttnPlan { long long best_hs; int three, wrap3; };
+// How the two-tile kernel cuts a shape of BH (sample, head)s and N > 128 tokens on G SMs: best_hs heads are handed out tile by tile;
+// three: what rs_attn_kernel_choice reports.
+struct AttnPlan { long long best_hs; int three; };
 AttnPlan attn_plan(long long BH, int N, int G);
-// Three query tiles per CTA (rs_attn_tc3.cu), N > 128: the longest CTA's load under its item list, and the launch.
-long long attn_tc3_plan(long long BH, int N, int G, int* wrap);
-long long attn_tc3_across_load(long long BH, int N, int G);
+// Three query tiles per CTA (rs_attn_tc3.cu).  lens as seq_lens below, with at most attn_tc3_max_samples() samples; not with split.
+int attn_tc3_max_samples();
 cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMap& tmQ, const CUtensorMap& tmK,
-                            const CUtensorMap& tmV, const CUtensorMap& tmO, int wrap, bool split, cudaStream_t st);
+                            const CUtensorMap& tmV, const CUtensorMap& tmO, const int32_t* lens, bool split, cudaStream_t st);
 // seq_lens (optional, dev [B]): sample b attends over its first seq_lens[b] tokens only.
 // split_weights: the softmax weights are multiplied with V as two bf16 parts (16 bits of mantissa); without seq_lens only.
 cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, const void* k, const void* v,
