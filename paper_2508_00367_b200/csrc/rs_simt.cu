@@ -279,28 +279,41 @@ template <typename T> cudaError_t dispatch_simt(SimtArgs& args, int sms, cudaStr
 // the query rows).
 // (One thread per query row with q and o in registers, the form this replaces, kept 24 of 148 SMs busy at 2 x 197
 // tokens of six heads and took 92 us.)
+// GROUPS: with a CTA or two to an SM a warp or two per scheduler walk through the key tiles one after the other, a chain of loads,
+// shuffles and exponentials each.  Then GROUPS times four warps share a CTA's rows, each group every GROUPS-th key tile in buffers of its own;
+// the groups' maxima, sums and outputs are merged through shared memory.  A group's tile may hold scores of -infinity only: exponents
+// are taken from 0 then, which makes all of its weights zeros.
 constexpr int AKV = 64, AWARPS = 4, ADH = 64;
 constexpr int KLD = ADH + 4;                                  // padded row length (floats): conflict-free 16-byte accesses
 constexpr int ATT_KV_FLOATS = AKV * KLD + AKV * ADH;          // one stage: keys (padded), values
-template <int AROWS> struct AttnSimt {
-    static constexpr int AQ = AWARPS * AROWS, PLD = AROWS == 8 ? 12 : 4;
-    static constexpr int SMEM = (AQ * ADH + 2 * ATT_KV_FLOATS + AWARPS * AKV * PLD) * 4;
+constexpr int OLD = ADH + 4;                                  // floats per row of a group's result: output, maximum, sum
+template <int AROWS, int GROUPS> struct AttnSimt {
+    static constexpr int AQ = AWARPS * AROWS, PLD = AROWS == 8 ? 12 : 4, STAGES = GROUPS > 1 ? 1 : 2, THREADS = 32 * AWARPS * GROUPS;
+    static constexpr int SMEM = (AQ * ADH + GROUPS * (STAGES * ATT_KV_FLOATS + AWARPS * AKV * PLD)) * 4;
+    static_assert(AQ * OLD <= ATT_KV_FLOATS && SMEM <= 227 * 1024, "a group's result takes the place of its keys");
 };
 
-template <typename T, int AROWS>
-__global__ void __launch_bounds__(32 * AWARPS, 2)
+template <typename T, int AROWS, int GROUPS>
+__global__ void __launch_bounds__((AttnSimt<AROWS, GROUPS>::THREADS), GROUPS == 1 ? 2 : 1)
 attn_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
                  T* __restrict__ out, int N, int H, float scale, long long qb, long long qr,
                  long long qh, long long kb, long long kr, long long kh, long long vb, long long vr,
                  long long vh) {
-    constexpr int AQ = AttnSimt<AROWS>::AQ, PLD = AttnSimt<AROWS>::PLD;
+    using A = AttnSimt<AROWS, GROUPS>;
+    constexpr int AQ = A::AQ, PLD = A::PLD, STAGES = A::STAGES;
     extern __shared__ __align__(16) float sm[];
-    float* Qs = sm;                                            // [AQ][64], scaled
-    float* KV = sm + AQ * ADH;                                 // [2 stages][keys 64 x 68 | values 64 x 64]
     grid_dep_launch();
     grid_dep_wait();
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    float* Ps = KV + 2 * ATT_KV_FLOATS + warp * AKV * PLD;     // [64 keys][AROWS] of this warp
+    const int group = GROUPS == 1 ? 0 : threadIdx.x / (32 * AWARPS);
+    const int tid = threadIdx.x - group * 32 * AWARPS, warp = tid >> 5, lane = tid & 31;     // within the group
+    float* Qs = sm;                                            // [AQ][64], scaled
+    float* const KV0 = sm + AQ * ADH;                          // a group: [stages][keys 64 x 68 | values 64 x 64]
+    float* KV = KV0 + group * STAGES * ATT_KV_FLOATS;
+    float* Ps = KV0 + GROUPS * STAGES * ATT_KV_FLOATS + (group * AWARPS + warp) * AKV * PLD;     // [64 keys][AROWS] of this warp
+    auto group_sync = [&]() {
+        if (GROUPS == 1) __syncthreads();
+        else tc::named_barrier(1 + group, 32 * AWARPS);
+    };
     const int h = blockIdx.y, b = blockIdx.z, q0 = blockIdx.x * AQ;
     const T* kp = k + b * kb + h * kh;
     const T* vp = v + b * vb + h * vh;
@@ -325,9 +338,9 @@ attn_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
             }
         }
     };
-    fetch(0, 0);
+    if (group < tiles) fetch(group, 0);
     cp_async_commit();
-    for (int e = tid; e < AQ * ADH; e += 32 * AWARPS) {
+    for (int e = threadIdx.x; e < AQ * ADH; e += A::THREADS) {
         const int r = e / ADH, c = e % ADH, i = q0 + r;
         Qs[e] = i < N ? to_float(q[b * qb + (long long)i * qr + h * qh + c]) * scale : 0.f;
     }
@@ -341,12 +354,17 @@ attn_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
 #pragma unroll
         for (int c = 0; c < 4; ++c) o[p][c] = 0ull;
 
-    for (int t = 0; t < tiles; ++t) {
-        const int stage = t & 1;
-        if (t + 1 < tiles) fetch(t + 1, stage ^ 1);
+    if (GROUPS > 1) __syncthreads();                           // Q is there
+    for (int t = group, n = 0; t < tiles; t += GROUPS, ++n) {
+        const int stage = STAGES == 1 ? 0 : n & 1;
+        if (STAGES > 1) {
+            if (t + GROUPS < tiles) fetch(t + GROUPS, stage ^ 1);
+        } else if (n) {
+            fetch(t, 0);
+        }
         cp_async_commit();
-        cp_async_wait<1>();
-        __syncthreads();
+        cp_async_wait<STAGES - 1>();
+        group_sync();
         const float* Ks = KV + stage * ATT_KV_FLOATS;
         const float* Vs = Ks + AKV * KLD;
         const int valid = min(AKV, N - t * AKV);
@@ -372,11 +390,12 @@ attn_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
             p0[r] = lane < valid ? pair_sum(s2[r][0]) : -INFINITY;
             p1[r] = lane + 32 < valid ? pair_sum(s2[r][1]) : -INFINITY;
             const float mx = fmaxf(m[r], warp_max(fmaxf(p0[r], p1[r])));
-            corr[r] = expf(m[r] - mx);                         // exp(-inf) = 0 on the first tile
+            const float from = GROUPS > 1 && mx == -INFINITY ? 0.f : mx;
+            corr[r] = expf(m[r] - from);                       // exp(-inf) = 0 on the first tile
             raised |= mx > m[r];
             m[r] = mx;
-            p0[r] = expf(p0[r] - mx);
-            p1[r] = expf(p1[r] - mx);
+            p0[r] = expf(p0[r] - from);
+            p1[r] = expf(p1[r] - from);
             l[r] = l[r] * corr[r] + (p0[r] + p1[r]);
         }
         if (raised) {                                          // the same for the whole warp
@@ -409,11 +428,55 @@ attn_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
                 }
             }
         }
-        __syncthreads();                                       // everyone is done with this stage
+        group_sync();                                          // everyone is done with this stage
     }
 #pragma unroll
-    for (int r = 0; r < AROWS; ++r) l[r] = 1.f / warp_sum(l[r]);
+    for (int r = 0; r < AROWS; ++r) l[r] = warp_sum(l[r]);
     const int half = lane >> 4, col = (lane & 15) * 4;
+    float scale_o[AROWS];                                      // what this group's output is multiplied by
+    if (GROUPS > 1) {
+        // a row's result, [64 outputs | maximum, sum], where the group's keys were
+        auto result = [&](int g, int r) { return KV0 + g * STAGES * ATT_KV_FLOATS + (warp * AROWS + r) * OLD; };
+        if (lane == 0) {
+#pragma unroll
+            for (int r = 0; r < AROWS; ++r) *reinterpret_cast<float2*>(result(group, r) + ADH) = make_float2(m[r], l[r]);
+        }
+        if (group) {
+#pragma unroll
+            for (int p = 0; p < AROWS / 2; ++p) {
+                float ra[4], rb[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    o[p][c] = fadd2(o[p][c], __shfl_xor_sync(0xffffffffu, o[p][c], 16));
+                    unpack2(o[p][c], ra[c], rb[c]);
+                }
+                *reinterpret_cast<float4*>(result(group, 2 * p + half) + col) = half ? make_float4(rb[0], rb[1], rb[2], rb[3]) : make_float4(ra[0], ra[1], ra[2], ra[3]);
+            }
+        }
+        __syncthreads();
+        if (group) return;
+#pragma unroll
+        for (int r = 0; r < AROWS; ++r) {
+            float2 ml[GROUPS];
+            float mx = m[r];
+#pragma unroll
+            for (int g = 1; g < GROUPS; ++g) {
+                ml[g] = *reinterpret_cast<const float2*>(result(g, r) + ADH);
+                mx = fmaxf(mx, ml[g].x);
+            }
+            scale_o[r] = expf(m[r] - mx);
+            float sum = scale_o[r] * l[r];
+#pragma unroll
+            for (int g = 1; g < GROUPS; ++g) sum += expf(ml[g].x - mx) * ml[g].y;
+            const float inv = 1.f / sum;
+            scale_o[r] *= inv;
+            l[r] = inv;
+            m[r] = mx;
+        }
+    } else {
+#pragma unroll
+        for (int r = 0; r < AROWS; ++r) scale_o[r] = 1.f / l[r];
+    }
 #pragma unroll
     for (int p = 0; p < AROWS / 2; ++p) {
         float ra[4], rb[4];
@@ -424,36 +487,52 @@ attn_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
         }
         // the lower half warp stores row 2p, the upper row 2p + 1
         const int i = q0 + warp * AROWS + 2 * p + half;
-        const float inv = half ? l[2 * p + 1] : l[2 * p];
+        const float f = half ? scale_o[2 * p + 1] : scale_o[2 * p];
         float w[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) w[c] = (half ? rb[c] : ra[c]) * inv;
+        for (int c = 0; c < 4; ++c) w[c] = (half ? rb[c] : ra[c]) * f;
+        if (GROUPS > 1) {
+            const float mx = half ? m[2 * p + 1] : m[2 * p], inv = half ? l[2 * p + 1] : l[2 * p];
+#pragma unroll
+            for (int g = 1; g < GROUPS; ++g) {
+                const float* rp = KV0 + g * STAGES * ATT_KV_FLOATS + (warp * AROWS + 2 * p + half) * OLD;
+                const float fg = expf(rp[ADH] - mx) * inv;
+                const float4 og = *reinterpret_cast<const float4*>(rp + col);
+                w[0] = fmaf(og.x, fg, w[0]); w[1] = fmaf(og.y, fg, w[1]); w[2] = fmaf(og.z, fg, w[2]); w[3] = fmaf(og.w, fg, w[3]);
+            }
+        }
         if (i < N) store_n<T, 4>(out + ((long long)b * N + i) * ((long long)H * ADH) + h * ADH + col, w);
     }
 }
 
-template <typename T, int AROWS>
+template <typename T, int AROWS, int GROUPS>
 cudaError_t attn_launch(const rs_attn_desc& d, const void* q, const void* k, const void* v, void* out, cudaStream_t st) {
-    using A = AttnSimt<AROWS>;
+    using A = AttnSimt<AROWS, GROUPS>;
     static PerDeviceOnce attr_once;
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     e = (cudaError_t)attr_once.run(dev, [] {
-        return (int)cudaFuncSetAttribute(attn_simt_kernel<T, AROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, A::SMEM);
+        return (int)cudaFuncSetAttribute(attn_simt_kernel<T, AROWS, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, A::SMEM);
     });
     if (e != cudaSuccess) return e;
     const float scale = d.scale != 0.f ? d.scale : 1.f / sqrtf((float)d.head_dim);
     const dim3 grid((d.N + A::AQ - 1) / A::AQ, d.H, d.B);
-    return launch_pdl(attn_simt_kernel<T, AROWS>, grid, dim3(32 * AWARPS), A::SMEM, st, (const T*)q, (const T*)k, (const T*)v, (T*)out, d.N, d.H,
+    return launch_pdl(attn_simt_kernel<T, AROWS, GROUPS>, grid, dim3(A::THREADS), A::SMEM, st, (const T*)q, (const T*)k, (const T*)v, (T*)out, d.N, d.H,
                       scale, d.q_batch_stride, d.q_row_stride, d.q_head_stride, d.k_batch_stride, d.k_row_stride,
                       d.k_head_stride, d.v_batch_stride, d.v_row_stride, d.v_head_stride);
 }
 
 template <typename T>
 cudaError_t attn_dispatch(const rs_attn_desc& d, const void* q, const void* k, const void* v, void* out, int sms, cudaStream_t st) {
-    const long long ctas = (long long)((d.N + 31) / 32) * d.H * d.B;
-    return ctas < 2ll * sms ? attn_launch<T, 4>(d, q, k, v, out, st) : attn_launch<T, 8>(d, q, k, v, out, st);
+    const long long ctas32 = (long long)((d.N + 31) / 32) * d.H * d.B, ctas16 = (long long)((d.N + 15) / 16) * d.H * d.B;
+    const int tiles = (d.N + AKV - 1) / AKV;
+    // Four groups where the CTAs fit the SMs one to each, of sixteen rows or else of 32.  One group / four, us: 1 x 3 x 65 6.2 / 5.2, 1 x 3 x 130 8.1 / 6.4,
+    // 1 x 3 x 577 21.3 / 17.3, 2 x 6 x 197 (84 CTAs of 32 rows) 17.0 / 12.4; with more CTAs they lose: 4 x 6 x 197 18.2 / 23.1, 1 x 12 x 577 40.6 / 50.6.
+    // Two groups: 15.6 at 2 x 6 x 197.  Error against 64 bits 2.50e-7 -> 2.09e-7 there, 3.53e-7 -> 2.43e-7 at 1 x 3 x 577 (shorter sums).
+    if (tiles >= 2 && ctas16 <= sms) return attn_launch<T, 4, 4>(d, q, k, v, out, st);
+    if (tiles >= 3 && ctas32 <= sms) return attn_launch<T, 8, 4>(d, q, k, v, out, st);
+    return ctas32 < 2ll * sms ? attn_launch<T, 4, 1>(d, q, k, v, out, st) : attn_launch<T, 8, 1>(d, q, k, v, out, st);
 }
 
 }  // namespace

@@ -61,3 +61,30 @@ def test_counts_per_sample(ctx, B):   # noqa: F811
     for b in range(0, B, 1 if B < 10 else 23):
         n = int(lens[b])
         assert _close(got[b:b + 1, :n], _reference(qkv[b:b + 1, :n]), qkv[b:b + 1, :n]), (b, n)
+
+
+@pytest.mark.parametrize("B,H,N", [(1, 3, 65), (1, 1, 127), (1, 2, 200), (1, 3, 257), (1, 9, 256), (2, 6, 197), (1, 2, 600)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_fp32_key_tiles_in_groups(ctx, B, H, N, dtype):   # noqa: F811
+    """The fp32-FMA kernel with its key tiles dealt out to four groups of warps (few query rows), a group without a tile among
+    them; bf16 takes that kernel with strides that tensor maps cannot express only, so a context without tensor cores runs it."""
+    import os
+    import paper_2508_00367_b200 as rs
+    c = ctx
+    if dtype == torch.bfloat16:
+        os.environ["RS_DISABLE_TC"] = "1"
+        try:
+            c = rs.Context(0)
+        finally:
+            del os.environ["RS_DISABLE_TC"]
+    g = torch.Generator(device="cuda").manual_seed(N)
+    qkv = torch.randn(B, N, 3, H, 64, generator=g, device="cuda").to(dtype)
+    qkv[:, :, 0, :, 0] = 1.0
+    if N > 128:
+        qkv[:, 64:128, 1, :, 0] = float("-inf")                  # a group's only tile without weight
+    got = c.attn_fwd(qkv[:, :, 0], qkv[:, :, 1], qkv[:, :, 2])
+    # fp32: errors of exp and of the sums, a few 2^-23 of |v| (the weights sum to one); bf16: one rounding of the output
+    bound = (2e-6 if dtype == torch.float32 else 2.0 ** -8) * qkv[:, :, 2].double().abs().max()
+    assert (got.double() - _reference(qkv)).abs().max() < bound
+    if c is not ctx:
+        c.close()
