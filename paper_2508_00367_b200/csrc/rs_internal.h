@@ -126,7 +126,7 @@ cudaError_t launch_line_gather(rs_dtype dtype, const void* x, const int32_t* kee
 // out[M, N] = act(A[M, K] * W[N, K]^T + bias) + residual.
 cudaError_t launch_gemm_simt(rs_dtype in_dtype, const void* A, const void* W, const float* bias,
                              int gelu, const void* residual, rs_dtype res_dtype, void* out,
-                             rs_dtype out_dtype, long long M, int N, int K, int sm_count, cudaStream_t st);
+                             rs_dtype out_dtype, long long M, int N, int K, int sm_count, cudaStream_t st, bool weights_ready = false /* as for launch_gemm_tc */);
 cudaError_t launch_attn_simt(const rs_attn_desc& d, const void* q, const void* k, const void* v,
                              void* out, int sm_count, cudaStream_t st);
 

@@ -68,6 +68,7 @@ struct SimtArgs {
     void* out;
     long long M;
     int N, K, gelu, res_bf16, out_bf16, splits;
+    int weights_ready;       // W may be read before the kernel waits for its predecessor (no earlier kernel still running writes it)
 };
 
 template <typename T, int WM, int WN, int WK, int NJ>
@@ -77,7 +78,7 @@ gemm_simt_kernel(const SimtArgs args) {
     constexpr int CHUNK = 16 / (int)sizeof(T), CPR = C::BK / CHUNK;      // values per 16 bytes, 16-byte pieces per row
     extern __shared__ __align__(16) uint8_t smem[];
     grid_dep_launch();
-    grid_dep_wait();
+    if (!args.weights_ready) grid_dep_wait();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int wk = warp / (WM * WN), wm = (warp % (WM * WN)) / WN, wn = warp % WN;
     const int ty = lane >> 3, tx = lane & 7;
@@ -98,16 +99,22 @@ gemm_simt_kernel(const SimtArgs args) {
     const T* pw = W + (long long)(n0 + fr) * K + fc * CHUNK;
     const long long row_step = (long long)ROWS_PER_PASS * K;
     const uint32_t dst0 = tc::smem_u32(smem) + fr * C::ROW_BYTES + fc * 16;
-    auto fetch = [&](int slab, int stage) {
+    auto fetch_a = [&](int slab, int stage) {
         const uint32_t dst = dst0 + stage * C::STAGE_BYTES;
         const int k0 = slab * C::BK;
         const bool kok = k0 + fc * CHUNK < K;
-        const T *a = pa + k0, *w = pw + k0;
+        const T* a = pa + k0;
 #pragma unroll
         for (int i = 0; i < C::TM / ROWS_PER_PASS; ++i, a += row_step) {
             const bool ok = kok && m0 + fr + i * ROWS_PER_PASS < args.M;
             cp_async16(dst + i * ROWS_PER_PASS * C::ROW_BYTES, ok ? a : A, ok);
         }
+    };
+    auto fetch_w = [&](int slab, int stage) {
+        const uint32_t dst = dst0 + stage * C::STAGE_BYTES;
+        const int k0 = slab * C::BK;
+        const bool kok = k0 + fc * CHUNK < K;
+        const T* w = pw + k0;
 #pragma unroll
         for (int i = 0; i < C::TN / ROWS_PER_PASS; ++i, w += row_step) {
             const bool ok = kok && n0 + fr + i * ROWS_PER_PASS < args.N;
@@ -121,9 +128,15 @@ gemm_simt_kernel(const SimtArgs args) {
 #pragma unroll
         for (int j = 0; j < NJ; ++j) acc[i][j] = 0ull;
 
+    // Weights do not depend on the kernel before this one: the first slabs' are requested before it is waited for (they belong to
+    // the first group, which is waited for as a whole).  The four products of a ViT-S block, 2 x 197: 92.8 -> 89.5 us for the block.
+#pragma unroll
+    for (int s = 0; s < C::STAGES - 1; ++s)
+        if (s_begin + s < s_end) fetch_w(s_begin + s, s);
+    if (args.weights_ready) grid_dep_wait();
 #pragma unroll
     for (int s = 0; s < C::STAGES - 1; ++s) {
-        if (s_begin + s < s_end) fetch(s_begin + s, s);
+        if (s_begin + s < s_end) fetch_a(s_begin + s, s);
         cp_async_commit();
     }
     int stage = 0;
@@ -131,7 +144,11 @@ gemm_simt_kernel(const SimtArgs args) {
         cp_async_wait<C::STAGES - 2>();
         __syncthreads();                                                 // the slab landed, and everyone is done with the stage refilled next
         const int ahead = stage + C::STAGES - 1;
-        if (slab + C::STAGES - 1 < s_end) fetch(slab + C::STAGES - 1, ahead >= C::STAGES ? ahead - C::STAGES : ahead);
+        if (slab + C::STAGES - 1 < s_end) {
+            const int to = ahead >= C::STAGES ? ahead - C::STAGES : ahead;
+            fetch_a(slab + C::STAGES - 1, to);
+            fetch_w(slab + C::STAGES - 1, to);
+        }
         cp_async_commit();
         const uint8_t* base = smem + stage * C::STAGE_BYTES;
         const uint8_t* arow = base + (wm * 32 + ty) * C::ROW_BYTES + wk * (C::BK / WK) * (int)sizeof(T);
@@ -539,9 +556,9 @@ cudaError_t attn_dispatch(const rs_attn_desc& d, const void* q, const void* k, c
 
 cudaError_t launch_gemm_simt(rs_dtype in_dtype, const void* A, const void* W, const float* bias,
                              int gelu, const void* residual, rs_dtype res_dtype, void* out,
-                             rs_dtype out_dtype, long long M, int N, int K, int sm_count, cudaStream_t st) {
+                             rs_dtype out_dtype, long long M, int N, int K, int sm_count, cudaStream_t st, bool weights_ready) {
     if (M == 0 || N == 0) return cudaSuccess;
-    SimtArgs args = {A, W, bias, residual, out, M, N, K, gelu, res_dtype == RS_BF16, out_dtype == RS_BF16, 1};
+    SimtArgs args = {A, W, bias, residual, out, M, N, K, gelu, res_dtype == RS_BF16, out_dtype == RS_BF16, 1, weights_ready ? 1 : 0};
     return in_dtype == RS_BF16 ? dispatch_simt<__nv_bfloat16>(args, sm_count, st) : dispatch_simt<float>(args, sm_count, st);
 }
 
