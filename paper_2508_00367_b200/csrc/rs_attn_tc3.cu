@@ -14,9 +14,10 @@
 // 1850, of which 1250 are exponentials; 4 x 16 x 4097 369 -> 337 us, 16 x 12 x 1569 181 -> 160, 32 x 16 x 577 82.8 -> 72.3, 64 x 12 x 197 30.5 -> 24.1.
 // An item is three consecutive 128-row query tiles of one (sample, head), which share the K/V
 // tiles streamed through the TMA ring, or of consecutive (sample, head)s.
-// SPLIT: the weights go to the second product as a bf16 and the bf16 of what that left over, one after the other
-// through the same tensor-memory columns: 16 bits of mantissa instead of 8, for the blocks that used to have fp32
-// weights (see rs_block_fwd).
+// SPLIT: the weights go to the second product as a bf16 and the bf16 of what that left over, 16 bits of mantissa instead of 8,
+// for the blocks that used to have fp32 weights (see rs_block_fwd).  The second parts take columns of the S that they came
+// from, so the next Q K^T waits for P V there.  (One after the other through the columns of P, with S handed back early, every key tile went
+// to the tensor core and back twice: DeiT-T, 256 images, 1042 -> 992 us for the pass, twelve blocks of 2 x 197 x 192 394 -> 383.)
 #include <math.h>
 
 #include "rs_internal.h"
@@ -194,7 +195,6 @@ __global__ void __launch_bounds__(kThreads, 1)
 attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO, const Attn3Args args) {
     static_assert(!RAGGED || (!SPLIT && !CUT), "neither comes with a count per sample");
-    constexpr int PARTS = SPLIT ? 2 : 1;     // products P V per key tile
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + OFF_BAR);
@@ -313,7 +313,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 return ok;
             };
             auto issue = [&](int g, uint32_t dq, uint32_t idesc_s) {
-                ok = ns[g] == 0 || mbar_wait(&s_free[g], (ns[g] - 1) & 1u, abort_flag);
+                ok = ns[g] == 0 || mbar_wait(SPLIT ? &o_done[g] : &s_free[g], (ns[g] - 1) & 1u, abort_flag);
                 if (!ok) return;
                 tc_fence_after();
                 const uint32_t dk = k_lo + (uint32_t)stage * kKV16;
@@ -377,6 +377,9 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 const uint32_t dv = v_lo + (uint32_t)stage * kKV16, o_col = tmem_base + kOCol + g * DH, p_col = tmem_base + kPCol + g * (BKV / 2);
                 for (int k = 0; k < ksteps; ++k)
                     mma_ts_lh(o_col, p_col + 8 * k, dv + 128u * k, desc_hi, idesc_o, !(first && k == 0));
+                if (SPLIT)
+                    for (int k = 0; k < ksteps; ++k)
+                        mma_ts_lh(o_col, tmem_base + kSCol + g * BKV + 8 * k, dv + 128u * k, desc_hi, idesc_o, 1u);
                 mma_commit(&o_done[g]);
                 ++np[g];
             };
@@ -385,23 +388,13 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 const int ksteps_last = (it.n - (it.nkv - 1) * BKV + 15) >> 4;
                 const bool cut = CUT && it.third;
                 for (int j = 0, steps = cut ? it.third : it.nkv; j < steps && ok; ++j) {
-                    if (cut || SPLIT) {
-                        int stage_of[NG];                // SPLIT: kept for the second part
+                    if (cut) {
 #pragma unroll
-                        for (int part = 0; part < PARTS; ++part) {
-#pragma unroll
-                            for (int g = 0; g < NG; ++g) {
-                                const int tile = j + g * it.third;
-                                if ((!cut && g >= it.ng) || tile >= it.nkv || !ok) continue;
-                                if (part == 0) {
-                                    if ((cut || it.starts(g)) && !next_stage()) continue;
-                                    stage_of[g] = stage;
-                                } else {
-                                    stage = stage_of[g];
-                                }
-                                issue(g, tile == it.nkv - 1 ? ksteps_last : BKV / 16, j == 0 && part == 0);
-                                if (ok && part == PARTS - 1 && (cut || it.ends(g))) mma_commit(&v_empty[stage]);
-                            }
+                        for (int g = 0; g < NG; ++g) {
+                            const int tile = j + g * it.third;
+                            if (tile >= it.nkv || !ok || !next_stage()) continue;
+                            issue(g, tile == it.nkv - 1 ? ksteps_last : BKV / 16, j == 0);
+                            if (ok) mma_commit(&v_empty[stage]);
                         }
                     } else {
                         const int ksteps = j == it.nkv - 1 ? ksteps_last : BKV / 16;
@@ -440,7 +433,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         };
         // what last read the P columns, and wrote O: P V of the previous key tile (before the first one the barrier lets the
         // parity of its last phase through at once)
-        auto wait_o = [&]() { wait(&o_done[g], (cnt * PARTS - 1) & 1u); };
+        auto wait_o = [&]() { wait(&o_done[g], (cnt - 1) & 1u); };
         // The key tiles of one query tile: nkv of them, the first nfull whole, the last one of valid_last keys otherwise.  Leaves the
         // running maximum (times scale * log2 e) and sum of this thread's row.
         // gap1: the gap of the second key tile.
@@ -461,19 +454,14 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                     have_s = __any_sync(0xffffffffu, mx_l2 > m_l2 + (j == 1 ? gap1 : kRescaleGap));
                     if (have_s) break;
                     float l_tile = exp_pass<0, BKV / 2, SPLIT>(r, lo, sl, -m_l2);
-                    arrive(&s_free[g]);                  // the next Q K^T may overwrite S
+                    if (!SPLIT) arrive(&s_free[g]);      // the next Q K^T may overwrite S
                     l_tile += exp_pass<BKV / 2, BKV / 2, SPLIT>(r, lo, sl, -m_l2);
                     l_run += l_tile;
-                    wait_o();
+                    if constexpr (SPLIT) tmem_st_32x32(s_addr, lo);      // (S was complete after P V of the key tile before)
+                    else wait_o();
                     tmem_st_32x32(p_addr, r);
                     tmem_wait_st();
                     arrive(&p_ready[g]);
-                    if constexpr (SPLIT) {               // the rest of the weights, when the product with the first part is done
-                        wait(&o_done[g], 0);
-                        tmem_st_32x32(p_addr, lo);
-                        tmem_wait_st();
-                        arrive(&p_ready[g]);
-                    }
                 }
                 if (j == nkv) break;
                 // A key tile that raises the maximum, or the last one with fewer keys than columns: 16 columns at a time from
@@ -514,26 +502,23 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                     }
                 }
 #pragma unroll 1
-                for (int part = 0; part < PARTS; ++part) {
-                    if (part) wait(&o_done[g], 0);
-#pragma unroll 1
-                    for (int c = 0; c < valid; c += 16) {
-                        uint32_t s[16];
-                        load16(c, s);
+                for (int c = 0; c < valid; c += 16) {
+                    uint32_t s[16], low[8];
+                    load16(c, s);
 #pragma unroll
-                        for (int i = 0; i < 16; i += 2) {
-                            const float p0 = ex2(fmaf(__uint_as_float(s[i]), sl, -m_l2)), p1 = ex2(fmaf(__uint_as_float(s[i + 1]), sl, -m_l2));
-                            uint32_t h = pack_bf16(p0, p1);
-                            if (part) h = pack_bf16(p0 - __uint_as_float(h << 16), p1 - __uint_as_float(h & 0xffff0000u));
-                            else l_run += p0 + p1;
-                            s[i >> 1] = h;
-                        }
-                        tmem_st_32x8(p_addr + (c >> 1), s);
+                    for (int i = 0; i < 16; i += 2) {
+                        const float p0 = ex2(fmaf(__uint_as_float(s[i]), sl, -m_l2)), p1 = ex2(fmaf(__uint_as_float(s[i + 1]), sl, -m_l2));
+                        const uint32_t h = pack_bf16(p0, p1);
+                        if (SPLIT) low[i >> 1] = pack_bf16(p0 - __uint_as_float(h << 16), p1 - __uint_as_float(h & 0xffff0000u));
+                        l_run += p0 + p1;
+                        s[i >> 1] = h;
                     }
-                    tmem_wait_st();
-                    arrive(&p_ready[g]);
+                    tmem_st_32x8(p_addr + (c >> 1), s);
+                    if (SPLIT) tmem_st_32x8(s_addr + (c >> 1), low);     // (columns already read)
                 }
-                if (lane == 0) mbar_arrive(&s_free[g]);  // (every lane's reads of S are complete at the arrival above)
+                tmem_wait_st();
+                arrive(&p_ready[g]);
+                if (!SPLIT && lane == 0) mbar_arrive(&s_free[g]);        // (every lane's reads of S are complete at the arrival above)
             }
         };
         // O / l -> bf16 -> global.  The warp's 32 rows x 64 values go to its own slab of shared memory (128-byte rows, 16-byte
