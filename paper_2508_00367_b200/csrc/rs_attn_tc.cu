@@ -1,6 +1,6 @@
 // Fused attention on the tensor cores (Eq. sa): out = Softmax(Q K^T * scale) V per
 // (sample, head), head dimension 64, without ever writing the N x N matrix.
-// This kernel serves batches of very many samples with a count each, and as the other kernel's cross-check (see launch_attn_tc).
+// This kernel serves small batches with a count per sample, and as the other kernel's cross-check (see launch_attn_tc).
 //
 // Persistent kernel, one CTA per SM, looping over work items.  An item is two 128-row query
 // tiles A and B: for N > 128 two consecutive query tiles of one (sample, head), which share
@@ -579,13 +579,23 @@ cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, co
         return (int)a;
     });
     if (e != cudaSuccess) return e;
+    // The kernel with three query tiles per CTA: two tiles / three, us, 4 x 16 x 4097 404 / 335, x 2305 151 / 122, 16 x 12 x 1569 207 / 160, 32 x 16 x 577
+    // 101 / 72, 64 x 12 x 197 31.8 / 24.1, x 101 14.1 / 11.8, x 17 9.4 / 7.4, 1 x 12 x 197 6.3 / 5.6.  With a count per sample it first sorts the samples,
+    // which pays from 129 tokens and two query tiles per SM on (whole ragged passes, two / three: 79 x 203 x 768 1339 / 1299, 7 x 468 x 768
+    // 1056 / 1011, 12 x 1177 x 768 2234 / 2168; but 12 x 181 x 768 1814 / 1824, 1 x 160 x 1024 1216 / 1234, 200 x 80 x 384 646 / 694).
+    // RS_ATTN_KERNEL pins one (tests compare each with the oracle).
+    const bool split = split_weights && !seq_lens;          // (this file's kernel has no such weights)
+    const bool sorted = d.B <= attn_tc3_max_samples() && (ctx->attn_kernel == 3 || (d.N > BQ && (long long)d.B * d.H * ((d.N + BQ - 1) / BQ) > 2ll * ctx->sm_count));
+    const bool three = split || (ctx->attn_kernel != 2 && (!seq_lens || sorted));
+    const int kv_rows = three ? 64 : 128;                   // keys of a tile
     CUtensorMap tmQ, tmK, tmV, tmO;
     // out is [B, N, H, 64] contiguous; a softmax warp stores its 32 rows of one head at a time
     if (!make_tmap_qkv(ctx, &tmO, out, d.B, d.N, d.H, (long long)d.N * d.H * 64, (long long)d.H * 64, 64, 32) ||
         !make_tmap_qkv(ctx, &tmQ, q, d.B, d.N, d.H, d.q_batch_stride, d.q_row_stride, d.q_head_stride) ||
-        !make_tmap_qkv(ctx, &tmK, k, d.B, d.N, d.H, d.k_batch_stride, d.k_row_stride, d.k_head_stride) ||
-        !make_tmap_qkv(ctx, &tmV, v, d.B, d.N, d.H, d.v_batch_stride, d.v_row_stride, d.v_head_stride))
+        !make_tmap_qkv(ctx, &tmK, k, d.B, d.N, d.H, d.k_batch_stride, d.k_row_stride, d.k_head_stride, kv_rows) ||
+        !make_tmap_qkv(ctx, &tmV, v, d.B, d.N, d.H, d.v_batch_stride, d.v_row_stride, d.v_head_stride, kv_rows))
         return cudaErrorInvalidValue;
+    if (three) return launch_attn_tc3(ctx, d, tmQ, tmK, tmV, tmO, seq_lens, split, st);
     AttnArgs args;
     args.out = (__nv_bfloat16*)out;
     args.N = d.N; args.H = d.H;
@@ -594,17 +604,6 @@ cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, co
     long long items = (long long)args.per * (args.dual ? d.B : (long long)d.B * d.H);
     if (items >= (1ll << 30)) return cudaErrorInvalidValue;
     args.n_pair_items = (int)items; args.first_single_bh = d.B * d.H; args.tile_count = (d.N + BQ - 1) / BQ;
-    // The kernel with three query tiles per CTA takes every shape but batches of very many samples with a count each: two tiles /
-    // three, us, 4 x 16 x 4097 404 / 335, x 2305 151 / 122, 16 x 12 x 1569 207 / 165, 32 x 16 x 577 101 / 72, 64 x 12 x 197 31.8 / 26.1, x 101 14.1 / 11.6,
-    // x 17 9.4 / 7.4, 1 x 12 x 197 6.3 / 6.0.  RS_ATTN_KERNEL=2 keeps this file's for all (tests compare each with the oracle).
-    const bool split = split_weights && !seq_lens;          // (this file's kernel has no such weights)
-    if (split || (ctx->attn_kernel != 2 && (!seq_lens || d.B <= attn_tc3_max_samples()))) {
-        CUtensorMap tmK3, tmV3;
-        if (!make_tmap_qkv(ctx, &tmK3, k, d.B, d.N, d.H, d.k_batch_stride, d.k_row_stride, d.k_head_stride, 64) ||
-            !make_tmap_qkv(ctx, &tmV3, v, d.B, d.N, d.H, d.v_batch_stride, d.v_row_stride, d.v_head_stride, 64))
-            return cudaErrorInvalidValue;
-        return launch_attn_tc3(ctx, d, tmQ, tmK3, tmV3, tmO, seq_lens, split, st);
-    }
     if (!args.dual) {
         const long long BH = (long long)d.B * d.H;
         const int nt = args.tile_count, per = args.per;

@@ -51,7 +51,7 @@ constexpr int OFF_OST = OFF_V + NS * KV_BYTES;  // output staging: 12 softmax wa
 constexpr int OFF_BAR = OFF_OST + 4 * NG * 4096;
 constexpr int kMaxSamples = 256;                 // of a launch with a count per sample
 constexpr int OFF_SAMPLES = OFF_BAR + 512;      // what those launches keep of the counts
-constexpr size_t kSmem = (size_t)OFF_SAMPLES + 4 * (kMaxSamples + 2) + kMaxSamples + 1024 /*alignment slack*/;
+constexpr size_t kSmem = (size_t)OFF_SAMPLES + 4 * (kMaxSamples + 3) + kMaxSamples + 1024 /*alignment slack*/;
 static_assert(kOCol + NG * DH <= kTmemCols, "tensor-memory columns");
 static_assert(kSmem <= 232448, "shared memory of one CTA");
 
@@ -95,7 +95,7 @@ struct Item3 {
 };
 // RAGGED: what the CTA knows of the samples, in shared memory.
 struct Samples {
-    int items;
+    int items, per;                                      // items in all; query tiles to an item (two or one where that leaves no CTA a second item)
     int first_item[kMaxSamples + 1];
     unsigned char order[kMaxSamples];
 };
@@ -114,8 +114,8 @@ template <bool RAGGED, bool CUT> __device__ __forceinline__ Item3 decode_item3(c
         it.b = sm->order[lo];
         it.n = sample_len(a, it.b);
         it.nt = (it.n + BQ - 1) / BQ;
-        const int tile = (w - sm->first_item[lo]) * NG;
-        it.ng = min(NG, a.H * it.nt - tile);
+        const int tile = (w - sm->first_item[lo]) * sm->per;
+        it.ng = min(sm->per, a.H * it.nt - tile);
         it.h = tile / it.nt;
         it.q = tile - it.h * it.nt;
     } else {
@@ -234,21 +234,34 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     grid_dep_wait();
     Samples* samples = RAGGED ? reinterpret_cast<Samples*>(smem + OFF_SAMPLES) : nullptr;
     if constexpr (RAGGED) {
-        // samples by length, the longest first (its place: how many come before it), and the items before each
-        static_assert(kMaxSamples <= kThreads, "a thread to a sample");
-        const int b = threadIdx.x, len = b < args.B ? sample_len(args, b) : 0;
-        int place = 0, before = 0;
-        for (int o = 0; o < args.B && b < args.B; ++o) {
-            const int l = sample_len(args, o);
-            if (l > len || (l == len && o < b)) {
-                ++place;
-                before += (args.H * ((l + BQ - 1) / BQ) + NG - 1) / NG;
+        // Samples by length, the longest first (its place: how many come before it), and the items before each; a warp to a
+        // sample.  (A thread to a sample: 30 x 89 tokens 4.7 us for the loops.)
+        static_assert(kMaxSamples <= kThreads, "a thread to a sample's count");
+        int* lens = reinterpret_cast<int*>(smem + OFF_OST);                  // (not in use yet)
+        if ((int)threadIdx.x < args.B) lens[threadIdx.x] = sample_len(args, threadIdx.x);
+        __syncthreads();
+        auto tiles_of = [&](int l) { return args.H * ((l + BQ - 1) / BQ); };
+        int tiles = 0;
+        for (int o = lane; o < args.B; o += 32) tiles += tiles_of(lens[o]);
+        const int per = min((__reduce_add_sync(0xffffffffu, tiles) + (int)gridDim.x - 1) / (int)gridDim.x, NG);
+        auto items_of = [&](int l) { return per == 1 ? tiles_of(l) : per == 2 ? (tiles_of(l) + 1) / 2 : (tiles_of(l) + 2) / 3; };
+        for (int b = warp; b < args.B; b += kThreads / 32) {
+            const int len = lens[b];
+            int place = 0, before = 0;
+            for (int o = lane; o < args.B; o += 32) {
+                const int l = lens[o];
+                if (l > len || (l == len && o < b)) { ++place; before += items_of(l); }
             }
-        }
-        if (b < args.B) {
-            samples->order[place] = (unsigned char)b;
-            samples->first_item[place] = before;
-            if (place == args.B - 1) samples->items = samples->first_item[args.B] = before + (args.H * ((len + BQ - 1) / BQ) + NG - 1) / NG;
+            place = __reduce_add_sync(0xffffffffu, place);
+            before = __reduce_add_sync(0xffffffffu, before);
+            if (lane == 0) {
+                samples->order[place] = (unsigned char)b;
+                samples->first_item[place] = before;
+                if (place == args.B - 1) {
+                    samples->items = samples->first_item[args.B] = before + items_of(len);
+                    samples->per = per;
+                }
+            }
         }
         __syncthreads();
     }
@@ -695,7 +708,7 @@ cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMa
     const float scale = d.scale != 0.f ? d.scale : 0.125f;
     args.scale_log2 = scale * 1.4426950408889634f;
     args.status = ctx->d_status;
-    const long long most = lens ? (long long)d.B * (((long long)d.H * nt + NG - 1) / NG) : args.n_items;
+    const long long most = lens ? BH * nt : args.n_items;
     const int grid = most < G ? (int)most : G;
     auto run = [&](auto kernel) { return launch_pdl(kernel, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args); };
     if (lens) return run(attn_tc3_kernel<false, true, false>);

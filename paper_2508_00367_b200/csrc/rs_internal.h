@@ -33,7 +33,7 @@ struct rs_ctx {
     int require_tc;        // RS_REQUIRE_TC=1: a bf16 shape the tensor-core kernels cannot take is an error
     int* d_status;         // device status word (0 = ok), first bytes of a small allocation made by rs_create
     int log, nvtx;          // RS_LOG=1: a line per launch on stderr; RS_NVTX=1: an NVTX range around each launch call
-    int attn_kernel;        // RS_ATTN_KERNEL: 2 the attention kernel with two query tiles per CTA, else the one with three
+    int attn_kernel;        // RS_ATTN_KERNEL: 2 / 3 always the attention kernel with two / three query tiles per CTA, else by the shape
     long long launches;    // kernels launched through this context
     void* encode_tiled;    // cuTensorMapEncodeTiled entry point (driver API), or null
     int timing;            // bracket launches with events

@@ -49,7 +49,7 @@ def test_a_sample_does_not_depend_on_its_place(ctx, B, H, N):   # noqa: F811
     assert _close(got[:1, -300:], _reference(qkv[:1])[:, -300:], qkv)
 
 
-@pytest.mark.parametrize("B", [1, 7, 256, 257])
+@pytest.mark.parametrize("B", [1, 7, 70, 256, 257])
 def test_counts_per_sample(ctx, B):   # noqa: F811
     N, H = 200, 3
     g = torch.Generator(device="cuda").manual_seed(B)
@@ -58,7 +58,7 @@ def test_counts_per_sample(ctx, B):   # noqa: F811
     lens[-1] = N
     got = ctx.attn_fwd_ragged(qkv[:, :, 0], qkv[:, :, 1], qkv[:, :, 2], lens)
     ctx.async_status()
-    for b in range(0, B, 1 if B < 10 else 23):
+    for b in range(0, B, 1 if B < 10 else 11):
         n = int(lens[b])
         assert _close(got[b:b + 1, :n], _reference(qkv[b:b + 1, :n]), qkv[b:b + 1, :n]), (b, n)
 
