@@ -139,13 +139,13 @@ template <bool RAGGED, bool CUT> __device__ __forceinline__ Item3 decode_item3(c
     return it;
 }
 
-// Maximum of a 64-column row of S in registers.
-__device__ __forceinline__ float row_max64(const uint32_t (&r)[BKV]) {
+// Maximum of N columns of a row of S in registers.
+template <int N> __device__ __forceinline__ float row_max(const uint32_t (&r)[N]) {
     float m[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) m[c] = -INFINITY;
 #pragma unroll
-    for (int i = 0; i < BKV; i += 16)                 // eight independent chains: latency, not count, is the cost
+    for (int i = 0; i < N; i += 16)                 // eight independent chains: latency, not count, is the cost
 #pragma unroll
         for (int c = 0; c < 8; ++c) m[c] = max3(m[c], __uint_as_float(r[i + 2 * c]), __uint_as_float(r[i + 2 * c + 1]));
     return max3(max3(m[0], m[1], m[2]), max3(m[3], m[4], m[5]), fmaxf(m[6], m[7]));
@@ -449,11 +449,48 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         auto wait_o = [&]() { wait(&o_done[g], (cnt - 1) & 1u); };
         // The key tiles of one query tile: nkv of them, the first nfull whole, the last one of valid_last keys otherwise.  Leaves the
         // running maximum (times scale * log2 e) and sum of this thread's row.
-        // gap1: the gap of the second key tile.
-        auto walk = [&](int nkv, int nfull, int valid_last, float gap1, float& m_l2, float& l_run) {
+        // gap1: the gap of the second key tile.  two_first: the running maximum starts as that of the first two key tiles, both whole.
+        // What rounding the weights to bf16 costs is decided by the largest ones.  The weight at the running maximum is 1 and exact; so up to 128 keys
+        // the maximum is the true one, and of more it starts as that of the first 128, as with key tiles of 128.  Where the true maximum `top` lies
+        // above the running one all the same, its weight goes into the sum as it was rounded: numerator and denominator then err together, and of
+        // a weight that outweighs the rest nothing remains of its error.  Error against 64 bits, 1e-3, scores of standard deviation 1 / 4: from the first 64
+        // keys' maximum, from 128, with the top weight as rounded: 64 x 12 x 197 2.272 / 2.104, 2.224 / 1.952, 2.217 / 1.786; 16 x 12 x 1569
+        // 2.335 / 2.098, 2.330 / 2.149, 2.328 / 1.886.  Time: 25.0 -> 27.3 us and 159 -> 161 (the wait for the second key tile's S, 1000 cycles an item).
+        // Keys cut in three have three running maxima, each exact for a part of the keys, and need neither (1 x 12 x 197: from 128 keys 2.262 / 1.954, cut 2.215 / 1.923).
+        auto walk = [&](int nkv, int nfull, int valid_last, float gap1, bool two_first, float& m_l2, float& l_run) {
+            float top = -INFINITY;                       // (not scaled)
             m_l2 = kLowest;
             l_run = 0.f;
-            for (int j = 0; j < nkv; ++j, ++cnt) {
+            int j = 0;
+            if (two_first) {
+                // S of the first key tile is handed back once it is in registers; of the second's, which stays where it is, only
+                // the maximum is taken before the first's exponentials.
+                uint32_t r[BKV];
+                wait(&s_full[g], cnt & 1u);
+                tmem_ld_32x32(s_addr, r);
+                tmem_ld_32x32(s_addr + 32, r + 32);
+                tmem_wait_ld();
+                arrive(&s_free[g]);
+                float mx = row_max<BKV>(r);
+                wait(&s_full[g], (cnt + 1) & 1u);
+#pragma unroll
+                for (int c = 0; c < BKV; c += 32) {
+                    uint32_t s[32];
+                    tmem_ld_32x32(s_addr + c, s);
+                    tmem_wait_ld();
+                    mx = fmaxf(mx, row_max<32>(s));
+                }
+                top = mx;
+                m_l2 = fmaxf(mx * sl, kLowest);
+                uint32_t unused[1];
+                l_run = exp_pass<0, BKV, false>(r, unused, sl, -m_l2);
+                wait_o();
+                tmem_st_32x32(p_addr, r);
+                tmem_wait_st();
+                arrive(&p_ready[g]);
+                ++j, ++cnt;
+            }
+            for (; j < nkv; ++j, ++cnt) {
                 // Whole key tiles whose maximum stays within 2^kRescaleGap of the running one: nearly all of them.
                 bool have_s = false;
                 for (; j < nfull; ++j, ++cnt) {
@@ -462,10 +499,11 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                     tmem_ld_32x32(s_addr, r);
                     tmem_ld_32x32(s_addr + 32, r + 32);
                     tmem_wait_ld();
-                    const float mx_l2 = row_max64(r) * sl;
+                    const float mx = row_max<BKV>(r), mx_l2 = mx * sl;
                     if (j == 0) m_l2 = fmaxf(mx_l2, kLowest);
                     have_s = __any_sync(0xffffffffu, mx_l2 > m_l2 + (j == 1 ? gap1 : kRescaleGap));
                     if (have_s) break;
+                    if (!SPLIT) top = fmaxf(top, mx);
                     float l_tile = exp_pass<0, BKV / 2, SPLIT>(r, lo, sl, -m_l2);
                     if (!SPLIT) arrive(&s_free[g]);      // the next Q K^T may overwrite S
                     l_tile += exp_pass<BKV / 2, BKV / 2, SPLIT>(r, lo, sl, -m_l2);
@@ -496,6 +534,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                     for (int i = 0; i < 16; i += 2) mx = max3(mx, __uint_as_float(s[i]), __uint_as_float(s[i + 1]));
                 }
                 const float mx_l2 = mx * sl;
+                if (!SPLIT) top = fmaxf(top, mx);
                 wait_o();
                 if (j == 0) {
                     m_l2 = fmaxf(mx_l2, kLowest);
@@ -533,6 +572,10 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 arrive(&p_ready[g]);
                 if (!SPLIT && lane == 0) mbar_arrive(&s_free[g]);        // (every lane's reads of S are complete at the arrival above)
             }
+            if (two_first) {                             // (a top that raised the running maximum has a weight of 1)
+                const float p = ex2(fmaf(top, sl, -m_l2));
+                l_run += __uint_as_float(pack_bf16(p, 0.f) << 16) - p;
+            }
         };
         // O / l -> bf16 -> global.  The warp's 32 rows x 64 values go to its own slab of shared memory (128-byte rows, 16-byte
         // pieces XOR-swizzled like the tensor map's box) and leave with one TMA store, which drops the rows past N.
@@ -549,9 +592,8 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 tma_store_commit();
             }
         };
-        // Up to 128 keys the maximum is exact, so that the largest weight is 1 and is not rounded (of a few weights it is a good part: error
-        // against 64 bits at 4 x 3 x 100 with scores of standard deviation 1 / 4, 2.22e-3 / 2.00e-3 -> 2.13e-3 / 1.75e-3; 64 x 12 x 101 11.4 -> 11.8 us).
-        auto first_gap = [](int n) { return n <= 2 * BKV ? 0.f : kRescaleGap; };
+        auto first_gap = [](int nkv) { return !SPLIT && nkv == 2 ? 0.f : kRescaleGap; };
+        auto two_first = [](int nkv) { return !SPLIT && nkv > 2; };
         const int nkv_all = (args.N + BKV - 1) / BKV, nfull_all = args.N / BKV, valid_all = args.N % BKV;
         const int whole = CUT ? args.n_whole : n_items;
         int w = blockIdx.x;
@@ -559,8 +601,8 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             const Item3 it = decode_item3<RAGGED, CUT>(args, samples, w);
             if (g >= it.ng) continue;
             float m_l2, l_run;
-            if constexpr (RAGGED) walk(it.nkv, it.n / BKV, it.n % BKV, first_gap(it.n), m_l2, l_run);
-            else walk(nkv_all, nfull_all, valid_all, first_gap(args.N), m_l2, l_run);
+            if constexpr (RAGGED) walk(it.nkv, it.n / BKV, it.n % BKV, first_gap(it.nkv), two_first(it.nkv), m_l2, l_run);
+            else walk(nkv_all, nfull_all, valid_all, first_gap(nkv_all), two_first(nkv_all), m_l2, l_run);
             wait_o();
             if (lane == 0) tma_store_wait_read<0>();     // the slab's previous store has read it
             __syncwarp();
@@ -587,7 +629,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 const Item3 it = decode_item3<RAGGED, CUT>(args, samples, w);
                 const int first = g * it.third, n = min(max(it.nkv - first, 0), it.third);
                 float m_l2, l_run;
-                walk(n, min(n, nfull_all - first), valid_all, kRescaleGap, m_l2, l_run);
+                walk(n, min(n, nfull_all - first), valid_all, kRescaleGap, false, m_l2, l_run);
                 wait_o();
                 if (lane == 0) tma_store_wait_read<0>();
                 __syncwarp();

@@ -60,3 +60,33 @@ def test_query_tiles_across_heads(pinned, B, H, N):   # noqa: F811
     want = torch.softmax(q @ k.transpose(2, 3) / 8.0, -1) @ v
     # weights rounded to bf16 (2^-9 each, they sum to one), values up to |v|max; one rounding of the output
     assert (got - want.transpose(1, 2).reshape(B, N, H * 64)).abs().max() < 2.0 ** -8 * v.abs().max()
+
+
+@pytest.mark.parametrize("B,H,N,counts", [(8, 12, 129, False), (8, 12, 197, False), (4, 16, 300, False), (2, 12, 2353, False),
+                                          (64, 3, 101, False), (30, 12, 300, True), (3, 3, 200, True)])
+@pytest.mark.parametrize("where", [70, 100, 127, 128])
+def test_the_largest_weight_is_not_rounded(ctx, B, H, N, counts, where):   # noqa: F811
+    """One key outweighs the rest by 3 to 5 nats (less than what raises the running maximum) and is the only one with values, so the
+    output is its share p of the weights times its value.  Its weight is exact, or rounded the same above and below the line: an
+    error e of it leaves e (1 - p), 1 - p <= 0.05, which changes the bf16 of at most 5 % of the outputs (all of e would: half)."""
+    if where >= N:
+        return
+    g = torch.Generator(device="cuda").manual_seed(where + N)
+    q, k, v = (torch.zeros(B, N, H, 64, device="cuda") for _ in range(3))
+    a = torch.rand(B, N, H, generator=g, device="cuda").mul_(2).add_(3).bfloat16()
+    q[..., 0], q[..., 1] = a.float(), 8.0
+    k[..., 1] = -12.0                                            # scores of -12 nats,
+    k[:, 3, :, 1] = 0.0                                          # one of 0
+    k[:, where, :, 0], k[:, where, :, 1] = 8.0, 0.0              # and one of a
+    v[:, where] = torch.rand(B, H, 64, generator=g, device="cuda").add_(1).bfloat16().float()
+    q, k, v = q.bfloat16(), k.bfloat16(), v.bfloat16()
+    lens = torch.randint(max(130, where + 1), N + 1, (B,), generator=g, device="cuda").to(torch.int32) if counts else torch.full((B,), N, device="cuda")
+    got = (ctx.attn_fwd_ragged(q, k, v, lens) if counts else ctx.attn_fwd(q, k, v)).view(B, N, H, 64)
+    w = a.double().exp()
+    p = w / (w + 1 + (lens.view(B, 1, 1) - 2) * np.exp(-12.0))
+    want = (p[..., None] * v[:, where].double()[:, None]).bfloat16()
+    # (2353: without the query tiles at the end that are cut by keys, which have a running maximum per part instead)
+    used = (torch.arange(N, device="cuda")[None] < lens.clamp(max=2048)[:, None])[:, :, None, None].expand_as(got)
+    if where < 128 or not counts or B > 3:                       # (small batches with counts: the kernel that knows no true maximum)
+        assert (got != want)[used].double().mean() < 0.05
+    assert ((got.float() - want.float()).abs() <= want.float() * 2.0 ** -7)[used].all()
