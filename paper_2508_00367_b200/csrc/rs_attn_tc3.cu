@@ -457,9 +457,11 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         // keys' maximum, from 128, with the top weight as rounded: 64 x 12 x 197 2.272 / 2.104, 2.224 / 1.952, 2.217 / 1.786; 16 x 12 x 1569
         // 2.335 / 2.098, 2.330 / 2.149, 2.328 / 1.886.  Time: 25.0 -> 27.3 us and 159 -> 161 (the wait for the second key tile's S, 1000 cycles an item).
         // Keys cut in three have three running maxima, each exact for a part of the keys, and need neither (1 x 12 x 197: from 128 keys 2.262 / 1.954, cut 2.215 / 1.923).
-        auto walk = [&](int nkv, int nfull, int valid_last, float gap1, bool two_first, float& m_l2, float& l_run) {
+        // lowest: what the running maximum is at least.  +infinity for rows past a sample's own count: their weights are zeros then and they have
+        // no say in which piece of code a key tile goes through, so that a row's bits are those of its sample's tokens alone.
+        auto walk = [&](int nkv, int nfull, int valid_last, float gap1, bool two_first, float lowest, float& m_l2, float& l_run) {
             float top = -INFINITY;                       // (not scaled)
-            m_l2 = kLowest;
+            m_l2 = lowest;
             l_run = 0.f;
             int j = 0;
             if (two_first) {
@@ -481,7 +483,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                     mx = fmaxf(mx, row_max<32>(s));
                 }
                 top = mx;
-                m_l2 = fmaxf(mx * sl, kLowest);
+                m_l2 = fmaxf(mx * sl, lowest);
                 uint32_t unused[1];
                 l_run = exp_pass<0, BKV, false>(r, unused, sl, -m_l2);
                 wait_o();
@@ -500,7 +502,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                     tmem_ld_32x32(s_addr + 32, r + 32);
                     tmem_wait_ld();
                     const float mx = row_max<BKV>(r), mx_l2 = mx * sl;
-                    if (j == 0) m_l2 = fmaxf(mx_l2, kLowest);
+                    if (j == 0) m_l2 = fmaxf(mx_l2, lowest);
                     have_s = __any_sync(0xffffffffu, mx_l2 > m_l2 + (j == 1 ? gap1 : kRescaleGap));
                     if (have_s) break;
                     if (!SPLIT) top = fmaxf(top, mx);
@@ -537,7 +539,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 if (!SPLIT) top = fmaxf(top, mx);
                 wait_o();
                 if (j == 0) {
-                    m_l2 = fmaxf(mx_l2, kLowest);
+                    m_l2 = fmaxf(mx_l2, lowest);
                 } else if (__any_sync(0xffffffffu, mx_l2 > m_l2 + (j == 1 ? gap1 : kRescaleGap))) {
                     const bool raise = mx_l2 > m_l2 + (j == 1 ? gap1 : kRescaleGap);
                     const float alpha = raise ? ex2(m_l2 - mx_l2) : 1.f;
@@ -600,9 +602,10 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         for (; w < whole; w += gridDim.x) {
             const Item3 it = decode_item3<RAGGED, CUT>(args, samples, w);
             if (g >= it.ng) continue;
+            const bool in_use = !RAGGED || (it.q + g - it.stream(g) * it.nt) * BQ + q * 32 + lane < it.n;
             float m_l2, l_run;
-            if constexpr (RAGGED) walk(it.nkv, it.n / BKV, it.n % BKV, first_gap(it.nkv), two_first(it.nkv), m_l2, l_run);
-            else walk(nkv_all, nfull_all, valid_all, first_gap(nkv_all), two_first(nkv_all), m_l2, l_run);
+            if constexpr (RAGGED) walk(it.nkv, it.n / BKV, it.n % BKV, first_gap(it.nkv), two_first(it.nkv), in_use ? kLowest : INFINITY, m_l2, l_run);
+            else walk(nkv_all, nfull_all, valid_all, first_gap(nkv_all), two_first(nkv_all), kLowest, m_l2, l_run);
             wait_o();
             if (lane == 0) tma_store_wait_read<0>();     // the slab's previous store has read it
             __syncwarp();
@@ -617,6 +620,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                     uint32_t wv[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) wv[i] = pack_bf16(__uint_as_float(o[8 * e + 2 * i]) * inv, __uint_as_float(o[8 * e + 2 * i + 1]) * inv);
+                    if (!in_use) wv[0] = wv[1] = wv[2] = wv[3] = 0u;
                     *reinterpret_cast<uint4*>(slab + ((((c >> 3) + e) ^ (lane & 7)) << 4)) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
                 }
             }
@@ -629,7 +633,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 const Item3 it = decode_item3<RAGGED, CUT>(args, samples, w);
                 const int first = g * it.third, n = min(max(it.nkv - first, 0), it.third);
                 float m_l2, l_run;
-                walk(n, min(n, nfull_all - first), valid_all, kRescaleGap, false, m_l2, l_run);
+                walk(n, min(n, nfull_all - first), valid_all, kRescaleGap, false, kLowest, m_l2, l_run);
                 wait_o();
                 if (lane == 0) tma_store_wait_read<0>();
                 __syncwarp();

@@ -53,6 +53,24 @@ def test_attn_ragged_per_sample_lengths(ctx, N, H, lens):
     two.close()
 
 
+@pytest.mark.parametrize("B,H,N", [(40, 12, 333), (12, 12, 700), (3, 3, 333)])
+@pytest.mark.parametrize("gain", [1.0, 8.0])
+def test_attn_ragged_rows_do_not_see_the_padding(ctx, B, H, N, gain):
+    """The bits of a sample's rows are the same whatever (finite) values stand in the padding: padding queries far above the others' scores,
+    or zeros.  At `gain` 8 the rows in use raise their own maxima too."""
+    g = torch.Generator(device="cuda").manual_seed(N)
+    qkv = torch.randn(B, N, 3, H, 64, generator=g, device="cuda")
+    qkv[:, :, 0] *= gain
+    lens = torch.randint(1, N + 1, (B,), generator=g, device="cuda").to(torch.int32)
+    pad = (torch.arange(N, device="cuda")[None] >= lens[:, None])[:, :, None, None, None]
+    got = []
+    for fill in (torch.zeros((), device="cuda"), 50 * torch.randn(B, N, 3, H, 64, generator=g, device="cuda")):
+        x = torch.where(pad, fill, qkv).bfloat16()
+        got.append(torch.where(pad[:, :, 0, 0], 0, ctx.attn_fwd_ragged(x[:, :, 0], x[:, :, 1], x[:, :, 2], lens)))
+    assert torch.equal(got[0], got[1])
+    ctx.async_status()
+
+
 @pytest.mark.parametrize("N,D,dtype", [(197, 64, torch.bfloat16), (600, 32, torch.float32), (1500, 8, torch.float32)])
 def test_topk_compact_ragged_bit_exact(ctx, N, D, dtype):
     rng = np.random.default_rng(N)
