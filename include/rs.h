@@ -266,8 +266,8 @@ RS_API rs_status rs_vit_fwd(rs_ctx* ctx, const rs_vit_desc* desc /*host*/,
  * Layout: padded.  Every sample owns N rows of its tensors; sample b's seq_lens[b] tokens sit at the
  * front of its rows, the rows behind them are padding.  Padding rows of an INPUT must hold finite
  * values (zeros will do): they are multiplied by zero weights, never selected.  Padding rows of the
- * token OUTPUT x_out are written as zeros, of keep_idx as -1; other outputs (attention rows, scores,
- * x_full) are unspecified but finite there.  seq_lens, drops, lens_out (dev): [B] int32.  Values are
+ * token OUTPUT x_out and of rs_attn_fwd_ragged's out are written as zeros, of keep_idx as -1; other outputs
+ * (scores, x_full) are unspecified but finite there.  seq_lens, drops, lens_out (dev): [B] int32.  Values are
  * read on the device and clamped there: seq_lens to [1, N], drops to [0, seq_lens[b] - 1], and the
  * kept count seq_lens[b] - drops[b] to at most the row stride of the outputs.  Tensor-core path only
  * (RS_BF16, head_dim 64; for the block D and D_mlp multiples of 128 or 192) and N <= 4608:

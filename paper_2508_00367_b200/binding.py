@@ -274,7 +274,7 @@ class Context:
     # ---- per-sample token counts (padded layout) ----
     def attn_fwd_ragged(self, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, seq_lens: torch.Tensor,
                         scale: float = 0.0, out: Optional[torch.Tensor] = None) -> torch.Tensor:
-        """rs_attn_fwd_ragged: sample b attends over its first seq_lens[b] tokens; rows behind them are unspecified."""
+        """rs_attn_fwd_ragged: sample b attends over its first seq_lens[b] tokens; rows behind them are zeros."""
         B, N, H, dh = q.shape
         assert seq_lens.dtype == torch.int32 and seq_lens.is_cuda and seq_lens.numel() == B
         if out is None:

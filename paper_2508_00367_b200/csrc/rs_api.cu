@@ -458,7 +458,7 @@ static rs_status block_fwd_impl(rs_ctx* ctx, const rs_block_desc* d, const rs_bl
         // Blocks that only the 192-column tiles take had fp32 attention weights on the fp32-FMA kernels: bf16 weights raised the
         // error of their attention score against 64 bits to 1.19x (4 x 50 tokens, D = 192; 1.08x at 32 x 197), two bf16 parts keep it.
         const bool split_weights = (D % 128) != 0 || (Dm % 128) != 0;
-        RS_CHECK_LAUNCH(ctx, RS_K_ATTN, st, rs::launch_attn_tc(ctx, ad, qkv, kp, vp, o, hk ? hk->seq_lens : nullptr, st, split_weights), "attention");
+        RS_CHECK_LAUNCH(ctx, RS_K_ATTN, st, rs::launch_attn_tc(ctx, ad, qkv, kp, vp, o, hk ? hk->seq_lens : nullptr, st, split_weights, x_full != nullptr), "attention");
         nparts = one_tail ? rs::tail_tc_parts() : rs::gemm_tc_score_parts(D);
         // shift through attention (operation choice (i)): partial sums of (SA(LN(x)) - x)^2 from this epilogue
         if (!one_tail)
@@ -552,7 +552,7 @@ rs_status rs_attn_fwd_ragged(rs_ctx* ctx, const rs_attn_desc* d, const void* q, 
     if (!(d->scale >= 0.f)) return fail(ctx, RS_ERR_INVALID_ARG, "rs_attn_fwd_ragged: scale must be >= 0");
     if (!ctx->use_tc || !rs::attn_tc_supported(*d))
         return fail(ctx, RS_ERR_UNSUPPORTED, "rs_attn_fwd_ragged: needs the tensor-core kernel (bf16, head_dim 64, strides multiples of 8)");
-    RS_CHECK_LAUNCH(ctx, RS_K_ATTN, (cudaStream_t)stream, rs::launch_attn_tc(ctx, *d, q, k, v, out, seq_lens, (cudaStream_t)stream), "tensor-core attention launch");
+    RS_CHECK_LAUNCH(ctx, RS_K_ATTN, (cudaStream_t)stream, rs::launch_attn_tc(ctx, *d, q, k, v, out, seq_lens, (cudaStream_t)stream, false, true), "tensor-core attention launch");
     return RS_OK;
 }
 

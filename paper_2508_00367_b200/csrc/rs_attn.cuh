@@ -79,5 +79,18 @@ __device__ __forceinline__ void ex2_pair_fma(uint64_t x2, float& p0, float& p1) 
     unpack2(ffma2(q, scale, 0ull), p0, p1);
 }
 
+// Zeros in the rows of out ([B, N, H, 64]) that no query tile writes: every box of 32 rows that lies past its sample's count (lens, clamped
+// to 1 .. N).  One warp per CTA, idle otherwise.
+__device__ __forceinline__ void zero_padding(__nv_bfloat16* out, const int* lens, int B, int N, int H, int lane) {
+    const int boxes = (N + 31) / 32;
+    const long long all = (long long)B * boxes;
+    for (long long i = blockIdx.x; i < all; i += gridDim.x) {
+        const int b = (int)(i / boxes), row0 = (int)(i - (long long)b * boxes) * 32;
+        if (row0 < min(max(__ldg(lens + b), 1), N)) continue;
+        uint4* p = reinterpret_cast<uint4*>(out + ((long long)b * N + row0) * H * 64);
+        for (int e = lane, n = min(32, N - row0) * H * 8; e < n; e += 32) p[e] = make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+
 }  // namespace attn
 }  // namespace rs

@@ -50,8 +50,8 @@ constexpr int OFF_BAR = OFF_OST + 8 * 4096;
 constexpr size_t kSmem = (size_t)OFF_BAR + 256 + 1024 /*alignment slack*/;
 
 struct AttnArgs {
-    __nv_bfloat16* out;      // [B, N, H*64]
-    int N, H;
+    __nv_bfloat16* out;      // [B, N, H, 64] where the caller sees the rows past a sample's own count: zeros; else null
+    int N, H, B;
     int dual;                // 1: N <= 128, an item is two heads; 0: an item is two query tiles of one head
     int per;                 // items per (sample, head) [dual = 0] or per sample [dual = 1]
     int n_items;
@@ -336,6 +336,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 cur = nxt;
             }
         }
+    } else if (warp == 10 && args.out) {
+        zero_padding(args.out, args.lens, args.B, args.N, args.H, lane);
     }
     } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftmaxRegs));
@@ -432,17 +434,18 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             if (lane == 0) tma_store_wait_read<0>();     // the slab's previous store has read it
             __syncwarp();
             uint8_t* slab = smem + OFF_OST + (g * 4 + q) * 4096 + (lane >> 3) * 1024 + (lane & 7) * 128;
+            const int row0 = (g ? it.q0[1] : it.q0[0]) + q * 32;
+            const bool in_use = row0 + lane < it.n;
 #pragma unroll
             for (int g8 = 0; g8 < 8; ++g8) {
                 uint32_t wv[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
                     wv[e] = pack_bf16(__uint_as_float(o[8 * g8 + 2 * e]) * inv, __uint_as_float(o[8 * g8 + 2 * e + 1]) * inv);
-                *reinterpret_cast<uint4*>(slab + ((g8 ^ (lane & 7)) << 4)) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
+                *reinterpret_cast<uint4*>(slab + ((g8 ^ (lane & 7)) << 4)) = in_use ? make_uint4(wv[0], wv[1], wv[2], wv[3]) : make_uint4(0u, 0u, 0u, 0u);
             }
             fence_async_smem();
             __syncwarp();
-            const int row0 = (g ? it.q0[1] : it.q0[0]) + q * 32;
             if (lane == 0 && row0 < it.n) {
                 tma_store_4d(&tmO, smem + OFF_OST + (g * 4 + q) * 4096, 0, g ? it.h[1] : it.h[0], row0, it.b);
                 tma_store_commit();
@@ -567,7 +570,7 @@ AttnPlan attn_plan(long long BH, int N, int G) {
 }
 
 cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, const void* k, const void* v,
-                           void* out, const int32_t* seq_lens, cudaStream_t st, bool split_weights) {
+                           void* out, const int32_t* seq_lens, cudaStream_t st, bool split_weights, bool write_padding) {
     if (!ctx->encode_tiled) return cudaErrorNotSupported;
     static PerDeviceOnce attr_once;   // the attribute belongs to the device current at the call
     int dev = -1;
@@ -587,6 +590,7 @@ cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, co
     const bool split = split_weights && !seq_lens;          // (this file's kernel has no such weights)
     const bool sorted = d.B <= attn_tc3_max_samples() && (ctx->attn_kernel == 3 || (d.N > BQ && (long long)d.B * d.H * ((d.N + BQ - 1) / BQ) > 2ll * ctx->sm_count));
     const bool three = split || (ctx->attn_kernel != 2 && (!seq_lens || sorted));
+    void* const padded_out = seq_lens && write_padding ? out : nullptr;
     const int kv_rows = three ? 64 : 128;                   // keys of a tile
     CUtensorMap tmQ, tmK, tmV, tmO;
     // out is [B, N, H, 64] contiguous; a softmax warp stores its 32 rows of one head at a time
@@ -595,10 +599,10 @@ cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, co
         !make_tmap_qkv(ctx, &tmK, k, d.B, d.N, d.H, d.k_batch_stride, d.k_row_stride, d.k_head_stride, kv_rows) ||
         !make_tmap_qkv(ctx, &tmV, v, d.B, d.N, d.H, d.v_batch_stride, d.v_row_stride, d.v_head_stride, kv_rows))
         return cudaErrorInvalidValue;
-    if (three) return launch_attn_tc3(ctx, d, tmQ, tmK, tmV, tmO, seq_lens, split, st);
+    if (three) return launch_attn_tc3(ctx, d, tmQ, tmK, tmV, tmO, padded_out, seq_lens, split, st);
     AttnArgs args;
-    args.out = (__nv_bfloat16*)out;
-    args.N = d.N; args.H = d.H;
+    args.out = (__nv_bfloat16*)padded_out;
+    args.N = d.N; args.H = d.H; args.B = d.B;
     args.dual = d.N <= BQ ? 1 : 0;
     args.per = args.dual ? (d.H + 1) / 2 : (d.N + 2 * BQ - 1) / (2 * BQ);
     long long items = (long long)args.per * (args.dual ? d.B : (long long)d.B * d.H);

@@ -70,6 +70,7 @@ struct Attn3Args {
     int full, rest;          // items of three tiles that fill whole rounds, tiles per item after those
     int n_whole, n_items;    // items before those with the keys cut, and in all
     const int* lens;         // RAGGED: [B], sample b attends over its first lens[b] tokens only (clamped to 1 .. N)
+    __nv_bfloat16* out;      // RAGGED: [B, N, H, 64] where the caller sees the rows past them: zeros; else null
     float scale_log2;        // scale * log2(e)
     int* status;
 };
@@ -421,6 +422,8 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 }
             }
         }
+    } else if (RAGGED && warp == 15 && args.out) {
+        zero_padding(args.out, args.lens, args.B, args.N, args.H, lane);
     }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftmaxRegs));
@@ -718,7 +721,7 @@ int attn_tc3_cut(long long BH, int N, int G) {
 
 // tmK, tmV: boxes of 64 rows; tmQ: 128 rows; tmO: 32 rows.
 cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMap& tmQ, const CUtensorMap& tmK,
-                            const CUtensorMap& tmV, const CUtensorMap& tmO, const int32_t* lens, bool split, cudaStream_t st) {
+                            const CUtensorMap& tmV, const CUtensorMap& tmO, void* padded_out, const int32_t* lens, bool split, cudaStream_t st) {
     static PerDeviceOnce attr_once;   // the attribute belongs to the device current at the call
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
@@ -751,6 +754,7 @@ cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMa
     args.n_whole = args.full + (int)((left + args.rest - 1) / args.rest);
     args.n_items = args.n_whole + (int)(BH * args.cut);
     args.lens = lens;
+    args.out = (__nv_bfloat16*)padded_out;
     const float scale = d.scale != 0.f ? d.scale : 0.125f;
     args.scale_log2 = scale * 1.4426950408889634f;
     args.status = ctx->d_status;

@@ -71,6 +71,21 @@ def test_attn_ragged_rows_do_not_see_the_padding(ctx, B, H, N, gain):
     ctx.async_status()
 
 
+@pytest.mark.parametrize("B,H,N", [(40, 12, 333), (12, 12, 700), (3, 3, 333), (5, 3, 128), (6, 2, 70)])
+def test_attn_ragged_writes_every_row(ctx, B, H, N):
+    """Rows past a sample's count are zeros over a buffer of NaN, in both kernels, whatever the padding queries hold."""
+    g = torch.Generator(device="cuda").manual_seed(N)
+    qkv = torch.randn(B, N, 3, H, 64, generator=g, device="cuda").bfloat16()
+    lens = torch.randint(1, N + 1, (B,), generator=g, device="cuda").to(torch.int32)
+    lens[0], lens[1], lens[2] = 1, N, 33
+    pad = torch.arange(N, device="cuda")[None] >= lens[:, None]
+    qkv[:, :, 0][pad] = 1e38
+    out = torch.full((B, N, H * 64), float("nan"), device="cuda").bfloat16()
+    ctx.attn_fwd_ragged(qkv[:, :, 0], qkv[:, :, 1], qkv[:, :, 2], lens, out=out)
+    ctx.async_status()
+    assert (out[pad] == 0).all() and out[~pad].isfinite().all() and (out[~pad] != 0).any(-1).all()
+
+
 @pytest.mark.parametrize("N,D,dtype", [(197, 64, torch.bfloat16), (600, 32, torch.float32), (1500, 8, torch.float32)])
 def test_topk_compact_ragged_bit_exact(ctx, N, D, dtype):
     rng = np.random.default_rng(N)

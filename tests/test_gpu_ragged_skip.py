@@ -46,10 +46,13 @@ def test_block_over_poisoned_buffers(ctx, lens, N, D):   # noqa: F811
         if parity.check_keep(ref["scores"], ref["keep_idx"], res["keep_idx"][b:b + 1, :k].numpy()) == 0:
             parity.check_float(res["x_out"][b, :k].double().numpy(), orc.round_to(ref["x_out"][0], "bf16"), "bf16", True)
         assert (res["x_out"][b, k:] == 0).all() and (res["keep_idx"][b, k:] == -1).all()
-    # with the un-pruned output asked for nothing is left out: the same rows
+    # with the un-pruned output asked for nothing is left out: the same rows, and finite ones in the padding
+    torch.cuda.empty_cache()
+    _poison()
     full = ctx.block_fwd_ragged(xd, dw, H, dl, dd, N, want_full=True)
     torch.cuda.synchronize()
     assert torch.equal(full["x_out"].cpu(), res["x_out"])
+    assert torch.isfinite(full["x_full"].float()).all() and torch.isfinite(full["scores"]).all()
     ctx.async_status()
 
 
