@@ -32,6 +32,10 @@ RS_API rs_status rs_timing_read(rs_ctx* ctx, void* stream, double* ms /*host[RS_
  * shape, box) and kept in a 128-slot cache of the context.  Hits and misses so far (host counters). */
 RS_API rs_status rs_tmap_cache_stats(const rs_ctx* ctx, long long* hits /*host*/, long long* misses /*host*/);
 
+/* The kernels' bounded waits by themselves: a small kernel whose warps wait `waits` times each for something that never happens.
+ * It ends after the limit of one wait, about two seconds, and rs_async_status then reports RS_ERR_TIMEOUT. */
+RS_API rs_status rs_wait_check(rs_ctx* ctx, int waits, void* stream);
+
 /* Which of two tensor-core attention kernels a cost model of their earlier forms expects to be the faster one for B
  * samples, H heads and N tokens on a GPU of sm_count SMs: 2 (two query tiles per thread block; also every N <= 128)
  * or 3 (three).  Host arithmetic only; needs no context and no GPU.  rs_attn_fwd takes 3 for every shape now. */

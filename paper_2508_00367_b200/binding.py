@@ -28,7 +28,8 @@ EXPORTS = ("rs_create", "rs_destroy", "rs_last_error", "rs_async_status", "rs_us
            "rs_block_workspace_bytes", "rs_block_fwd", "rs_timing_enable", "rs_timing_read",
            "rs_static_scratch_bytes", "rs_block_fwd_static", "rs_linear_fwd", "rs_vit_workspace_bytes", "rs_vit_fwd",
            "rs_vit_fwd_taps", "rs_linewise_compact", "rs_static_async_status", "rs_linear_uses_tensor_cores",
-           "rs_block_uses_tensor_cores", "rs_attn_fwd_ragged", "rs_topk_compact_ragged", "rs_block_fwd_ragged", "rs_vit_fwd_ragged", "rs_prepare_ln1_fold", "rs_attn_kernel_choice", "rs_tmap_cache_stats")
+           "rs_block_uses_tensor_cores", "rs_attn_fwd_ragged", "rs_topk_compact_ragged", "rs_block_fwd_ragged", "rs_vit_fwd_ragged", "rs_prepare_ln1_fold", "rs_attn_kernel_choice", "rs_tmap_cache_stats",
+           "rs_wait_check")
 LIN_EPILOGUE = {"bias": 0, "gelu": 1, "residual": 2}
 KERNEL_CLASSES = ("layernorm", "gemm", "attn", "score", "select", "gather")
 
@@ -155,6 +156,8 @@ def load_library() -> ctypes.CDLL:
     lib.rs_prepare_ln1_fold.restype = ci
     lib.rs_attn_kernel_choice.argtypes = [ci, ci, ci, ci]
     lib.rs_attn_kernel_choice.restype = ci
+    lib.rs_wait_check.argtypes = [vp, ci, vp]
+    lib.rs_wait_check.restype = ci
     _lib = lib
     return lib
 
@@ -226,6 +229,10 @@ class Context:
 
     def async_status(self):
         self._check(self.lib.rs_async_status(self.handle, _stream(self.device)))
+
+    def wait_check(self, waits: int):
+        """rs_wait_check: warps that wait `waits` times each for something that never happens; async_status raises afterwards."""
+        self._check(self.lib.rs_wait_check(self.handle, int(waits), _stream(self.device)))
 
     def uses_tensor_cores(self, dtype=torch.bfloat16) -> bool:
         return bool(self.lib.rs_uses_tensor_cores(self.handle, RS_BF16 if dtype == torch.bfloat16 else RS_F32))

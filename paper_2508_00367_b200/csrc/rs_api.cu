@@ -196,6 +196,13 @@ int rs_attn_kernel_choice(int sm_count, int B, int H, int N) {
     return rs::attn_plan((long long)B * H, N, sm_count).three ? 3 : 2;
 }
 
+rs_status rs_wait_check(rs_ctx* ctx, int waits, void* stream) {
+    if (!ctx) return RS_ERR_INVALID_ARG;
+    if (waits < 1) return fail(ctx, RS_ERR_INVALID_ARG, "rs_wait_check: waits must be >= 1");
+    const cudaError_t e = rs::launch_wait_check(ctx, waits, (cudaStream_t)stream);
+    return e == cudaSuccess ? RS_OK : cuda_fail(ctx, e, "wait check");
+}
+
 rs_status rs_tmap_cache_stats(const rs_ctx* ctx, long long* hits, long long* misses) {
     if (!ctx || !hits || !misses) return RS_ERR_INVALID_ARG;
     *hits = ctx->tmap_hits;

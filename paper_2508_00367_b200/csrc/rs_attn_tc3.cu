@@ -438,7 +438,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         // A wait that runs out ends the issuing threads and is reported through the status word; these warps walk on to the end
         // of their items, whose results are void then, so that no lane ever leaves a collective access to the others.
         auto wait = [&](uint64_t* bar, uint32_t parity) {
-            mbar_wait(bar, parity, abort_flag);
+            mbar_wait<false, true>(bar, parity, abort_flag);
             __syncwarp();
             tc_fence_after();
         };
@@ -691,7 +691,30 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     }
 }
 
+// The bounded waits by themselves: every warp waits n times, as the softmax warps do, for a barrier that nothing arrives at.
+__global__ void __launch_bounds__(128) wait_check_kernel(int n, int* status) {
+    __shared__ uint64_t bar;
+    __shared__ volatile int abort_flag;
+    if (threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        abort_flag = 0;
+        mbar_fence_init();
+    }
+    __syncthreads();
+    for (int i = 0; i < n; ++i) {
+        mbar_wait<false, true>(&bar, 0, &abort_flag);
+        __syncwarp();
+    }
+    __syncthreads();
+    if (abort_flag && threadIdx.x == 0) atomicExch(status, RS_DEV_TIMEOUT);
+}
+
 }  // namespace
+
+cudaError_t launch_wait_check(rs_ctx* ctx, int n, cudaStream_t st) {
+    wait_check_kernel<<<1, 128, 0, st>>>(n, ctx->d_status);
+    return cudaGetLastError();
+}
 
 int attn_tc3_max_samples() { return kMaxSamples; }
 

@@ -199,6 +199,7 @@ struct AttnPlan { long long best_hs; int three; };
 AttnPlan attn_plan(long long BH, int N, int G);
 // Three query tiles per CTA (rs_attn_tc3.cu).  padded_out: out where the rows past a sample's count are to be written.  lens as seq_lens below, with at most attn_tc3_max_samples() samples; not with split.
 int attn_tc3_max_samples();
+cudaError_t launch_wait_check(rs_ctx* ctx, int n, cudaStream_t st);
 cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMap& tmQ, const CUtensorMap& tmK,
                             const CUtensorMap& tmV, const CUtensorMap& tmO, void* padded_out, const int32_t* lens, bool split, cudaStream_t st);
 // seq_lens (optional, dev [B]): sample b attends over its first seq_lens[b] tokens only.

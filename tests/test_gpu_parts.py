@@ -378,3 +378,25 @@ def test_linear(ctx, dtype, epilogue, M, N, K):
         parity.check_float(got[rows], want, dtype, rounded_output=False)
     else:
         parity.check_float(got[rows], orc.round_to(want, dtype), dtype, rounded_output=True)
+
+
+def test_waits_that_run_out_end_the_kernel_once():
+    """A wait that nothing ends gives up after two seconds; the same thread's later ones, tens of thousands here (a thread may wait
+    twice per key tile), end at their first try, 4 us each: 0.2 s in all, where 256 tries each are 50 s.  The status says so, and
+    the context stays usable."""
+    import time
+    import paper_2508_00367_b200 as rs
+    c = rs.Context(0)
+    t0 = time.monotonic()
+    c.wait_check(50000)
+    with pytest.raises(rs.RsError) as e:
+        c.async_status()
+    assert e.value.status == 5 and 1.9 < time.monotonic() - t0 < 3.5
+    c.async_status()                                             # read once
+    a = _tok((2, 33, 768), torch.bfloat16, 3).cuda()
+    assert (c.shift_score(a, a) == 0).all()
+    c.async_status()
+    with pytest.raises(rs.RsError) as e:
+        c.wait_check(0)
+    assert e.value.status == 1
+    c.close()
