@@ -6,6 +6,8 @@
 namespace rs {
 namespace attn {
 
+constexpr float kLowest = -3.402823466e38f;      // stands for a maximum of -infinity, below which no finite one is: such scores are weights of 0
+
 __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

@@ -381,7 +381,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                           : ncol == 64 ? row_max<64, 1>(r, valid) : row_max<32, 1>(r, valid);
                 const float mx_l2 = mx * sl;
                 if (j == 0) {
-                    m_l2 = mx_l2;
+                    m_l2 = fmaxf(mx_l2, kLowest);
                 } else if (__any_sync(0xffffffffu, mx_l2 > m_l2 + kRescaleGap)) {
                     // rare: rescale O and the sum; O += P V of the previous key tile must have retired
                     if (!__all_sync(0xffffffffu, mbar_wait(&o_done[g], (cnt - 1) & 1u, abort_flag))) { ok = false; break; }

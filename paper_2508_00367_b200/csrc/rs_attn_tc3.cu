@@ -43,7 +43,6 @@ constexpr int kLaunchRegs = 128, kSoftmaxRegs = 152, kOtherRegs = 56;
 static_assert(384 * kSoftmaxRegs + 128 * kOtherRegs <= kThreads * kLaunchRegs, "register pool of the CTA");
 constexpr int kSCol = 0, kPCol = NG * BKV, kOCol = kPCol + NG * (BKV / 2);   // S 0..191, P 192..287, O 288..479
 constexpr int kTmemCols = 512;
-constexpr float kLowest = -3.402823466e38f;      // stands for a maximum of -infinity, below which no finite one is: such scores are weights of 0
 constexpr float kRescaleGap = 8.f;              // log2 units the tile maximum may exceed the running one
 // shared memory: Q[2 buffers][NG] | K[NS] | V[NS] | output staging | barriers
 constexpr int OFF_Q = 0, OFF_K = 2 * NG * Q_BYTES, OFF_V = OFF_K + NS * KV_BYTES;

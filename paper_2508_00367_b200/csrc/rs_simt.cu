@@ -298,8 +298,8 @@ template <typename T> cudaError_t dispatch_simt(SimtArgs& args, int sms, cudaStr
 // tokens of six heads and took 92 us.)
 // GROUPS: with a CTA or two to an SM a warp or two per scheduler walk through the key tiles one after the other, a chain of loads,
 // shuffles and exponentials each.  Then GROUPS times four warps share a CTA's rows, each group every GROUPS-th key tile in buffers of its own;
-// the groups' maxima, sums and outputs are merged through shared memory.  A group's tile may hold scores of -infinity only: exponents
-// are taken from 0 then, which makes all of its weights zeros.
+// the groups' maxima, sums and outputs are merged through shared memory.
+// A first key tile may hold scores of -infinity only: the maximum starts from the lowest finite number, which makes all of its weights zeros.
 constexpr int AKV = 64, AWARPS = 4, ADH = 64;
 constexpr int KLD = ADH + 4;                                  // padded row length (floats): conflict-free 16-byte accesses
 constexpr int ATT_KV_FLOATS = AKV * KLD + AKV * ADH;          // one stage: keys (padded), values
@@ -365,7 +365,7 @@ attn_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
     float m[AROWS], l[AROWS];                                  // running maximum (the warp's), this lane's share of the sum
     uint64_t o[AROWS / 2][4];                                  // rows (2p, 2p + 1) x columns 4 (lane & 15) .. + 3, keys of this half warp
 #pragma unroll
-    for (int r = 0; r < AROWS; ++r) { m[r] = -INFINITY; l[r] = 0.f; }
+    for (int r = 0; r < AROWS; ++r) { m[r] = attn::kLowest; l[r] = 0.f; }
 #pragma unroll
     for (int p = 0; p < AROWS / 2; ++p)
 #pragma unroll
@@ -407,12 +407,11 @@ attn_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
             p0[r] = lane < valid ? pair_sum(s2[r][0]) : -INFINITY;
             p1[r] = lane + 32 < valid ? pair_sum(s2[r][1]) : -INFINITY;
             const float mx = fmaxf(m[r], warp_max(fmaxf(p0[r], p1[r])));
-            const float from = GROUPS > 1 && mx == -INFINITY ? 0.f : mx;
-            corr[r] = expf(m[r] - from);                       // exp(-inf) = 0 on the first tile
+            corr[r] = expf(m[r] - mx);                         // 0 on the first tile
             raised |= mx > m[r];
             m[r] = mx;
-            p0[r] = expf(p0[r] - from);
-            p1[r] = expf(p1[r] - from);
+            p0[r] = expf(p0[r] - mx);
+            p1[r] = expf(p1[r] - mx);
             l[r] = l[r] * corr[r] + (p0[r] + p1[r]);
         }
         if (raised) {                                          // the same for the whole warp

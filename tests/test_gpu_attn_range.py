@@ -90,3 +90,23 @@ def test_the_largest_weight_is_not_rounded(ctx, B, H, N, counts, where):   # noq
     if where < 128 or not counts or B > 3:                       # (small batches with counts: the kernel that knows no true maximum)
         assert (got != want)[used].double().mean() < 0.05
     assert ((got.float() - want.float()).abs() <= want.float() * 2.0 ** -7)[used].all()
+
+
+@pytest.mark.parametrize("B,H,N", [(1, 2, 197), (4, 6, 197), (1, 12, 577), (30, 12, 300)])
+@pytest.mark.parametrize("last", [64, 128, 150])
+def test_first_keys_without_weight(ctx, pinned, B, H, N, last):   # noqa: F811
+    """Keys at -infinity that fill the first key tile (or tiles) are weights of zero in every kernel: both on the tensor cores, with and
+    without counts, and the fp32 one with one group of warps and with four."""
+    g = torch.Generator(device="cuda").manual_seed(last + N)
+    qkv = torch.randn(B, N, 3, H, 64, generator=g, device="cuda").bfloat16()
+    qkv[:, :, 0, :, 0] = 1.0
+    qkv[:, :last, 1, :, 0] = float("-inf")
+    q, k, v = (qkv[:, :, i].transpose(1, 2).double() for i in range(3))
+    want = (torch.softmax(q @ k.transpose(2, 3) / 8.0, -1) @ v).transpose(1, 2).reshape(B, N, H * 64)
+    bound = 2.0 ** -8 * v.abs().max()                                # as above
+    a = [qkv[:, :, i] for i in range(3)]
+    lens = torch.full((B,), N, dtype=torch.int32, device="cuda")
+    for c in (ctx, pinned[2], pinned[3]):
+        assert (c.attn_fwd(*a).double() - want).abs().max() < bound
+        assert (c.attn_fwd_ragged(*a, lens).double() - want).abs().max() < bound
+    assert (ctx.attn_fwd(*(t.float() for t in a)).double() - want).abs().max() < 2e-6 * v.abs().max()     # (errors of exp and of the sums)
