@@ -36,10 +36,12 @@ RS_API rs_status rs_tmap_cache_stats(const rs_ctx* ctx, long long* hits /*host*/
  * It ends after the limit of one wait, about two seconds, and rs_async_status then reports RS_ERR_TIMEOUT. */
 RS_API rs_status rs_wait_check(rs_ctx* ctx, int waits, void* stream);
 
-/* Which of two tensor-core attention kernels a cost model of their earlier forms expects to be the faster one for B
- * samples, H heads and N tokens on a GPU of sm_count SMs: 2 (two query tiles per thread block; also every N <= 128)
- * or 3 (three).  Host arithmetic only; needs no context and no GPU.  rs_attn_fwd takes 3 for every shape now. */
+/* Which of the two tensor-core attention kernels runs B samples of H heads and N tokens on a GPU of sm_count SMs: 2 (two query tiles
+ * per thread block) or 3 (three), 0 for arguments below 1.  rs_attn_fwd takes 3 for every shape; rs_attn_fwd_ragged 3 for N > 128,
+ * B <= 256 and more than two query tiles per SM, else 2.  Host arithmetic only; needs no context and no GPU, and knows
+ * nothing of RS_ATTN_KERNEL. */
 RS_API int rs_attn_kernel_choice(int sm_count, int B, int H, int N);
+RS_API int rs_attn_ragged_kernel_choice(int sm_count, int B, int H, int N);
 
 #ifdef __cplusplus
 }

@@ -191,9 +191,11 @@ int rs_uses_tensor_cores(const rs_ctx* ctx, rs_dtype dtype) {
 long long rs_launch_count(const rs_ctx* ctx) { return ctx ? ctx->launches : 0; }
 
 int rs_attn_kernel_choice(int sm_count, int B, int H, int N) {
-    if (sm_count < 1 || B < 1 || H < 1 || N < 1) return 0;
-    if (N <= 128) return 2;
-    return rs::attn_plan((long long)B * H, N, sm_count).three ? 3 : 2;
+    return sm_count < 1 || B < 1 || H < 1 || N < 1 ? 0 : rs::attn_tc_tiles(sm_count, B, H, N, false);
+}
+
+int rs_attn_ragged_kernel_choice(int sm_count, int B, int H, int N) {
+    return sm_count < 1 || B < 1 || H < 1 || N < 1 ? 0 : rs::attn_tc_tiles(sm_count, B, H, N, true);
 }
 
 rs_status rs_wait_check(rs_ctx* ctx, int waits, void* stream) {

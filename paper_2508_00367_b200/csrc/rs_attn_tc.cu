@@ -1,6 +1,6 @@
 // Fused attention on the tensor cores (Eq. sa): out = Softmax(Q K^T * scale) V per
 // (sample, head), head dimension 64, without ever writing the N x N matrix.
-// This kernel serves small batches with a count per sample, and as the other kernel's cross-check (see launch_attn_tc).
+// This kernel serves small, short or very many samples with a count each, and as the other kernel's cross-check (see attn_tc_tiles).
 //
 // Persistent kernel, one CTA per SM, looping over work items.  An item is two 128-row query
 // tiles A and B: for N > 128 two consecutive query tiles of one (sample, head), which share
@@ -492,45 +492,13 @@ bool attn_tc_supported(const rs_attn_desc& d) {
     return true;
 }
 
-// The load of the longest CTA, in tenths of three query tiles of one head, when the kernel with three tiles per CTA takes its items
-// within heads: the one or two tiles left over per head (two cost as much as three, one 7) follow the groups, on the CTAs that
-// the last round of groups left out, up to two each (wrap = 0; -1: too many), or round robin over all (wrap = 1).
-static long long three_tile_load(long long BH, int N, int G, int wrap) {
-    constexpr int NG = 3;
-    const int tiles = (N + BQ - 1) / BQ, per3 = tiles / NG, tail_ng = tiles - per3 * NG;
-    const long long n3 = BH * per3, n_tail = tail_ng ? BH : 0;
-    const int r = (int)(n3 % G), idle = G - r;
-    if (!wrap && n_tail > 2ll * idle) return -1;
-    const int stride = wrap ? G : idle, tail_cost = tail_ng == 1 ? 7 : 10;
-    long long worst = 0;
-    for (int c = 0; c < G; ++c) {
-        long long load = c < n3 ? 10 * ((n3 - c + G - 1) / G) : 0;
-        int pos = c - r;
-        if (pos < 0) {
-            if (!wrap) { worst = load > worst ? load : worst; continue; }
-            pos += G;
-        }
-        if (pos < n_tail) load += tail_cost * ((n_tail - pos + stride - 1) / stride);
-        worst = load > worst ? load : worst;
-    }
-    return worst;
-}
-// The same with items across heads.
-static long long three_tile_across_load(long long BH, int N, int G) {
-    const long long tiles = BH * ((N + BQ - 1) / BQ), left = tiles % (3ll * G);
-    return (tiles - left) / (3ll * G) * 10 + (left == 0 ? 0 : left <= G ? 7 : 10);
-}
-
 // How this kernel cuts a shape with more than one query tile per head (host side, remembered per shape).  Items go to the CTAs
 // round robin, and a pair of query tiles costs
 // twice a single one, so a last round with few pairs left keeps most SMs idle for a whole pair's time.
 // The tiles of the last few (sample, head)s are therefore handed out one by one where that shortens the
-// longest CTA: best_hs is the count with the smallest makespan under the cost model pair = 10, single = 7
+// longest CTA: their count is the one with the smallest makespan under the cost model pair = 10, single = 7
 // (a query tile alone runs faster than next to another, but not twice as fast: measured).
-// `three` is what a cost model of two earlier kernels says of this one against the one with three tiles per CTA: both paced by
-// the longest CTA, its items (in tenths) times the key tiles of an item plus a cost per item, microseconds fitted to thirteen
-// shapes from N = 197 to 4097.  rs_attn_kernel_choice reports it; the dispatch does not follow it any more (see launch_attn_tc).
-AttnPlan attn_plan(long long BH, int N, int G) {
+static long long heads_handed_out_singly(long long BH, int N, int G) {
     const int nt = (N + BQ - 1) / BQ, per = (N + 2 * BQ - 1) / (2 * BQ);
     auto makespan = [&](long long hs) {
         const long long pair_items = (BH - hs) * per, singles = hs * nt, all = pair_items + singles;
@@ -544,8 +512,8 @@ AttnPlan attn_plan(long long BH, int N, int G) {
         return worst;
     };
     static std::mutex memo_mu;
-    static std::map<std::tuple<long long, int, int>, AttnPlan> memo;
-    AttnPlan plan = {0, 0};
+    static std::map<std::tuple<long long, int, int>, long long> memo;
+    long long best_hs = 0;
     const auto key = std::make_tuple(BH, N, G);
     std::lock_guard<std::mutex> lock(memo_mu);
     const auto hit = memo.find(key);
@@ -556,17 +524,21 @@ AttnPlan attn_plan(long long BH, int N, int G) {
     if (N > BQ && BH * per <= 200000) {                   // (a host loop over the items for every candidate)
         for (long long hs = 0; hs <= hs_max; ++hs) {
             const long long m = makespan(hs);
-            if (best < 0 || m < best) { best = m; plan.best_hs = hs; }
+            if (best < 0 || m < best) { best = m; best_hs = hs; }
         }
-        const long long u_in = three_tile_load(BH, N, G, 0), u_wrap = three_tile_load(BH, N, G, 1), u3 = u_in < 0 || u_wrap < u_in ? u_wrap : u_in;
-        const double t2 = best / 10.0 * (((N + BKV - 1) / BKV) * 1.505 + 2.51) + 2.32;
-        const double t3 = u3 / 10.0 * (((N + 63) / 64) * 1.136 + 1.00) + 6.71;
-        const double two_streams = 1.0 + 0.12 * (nt % 3 ? 2.0 / nt : 0.0);
-        const double t3a = three_tile_across_load(BH, N, G) / 10.0 * (((N + 63) / 64) * 1.136 + 1.00) * two_streams + 6.71;
-        plan.three = t3 < t2 || t3a < 0.92 * t2;
     }
-    memo[key] = plan;
-    return plan;
+    memo[key] = best_hs;
+    return best_hs;
+}
+
+// Query tiles per CTA, two (this file's kernel) or three: two tiles / three, us, 4 x 16 x 4097 404 / 337, x 2305 151 / 122, 16 x 12 x 1569 207 / 160,
+// 32 x 16 x 577 101 / 74, 64 x 12 x 197 31.8 / 27.2, x 101 14.6 / 13.2, x 17 9.4 / 7.4, 1 x 12 x 197 6.3 / 5.6.  With a count per sample the kernel of three
+// first sorts the samples (up to attn_tc3_max_samples() of them), which pays from 129 tokens and two query tiles per SM on (whole ragged
+// passes, two / three: 79 x 203 x 768 1339 / 1299, 7 x 468 x 768 1056 / 1011, 12 x 1177 x 768 2234 / 2168; but 12 x 181 x 768 1814 / 1824, 1 x 160 x 1024
+// 1216 / 1234, 200 x 80 x 384 646 / 694).  RS_ATTN_KERNEL pins one (tests compare each with the oracle).
+int attn_tc_tiles(int sm_count, int B, int H, int N, bool counts) {
+    if (!counts) return 3;
+    return B <= attn_tc3_max_samples() && N > BQ && (long long)B * H * ((N + BQ - 1) / BQ) > 2ll * sm_count ? 3 : 2;
 }
 
 cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, const void* k, const void* v,
@@ -582,14 +554,10 @@ cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, co
         return (int)a;
     });
     if (e != cudaSuccess) return e;
-    // The kernel with three query tiles per CTA: two tiles / three, us, 4 x 16 x 4097 404 / 335, x 2305 151 / 122, 16 x 12 x 1569 207 / 160, 32 x 16 x 577
-    // 101 / 72, 64 x 12 x 197 31.8 / 24.1, x 101 14.1 / 11.8, x 17 9.4 / 7.4, 1 x 12 x 197 6.3 / 5.6.  With a count per sample it first sorts the samples,
-    // which pays from 129 tokens and two query tiles per SM on (whole ragged passes, two / three: 79 x 203 x 768 1339 / 1299, 7 x 468 x 768
-    // 1056 / 1011, 12 x 1177 x 768 2234 / 2168; but 12 x 181 x 768 1814 / 1824, 1 x 160 x 1024 1216 / 1234, 200 x 80 x 384 646 / 694).
-    // RS_ATTN_KERNEL pins one (tests compare each with the oracle).
     const bool split = split_weights && !seq_lens;          // (this file's kernel has no such weights)
-    const bool sorted = d.B <= attn_tc3_max_samples() && (ctx->attn_kernel == 3 || (d.N > BQ && (long long)d.B * d.H * ((d.N + BQ - 1) / BQ) > 2ll * ctx->sm_count));
-    const bool three = split || (ctx->attn_kernel != 2 && (!seq_lens || sorted));
+    const int tiles = split ? 3 : ctx->attn_kernel == 2 ? 2 : ctx->attn_kernel == 3 && (!seq_lens || d.B <= attn_tc3_max_samples()) ? 3
+                      : attn_tc_tiles(ctx->sm_count, d.B, d.H, d.N, seq_lens != nullptr);
+    const bool three = tiles == 3;
     void* const padded_out = seq_lens && write_padding ? out : nullptr;
     const int kv_rows = three ? 64 : 128;                   // keys of a tile
     CUtensorMap tmQ, tmK, tmV, tmO;
@@ -611,8 +579,7 @@ cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, co
     if (!args.dual) {
         const long long BH = (long long)d.B * d.H;
         const int nt = args.tile_count, per = args.per;
-        const AttnPlan plan = attn_plan(BH, d.N, ctx->sm_count);
-        const long long best_hs = plan.best_hs;
+        const long long best_hs = heads_handed_out_singly(BH, d.N, ctx->sm_count);
         args.n_pair_items = (int)((BH - best_hs) * per);
         args.first_single_bh = (int)(BH - best_hs);
         items = (BH - best_hs) * per + best_hs * nt;

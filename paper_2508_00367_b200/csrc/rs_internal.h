@@ -193,10 +193,8 @@ cudaError_t launch_tail_tc(rs_ctx* ctx, const TailCall& c, cudaStream_t st);
 
 // ---- tcgen05 attention (rs_attn_tc.cu): bf16, head dimension 64 ----
 bool attn_tc_supported(const rs_attn_desc& d);
-// How the two-tile kernel cuts a shape of BH (sample, head)s and N > 128 tokens on G SMs: best_hs heads are handed out tile by tile;
-// three: what rs_attn_kernel_choice reports.
-struct AttnPlan { long long best_hs; int three; };
-AttnPlan attn_plan(long long BH, int N, int G);
+// Query tiles per CTA, two (rs_attn_tc.cu) or three (rs_attn_tc3.cu), that a shape is run with on a GPU of sm_count SMs, with a count per sample or without.
+int attn_tc_tiles(int sm_count, int B, int H, int N, bool counts);
 // Three query tiles per CTA (rs_attn_tc3.cu).  padded_out: out where the rows past a sample's count are to be written.  lens as seq_lens below, with at most attn_tc3_max_samples() samples; not with split.
 int attn_tc3_max_samples();
 cudaError_t launch_wait_check(rs_ctx* ctx, int n, cudaStream_t st);

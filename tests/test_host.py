@@ -241,26 +241,28 @@ def test_ex2_polynomial_and_its_ends():
     assert (ends[:3] == 0).all() and np.isnan(ends[3])
 
 
-def test_attention_kernel_choice_follows_the_measured_winners():
-    """The cost model that picks between the two attention kernels (two or three query tiles per thread
-    block) against the kernel that is the faster one when both are timed on a B200 of 148 SMs (CUDA
-    events over graph replays), and the shapes that it is known to get wrong."""
+def test_attention_kernel_choice_is_the_rule_that_runs():
+    """Which attention kernel runs a shape (two or three query tiles per thread block) on a B200 of 148 SMs: without counts the one of
+    three, the faster one at every shape that both were timed at; with a count per sample where sorting the samples pays."""
     import paper_2508_00367_b200 as rs
-    measured = {  # (B, H, N): faster kernel
-        (4, 16, 4097): 3, (4, 16, 3073): 3, (4, 16, 1297): 3, (16, 12, 1569): 3, (16, 12, 1099): 3, (16, 12, 770): 3,
-        (32, 16, 577): 3, (32, 16, 337): 3, (64, 12, 181): 3, (64, 12, 133): 3, (1, 16, 4097): 2, (2, 12, 2353): 2,
+    measured = {  # (B, H, N): us with two tiles, with three
+        (4, 16, 4097): (404, 337), (4, 16, 2305): (151, 122), (16, 12, 1569): (207, 160), (32, 16, 577): (101, 74), (64, 12, 197): (31.8, 27.2),
+        (64, 12, 101): (14.6, 13.2), (64, 12, 17): (9.4, 7.4), (1, 12, 197): (6.3, 5.6),
     }
-    for (B, H, N), want in measured.items():
-        assert rs.attn_kernel_choice(148, B, H, N) == want, (B, H, N)
-    misses = {  # the three-tile kernel is the faster one: us with two tiles, with three
-        (4, 16, 2305): (151.3, 133.6), (4, 16, 1729): (92.1, 90.2), (16, 12, 539): (38.8, 36.7), (32, 16, 457): (59.8, 59.2),
-        (64, 12, 197): (31.8, 30.5), (8, 16, 577): (32.1, 30.3),
+    for (B, H, N), (two, three) in measured.items():
+        assert rs.attn_kernel_choice(148, B, H, N) == 3 and three < two, (B, H, N)
+    ragged = {  # (B, N, D): us of a whole pass with two tiles, with three
+        (79, 203, 768): (1339, 1299), (7, 468, 768): (1056, 1011), (12, 1177, 768): (2234, 2168), (12, 181, 768): (1814, 1824), (1, 160, 1024): (1216, 1234),
+        (200, 80, 384): (646, 694),
     }
-    for (B, H, N), (two, three) in misses.items():
-        assert rs.attn_kernel_choice(148, B, H, N) == 2 and three < two, (B, H, N)
-    for N in (1, 64, 128):
-        assert rs.attn_kernel_choice(148, 64, 12, N) == 2        # one query tile per head: two heads per item
-    assert rs.attn_kernel_choice(0, 1, 1, 1) == 0
+    for (B, N, D), (two, three) in ragged.items():
+        assert rs.attn_kernel_choice(148, B, D // 64, N, counts=True) == (3 if three < two else 2), (B, N, D)
+    assert rs.attn_kernel_choice(148, 256, 12, 1000, counts=True) == 3
+    assert rs.attn_kernel_choice(148, 257, 12, 1000, counts=True) == 2       # (the sorting kernel's limit)
+    assert [rs.attn_kernel_choice(148, B, 1, 256, counts=True) for B in (148, 149)] == [2, 3]
+    assert [rs.attn_kernel_choice(148, 256, 12, N, counts=True) for N in (128, 129)] == [2, 3]
+    for counts in (False, True):
+        assert rs.attn_kernel_choice(0, 1, 1, 1, counts) == 0 and rs.attn_kernel_choice(148, 1, 1, 0, counts) == 0
 
 
 def test_a_layer_loop_of_no_blocks_can_be_made():
