@@ -535,10 +535,11 @@ static long long heads_handed_out_singly(long long BH, int N, int G) {
 // 32 x 16 x 577 101 / 74, 64 x 12 x 197 31.8 / 27.2, x 101 14.6 / 13.2, x 17 9.4 / 7.4, 1 x 12 x 197 6.3 / 5.6.  With a count per sample the kernel of three
 // first sorts the samples (up to attn_tc3_max_samples() of them), which pays from 129 tokens and two query tiles per SM on (whole ragged
 // passes, two / three: 79 x 203 x 768 1339 / 1299, 7 x 468 x 768 1056 / 1011, 12 x 1177 x 768 2234 / 2168; but 12 x 181 x 768 1814 / 1824, 1 x 160 x 1024
-// 1216 / 1234, 200 x 80 x 384 646 / 694).  RS_ATTN_KERNEL pins one (tests compare each with the oracle).
+// 1216 / 1234, 200 x 80 x 384 646 / 694).  0: more tiles than the kernel counts.  RS_ATTN_KERNEL pins one (tests compare each with the oracle).
 int attn_tc_tiles(int sm_count, int B, int H, int N, bool counts) {
-    if (!counts) return 3;
-    return B <= attn_tc3_max_samples() && N > BQ && (long long)B * H * ((N + BQ - 1) / BQ) > 2ll * sm_count ? 3 : 2;
+    const long long tiles = (long long)B * H * ((N + BQ - 1) / BQ);
+    if (!counts) return tiles < attn_tc3_max_tiles() ? 3 : 0;
+    return B <= attn_tc3_max_samples() && N > BQ && tiles > 2ll * sm_count && tiles < attn_tc3_max_tiles() ? 3 : 2;
 }
 
 cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, const void* k, const void* v,
@@ -557,6 +558,7 @@ cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, co
     const bool split = split_weights && !seq_lens;          // (this file's kernel has no such weights)
     const int tiles = split ? 3 : ctx->attn_kernel == 2 ? 2 : ctx->attn_kernel == 3 && (!seq_lens || d.B <= attn_tc3_max_samples()) ? 3
                       : attn_tc_tiles(ctx->sm_count, d.B, d.H, d.N, seq_lens != nullptr);
+    if (!tiles) return cudaErrorInvalidValue;
     const bool three = tiles == 3;
     void* const padded_out = seq_lens && write_padding ? out : nullptr;
     const int kv_rows = three ? 64 : 128;                   // keys of a tile

@@ -716,6 +716,8 @@ cudaError_t launch_wait_check(rs_ctx* ctx, int n, cudaStream_t st) {
 }
 
 int attn_tc3_max_samples() { return kMaxSamples; }
+// Tiles and items are counted in ints, with room for a stride of the grid past the last.
+long long attn_tc3_max_tiles() { return (1ll << 31) - (1 << 20); }
 
 // How many query tiles of every head are taken with the keys cut in three: the count with the shortest longest CTA.  An item of one, two
 // or three query tiles takes 0.62, 0.80 or 1.03 us per key tile and 1.3, one with the keys cut 1.03 per key tile of a third and 1.4;
@@ -761,7 +763,7 @@ cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMa
     const int G = ctx->sm_count;
     const long long BH = (long long)d.B * d.H;
     const int nt = (d.N + BQ - 1) / BQ;
-    if (BH * nt >= (1ll << 30)) return cudaErrorInvalidValue;
+    if (BH * nt >= attn_tc3_max_tiles()) return cudaErrorInvalidValue;
     args.cut = lens ? 0 : attn_tc3_cut(BH, d.N, G);
     args.nt = nt - args.cut;
     const long long tiles = BH * args.nt, left = tiles % (NG * (long long)G);

@@ -193,10 +193,12 @@ cudaError_t launch_tail_tc(rs_ctx* ctx, const TailCall& c, cudaStream_t st);
 
 // ---- tcgen05 attention (rs_attn_tc.cu): bf16, head dimension 64 ----
 bool attn_tc_supported(const rs_attn_desc& d);
-// Query tiles per CTA, two (rs_attn_tc.cu) or three (rs_attn_tc3.cu), that a shape is run with on a GPU of sm_count SMs, with a count per sample or without.
+// Query tiles per CTA, two (rs_attn_tc.cu) or three (rs_attn_tc3.cu), that a shape is run with on a GPU of sm_count SMs, with a count per sample or without;
+// 0: refused.
 int attn_tc_tiles(int sm_count, int B, int H, int N, bool counts);
 // Three query tiles per CTA (rs_attn_tc3.cu).  padded_out: out where the rows past a sample's count are to be written.  lens as seq_lens below, with at most attn_tc3_max_samples() samples; not with split.
 int attn_tc3_max_samples();
+long long attn_tc3_max_tiles();
 cudaError_t launch_wait_check(rs_ctx* ctx, int n, cudaStream_t st);
 cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMap& tmQ, const CUtensorMap& tmK,
                             const CUtensorMap& tmV, const CUtensorMap& tmO, void* padded_out, const int32_t* lens, bool split, cudaStream_t st);

@@ -261,6 +261,8 @@ def test_attention_kernel_choice_is_the_rule_that_runs():
     assert rs.attn_kernel_choice(148, 257, 12, 1000, counts=True) == 2       # (the sorting kernel's limit)
     assert [rs.attn_kernel_choice(148, B, 1, 256, counts=True) for B in (148, 149)] == [2, 3]
     assert [rs.attn_kernel_choice(148, 256, 12, N, counts=True) for N in (128, 129)] == [2, 3]
+    assert rs.attn_kernel_choice(148, 32768, 32768, 1) == 3                  # 2^30 query tiles of one token: 137 GB of output
+    assert rs.attn_kernel_choice(148, 65535, 65535, 1) == 0
     for counts in (False, True):
         assert rs.attn_kernel_choice(0, 1, 1, 1, counts) == 0 and rs.attn_kernel_choice(148, 1, 1, 0, counts) == 0
 
