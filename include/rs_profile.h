@@ -43,6 +43,8 @@ RS_API rs_status rs_wait_check(rs_ctx* ctx, int waits, void* stream);
  * nothing of RS_ATTN_KERNEL. */
 RS_API int rs_attn_kernel_choice(int sm_count, int B, int H, int N);
 RS_API int rs_attn_ragged_kernel_choice(int sm_count, int B, int H, int N);
+/* How many of a head's ceil(N / 128) query tiles rs_attn_fwd takes with their keys cut in three (the last ones of every head). */
+RS_API int rs_attn_key_cut(int sm_count, int B, int H, int N);
 
 #ifdef __cplusplus
 }

@@ -29,7 +29,7 @@ EXPORTS = ("rs_create", "rs_destroy", "rs_last_error", "rs_async_status", "rs_us
            "rs_static_scratch_bytes", "rs_block_fwd_static", "rs_linear_fwd", "rs_vit_workspace_bytes", "rs_vit_fwd",
            "rs_vit_fwd_taps", "rs_linewise_compact", "rs_static_async_status", "rs_linear_uses_tensor_cores",
            "rs_block_uses_tensor_cores", "rs_attn_fwd_ragged", "rs_topk_compact_ragged", "rs_block_fwd_ragged", "rs_vit_fwd_ragged", "rs_prepare_ln1_fold", "rs_attn_kernel_choice", "rs_tmap_cache_stats",
-           "rs_wait_check", "rs_attn_ragged_kernel_choice")
+           "rs_wait_check", "rs_attn_ragged_kernel_choice", "rs_attn_key_cut")
 LIN_EPILOGUE = {"bias": 0, "gelu": 1, "residual": 2}
 KERNEL_CLASSES = ("layernorm", "gemm", "attn", "score", "select", "gather")
 
@@ -154,7 +154,7 @@ def load_library() -> ctypes.CDLL:
     lib.rs_vit_fwd_ragged.restype = ci
     lib.rs_prepare_ln1_fold.argtypes = [vp, ci, ci, vp, vp, vp, vp, vp, vp, vp, vp]
     lib.rs_prepare_ln1_fold.restype = ci
-    for choice in (lib.rs_attn_kernel_choice, lib.rs_attn_ragged_kernel_choice):
+    for choice in (lib.rs_attn_kernel_choice, lib.rs_attn_ragged_kernel_choice, lib.rs_attn_key_cut):
         choice.argtypes = [ci, ci, ci, ci]
         choice.restype = ci
     lib.rs_wait_check.argtypes = [vp, ci, vp]
@@ -168,6 +168,11 @@ def attn_kernel_choice(sm_count: int, B: int, H: int, N: int, counts: bool = Fal
     attention kernel that runs the shape (host arithmetic only)."""
     lib = load_library()
     return int((lib.rs_attn_ragged_kernel_choice if counts else lib.rs_attn_kernel_choice)(sm_count, B, H, N))
+
+
+def attn_key_cut(sm_count: int, B: int, H: int, N: int) -> int:
+    """rs_attn_key_cut: query tiles of every head that attention without counts takes with their keys cut in three (host arithmetic only)."""
+    return int(load_library().rs_attn_key_cut(sm_count, B, H, N))
 
 
 def _dt(t: torch.Tensor) -> int:

@@ -194,6 +194,10 @@ int rs_attn_kernel_choice(int sm_count, int B, int H, int N) {
     return sm_count < 1 || B < 1 || H < 1 || N < 1 ? 0 : rs::attn_tc_tiles(sm_count, B, H, N, false);
 }
 
+int rs_attn_key_cut(int sm_count, int B, int H, int N) {
+    return sm_count < 1 || B < 1 || H < 1 || N < 1 || rs::attn_tc_tiles(sm_count, B, H, N, false) != 3 ? 0 : rs::attn_tc3_cut((long long)B * H, N, sm_count);
+}
+
 int rs_attn_ragged_kernel_choice(int sm_count, int B, int H, int N) {
     return sm_count < 1 || B < 1 || H < 1 || N < 1 ? 0 : rs::attn_tc_tiles(sm_count, B, H, N, true);
 }

@@ -199,6 +199,7 @@ int attn_tc_tiles(int sm_count, int B, int H, int N, bool counts);
 // Three query tiles per CTA (rs_attn_tc3.cu).  padded_out: out where the rows past a sample's count are to be written.  lens as seq_lens below, with at most attn_tc3_max_samples() samples; not with split.
 int attn_tc3_max_samples();
 long long attn_tc3_max_tiles();
+int attn_tc3_cut(long long BH, int N, int G);       // query tiles of every head with the keys cut in three
 cudaError_t launch_wait_check(rs_ctx* ctx, int n, cudaStream_t st);
 cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMap& tmQ, const CUtensorMap& tmK,
                             const CUtensorMap& tmV, const CUtensorMap& tmO, void* padded_out, const int32_t* lens, bool split, cudaStream_t st);
