@@ -59,7 +59,7 @@ struct AttnArgs {
     // tile_count of them for each (sample, head) from first_single_bh on (see launch_attn_tc)
     int n_pair_items, first_single_bh, tile_count;
     float scale_log2;        // scale * log2(e)
-    const int* lens;         // optional [B]: sample b attends over its first lens[b] tokens only (clamped to 1 .. N)
+    const int* lens;         // COUNTS: [B], sample b attends over its first lens[b] tokens only (clamped to 1 .. N)
     int* status;
 };
 
@@ -71,14 +71,14 @@ struct Item {
     int nkv;                 // key tiles per query tile
     int slots;               // K/V ring stages the item consumes
 };
-__device__ __forceinline__ Item decode_item(const AttnArgs& a, int w) {
+template <bool COUNTS> __device__ __forceinline__ Item decode_item(const AttnArgs& a, int w) {
     Item it;
     if (a.dual) {
         const int hp = w % a.per;
         it.b = w / a.per;
         it.h[0] = 2 * hp; it.h[1] = 2 * hp + 1;
         it.q0[0] = it.q0[1] = 0;
-        it.n = a.lens ? min(max(__ldg(a.lens + it.b), 1), a.N) : a.N;
+        it.n = COUNTS ? min(max(__ldg(a.lens + it.b), 1), a.N) : a.N;
         it.ng = it.h[1] < a.H ? 2 : 1;
         it.nkv = 1;
         it.slots = it.ng;
@@ -95,7 +95,7 @@ __device__ __forceinline__ Item decode_item(const AttnArgs& a, int w) {
         }
         it.b = bh / a.H;
         it.h[0] = it.h[1] = bh % a.H;
-        it.n = a.lens ? min(max(__ldg(a.lens + it.b), 1), a.N) : a.N;
+        it.n = COUNTS ? min(max(__ldg(a.lens + it.b), 1), a.N) : a.N;
         it.ng = (it.q0[0] < it.n ? 1 : 0) + (it.q0[1] < it.n ? 1 : 0);
         it.nkv = (it.n + BKV - 1) / BKV;
         it.slots = it.nkv;
@@ -103,9 +103,9 @@ __device__ __forceinline__ Item decode_item(const AttnArgs& a, int w) {
     return it;
 }
 // First item at or after w (in this CTA's stride) that has work; n_items if none.
-__device__ __forceinline__ int next_item(const AttnArgs& a, int w, int stride) {
-    if (!a.lens) return w;
-    while (w < a.n_items && decode_item(a, w).ng == 0) w += stride;
+template <bool COUNTS> __device__ __forceinline__ int next_item(const AttnArgs& a, int w, int stride) {
+    if (!COUNTS) return w;
+    while (w < a.n_items && decode_item<COUNTS>(a, w).ng == 0) w += stride;
     return w;
 }
 
@@ -164,7 +164,8 @@ __device__ __forceinline__ float exp_pass(uint32_t (&r)[128], float sl, float mn
 // FINE: partial key tiles are handled by 32-column groups (worth it when a sequence is a few
 // tiles long).  Without it the one partial tile of a long sequence is a full tile with every
 // element tested, and the kernel carries less code around its inner loop, which that loop feels.
-template <bool FINE>
+// COUNTS: with a count per sample (args.lens).
+template <bool FINE, bool COUNTS>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO, const AttnArgs args) {
@@ -213,8 +214,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         if (elect_one()) {
             uint32_t kv_it = 0, item_n = 0;
             bool ok = true;
-            for (int w = next_item(args, blockIdx.x, gridDim.x); w < args.n_items && ok; w = next_item(args, w + gridDim.x, gridDim.x), ++item_n) {
-                const Item it = decode_item(args, w);
+            for (int w = next_item<COUNTS>(args, blockIdx.x, gridDim.x); w < args.n_items && ok; w = next_item<COUNTS>(args, w + gridDim.x, gridDim.x), ++item_n) {
+                const Item it = decode_item<COUNTS>(args, w);
                 const uint32_t qb = item_n & 1u;
                 if (!mbar_wait(&q_empty[qb], ((item_n >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
                 mbar_expect_tx(&q_full[qb], it.ng * TILE_BYTES);
@@ -239,7 +240,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         }
     } else if (warp == 9) {
         // ---------------- MMA issuer ----------------
-        if (elect_one() && next_item(args, blockIdx.x, gridDim.x) < args.n_items) {
+        if (elect_one() && next_item<COUNTS>(args, blockIdx.x, gridDim.x) < args.n_items) {
             constexpr uint32_t idesc_o = idesc_bf16(BQ, DH, 0, 1), idesc_s_full = idesc_bf16(BQ, BKV, 0, 0);
             // descriptors as halves: per product only the low half moves (address >> 4)
             constexpr uint32_t kTile16 = TILE_BYTES >> 4;
@@ -290,15 +291,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             };
 
             uint32_t item_n = 0, kv0 = 0;
-            int w = next_item(args, blockIdx.x, gridDim.x);
-            Item cur = decode_item(args, w);
+            int w = next_item<COUNTS>(args, blockIdx.x, gridDim.x);
+            Item cur = decode_item<COUNTS>(args, w);
             ok = mbar_wait(&q_full[0], 0, abort_flag);
 #pragma unroll
             for (int g = 0; g < 2; ++g)
                 if (ok && g < cur.ng) issue_s_one(cur, 0, kv0, 0, g);
             while (ok) {
                 const uint32_t qb = item_n & 1u;
-                const int wn = next_item(args, w + gridDim.x, gridDim.x);
+                const int wn = next_item<COUNTS>(args, w + gridDim.x, gridDim.x);
                 Item nxt = cur;
                 for (int j = 0; j < cur.nkv && ok; ++j) {
                     // Look ahead, per query tile: the tile's next Q K^T (of this item, or the first of the
@@ -309,7 +310,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                     const bool ahead = !last || wn < args.n_items;
                     const uint32_t nb = last ? (item_n + 1) & 1u : qb;
                     if (last && ahead) {
-                        nxt = decode_item(args, wn);
+                        nxt = decode_item<COUNTS>(args, wn);
                         if (!mbar_wait(&q_full[nb], ((item_n + 1) >> 1) & 1u, abort_flag)) { ok = false; break; }
                     }
                     const Item& sit = last ? nxt : cur;
@@ -336,7 +337,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 cur = nxt;
             }
         }
-    } else if (warp == 10 && args.out) {
+    } else if (COUNTS && warp == 10 && args.out) {
         zero_padding(args.out, args.lens, args.B, args.N, args.H, lane);
     }
     } else {
@@ -352,7 +353,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         uint32_t cnt = 0, item_n = 0;                    // tiles / items this warpgroup has walked through
         bool ok = true;
         for (int w = blockIdx.x; w < args.n_items && ok; w += gridDim.x, ++item_n) {
-            const Item it = decode_item(args, w);
+            const Item it = decode_item<COUNTS>(args, w);
             if (g >= it.ng) continue;
             float m_l2 = 0.f, l_run = 0.f;               // running maximum (times scale*log2 e) and sum
             for (int j = 0; j < it.nkv && ok; ++j, ++cnt) {
@@ -435,7 +436,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             __syncwarp();
             uint8_t* slab = smem + OFF_OST + (g * 4 + q) * 4096 + (lane >> 3) * 1024 + (lane & 7) * 128;
             const int row0 = (g ? it.q0[1] : it.q0[0]) + q * 32;
-            const bool in_use = row0 + lane < it.n;
+            const bool in_use = !COUNTS || row0 + lane < it.n;
 #pragma unroll
             for (int g8 = 0; g8 < 8; ++g8) {
                 uint32_t wv[4];
@@ -538,6 +539,10 @@ static long long heads_handed_out_singly(long long BH, int N, int G) {
 // 1216 / 1234, 200 x 80 x 384 646 / 694).  0: more tiles than the kernel counts.  RS_ATTN_KERNEL pins one (tests compare each with the oracle).
 int attn_tc_tiles(int sm_count, int B, int H, int N, bool counts) {
     const long long tiles = (long long)B * H * ((N + BQ - 1) / BQ);
+    // Nearly 128 tokens, a round of this kernel's pairs but two tiles a CTA of the other's: there the second key tile, which raises the maximum of most
+    // rows, is not hidden behind a third tile.  Two / three, us, 20 x 12 heads: x 112 6.7 / 6.6, x 120 6.6 / 7.0, x 128 6.4 / 7.2; of 128 tokens, whose one
+    // key tile is whole here, already with a tile a CTA, 12 x 12 5.7 / 5.9 (x 120 5.9 / 5.8); 37 x 12 x 128 10.3 / 9.5, x 120 10.9 / 9.1.
+    if (!counts && N > 112 && N <= BQ && tiles <= 2ll * sm_count && (N == BQ || tiles > sm_count)) return 2;
     if (!counts) return tiles < attn_tc3_max_tiles() ? 3 : 0;
     return B <= attn_tc3_max_samples() && N > BQ && tiles > 2ll * sm_count && tiles < attn_tc3_max_tiles() ? 3 : 2;
 }
@@ -550,8 +555,9 @@ cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, co
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     e = (cudaError_t)attr_once.run(dev, [] {
-        cudaError_t a = cudaFuncSetAttribute(attn_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-        if (a == cudaSuccess) a = cudaFuncSetAttribute(attn_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+        cudaError_t a = cudaSuccess;
+        for (const void* f : {(const void*)attn_tc_kernel<true, false>, (const void*)attn_tc_kernel<true, true>, (const void*)attn_tc_kernel<false, false>, (const void*)attn_tc_kernel<false, true>})
+            if (a == cudaSuccess) a = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
         return (int)a;
     });
     if (e != cudaSuccess) return e;
@@ -596,8 +602,9 @@ cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, co
     const int nkv = (d.N + BKV - 1) / BKV;
     const int grid = args.n_items < ctx->sm_count ? args.n_items : ctx->sm_count;
     // a partial key tile is worth its own code when it is a good part of the sequence
-    if (nkv <= 12) return launch_pdl(attn_tc_kernel<true>, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args);
-    return launch_pdl(attn_tc_kernel<false>, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args);
+    auto run = [&](auto kernel) { return launch_pdl(kernel, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args); };
+    if (nkv <= 12) return seq_lens ? run(attn_tc_kernel<true, true>) : run(attn_tc_kernel<true, false>);
+    return seq_lens ? run(attn_tc_kernel<false, true>) : run(attn_tc_kernel<false, false>);
 }
 
 }  // namespace rs

@@ -505,7 +505,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                     tmem_wait_ld();
                     const float mx = row_max<BKV>(r), mx_l2 = mx * sl;
                     if (j == 0) m_l2 = fmaxf(mx_l2, lowest);
-                    have_s = __any_sync(0xffffffffu, mx_l2 > m_l2 + (j == 1 ? gap1 : kRescaleGap));
+                    have_s = __any_sync(0xffffffffu, mx_l2 > m_l2 + kRescaleGap);
                     if (have_s) break;
                     if (!SPLIT) top = fmaxf(top, mx);
                     float l_tile = exp_pass<0, BKV / 2, SPLIT>(r, lo, sl, -m_l2);
@@ -598,7 +598,9 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         };
         auto first_gap = [](int nkv) { return !SPLIT && nkv == 2 ? 0.f : kRescaleGap; };
         auto two_first = [](int nkv) { return !SPLIT && nkv > 2; };
-        const int nkv_all = (args.N + BKV - 1) / BKV, nfull_all = args.N / BKV, valid_all = args.N % BKV;
+        // Whole key tiles.  The second of two counts as one with 64 keys: nearly all of them raise the maximum.
+        auto whole_tiles = [](int n) { return !SPLIT && n <= 2 * BKV ? n >= BKV : n / BKV; };
+        const int nkv_all = (args.N + BKV - 1) / BKV, nfull_all = whole_tiles(args.N), valid_all = args.N - nfull_all * BKV;
         const int whole = CUT ? args.n_whole : n_items;
         int w = blockIdx.x;
         for (; w < whole; w += gridDim.x) {
@@ -606,7 +608,7 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             if (g >= it.ng) continue;
             const bool in_use = !RAGGED || (it.q + g - it.stream(g) * it.nt) * BQ + q * 32 + lane < it.n;
             float m_l2, l_run;
-            if constexpr (RAGGED) walk(it.nkv, it.n / BKV, it.n % BKV, first_gap(it.nkv), two_first(it.nkv), in_use ? kLowest : INFINITY, m_l2, l_run);
+            if constexpr (RAGGED) walk(it.nkv, whole_tiles(it.n), it.n - whole_tiles(it.n) * BKV, first_gap(it.nkv), two_first(it.nkv), in_use ? kLowest : INFINITY, m_l2, l_run);
             else walk(nkv_all, nfull_all, valid_all, first_gap(nkv_all), two_first(nkv_all), kLowest, m_l2, l_run);
             wait_o();
             if (lane == 0) tma_store_wait_read<0>();     // the slab's previous store has read it
