@@ -82,15 +82,18 @@ __device__ __forceinline__ void ex2_pair_fma(uint64_t x2, float& p0, float& p1) 
 }
 
 // Zeros in the rows of out ([B, N, H, 64]) that no query tile writes: every box of 32 rows that lies past its sample's count (lens, clamped
-// to 1 .. N).  One warp per CTA, idle otherwise.
+// to 1 .. N).  One warp per CTA, idle otherwise; eight rows at a time, so that few samples are spread over the CTAs too, and a lane
+// to look up whether they are to be written.
 __device__ __forceinline__ void zero_padding(__nv_bfloat16* out, const int* lens, int B, int N, int H, int lane) {
-    const int boxes = (N + 31) / 32;
-    const long long all = (long long)B * boxes;
-    for (long long i = blockIdx.x; i < all; i += gridDim.x) {
-        const int b = (int)(i / boxes), row0 = (int)(i - (long long)b * boxes) * 32;
-        if (row0 < min(max(__ldg(lens + b), 1), N)) continue;
-        uint4* p = reinterpret_cast<uint4*>(out + ((long long)b * N + row0) * H * 64);
-        for (int e = lane, n = min(32, N - row0) * H * 8; e < n; e += 32) p[e] = make_uint4(0u, 0u, 0u, 0u);
+    const int parts = (N + 7) / 8, all = B * parts;          // (B * N rows of 128 bytes fit a GPU)
+    for (int first = blockIdx.x; first < all; first += 32 * gridDim.x) {
+        const int i = first + lane * gridDim.x, b = i / parts, row0 = (i - b * parts) * 8;
+        uint32_t left = __ballot_sync(0xffffffffu, i < all && (row0 & ~31) >= min(max(__ldg(lens + min(b, B - 1)), 1), N));
+        for (; left; left &= left - 1) {
+            const int src = __ffs(left) - 1, fb = __shfl_sync(0xffffffffu, b, src), fr = __shfl_sync(0xffffffffu, row0, src);
+            uint4* p = reinterpret_cast<uint4*>(out + ((long long)fb * N + fr) * H * 64);
+            for (int e = lane, n = min(8, N - fr) * H * 8; e < n; e += 32) p[e] = make_uint4(0u, 0u, 0u, 0u);
+        }
     }
 }
 

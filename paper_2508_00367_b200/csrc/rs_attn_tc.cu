@@ -566,7 +566,7 @@ cudaError_t launch_attn_tc(rs_ctx* ctx, const rs_attn_desc& d, const void* q, co
                       : attn_tc_tiles(ctx->sm_count, d.B, d.H, d.N, seq_lens != nullptr);
     if (!tiles) return cudaErrorInvalidValue;
     const bool three = tiles == 3;
-    void* const padded_out = seq_lens && write_padding ? out : nullptr;
+    void* const padded_out = seq_lens && write_padding && d.N > 32 ? out : nullptr;     // (the first box of 32 rows holds a token)
     const int kv_rows = three ? 64 : 128;                   // keys of a tile
     CUtensorMap tmQ, tmK, tmV, tmO;
     // out is [B, N, H, 64] contiguous; a softmax warp stores its 32 rows of one head at a time
