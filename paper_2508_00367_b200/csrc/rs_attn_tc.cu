@@ -104,8 +104,9 @@ template <bool COUNTS> __device__ __forceinline__ Item decode_item(const AttnArg
 }
 // First item at or after w (in this CTA's stride) that has work; n_items if none.
 template <bool COUNTS> __device__ __forceinline__ int next_item(const AttnArgs& a, int w, int stride) {
-    if (!COUNTS) return w;
-    while (w < a.n_items && decode_item<COUNTS>(a, w).ng == 0) w += stride;
+    if constexpr (COUNTS) {
+        while (w < a.n_items && decode_item<COUNTS>(a, w).ng == 0) w += stride;
+    }
     return w;
 }
 
