@@ -97,6 +97,22 @@ def test_counts_per_sample_sorted(ctx, B, H, N, longest, per, gain):   # noqa: F
         assert err.abs().max() < 2.0 ** -8 * qkv[b, :n, 2].double().abs().max(), (b, n)
 
 
+@pytest.mark.parametrize("counts", ["equal", "one key tile apart", "one long"])
+def test_every_sample_of_a_sorted_batch(ctx, counts):   # noqa: F811
+    """256 samples, the most that are sorted, and ties in their order: every row of every sample is written, once, with its own sample's result."""
+    B, H, N = 256, 3, 197
+    g = torch.Generator(device="cuda").manual_seed(B)
+    qkv = torch.randn(B, N, 3, H, 64, generator=g, device="cuda").bfloat16()
+    lens = {"equal": torch.full((B,), 150), "one key tile apart": torch.arange(B) % 4 * 64 + 1, "one long": torch.tensor([1] * (B - 1) + [N])}[counts].to(torch.int32).cuda()
+    got = ctx.attn_fwd_ragged(qkv[:, :, 0], qkv[:, :, 1], qkv[:, :, 2], lens, out=torch.full((B, N, H * 64), float("nan"), dtype=torch.bfloat16, device="cuda"))
+    ctx.async_status()
+    q, k, v = (qkv[:, :, i].transpose(1, 2).double() for i in range(3))
+    past = torch.arange(N, device="cuda")[None] >= lens[:, None]
+    s = (q @ k.transpose(2, 3) / 8.0).masked_fill(past[:, None, None], float("-inf"))
+    want = (torch.softmax(s, -1) @ v).transpose(1, 2).reshape(B, N, -1).masked_fill(past[..., None], 0.0)
+    assert _close(got, want, qkv)
+
+
 @pytest.mark.parametrize("B,H,N", [(1, 3, 65), (1, 1, 127), (1, 2, 200), (1, 3, 257), (1, 9, 256), (2, 6, 197), (1, 2, 600)])
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 def test_fp32_key_tiles_in_groups(ctx, B, H, N, dtype):   # noqa: F811
