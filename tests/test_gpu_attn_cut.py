@@ -113,6 +113,24 @@ def test_every_sample_of_a_sorted_batch(ctx, counts):   # noqa: F811
     assert _close(got, want, qkv)
 
 
+@pytest.mark.parametrize("B", [74, 75])
+@pytest.mark.parametrize("H", [1, 2, 3, 4])
+def test_tiles_to_an_item_of_a_sorted_batch(ctx, B, H):   # noqa: F811
+    """Two query tiles per head: as many as fill one, two, three and four rounds of 148, and a sample more, on both sides of where one, two or
+    three go to an item."""
+    import paper_2508_00367_b200 as rs
+    N = 600
+    assert rs.attn_kernel_choice(148, B, H, N, counts=True) == 3
+    g = torch.Generator(device="cuda").manual_seed(B + H)
+    qkv = torch.randn(B, N, 3, H, 64, generator=g, device="cuda").bfloat16()
+    lens = (129 + torch.arange(B) * 50 % 128).to(torch.int32).cuda()
+    got = ctx.attn_fwd_ragged(qkv[:, :, 0], qkv[:, :, 1], qkv[:, :, 2], lens)
+    ctx.async_status()
+    for b in range(0, B, 3):
+        n = int(lens[b])
+        assert _close(got[b:b + 1, :n], _reference(qkv[b:b + 1, :n]), qkv[b:b + 1, :n]), (b, n)
+
+
 @pytest.mark.parametrize("B,H,N", [(1, 3, 65), (1, 1, 127), (1, 2, 200), (1, 3, 257), (1, 9, 256), (2, 6, 197), (1, 2, 600)])
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 def test_fp32_key_tiles_in_groups(ctx, B, H, N, dtype):   # noqa: F811
