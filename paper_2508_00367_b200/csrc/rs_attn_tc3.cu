@@ -236,8 +236,8 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     if constexpr (RAGGED) {
         // Samples by key tiles, the most first (its place: how many come before it), and the items before each; a warp to a
         // sample, whose lanes keep what they compare it with in registers.  (A thread to a sample: 30 x 89 tokens 4.7 us for the loops.
-        // Tiles and items worked out at each comparison: 256 x 3 x 129 30.6 us instead
-        // of 18.6, 256 x 3 x 197 38.3 of 25.9, 64 x 12 x 197 24.0 of 23.0.)
+        // Tiles and items worked out at each comparison: 256 x 3 x 129 30.6 us instead of
+        // 18.6, 256 x 3 x 197 38.3 of 25.9, 64 x 12 x 197 24.0 of 23.0.)
         static_assert(kMaxSamples <= kThreads && kMaxSamples <= 256, "a thread to a sample's count, its index in eight bits");
         constexpr int PER_LANE = kMaxSamples / 32;
         uint32_t* keys = reinterpret_cast<uint32_t*>(smem + OFF_OST);        // (not in use yet)
@@ -249,17 +249,22 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         }
         __syncthreads();
         uint32_t key[PER_LANE];
-        int items[PER_LANE], all = 0;
+        int items[PER_LANE], n1 = 0, n2 = 0, n3 = 0;                         // items in all with one, two or three query tiles each
 #pragma unroll
         for (int i = 0; i < PER_LANE; ++i) {
             key[i] = keys[lane + 32 * i];
             items[i] = tiles[lane + 32 * i];
-            all += items[i];
+            n1 += items[i];
+            n2 += (items[i] + 1) / 2;
+            n3 += (items[i] + 2) / 3;
         }
-        all = __reduce_add_sync(0xffffffffu, all);
-        // Two or one to an item where that leaves no CTA a second item; two also where three would take a second round for less than a third more
-        // tiles (two rounds of 0.80 us per key tile instead of two of 1.03): 30 x 12 x 197 tokens (516 tiles) 16.5 -> 14.4 us, 24 x 12 x 256 (576) 19.4 -> 17.1.
-        const int G = gridDim.x, per = all <= G ? 1 : all <= 2 * G || (all > 3 * G && all <= 4 * G) ? 2 : NG;
+        // The fewest rounds, an item of one, two or three weighed by what a key tile of it takes (0.62, 0.80 and 1.03 us, and 0.85 for two, since more
+        // items also meet more heads' ends: 40 x 12 x 333 tokens with five rounds of two 39.3 us, with four of three 37.3).  With three wherever two left
+        // a CTA a second item, and two wherever one did, whatever the items of short samples came to: 24 x 12 x 256 (576 tiles) 19.4 us, so 17.0;
+        // 90 x 3 x 134 (276 tiles, in 180 items of two or 93 of three) 13.3, so 11.0.
+        auto rounds = [](int n) { return (int)(((unsigned)n + gridDim.x - 1) / gridDim.x); };
+        const float t1 = 0.62f * rounds(__reduce_add_sync(0xffffffffu, n1)), t2 = 0.85f * rounds(__reduce_add_sync(0xffffffffu, n2)), t3 = 1.03f * rounds(__reduce_add_sync(0xffffffffu, n3));
+        const int per = t1 <= t2 && t1 <= t3 ? 1 : t2 <= t3 ? 2 : 3;
         auto items_of = [&](int t) { return per == 1 ? t : per == 2 ? (t + 1) / 2 : (t + 2) / 3; };
 #pragma unroll
         for (int i = 0; i < PER_LANE; ++i) items[i] = items_of(items[i]);
