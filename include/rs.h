@@ -91,7 +91,8 @@ RS_API int rs_linear_uses_tensor_cores(const rs_ctx* ctx, rs_dtype dtype, long l
  * out (dev): [B, N, H*head_dim] contiguous, same dtype.  No [N, N] buffer is
  * ever written to global memory.  scale == 0 selects 1/sqrt(head_dim).
  * Two tensor-core kernels serve bf16 (two or three 128-row query tiles per thread block): the one with
- * three, but for some batches of 113 to 128 tokens and at most two heads per SM (rs_attn_kernel_choice) and with a count per sample of at most 128 tokens, more than 256 samples, or at most two
+ * three, but for shapes that come to a round or two of pairs of query tiles over the SMs (rs_attn_kernel_choice),
+ * and with a count per sample those of at most 128 tokens, more than 256 samples, or at most two
  * query tiles per SM (rs_attn_ragged_kernel_choice).  The result for one shape is reproducible bit for
  * bit and does not depend on a sample's place in the batch; the rounding order may differ between shapes.
  * RS_ATTN_KERNEL=2 or =3 in the environment at rs_create pins one of them where it applies. */

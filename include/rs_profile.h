@@ -38,8 +38,9 @@ RS_API rs_status rs_wait_check(rs_ctx* ctx, int waits, void* stream);
 
 /* Which of the two tensor-core attention kernels runs B samples of H heads and N tokens on a GPU of sm_count SMs: 2 (two query tiles
  * per thread block) or 3 (three), 0 for arguments below 1 and shapes of about 2^31 query
- * tiles and more.  rs_attn_fwd takes 3 for every other shape but
- * some of 113 to 128 tokens and at most two heads per SM; rs_attn_fwd_ragged 3 for N > 128,
+ * tiles and more.  rs_attn_fwd takes 2 for some shapes of 113 to 128 tokens and at most two heads per SM, and for those of more
+ * than 512 tokens whose query tiles, in pairs within a head, fill one round of the SMs (more tiles than SMs) or two (more than three
+ * times as many) and whose keys 3 would not cut; else 3.  rs_attn_fwd_ragged takes 3 for N > 128,
  * B <= 256 and more than two query tiles per SM, else 2.  Host arithmetic only; needs no context and no GPU, and knows
  * nothing of RS_ATTN_KERNEL. */
 RS_API int rs_attn_kernel_choice(int sm_count, int B, int H, int N);

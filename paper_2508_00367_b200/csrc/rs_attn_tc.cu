@@ -544,6 +544,13 @@ int attn_tc_tiles(int sm_count, int B, int H, int N, bool counts) {
     // rows, is not hidden behind a third tile.  Two / three, us, 20 x 12 heads: x 112 6.7 / 6.6, x 120 6.6 / 7.0, x 128 6.4 / 7.2; of 128 tokens, whose one
     // key tile is whole here, already with a tile a CTA, 12 x 12 5.7 / 5.9 (x 120 5.9 / 5.8); 37 x 12 x 128 10.3 / 9.5, x 120 10.9 / 9.1.
     if (!counts && N > 112 && N <= BQ && tiles <= 2ll * sm_count && (N == BQ || tiles > sm_count)) return 2;
+    // A round or two of pairs, where the other kernel has a round of two tiles, or of three and one, and does not cut the keys: two of its tiles to a CTA
+    // take as long as a pair here, with twice the key tiles to wait for.  From 513 tokens on; below that what counts is how a last key tile fills
+    // (4 x 16 x 512 12.0 / 12.4, 12 x 12 x 192 8.5 / 8.0, 8 x 12 x 160 7.9 / 7.8).  Two / three, us: 1 x 12 x 2353 36.0 / 37.8, 1 x 16 x 2043 31.9 / 33.6, 1 x 12 x 1569
+    // 25.9 / 27.1, 2 x 12 x 1201 21.6 / 22.6, 4 x 12 x 638 13.9 / 14.9, 8 x 12 x 700 26.0 / 27.3, 30 x 3 x 750 27.4 / 28.2.
+    const long long pairs = (long long)B * H * (((N + BQ - 1) / BQ + 1) / 2);
+    if (!counts && N > 4 * BQ && ((tiles > sm_count && pairs <= sm_count) || (tiles > 3ll * sm_count && pairs <= 2ll * sm_count)) &&
+        !attn_tc3_cut((long long)B * H, N, sm_count)) return 2;
     if (!counts) return tiles < attn_tc3_max_tiles() ? 3 : 0;
     return B <= attn_tc3_max_samples() && N > BQ && tiles > 2ll * sm_count && tiles < attn_tc3_max_tiles() ? 3 : 2;
 }

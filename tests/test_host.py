@@ -241,6 +241,23 @@ def test_ex2_polynomial_and_its_ends():
     assert (ends[:3] == 0).all() and np.isnan(ends[3])
 
 
+def test_attention_kernel_choice_of_rounds_of_pairs():
+    """Shapes that come to one or two rounds of pairs of query tiles on 148 SMs, and shapes beside them: the faster kernel where both were timed."""
+    import paper_2508_00367_b200 as rs
+    measured = {  # (B, H, N): us with two tiles, with three
+        (1, 12, 2353): (36.0, 37.8), (1, 12, 1569): (25.9, 27.1), (1, 16, 2043): (31.9, 33.6), (2, 12, 1201): (21.6, 22.6), (2, 12, 785): (16.1, 16.7),
+        (4, 12, 638): (13.9, 14.9), (6, 3, 1033): (19.3, 19.9), (8, 12, 700): (26.0, 27.2), (6, 16, 736): (27.1, 27.7), (30, 3, 750): (27.4, 28.2),
+        (1, 12, 1671): (28.0, 26.5), (4, 3, 1878): (30.3, 29.0), (1, 12, 1515): (20.9, 15.0), (12, 12, 192): (8.5, 8.0), (30, 6, 371): (22.5, 18.8),
+        (3, 6, 3128): (85.0, 77.9), (4, 16, 872): (30.7, 29.3), (20, 3, 1147): (47.0, 36.0),
+    }
+    for (B, H, N), (two, three) in measured.items():
+        assert rs.attn_kernel_choice(148, B, H, N) == (2 if two < three else 3), (B, H, N)
+    # on both sides of the lines: 513 tokens, 148 tiles, 148 pairs, 444 tiles and no keys cut, 296 pairs
+    for shape, tiles in (((4, 10, 512), 3), ((4, 10, 513), 2), ((37, 1, 513), 2), ((49, 1, 513), 2), ((50, 1, 513), 3), ((74, 1, 700), 3), ((98, 1, 700), 2), ((99, 1, 700), 3)):
+        assert rs.attn_kernel_choice(148, *shape) == tiles, (shape, rs.attn_key_cut(148, *shape))
+        assert tiles == 3 or rs.attn_key_cut(148, *shape) == 0
+
+
 def test_attention_kernel_choice_is_the_rule_that_runs():
     """Which attention kernel runs a shape (two or three query tiles per thread block) on a B200 of 148 SMs: without counts the
     faster one at the shapes that both were timed at, with a count per sample the one of three where sorting the samples pays."""
