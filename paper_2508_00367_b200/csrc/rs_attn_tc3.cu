@@ -10,8 +10,9 @@
 // The softmax warps' loop over whole key tiles carries nothing else: no masks, no rescaling of O, no second form of the
 // exponentials.  A tile that needs any of these goes through a second, short piece of code (16 columns at a time from tensor
 // memory).  What a loop that long also carries is paid for at every tile and in instruction fetches (32 KB at full rate,
-// then a third of it): with masked and rescaling forms in the loop a key tile of three query tiles took 2000 to 2200 cycles, so 1750 to
-// 1850, of which 1250 are exponentials; 4 x 16 x 4097 369 -> 337 us, 16 x 12 x 1569 181 -> 160, 32 x 16 x 577 82.8 -> 72.3, 64 x 12 x 197 30.5 -> 24.1.
+// then a third of it): with masked and rescaling forms out of the loop 4 x 16 x 4097 369 -> 337 us, 16 x 12 x 1569 181 -> 160, 32 x 16 x 577 82.8 ->
+// 72.3, 64 x 12 x 197 30.5 -> 24.1 (339, 163, 78 and 25.9 with the maximum of the first 128 keys, see walk).  A key tile of three query tiles takes about 1980 cycles
+// (647 000 SM cycles by ncu for five items of 65, their ends included), of which 1250 are exponentials.
 // An item is three consecutive 128-row query tiles of one (sample, head), which share the K/V
 // tiles streamed through the TMA ring, or of consecutive (sample, head)s.
 // SPLIT: the weights go to the second product as a bf16 and the bf16 of what that left over, 16 bits of mantissa instead of 8,
