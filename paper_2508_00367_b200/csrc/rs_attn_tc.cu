@@ -552,6 +552,8 @@ int attn_tc_tiles(int sm_count, int B, int H, int N, bool counts) {
     if (!counts && N > 4 * BQ && ((tiles > sm_count && pairs <= sm_count) || (tiles > 3ll * sm_count && pairs <= 2ll * sm_count)) &&
         !attn_tc3_cut((long long)B * H, N, sm_count)) return 2;
     if (!counts) return tiles < attn_tc3_max_tiles() ? 3 : 0;
+    // (Up to two query tiles per head and three to four tiles per SM: with nearly full counts two rounds of pairs are shorter, with counts from a third of N
+    // the kernel of three is: 20 x 12 x 178 13.7 / 15.0 and 13.6 / 11.5, 24 x 12 x 197 14.3 / 15.5 and 13.9 / 12.3, 20 x 12 x 157 13.3 / 13.9 and 13.0 / 10.6.)
     return B <= attn_tc3_max_samples() && N > BQ && tiles > 2ll * sm_count && tiles < attn_tc3_max_tiles() ? 3 : 2;
 }
 
