@@ -191,11 +191,16 @@ __device__ __forceinline__ float exp_pass(uint32_t (&r)[BKV], uint32_t (&lo)[SPL
 }
 
 // CUT: there are items with the keys cut in three.  (Without, the loops carry nothing of them: 4 x 16 x 3073 205 -> 198 us.)
-template <bool SPLIT, bool RAGGED, bool CUT>
+// FIRST: there are query tiles that see more than 128 keys at once, whose running maximum starts from the first two key tiles (two_first).
+// (Without, a short sequence and one with all query tiles cut carry nothing of them: twelve blocks of one image, ViT-B, 477 -> 472 us, where every
+// launch fetches the kernel's instructions anew; and with it known, 4 x 16 x 4097 338.5 -> 335.4, 16 x 12 x 539 33.4 -> 32.6.)
+template <bool SPLIT, bool RAGGED, bool CUT, bool FIRST>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO, const Attn3Args args) {
     static_assert(!RAGGED || (!SPLIT && !CUT), "neither comes with a count per sample");
+    static_assert(!FIRST || !SPLIT, "weights of 16 bits");
+    constexpr bool WHOLE = !CUT || FIRST || SPLIT;       // (else all query tiles have their keys cut)
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + OFF_BAR);
@@ -619,14 +624,14 @@ attn_tc3_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 tma_store_commit();
             }
         };
-        auto first_gap = [](int nkv) { return !SPLIT && nkv == 2 ? 0.f : kRescaleGap; };
-        auto two_first = [](int nkv) { return !SPLIT && nkv > 2; };
+        auto first_gap = [](int nkv) { return !SPLIT && (RAGGED || !FIRST) && nkv == 2 ? 0.f : kRescaleGap; };
+        auto two_first = [](int nkv) { return FIRST && (!RAGGED || nkv > 2); };
         // Whole key tiles.  The second of two counts as one with 64 keys: nearly all of them raise the maximum.
         auto whole_tiles = [](int n) { return !SPLIT && n <= 2 * BKV ? n >= BKV : n / BKV; };
         const int nkv_all = (args.N + BKV - 1) / BKV, nfull_all = whole_tiles(args.N), valid_all = args.N - nfull_all * BKV;
         const int whole = CUT ? args.n_whole : n_items;
         int w = blockIdx.x;
-        for (; w < whole; w += gridDim.x) {
+        for (; WHOLE && w < whole; w += gridDim.x) {
             const Item3 it = decode_item3<RAGGED, CUT>(args, samples, w);
             if (g >= it.ng) continue;
             const bool in_use = !RAGGED || (it.q + g - it.stream(g) * it.nt) * BQ + q * 32 + lane < it.n;
@@ -777,8 +782,9 @@ cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMa
     if (e != cudaSuccess) return e;
     e = (cudaError_t)attr_once.run(dev, [] {
         cudaError_t a = cudaSuccess;
-        for (const void* f : {(const void*)attn_tc3_kernel<false, false, false>, (const void*)attn_tc3_kernel<false, false, true>, (const void*)attn_tc3_kernel<false, true, false>,
-                              (const void*)attn_tc3_kernel<true, false, false>, (const void*)attn_tc3_kernel<true, false, true>})
+        for (const void* f : {(const void*)attn_tc3_kernel<false, false, false, false>, (const void*)attn_tc3_kernel<false, false, false, true>, (const void*)attn_tc3_kernel<false, false, true, false>,
+                              (const void*)attn_tc3_kernel<false, false, true, true>, (const void*)attn_tc3_kernel<false, true, false, true>, (const void*)attn_tc3_kernel<true, false, false, false>,
+                              (const void*)attn_tc3_kernel<true, false, true, false>})
             if (a == cudaSuccess) a = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
         return (int)a;
     });
@@ -810,9 +816,11 @@ cudaError_t launch_attn_tc3(rs_ctx* ctx, const rs_attn_desc& d, const CUtensorMa
     const long long most = lens ? BH * nt : args.n_items;
     const int grid = most < G ? (int)most : G;
     auto run = [&](auto kernel) { return launch_pdl(kernel, dim3(grid), dim3(kThreads), kSmem, st, tmQ, tmK, tmV, tmO, args); };
-    if (lens) return run(attn_tc3_kernel<false, true, false>);
-    if (split) return args.cut ? run(attn_tc3_kernel<true, false, true>) : run(attn_tc3_kernel<true, false, false>);
-    return args.cut ? run(attn_tc3_kernel<false, false, true>) : run(attn_tc3_kernel<false, false, false>);
+    if (lens) return run(attn_tc3_kernel<false, true, false, true>);
+    if (split) return args.cut ? run(attn_tc3_kernel<true, false, true, false>) : run(attn_tc3_kernel<true, false, false, false>);
+    // Short sequences, and those with all query tiles cut by keys, run without the code that only the others need.
+    if (args.cut) return args.nt ? run(attn_tc3_kernel<false, false, true, true>) : run(attn_tc3_kernel<false, false, true, false>);
+    return d.N > 2 * BKV ? run(attn_tc3_kernel<false, false, false, true>) : run(attn_tc3_kernel<false, false, false, false>);
 }
 
 }  // namespace rs
